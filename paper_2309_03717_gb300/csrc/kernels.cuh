@@ -524,7 +524,7 @@ __device__ __forceinline__ RefrGrad<T> refraction_grad(int kind, T R, T x, T E, 
     drho = T(-0.5) + x * (T(1) / T(3) + x * (T(-1) / T(8) + x * (T(1) / T(30))));
   } else if constexpr (std::is_same<T, float>::value) {
     // FP32 gradients: the approximate exponential and quotient (a few ulp)
-    const float em = __expf(-x);
+    const float em = exp_ap(-x);
     const float ix = __frcp_rn(x);
     rho = (1.0f - em) * ix;
     drho = (em - rho) * ix;

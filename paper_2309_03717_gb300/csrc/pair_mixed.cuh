@@ -386,8 +386,8 @@ struct OpsMixed {
     const int Jb = lin_cell(e.ub, N, sb);
     const float amp = t.amp;
     if (e.branch == 0) {
-      const float c0 = __fdividef(amp, e.f0.D * e.g0.R0) * (e.f0.invR * e.f0.invR);
-      const float c1 = __fdividef(-amp, e.f1.D * e.g1.R0) * (e.f1.invR * e.f1.invR);
+      const float c0 = div_ap(amp, e.f0.D * e.g0.R0) * (e.f0.invR * e.f0.invR);
+      const float c1 = div_ap(-amp, e.f1.D * e.g1.R0) * (e.f1.invR * e.f1.invR);
       if (Ja == Jb) {
         // both in one cell: add them in registers, two reductions
         const float a0 = c0 * (1.0f - sa), b0 = c1 * (1.0f - sb), a1 = c0 * sa, b1 = c1 * sb;
@@ -410,7 +410,7 @@ struct OpsMixed {
       if (Ja >= 0 && Ja < N) out.dep(Ja, -c * e.fm.V[0], -c * e.fm.V[1], -c * e.fm.V[2]);
       return;
     }
-    const float c = __fdividef(amp, e.fm.D * e.gm.R0) * i2;
+    const float c = div_ap(amp, e.fm.D * e.gm.R0) * i2;
     dep_lin(out, N, Ja, sa, c * e.fm.V[0], c * e.fm.V[1], c * e.fm.V[2]);
     dep_lin(out, N, Jb, sb, -c * e.fm.V[0], -c * e.fm.V[1], -c * e.fm.V[2]);
   }
@@ -430,8 +430,8 @@ struct OpsMixed {
     const bool ina = ka >= 0 && ka < N, inb = kb >= 0 && kb < N;
     const float amp = t.amp;
     if (e.branch == 0) {
-      const float c0 = __fdividef(amp, e.f0.D * e.g0.R0) * (e.f0.invR * e.f0.invR);
-      const float c1 = __fdividef(-amp, e.f1.D * e.g1.R0) * (e.f1.invR * e.f1.invR);
+      const float c0 = div_ap(amp, e.f0.D * e.g0.R0) * (e.f0.invR * e.f0.invR);
+      const float c1 = div_ap(-amp, e.f1.D * e.g1.R0) * (e.f1.invR * e.f1.invR);
       if (ina && inb && ka == kb) {
         // both deposits in one bin: add them in registers, one reduction
         out.dep(ka, c0 * e.f0.V[0] + c1 * e.f1.V[0], c0 * e.f0.V[1] + c1 * e.f1.V[1],
@@ -443,7 +443,7 @@ struct OpsMixed {
       return;
     }
     if (ka == kb) return;  // one bin (or both outside on one side): the bin average of E vanishes
-    const float c = __fdividef(amp, e.fm.D * e.gm.R0) * (e.fm.invR * e.fm.invR);
+    const float c = div_ap(amp, e.fm.D * e.gm.R0) * (e.fm.invR * e.fm.invR);
     if (ina) out.dep(ka, c * e.fm.V[0], c * e.fm.V[1], c * e.fm.V[2]);
     if (inb) out.dep(kb, -c * e.fm.V[0], -c * e.fm.V[1], -c * e.fm.V[2]);
   }
@@ -513,7 +513,7 @@ struct OpsMixed {
         dep_lin(out, N, Jlo, 0.5f * (slo + shi), Mx, My, Mz);
         return;
       }
-      const float invW = __fdividef(1.0f, 2.0f * hh);
+      const float invW = div_ap(1.0f, 2.0f * hh);
       const LinEnds z = lin_ends(Jlo, slo, Jhi, shi, invW);
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -527,7 +527,7 @@ struct OpsMixed {
     // bin: weight 1, M x 1 = M exactly) or the share it covers, in one
     // reduction either way, so that lanes of both kinds take one path
     const bool one = klo == khi;
-    const float invW = __fdividef(1.0f, 2.0f * hh);  // 1 / interval length in bins (unused when one)
+    const float invW = div_ap(1.0f, 2.0f * hh);  // 1 / interval length in bins (unused when one)
     const float wlo = one ? 1.0f : gap_to_next_edge(ulo, klo) * invW;
     if (klo >= 0 && klo < N && wlo > 0.0f) out.dep(klo, Mx * wlo, My * wlo, Mz * wlo);
     if (one) return;
@@ -579,8 +579,8 @@ struct OpsMixed {
       if (!(fminf(fabsf(f0.D), fabsf(f1.D)) >= M.eps_C)) return kDeferPair;
       const bool ina = ka >= 0, inb = kb >= 0;  // decided and inside the window
       const float amp = t.amp;
-      const float c0 = __fdividef(amp, f0.D * g0.R0) * (f0.invR * f0.invR);
-      const float c1 = __fdividef(-amp, f1.D * g1.R0) * (f1.invR * f1.invR);
+      const float c0 = div_ap(amp, f0.D * g0.R0) * (f0.invR * f0.invR);
+      const float c1 = div_ap(-amp, f1.D * g1.R0) * (f1.invR * f1.invR);
       // both deposits in one bin add in registers (one reduction); otherwise
       // one each.  One code path for both kinds of lane: the start's deposit
       // carries the end's when they share the bin (the end's weight 0 else)
@@ -631,7 +631,7 @@ struct OpsMixed {
       g.s[2] = 0.5f * __fadd_rn(a0z, a1z);
       const float rho2 = __fmaf_rn(g.s[0], g.s[0], __fmul_rn(g.s[1], g.s[1]));
       const float S = __fmaf_rn(g.s[2], g.s[2], rho2);
-      g.y = rsqrtf(S);
+      g.y = rsqrt_ap(S);
       g.R0 = __fmul_rn(S, g.y);
       g.R1 = 0.0f;
       if (g.R0 == 0.0f) return true;  // the midpoint on the antenna: no deposit
@@ -708,7 +708,7 @@ struct OpsMixed {
       float fr;
       const int k = bin_raw(ua, N, fr);
       if (k < 0 || k >= N) return;
-      const float c = __fdividef(j ? -amp : amp, f.D * g.R0) * (f.invR * f.invR);
+      const float c = div_ap(j ? -amp : amp, f.D * g.R0) * (f.invR * f.invR);
       out.dep(k, c * f.V[0], c * f.V[1], c * f.V[2]);
     }
   }
@@ -1001,7 +1001,7 @@ struct OpsMixed {
         gather_lin(G, N, Jlo, 0.5f * (slo + shi), S, sl);
         dLdu = Av[0] * sl[0] + Av[1] * sl[1] + Av[2] * sl[2];
       } else {
-        const float invW = __fdividef(1.0f, 2.0f * hh);
+        const float invW = div_ap(1.0f, 2.0f * hh);
         const LinEnds z = lin_ends(Jlo, slo, Jhi, shi, invW);
         float ix = 0.0f, iy = 0.0f, iz = 0.0f;  // G summed over the bins strictly between the ends
         const int kb = Jlo + 1 < 0 ? 0 : Jlo + 1;
@@ -1035,7 +1035,7 @@ struct OpsMixed {
       const bool one = klo == khi;
       const bool inlo = klo >= 0 && klo < N, inhi = !one && khi >= 0 && khi < N;
       if (one && !inlo) return;
-      const float invW = one ? 0.0f : __fdividef(1.0f, 2.0f * hh);
+      const float invW = one ? 0.0f : div_ap(1.0f, 2.0f * hh);
       const float4 glo = inlo ? G[klo] : make_float4(0.f, 0.f, 0.f, 0.f);
       const float4 ghi = inhi ? G[khi] : make_float4(0.f, 0.f, 0.f, 0.f);
       const float wlo = inlo ? (one ? 1.0f : gap_to_next_edge(ulo, klo) * invW) : 0.0f, whi = fhi * invW;
@@ -1064,7 +1064,7 @@ struct OpsMixed {
       dLdr[k] = -c * sb[k] - sbr * b[k];
     }
     const float dtau = t.dtauh;  // (t1 - t0)/dt
-    float dLd_dtau = __fdividef(AS, dtau);
+    float dLd_dtau = div_ap(AS, dtau);
     float dLdR = -AS * invR;
     // through h = |D| dtau / 2
     const float absD = aD.h;
@@ -1138,7 +1138,7 @@ struct OpsMixed {
         }
         tg[3 * j + 2] += dns * dNdz_fac * E;
         dn += dns * E;
-        const float cj = __fdividef(kap, f.D * g.R0) * (f.invR * f.invR);
+        const float cj = div_ap(kap, f.D * g.R0) * (f.invR * f.invR);
         const float dLdu = cj * (f.V[0] * sl[0] + f.V[1] * sl[1] + f.V[2] * sl[2]);
         arrival_grad(g, f.invR, E, M, dLdu, tg + 3 * j, nullptr, 1.0f, ga, dn);
         tg[6 + j] += dLdu * idt;
@@ -1188,7 +1188,7 @@ struct OpsMixed {
     dn += dns * t.Emh;
     // the slide of the two spread deposits +/- c V
     const float Dm = e.fm.D;
-    const float cm = __fdividef(amp, Dm * e.gm.R0) * (invR * invR);
+    const float cm = div_ap(amp, Dm * e.gm.R0) * (invR * invR);
     const float dLdua = cm * (e.fm.V[0] * sla[0] + e.fm.V[1] * sla[1] + e.fm.V[2] * sla[2]);
     const float dLdub = -cm * (e.fm.V[0] * slb[0] + e.fm.V[1] * slb[1] + e.fm.V[2] * slb[2]);
     const float dLdum = dLdua + dLdub;
