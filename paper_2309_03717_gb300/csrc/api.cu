@@ -177,8 +177,14 @@ struct c8r_ctx {
   double dt_ns = 0.0;
   std::vector<double> pos, t_start;
   AntRec* d_ants = nullptr;
-  void* d_acc = nullptr;     // accumulator [n_ant][n_bins][x, y, z, pad]
-  size_t acc_bytes = 0;
+  void* d_acc = nullptr;     // accumulator [copies][n_ant][rows][n_bins][x, y, z, pad]
+  size_t acc_bytes = 0;      // of all copies (shape.replicas of them)
+  // copies that may hold deposits (the first copies_used; the others are zero),
+  // which is what a fetch sums and a reset zeroes.  Work captured into a CUDA
+  // graph runs when the host does not see it: once anything was captured, every
+  // copy counts as used for good
+  int copies_used = 1;
+  bool copies_all = false;
   void* d_stage = nullptr;   // [n_ant][3][n_bins] staging for copies to host
   void* d_gbm = nullptr;     // backward: dL/dtraces, bin-major [n_ant][n_bins] accumulator elements
   PrefixFF* d_gpre = nullptr;  // backward (mixed ZHS): running sums of d_gbm over the bins, [n_ant][n_bins + 1]
@@ -219,6 +225,15 @@ int cuda_fail(c8r_ctx* c, cudaError_t e, const char* where) {
   return fail(c, C8R_ECUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
+// whether work enqueued on st runs later, from a graph (also when that cannot
+// be told)
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const bool plain = cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+  if (!plain) cudaGetLastError();
+  return !plain;
+}
+
 // the arrival form of the one-bin Endpoint kernels (MedParams::split), from the
 // ingest's votes of earlier pushes: the split form when at least half of the
 // tracks counted see the antenna array's centroid from above within 45
@@ -246,11 +261,7 @@ void form_poll(c8r_ctx* c) {
 void form_fetch(c8r_ctx* c, cudaStream_t st) {
   if (c->form_mode != C8R_FORM_AUTO || c->form_pending || !c->h_form || !c->ev_form || c->precision != C8R_MIXED)
     return;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return;
-  }
+  if (capturing(st)) return;
   if (cudaMemcpyAsync(c->h_form, c->d_kept + 1, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st) !=
           cudaSuccess ||
       cudaEventRecord(c->ev_form, st) != cudaSuccess) {
@@ -258,6 +269,20 @@ void form_fetch(c8r_ctx* c, cudaStream_t st) {
     return;
   }
   c->form_pending = true;
+}
+
+// copies of the accumulator that work enqueued on st has to reckon with
+int copies_in_use(c8r_ctx* c, cudaStream_t st) {
+  if (capturing(st)) c->copies_all = true;
+  return c->copies_all ? c->shape.replicas : c->copies_used;
+}
+
+// zero the accumulator
+cudaError_t zero_acc(c8r_ctx* c, cudaStream_t st) {
+  const int n = copies_in_use(c, st);
+  const cudaError_t e = cudaMemsetAsync(c->d_acc, 0, c->acc_bytes / c->shape.replicas * n, st);
+  if (e == cudaSuccess) c->copies_used = 1;
+  return e;
 }
 
 // a new antenna layout or medium: earlier votes no longer apply
@@ -502,6 +527,7 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
     c->t_start.assign(t_start, t_start + n_ant);
     cudaError_t e = cudaMemset(c->d_acc, 0, c->acc_bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "trace reset");
+    c->copies_used = 1;
     c->pushed = 0;
     cudaMemset(c->d_kept, 0, sizeof(unsigned long long));
     return rebuild_tables(c);
@@ -526,6 +552,8 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   c->acc_bytes = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(precision, formalism);
   c->shape.replicas = acc_replicas(precision, formalism, n_ant, n_bins, c->shape.a_tile, c->sm_count);
   c->acc_bytes *= c->shape.replicas;
+  c->copies_used = 1;
+  c->copies_all = false;
   cudaError_t e = dev_malloc(&c->d_ants, sizeof(AntRec) * n_ant);
   if (e == cudaSuccess) e = dev_malloc(&c->d_acc, c->acc_bytes);
   if (e == cudaSuccess) e = cudaMemset(c->d_acc, 0, c->acc_bytes);
@@ -580,6 +608,10 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
   if ((r = ensure_tiles(c, chunk)) != C8R_OK) return r;
   const bool lin = c->deposit == C8R_DEPOSIT_LINEAR;
   form_poll(c);
+  FwdShape shape = c->shape;  // of this push: with the accumulator copies it uses
+  shape.replicas = push_replicas(shape.replicas, n, c->n_bins);
+  if (capturing(st)) c->copies_all = true;
+  if (shape.replicas > c->copies_used) c->copies_used = shape.replicas;
   for (int64_t off = 0; off < n; off += chunk) {
     const int64_t m = (n - off) < chunk ? (n - off) : chunk;
     TrackPtrs p = offset_tracks(t, off);
@@ -598,9 +630,9 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
     M.wait_limit = current_wait_limit();
     e = (c->precision == C8R_FP64)
             ? launch_forward_f64(c->formalism, lin, c->d_tiles, n_tiles, c->d_ants, c->n_ant, M, c->d_acc,
-                                 c->shape, c->sm_count, c->d_err, st)
+                                 shape, c->sm_count, c->d_err, st)
             : launch_forward_mixed(c->formalism, lin, c->d_tiles, n_tiles, c->d_ants, c->n_ant, M, c->d_acc,
-                                   c->shape, c->sm_count, c->d_err, st);
+                                   shape, c->sm_count, c->d_err, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "forward launch");
     if (c->profiling) {
       cudaEventRecord(e2, st);
@@ -613,9 +645,19 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
   return C8R_OK;
 }
 
-static cudaError_t fetch_acc(c8r_ctx* c, void* dst, cudaStream_t st) {
-  return launch_acc_to_traces(c->precision, c->d_acc, c->n_ant, c->n_bins, acc_rows(c->precision, c->formalism), dst,
-                              0, st, c->shape.replicas);
+// the traces into dst, and the accumulator zeroed if `clear`: by the same kernel
+// while the accumulator is small (a launch fewer, which is what a small event
+// waits for), else by a memset, whose plain writes run faster than a kernel's
+// reads and writes in turn
+constexpr size_t kFusedClear = (size_t)4 << 20;
+static cudaError_t fetch_acc(c8r_ctx* c, void* dst, bool clear, cudaStream_t st) {
+  const int n = copies_in_use(c, st);
+  const bool fused = clear && c->acc_bytes / c->shape.replicas * n <= kFusedClear;
+  cudaError_t e = launch_acc_to_traces(c->precision, c->d_acc, c->n_ant, c->n_bins,
+                                       acc_rows(c->precision, c->formalism), dst, false, fused, st, n);
+  if (e == cudaSuccess && fused) c->copies_used = 1;
+  if (e == cudaSuccess && clear && !fused) e = zero_acc(c, st);
+  return e;
 }
 
 int c8r_fetch_traces(c8r_ctx* c, void* dst, int dst_is_device, int reset, void* stream) {
@@ -626,7 +668,7 @@ int c8r_fetch_traces(c8r_ctx* c, void* dst, int dst_is_device, int reset, void* 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
   if (dst_is_device) {
-    e = fetch_acc(c, dst, st);
+    e = fetch_acc(c, dst, reset != 0, st);
   } else {
     if (!c->d_stage) {
       e = dev_malloc(&c->d_stage, c->trace_bytes);
@@ -636,14 +678,11 @@ int c8r_fetch_traces(c8r_ctx* c, void* dst, int dst_is_device, int reset, void* 
         return fail(c, C8R_ENOMEM, "staging buffer for the host copy");
       }
     }
-    e = fetch_acc(c, c->d_stage, st);
+    e = fetch_acc(c, c->d_stage, false, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dst, c->d_stage, c->trace_bytes, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && reset) e = zero_acc(c, st);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "trace copy");
-  if (reset) {
-    e = cudaMemsetAsync(c->d_acc, 0, c->acc_bytes, st);
-    if (e != cudaSuccess) return cuda_fail(c, e, "trace reset");
-  }
   if (!dst_is_device) {
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(c, e, "stream synchronise");
@@ -656,7 +695,7 @@ int c8r_reset(c8r_ctx* c, void* stream) {
   if (!c->ants_set) return fail(c, C8R_ESTATE, "c8r_set_antennas has not been called");
   cudaSetDevice(c->device);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaMemsetAsync(c->d_acc, 0, c->acc_bytes, st);
+  cudaError_t e = zero_acc(c, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_kept, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return cuda_fail(c, e, "reset");
   c->pushed = 0;

@@ -379,7 +379,7 @@ int enqueue(c8r_batch* b, const TrackPtrs& tp, float* out, int n_items_limit, cu
   if (r != C8R_OK) return r;
   if (out) {
     cudaError_t e = launch_acc_to_traces(C8R_MIXED, b->d_acc, b->total_ant, b->M.n_bins,
-                                         acc_rows(C8R_MIXED, b->formalism), out, 1, st, b->replicas);
+                                         acc_rows(C8R_MIXED, b->formalism), out, true, false, st, b->replicas);
     if (e != cudaSuccess) return bfail(b, C8R_ECUDA, std::string("batch fetch: ") + cudaGetErrorString(e));
   }
   return C8R_OK;

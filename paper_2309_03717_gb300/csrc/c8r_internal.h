@@ -29,43 +29,53 @@ inline size_t acc_elem_bytes(int precision) { return precision == C8R_FP64 ? 32 
 inline int acc_rows(int precision, int formalism) { return precision == C8R_MIXED && formalism == C8R_ZHS ? 2 : 1; }
 // copies of the accumulator the forward kernel spreads its reductions over (CTA
 // range r adds into copy r % replicas; the fetch sums them).  Most reductions go
-// into the few bins per antenna that the pulse arrives in, and with many CTAs
-// on one antenna tile at a time those bins' L2 slices become the bottleneck.
-// The copies split each hot bin over several addresses.  Measured (pair-kernel
-// time): ZHS on a 160-antenna array (5 antenna tiles) 41 -> 34 ms with 2
-// copies, no better with 4; Endpoint there unchanged (issue-bound) and 2 %
-// slower with the linear deposit; on a 64-antenna array (2 tiles) Endpoint
-// 1.18 -> 0.97 ms with 2 (0.95 with 8), ZHS 1.10 -> 0.73 ms with 4, and with
-// the linear deposit Endpoint 2.68 -> 1.70 ms with 2.  So the count follows the
-// CTAs per antenna tile (resident CTAs / antenna tiles): about one copy per 200
-// for Endpoint and per 100 for ZHS, rounded down to a power of two, at most 8,
-// and only as many as fit the 48 MB of L2 the forward grid budgets for
-// accumulator rows (more would split the antenna tiles into more L2 blocks,
-// with more CTAs per tile again).
+// into the few bins per antenna that the pulse arrives in, and with many CTAs on
+// one antenna tile at a time those bins' addresses become the bottleneck: on 4e6
+// tracks of a vertical shower x 160 antennas the Endpoint kernel took 7.8 ms with
+// one copy, 5.7 / 5.48 / 5.49 with 2 / 4 / 8, and 5.4 with no reductions at all.
+// A copy costs its bytes once to zero and once to read per fetch, so few tracks
+// take few copies.  Measured (us per push and fetch, 4096 bins, 1 / 4 / 16
+// copies): Endpoint, 8 antennas, 1e6 tracks 646 / 224 / 152, 64 antennas 1123 /
+// 752 / 625, 160 antennas 1749 / 1412 / 1422, 512 antennas x 3e5 1303 / 1310 /
+// 1310; ZHS, 8 antennas 576 / 257 / 213, 160 antennas 1955 / 1552 / 1552 (the
+// budget allows 4); linear deposit, 64 antennas 2487 / 1612 / 1242.  With 3e4
+// tracks: Endpoint, 64 antennas 76 / 61 / 64, ZHS, 160 antennas 141 / 120 / 121.
+//
 // the batched launch: its many showers' antenna tiles spread the CTAs, so 2
 // copies for ZHS and 1 for Endpoint
 inline int acc_replicas(int precision, int formalism) { return acc_rows(precision, formalism) == 2 ? 2 : 1; }
-// a context: from its antenna count, bins and antenna tile
+// bytes of L2 that the accumulator rows in use at a time may take (forward_grid
+// groups the antenna tiles by it)
+constexpr size_t kAccL2Budget = (size_t)96 << 20;
+// the most copies a context uses (its accumulator is allocated for this many):
+// one per 29 resident CTAs of an antenna tile (6 CTAs per SM), at most 16 and
+// within the L2 budget, as a power of two.  29 is where the measurements above
+// part: 456 CTAs per tile (64 antennas) gain from 8 copies on, 182 (160
+// antennas) up to 4, 57 (512 antennas) not at all
 inline int acc_replicas(int precision, int formalism, int n_ant, int n_bins, int a_tile, int sm_count) {
   if (precision != C8R_MIXED) return 1;
   const int64_t ant_tiles = (n_ant + a_tile - 1) / a_tile;
-  const int64_t resident = (int64_t)sm_count * (formalism == C8R_ZHS ? 7 : 6);
-  const int64_t per_tile = resident / (ant_tiles > 0 ? ant_tiles : 1);
-  const int64_t per_copy = formalism == C8R_ZHS ? 100 : 200;
-  int64_t want = (per_tile + per_copy - 1) / per_copy;
+  const int64_t want = (int64_t)sm_count * 6 / (ant_tiles > 0 ? ant_tiles : 1) / 29;
   const size_t one = (size_t)n_ant * n_bins * 16 * acc_rows(precision, formalism);
-  const int64_t fit = (int64_t)(((size_t)48 << 20) / (one > 0 ? one : 1));
-  if (want > fit) want = fit;
-  if (want > 8) want = 8;
+  const int64_t fit = (int64_t)(kAccL2Budget / (one > 0 ? one : 1));
   int r = 1;
-  while (r * 2 <= want) r *= 2;  // a power of two
+  while (r < 16 && r * 2 <= want && r * 2 <= fit) r *= 2;
+  return r;
+}
+// the copies that a push of n tracks uses, of the `most` allocated: a track per
+// bin and copy at least, where the cost of a copy (about 32 bytes per bin and
+// antenna) falls below what it takes off the reductions of the tracks
+inline int push_replicas(int most, int64_t n, int n_bins) {
+  int r = 1;
+  while (r * 2 <= most && (int64_t)r * 2 * n_bins <= n) r *= 2;
   return r;
 }
 // accumulator [replicas][n_ant][rows][n_bins] -> traces [n_ant][3][n_bins]: the
 // copies are summed; with rows == 2 the second row (box edges) is integrated over
-// the bins and added; add != 0 adds into out.  FP32 only for add or replicas > 1
-cudaError_t launch_acc_to_traces(int precision, const void* acc, int n_ant, int n_bins, int rows, void* out, int add,
-                                 cudaStream_t st, int replicas = 1);
+// the bins and added; add adds into out; clear zeroes the accumulator (the copies
+// given) as it is read.  FP32 only for add or replicas > 1
+cudaError_t launch_acc_to_traces(int precision, void* acc, int n_ant, int n_bins, int rows, void* out, bool add,
+                                 bool clear, cudaStream_t st, int replicas = 1);
 
 // dL/dtraces [n_ant][3][n_bins] -> bin-major [n_ant][n_bins] accumulator elements
 cudaError_t launch_traces_to_bin_major(int precision, const void* g, int n_ant, int n_bins, void* out,

@@ -15,7 +15,7 @@
 // L2-resident accumulator [antenna][bin][x, y, z, 0] with one native vector
 // reduction (atomicAdd on float4; three FP64 reductions in the FP64 path); a
 // constant run of bins (ZHS) is added as its two edges into a second row that
-// the fetch integrates.  The mixed accumulator has 1 to 8 copies (CTA range r
+// the fetch integrates.  The mixed accumulator has 1 to 16 copies (CTA range r
 // adds into copy r % copies, acc_replicas) that the fetch sums.  Shared-memory
 // float atomics are not used: they stall the issuing warp, while the global
 // reductions are fire-and-forget.
@@ -395,14 +395,13 @@ inline int forward_threads(int a_tile) {
 // grid of the forward launch: about `waves` full waves of resident CTAs (a whole
 // number of them when the antenna tiles allow, so no wave runs part-empty);
 // antenna tiles grouped so that one block's accumulator rows take at most
-// l2_budget bytes
+// kAccL2Budget bytes
 inline int64_t forward_grid(FwdArgs& a, const FwdShape& shape, int resident, size_t acc_elem_bytes) {
   FwdGrid& g = a.g;
   g.ant_tiles = (a.n_ant + shape.a_tile - 1) / shape.a_tile;
-  const size_t l2_budget = (size_t)48 << 20;
   // an antenna tile's rows in every copy of the accumulator
   const size_t tile_bytes = (size_t)shape.a_tile * a.M.n_bins * acc_elem_bytes * (shape.replicas > 1 ? shape.replicas : 1);
-  int tpb = (int)(l2_budget / (tile_bytes > 0 ? tile_bytes : 1));
+  int tpb = (int)(kAccL2Budget / (tile_bytes > 0 ? tile_bytes : 1));
   g.tiles_per_block = tpb < 1 ? 1 : (tpb > g.ant_tiles ? g.ant_tiles : tpb);
   int64_t target = (int64_t)shape.waves * resident;
   int64_t ranges = (target + g.ant_tiles - 1) / g.ant_tiles;

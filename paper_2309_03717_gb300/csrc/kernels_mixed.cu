@@ -1,6 +1,8 @@
 // kernels_mixed.cu -- instantiation of the mixed-precision forward,
 // arrival-listing and adjoint kernels (FP32 field arithmetic, float-float
 // arrival times).
+#include <cooperative_groups.h>
+
 #include "pair_mixed.cuh"
 
 namespace c8r {
@@ -13,41 +15,56 @@ cudaError_t launch_forward_mixed(int formalism, bool lin, const void* tiles, int
 }
 
 // accumulator [n_ant][n_bins] float4 -> traces [n_ant][3][n_bins] (added or
-// stored); `replicas` copies of the accumulator, `stride` elements apart, are summed
-__global__ void k_acc_to_traces_f32(const float4* acc, int64_t n_ant_bins, int n_bins, float* out, int add,
-                                    int replicas, int64_t stride) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_ant_bins) return;
-  const int64_t a = i / n_bins;
-  const int k = (int)(i - a * n_bins);
-  float4 v = acc[i];
-  for (int r = 1; r < replicas; ++r) {
-    const float4 u = acc[i + r * stride];
-    v.x += u.x;
-    v.y += u.y;
-    v.z += u.z;
+// stored); `replicas` copies of the accumulator, `stride` elements apart, are
+// summed, and zeroed if `clear`.  Bound by DRAM for large arrays and by the
+// latency of its loads otherwise, so a thread has kFetchE bins (a block apart,
+// coalesced) in flight.
+constexpr int kFetchT = 256;
+constexpr int kFetchE = 4;
+__global__ void __launch_bounds__(kFetchT) k_acc_to_traces_f32(float4* acc, int64_t n_ant_bins, int n_bins, float* out,
+                                                               bool add, bool clear, int replicas, int64_t stride) {
+  const int64_t i0 = (int64_t)blockIdx.x * (kFetchT * kFetchE) + threadIdx.x;
+  const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  float4 v[kFetchE];
+#pragma unroll
+  for (int e = 0; e < kFetchE; ++e) v[e] = zero;
+#pragma unroll 2
+  for (int r = 0; r < replicas; ++r) {
+#pragma unroll
+    for (int e = 0; e < kFetchE; ++e) {
+      const int64_t i = i0 + e * kFetchT;
+      if (i < n_ant_bins) {
+        const float4 u = acc[i + r * stride];
+        v[e].x += u.x;
+        v[e].y += u.y;
+        v[e].z += u.z;
+      }
+    }
   }
-  float* o = out + a * 3 * n_bins + k;
-  if (add) {
-    o[0] += v.x;
-    o[n_bins] += v.y;
-    o[2 * n_bins] += v.z;
-  } else {
-    o[0] = v.x;
-    o[n_bins] = v.y;
-    o[2 * n_bins] = v.z;
+  if (clear)
+    for (int r = 0; r < replicas; ++r)
+#pragma unroll
+      for (int e = 0; e < kFetchE; ++e)
+        if (i0 + e * kFetchT < n_ant_bins) acc[i0 + e * kFetchT + r * stride] = zero;
+  float* o[kFetchE];
+  float4 w[kFetchE];
+#pragma unroll
+  for (int e = 0; e < kFetchE; ++e) {
+    const int64_t i = i0 + e * kFetchT;
+    const int64_t a = i / n_bins;
+    o[e] = out + a * 3 * n_bins + (i - a * n_bins);
+    w[e] = zero;
+    if (add && i < n_ant_bins) w[e] = make_float4(o[e][0], o[e][n_bins], o[e][2 * (int64_t)n_bins], 0.0f);
   }
+#pragma unroll
+  for (int e = 0; e < kFetchE; ++e)
+    if (i0 + e * kFetchT < n_ant_bins) {
+      o[e][0] = w[e].x + v[e].x;
+      o[e][n_bins] = w[e].y + v[e].y;
+      o[e][2 * (int64_t)n_bins] = w[e].z + v[e].z;
+    }
 }
 
-// accumulator with a row of box edges [n_ant][2][n_bins] float4 -> traces:
-// out[k] = direct[k] + sum_{j <= k} edge[j], each summed over the `replicas`
-// copies of the accumulator (`stride` elements apart).  One CTA per antenna
-// walks the bins in chunks of kScanT x kScanE, each thread kScanE consecutive
-// bins: the thread's total of the edges, an exclusive scan of the totals over
-// the CTA, then the running sum over the thread's bins from there, plus the
-// carry of the chunks before.  All sums in float-float on the FP32 pipe
-// (~2^-44 relative after 2^24 bins, far below the FP32 output); FP64 runs at
-// 1/64 of the FP32 rate on this part.
 constexpr int kScanT = 256;         // threads of the float-float scans
 constexpr int kScanE = 8;           // consecutive bins per thread and chunk
 
@@ -102,87 +119,188 @@ __device__ __forceinline__ void cta_exclusive_scan_ff3(const ff v[3], ff excl[3]
   }
 }
 
-// the edges of bin k summed over the accumulator copies, added to run[]
-__device__ __forceinline__ void add_edges(const float4* edge, int64_t k, int replicas, int64_t stride, ff run[3]) {
-  for (int r = 0; r < replicas; ++r) {
-    const float4 e = edge[k + r * stride];
-    run[0] = ff_add_f(run[0], e.x);
-    run[1] = ff_add_f(run[1], e.y);
-    run[2] = ff_add_f(run[2], e.z);
+// accumulator with a row of box edges [n_ant][2][n_bins] float4 -> traces:
+// out[k] = direct[k] + sum_{j <= k} edge[j], each summed over the `replicas`
+// copies of the accumulator (`stride` elements apart; zeroed if `clear`).  A
+// cluster of up to kFetchCluster CTAs has an antenna, each CTA kScanT x kFetchBins
+// consecutive bins and each thread kFetchBins of them, read once: the thread's
+// total of the edges, an exclusive scan over the CTA, the totals of the CTAs
+// before through distributed shared memory, then the running sum over the
+// thread's bins.  Longer windows take several rounds with a carry.  All sums in
+// float-float on the FP32 pipe (~2^-44 relative after 2^24 bins, far below the
+// FP32 output; FP64 runs at 1/64 of the FP32 rate on this part).  Bound by the
+// latency of its loads on small arrays.  Against one CTA per antenna that read
+// each bin twice: 4096 bins, 8 antennas with 8 copies 76 us, now 29 with 16;
+// 160 antennas with 2 copies 45 us, now 30 with 4; 512 antennas 58 -> 43 us; 1024
+// antennas x 8192 bins 200 -> 164 us.
+constexpr int kFetchBins = 4;
+constexpr int kFetchCluster = 8;
+static_assert(kScanT / 32 == 8 && kFetchCluster == 8, "sum_before8 takes eight totals");
+
+// From eight float-float totals of three components (t[c][q]), the sum of the
+// first `n` (before) and of all (tot), in every lane of the warp: lane 8c + q
+// takes one total and three shuffles add them
+__device__ __forceinline__ void sum_before8(const ff (*t)[8], int n, ff before[3], ff tot[3]) {
+  const int lane = threadIdx.x & 31, q = lane & 7;
+  ff all = lane < 24 ? t[lane >> 3][q] : ff{0.0f, 0.0f};
+  ff pre = q < n ? all : ff{0.0f, 0.0f};
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1) {
+    all = ff_sum(all, ff{__shfl_xor_sync(0xffffffffu, all.h, d), __shfl_xor_sync(0xffffffffu, all.l, d)});
+    pre = ff_sum(pre, ff{__shfl_xor_sync(0xffffffffu, pre.h, d), __shfl_xor_sync(0xffffffffu, pre.l, d)});
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    before[c] = ff{__shfl_sync(0xffffffffu, pre.h, 8 * c), __shfl_sync(0xffffffffu, pre.l, 8 * c)};
+    tot[c] = ff{__shfl_sync(0xffffffffu, all.h, 8 * c), __shfl_sync(0xffffffffu, all.l, 8 * c)};
   }
 }
 
-__global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(const float4* acc, int n_bins, float* out, int add,
-                                                               int replicas, int64_t stride) {
+__global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(float4* acc, int n_bins, float* out, bool add,
+                                                               bool clear, int replicas, int64_t stride) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), n_cta = (int)cluster.num_blocks();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   __shared__ ff warp_tot[3][kScanT / 32];
-  const int a = blockIdx.x;
-  const float4* direct = acc + (size_t)a * 2 * n_bins;
-  const float4* edge = direct + n_bins;
+  __shared__ ff cta_tot[2][3][kFetchCluster];  // the cluster's totals, of this round and the next
+  if (threadIdx.x < 6 * kFetchCluster) cta_tot[0][0][threadIdx.x] = ff{0.0f, 0.0f};  // absent CTAs count as zero
+  cluster.sync();
+  const int a = blockIdx.x / n_cta;
+  float4* direct = acc + (size_t)a * 2 * n_bins;
   float* o = out + (size_t)a * 3 * n_bins;
   ff carry[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
-  for (int base = 0; base < n_bins; base += kScanT * kScanE) {
-    const int k0 = base + threadIdx.x * kScanE;
-    const int k1 = min(k0 + kScanE, n_bins);
-    // this thread's total of the edges, and the edges before its bins
-    ff v[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
-    for (int k = k0; k < k1; ++k) add_edges(edge, k, replicas, stride, v);
-    ff excl[3], tot[3], run[3];
-    cta_exclusive_scan_ff3(v, excl, tot, warp_tot);
+  int buf = 0;
+  for (int64_t base = 0; base < n_bins; base += (int64_t)n_cta * kScanT * kFetchBins, buf ^= 1) {
+    const int64_t k0 = base + ((int64_t)rank * kScanT + threadIdx.x) * kFetchBins;
+    ff e[kFetchBins][3], d[kFetchBins][3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) run[c] = ff_sum(carry[c], excl[c]);
-    // the running sum over this thread's bins, plus the direct deposits
-    for (int k = k0; k < k1; ++k) {
-      add_edges(edge, k, replicas, stride, run);
-      ff d[3] = {run[0], run[1], run[2]};
-      for (int r = 0; r < replicas; ++r) {
-        const float4 u = direct[k + r * stride];
-        d[0] = ff_add_f(d[0], u.x);
-        d[1] = ff_add_f(d[1], u.y);
-        d[2] = ff_add_f(d[2], u.z);
-      }
+    for (int b = 0; b < kFetchBins; ++b)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float r = __fadd_rn(d[c].h, d[c].l);
-        if (add)
-          o[(size_t)c * n_bins + k] += r;
-        else
-          o[(size_t)c * n_bins + k] = r;
+      for (int c = 0; c < 3; ++c) e[b][c] = d[b][c] = ff{0.0f, 0.0f};
+#pragma unroll 2
+    for (int r = 0; r < replicas; ++r) {
+#pragma unroll
+      for (int b = 0; b < kFetchBins; ++b) {
+        if (k0 + b >= n_bins) continue;
+        const float4* p = direct + k0 + b + r * stride;
+        const float4 u = p[0], w = p[n_bins];
+        d[b][0] = ff_add_f(d[b][0], u.x);
+        d[b][1] = ff_add_f(d[b][1], u.y);
+        d[b][2] = ff_add_f(d[b][2], u.z);
+        e[b][0] = ff_add_f(e[b][0], w.x);
+        e[b][1] = ff_add_f(e[b][1], w.y);
+        e[b][2] = ff_add_f(e[b][2], w.z);
       }
     }
+    if (clear) {
+      const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      for (int r = 0; r < replicas; ++r)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) carry[c] = ff_sum(carry[c], tot[c]);
-    __syncthreads();  // warp_tot is rewritten by the next chunk
+        for (int b = 0; b < kFetchBins; ++b)
+          if (k0 + b < n_bins) direct[k0 + b + r * stride] = direct[n_bins + k0 + b + r * stride] = zero;
+    }
+    // the edges before this thread's bins: of the lanes before it, of the warps
+    // before its own, and of the CTAs before its own
+    ff lanes[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      ff inc = e[0][c];
+#pragma unroll
+      for (int b = 1; b < kFetchBins; ++b) inc = ff_sum(inc, e[b][c]);
+#pragma unroll
+      for (int s = 1; s < 32; s <<= 1) {
+        const ff u{__shfl_up_sync(0xffffffffu, inc.h, s), __shfl_up_sync(0xffffffffu, inc.l, s)};
+        if (lane >= s) inc = ff_sum(inc, u);
+      }
+      if (lane == 31) warp_tot[c][wid] = inc;
+      lanes[c] = ff{__shfl_up_sync(0xffffffffu, inc.h, 1), __shfl_up_sync(0xffffffffu, inc.l, 1)};
+      if (lane == 0) lanes[c] = ff{0.0f, 0.0f};
+    }
+    __syncthreads();
+    ff run[3], tot[3];
+    sum_before8(warp_tot, wid, run, tot);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) run[c] = ff_sum(run[c], lanes[c]);
+    if (n_cta > 1) {
+      // every CTA's totals to every CTA; two buffers, so that a round's totals
+      // are not overwritten before the slowest CTA has read them
+      if (threadIdx.x < n_cta) {
+        ff(*peer)[3][kFetchCluster] = cluster.map_shared_rank(cta_tot, threadIdx.x);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) peer[buf][c][rank] = tot[c];
+      }
+      cluster.sync();
+      ff before[3];
+      sum_before8(cta_tot[buf], rank, before, tot);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) run[c] = ff_sum(before[c], run[c]);
+    } else {
+      __syncthreads();  // warp_tot is rewritten by the next round
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      run[c] = ff_sum(carry[c], run[c]);
+      carry[c] = ff_sum(carry[c], tot[c]);
+    }
+#pragma unroll
+    for (int b = 0; b < kFetchBins; ++b) {
+      if (k0 + b >= n_bins) continue;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        run[c] = ff_sum(run[c], e[b][c]);
+        const ff s = ff_sum(run[c], d[b][c]);
+        const float x = __fadd_rn(s.h, s.l);
+        float* q = o + (size_t)c * n_bins + k0 + b;
+        *q = add ? *q + x : x;
+      }
+    }
   }
 }
 
-__global__ void k_acc_to_traces_f64(const Acc4D* acc, int64_t n_ant_bins, int n_bins, double* out) {
+__global__ void k_acc_to_traces_f64(Acc4D* acc, int64_t n_ant_bins, int n_bins, double* out, bool clear) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_ant_bins) return;
   const int64_t a = i / n_bins;
   const int k = (int)(i - a * n_bins);
   const Acc4D v = acc[i];
+  if (clear) acc[i] = Acc4D{0.0, 0.0, 0.0, 0.0};
   double* o = out + a * 3 * n_bins + k;
   o[0] = v.x;
   o[n_bins] = v.y;
   o[2 * n_bins] = v.z;
 }
 
-cudaError_t launch_acc_to_traces(int precision, const void* acc, int n_ant, int n_bins, int rows, void* out, int add,
-                                 cudaStream_t st, int replicas) {
+cudaError_t launch_acc_to_traces(int precision, void* acc, int n_ant, int n_bins, int rows, void* out, bool add,
+                                 bool clear, cudaStream_t st, int replicas) {
   const int64_t n = (int64_t)n_ant * n_bins;
   if (n <= 0) return cudaSuccess;
   const int64_t stride = n * rows;  // accumulator elements per copy
   if (rows == 2) {
-    k_acc_scan_to_traces<<<(unsigned)n_ant, kScanT, 0, st>>>(static_cast<const float4*>(acc), n_bins,
-                                                               static_cast<float*>(out), add, replicas, stride);
-    return cudaGetLastError();
+    // a cluster of CTAs per antenna, as many as one round over the window needs
+    int n_cta = 1;
+    while (n_cta < kFetchCluster && n_cta * kScanT * kFetchBins < n_bins) n_cta *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n_ant * n_cta);
+    cfg.blockDim = dim3(kScanT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = n_cta;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_acc_scan_to_traces, static_cast<float4*>(acc), n_bins, static_cast<float*>(out),
+                              add, clear, replicas, stride);
   }
-  const unsigned blocks = (unsigned)((n + 255) / 256);
-  if (precision == C8R_FP64)
-    k_acc_to_traces_f64<<<blocks, 256, 0, st>>>(static_cast<const Acc4D*>(acc), n, n_bins, static_cast<double*>(out));
-  else
-    k_acc_to_traces_f32<<<blocks, 256, 0, st>>>(static_cast<const float4*>(acc), n, n_bins, static_cast<float*>(out),
-                                                  add, replicas, stride);
+  if (precision == C8R_FP64) {
+    k_acc_to_traces_f64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(static_cast<Acc4D*>(acc), n, n_bins,
+                                                                    static_cast<double*>(out), clear);
+  } else {
+    constexpr int per = kFetchT * kFetchE;
+    k_acc_to_traces_f32<<<(unsigned)((n + per - 1) / per), kFetchT, 0, st>>>(
+        static_cast<float4*>(acc), n, n_bins, static_cast<float*>(out), add, clear, replicas, stride);
+  }
   return cudaGetLastError();
 }
 
