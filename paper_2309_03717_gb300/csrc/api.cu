@@ -83,6 +83,7 @@ void fill_medium(MedParams& M, int kind, double n_or_N0, double H, int n_bins, d
     split(n_or_N0 * H * kc, M.cN_h, M.cN_l);
     split(1.0 / H, M.invH_h, M.invH_l);
     M.N0f = (float)n_or_N0;
+    M.dz_series = (float)(-1.001e-3 * H);
     M.nf = 1.0f;
     M.R_E = earth_radius;
     M.RE_f = (float)earth_radius;

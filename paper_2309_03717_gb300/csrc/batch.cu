@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kTileT, Ops::kMinBlocks) k_batch(const BatchAr
   const MedParams& M = a.M;
   const FwdLayout L = fwd_layout(Ops::kPrec, a.a_tile, Ops::kDefers);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.bar_off);
-  AntRec* ant_s = reinterpret_cast<AntRec*>(smem + L.ant_off);
+  typename Ops::Ant* ant_s = reinterpret_cast<typename Ops::Ant*>(smem + L.ant_off);
   __shared__ int s_item;
   const int tid = threadIdx.x, nthr = blockDim.x;
   if (tid == 0) {
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kTileT, Ops::kMinBlocks) k_batch(const BatchAr
     const int idx = s_item;
     if (idx < 0 || idx >= a.n_items) break;
     const WorkItem w = a.items[idx];
-    for (int i = tid; i < w.n_here; i += nthr) ant_s[i] = a.ants[w.ant0 + i];
+    for (int i = tid; i < w.n_here; i += nthr) Ops::stage_ant(ant_s + i, a.ants[w.ant0 + i]);
     __syncthreads();
     float4* acc = a.acc + (size_t)(idx % a.replicas) * a.replica_stride + (size_t)w.ant0 * M.n_bins * Ops::kAccRows;
     if (!stream_range<Ops>(smem, L, bar, ant_s, acc, w.n_here,

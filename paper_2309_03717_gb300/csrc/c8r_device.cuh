@@ -11,6 +11,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <type_traits>
 
 #include "../../include/c8r.h"
 
@@ -105,6 +106,7 @@ struct MedParams {
   float nm1f;            // uniform: n - 1 formed in FP64, then rounded (never (1 + x) - 1 in FP32)
   float RE_f;            // spherical: Earth radius (m)
   float eps_C;           // near-Cherenkov threshold
+  float dz_series;       // exponential: -1.001e-3 H, the altitude difference from where the quotient's series may apply
   uint32_t wait_limit;   // polls of a bounded wait on a staged track tile before it gives up
   // the form of the FP32 arrival (Endpoint, one-bin deposit, plain media): the
   // centroid of the antenna array, which the ingest's count of tracks seen
@@ -152,6 +154,46 @@ __device__ __forceinline__ float exp_ap(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__fmul_rn(x, 1.44269504088896341f)));
   return r;
 }
+
+// ---------------------------------------------------------------------------
+// Two FP32 values at a time.  One add, multiply or fused multiply-add of a pair
+// (add/mul/fma.rn.f32x2) takes one issue slot and rounds each half as the plain
+// operation does; negations, absolute values and broadcast operands are free
+// (counted on this part), while the FP32 pipe's rate per value stays the same.
+// The pair kernels are bound by issue, so the per-pair arithmetic is written
+// once for T = float or float2 and the main passes run it on pairs: a pair's
+// two endpoints (Endpoint).  Comparisons and the approximate reciprocals take
+// each half apart.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float neg(float a) { return -a; }
+__device__ __forceinline__ float abs_of(float a) { return fabsf(a); }
+__device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 abs_of(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
+__device__ __forceinline__ float2 add_rn(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub_rn(float2 a, float2 b) { return __fadd2_rn(a, neg(b)); }
+__device__ __forceinline__ float2 mul_rn(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma_rn(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 rsqrt_ap(float2 x) { return make_float2(rsqrt_ap(x.x), rsqrt_ap(x.y)); }
+__device__ __forceinline__ float2 rcp_ap(float2 x) { return make_float2(rcp_ap(x.x), rcp_ap(x.y)); }
+__device__ __forceinline__ float2 div_ap(float2 a, float2 b) { return __fmul2_rn(a, rcp_ap(b)); }
+// a value in every half
+template <typename T>
+__device__ __forceinline__ T bc(float a);
+template <>
+__device__ __forceinline__ float bc<float>(float a) { return a; }
+template <>
+__device__ __forceinline__ float2 bc<float2>(float a) { return make_float2(a, a); }
+// Conditions that hold for nearly every pair (an emission point well above or
+// below the antenna, an antenna ahead of the track) pick between two forms in
+// the arithmetic below.  A plain value takes either; a float2 takes the usual
+// form in both halves, and the caller, which tests all the conditions of a pair
+// in one branch, redoes the rare pair half by half.
+template <typename T>
+constexpr bool kUsualForm = std::is_same<T, float2>::value;
 
 // ---------------------------------------------------------------------------
 // float-float ("double-float") arithmetic: error-free transformations after
@@ -438,11 +480,13 @@ __device__ __forceinline__ double arrival_f64(const MedParams& M, const GeoD& g,
 // ---------------------------------------------------------------------------
 // mixed path: FP32 field arithmetic; arrival time in float-float
 // ---------------------------------------------------------------------------
-struct GeoM {
-  float s[3], e[3];  // d = x_a - x_e as float-float per component
-  float R0, R1;      // |d| as float-float (R1 = 0 until geo_refine)
-  float y;           // ~1/R0 (rsqrt estimate)
+template <typename T>
+struct GeoT {
+  T s[3], e[3];  // d = x_a - x_e as float-float per component
+  T R0, R1;      // |d| as float-float (R1 = 0 until geo_refine)
+  T y;           // ~1/R0 (rsqrt estimate)
 };
+using GeoM = GeoT<float>;
 
 // d = a - p (p given as float-float; p_l = 0 for the FP32-exact endpoints) and
 // an FP32 estimate of R = |d| (enough for the Doppler factor and amplitudes)
@@ -730,16 +774,16 @@ constexpr int kFastUndecided = -2;  // an edge lies within the bound: the float-
 
 // d = a_h - p in FP32 (no low parts), rho^2 = d_x^2 + d_y^2, S = |d|^2 and
 // R0 = |d| as geo_lite forms them (the same s, y and R0 bit for bit)
-__device__ __forceinline__ void geo_fast(const AntRec& A, float px, float py, float pz, GeoM& g, float& S,
-                                         float& rho2) {
-  g.s[0] = __fadd_rn(A.xh, -px);
-  g.s[1] = __fadd_rn(A.yh, -py);
-  g.s[2] = __fadd_rn(A.zh, -pz);
-  rho2 = __fmaf_rn(g.s[0], g.s[0], __fmul_rn(g.s[1], g.s[1]));
-  S = __fmaf_rn(g.s[2], g.s[2], rho2);
+template <typename T>
+__device__ __forceinline__ void geo_fast(T ax, T ay, T az, T px, T py, T pz, GeoT<T>& g, T& S, T& rho2) {
+  g.s[0] = sub_rn(ax, px);
+  g.s[1] = sub_rn(ay, py);
+  g.s[2] = sub_rn(az, pz);
+  rho2 = fma_rn(g.s[0], g.s[0], mul_rn(g.s[1], g.s[1]));
+  S = fma_rn(g.s[2], g.s[2], rho2);
   g.y = rsqrt_ap(S);
-  g.R0 = __fmul_rn(S, g.y);
-  g.R1 = 0.0f;
+  g.R0 = mul_rn(S, g.y);
+  g.R1 = bc<T>(0.0f);
 }
 
 // T = tau + k z as float-float, the shifted time of arrival_fast, for a height
@@ -755,78 +799,94 @@ __device__ __forceinline__ void shifted_time(float tauh, float taul, float zh, f
   fast_two_sum(s, e2, Th, Tl);
 }
 
-// whether the split form of x pays for the emission point of g: within 45
-// degrees of the antenna's vertical and above it
-__device__ __forceinline__ bool split_pays(const GeoM& g, float S, float rho2) {
-  return g.s[2] < 0.0f && __fadd_rn(rho2, rho2) < S;
-}
-
 // the FP32 quotient (E_e - E_a)/dz of the refractivity term for the FP32
-// arrival (exponential medium): dz = s_z, the FP32 a_h - p of the emission
+// arrival (exponential medium); dz = s_z, the FP32 a_h - p of the emission
 // point (the same for every antenna of a flat array); for |dz/H| <= 1e-3 its
 // series (E_e/H)(1 + f)
-__device__ __forceinline__ float fast_quotient(const MedParams& M, float Eah, float Eal, float sz, float Eeh,
-                                               float Eel) {
-  const float x = __fmul_rn(sz, M.invH_h);
-  if (fabsf(x) > 1e-3f) return div_ap(__fadd_rn(__fsub_rn(Eeh, Eah), __fsub_rn(Eel, Eal)), sz);
-  const float f = __fmul_rn(x, __fmaf_rn(x, __fmaf_rn(x, -1.0f / 24.0f, 1.0f / 6.0f), -0.5f));
-  return __fmul_rn(__fmul_rn(Eeh, M.invH_h), __fadd_rn(1.0f, f));
+template <typename T>
+__device__ __forceinline__ T fast_quotient(const MedParams& M, T Eah, T Eal, T sz, T Eeh, T Eel) {
+  if constexpr (!kUsualForm<T>) {
+    const float x = __fmul_rn(sz, M.invH_h);
+    if (!(fabsf(x) > 1e-3f)) {
+      const float f = __fmul_rn(x, __fmaf_rn(x, __fmaf_rn(x, -1.0f / 24.0f, 1.0f / 6.0f), -0.5f));
+      return __fmul_rn(__fmul_rn(Eeh, M.invH_h), __fadd_rn(1.0f, f));
+    }
+  }
+  return div_ap(add_rn(sub_rn(Eeh, Eah), sub_rn(Eel, Eal)), sz);
 }
 
 // The FP32 arrival uf of the emission point of g (S = |d|^2, rho2 = d_x^2 +
-// d_y^2, T_e = Teh + Tel, qv the refractivity quotient of fast_quotient) and
-// its error bound, returned; SPLIT picks the form of x; q_extra adds a term
+// d_y^2, T_e = Teh + Tel, the antenna's T_a = Tah + Tal and bound constants, qv
+// the refractivity quotient of fast_quotient) and its error bound, returned; SPLIT picks the form of x; q_extra adds a term
 // u * q_extra * k x for geometry whose d carries more than the one rounding of
 // a_h - p (the midpoint)
-template <int KIND, bool SPLIT>
-__device__ __forceinline__ float arrival_fast(const MedParams& M, const AntRec& A, const GeoM& g, float S, float rho2,
-                                              float Teh, float Tel, float qv, float q_extra, float& uf_out) {
+template <int KIND, bool SPLIT, typename T>
+__device__ __forceinline__ T arrival_fast(const MedParams& M, const GeoT<T>& g, T S, T rho2, T Teh, T Tel, T Tah, T Tal,
+                                          float fb_abs, float fb_rel_v, T qv, float q_extra, T& uf_out) {
   static_assert(KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL, "plain straight-line media only");
   constexpr float u = 5.9604644775390625e-8f;  // 2^-24
   // R' = sqrt(S) rounded once (the direct form), or the unrefined R0 (the
   // split form, whose x is small: R enters it only through its denominator)
-  float R;
-  if constexpr (SPLIT) {
-    R = g.R0;
-  } else {
-    const float r = __fmaf_rn(-g.R0, g.R0, S);
-    R = __fmaf_rn(r, __fmul_rn(0.5f, g.y), g.R0);
-  }
+  T R = g.R0;
+  if constexpr (!SPLIT) R = fma_rn(fma_rn(neg(g.R0), g.R0, S), mul_rn(bc<T>(0.5f), g.y), g.R0);
   // x = R - w, w = z_e - z_a = -s_z
-  const float sz = g.s[2];
-  float x;
+  const T sz = g.s[2];
+  T x;
   if constexpr (SPLIT) {
-    x = sz < 0.0f ? div_ap(rho2, __fsub_rn(R, sz)) : __fadd_rn(R, sz);
+    x = div_ap(rho2, sub_rn(R, sz));
+    if constexpr (!kUsualForm<T>) x = sz < 0.0f ? x : __fadd_rn(R, sz);
   } else {
-    x = __fadd_rn(R, sz);
+    x = add_rn(R, sz);
   }
   const float kh = KIND == C8R_UNIFORM ? M.s_h : M.kc_h;
-  const float q = __fmul_rn(x, kh);
-  const float Td = __fadd_rn(__fsub_rn(Teh, A.Tah), __fsub_rn(Tel, A.Tal));
-  float v = 0.0f;
-  if constexpr (KIND == C8R_EXPONENTIAL) v = __fmul_rn(__fmul_rn(qv, R), M.cN_h);
-  const float uf = __fadd_rn(__fadd_rn(Td, q), v);
+  const T q = mul_rn(x, bc<T>(kh));
+  const T Td = add_rn(sub_rn(Teh, Tah), sub_rn(Tel, Tal));
+  T v = bc<T>(0.0f);
+  if constexpr (KIND == C8R_EXPONENTIAL) v = mul_rn(mul_rn(qv, R), bc<T>(M.cN_h));
+  const T uf = add_rn(add_rn(Td, q), v);
   uf_out = uf;
-  const float tail = __fmaf_rn(2.25f * u, fabsf(Td),
-                               __fmaf_rn(__fmaf_rn(SPLIT ? 22.0f : 17.0f, u, A.fb_rel_v), fabsf(v),
-                                         __fmaf_rn(3.25f * u, fabsf(uf), A.fb_abs)));
+  const T tail = fma_rn(bc<T>(2.25f * u), abs_of(Td),
+                        fma_rn(bc<T>(__fmaf_rn(SPLIT ? 22.0f : 17.0f, u, fb_rel_v)), abs_of(v),
+                               fma_rn(bc<T>(3.25f * u), abs_of(uf), bc<T>(fb_abs))));
   if constexpr (SPLIT) {
-    return __fmaf_rn(__fmaf_rn(q_extra, u, 19.0f * u), q, tail);
+    return fma_rn(bc<T>(__fmaf_rn(q_extra, u, 19.0f * u)), q, tail);
   } else {
-    return __fmaf_rn(__fmaf_rn(q_extra, u, 6.25f * u), q, __fmaf_rn(__fmul_rn(2.5f * u, kh), R, tail));
+    return fma_rn(bc<T>(__fmaf_rn(q_extra, u, 6.25f * u)), q, fma_rn(bc<T>(__fmul_rn(2.5f * u, kh)), R, tail));
   }
 }
 
-template <int KIND, bool SPLIT>
-__device__ __forceinline__ int arrival_bin_fast(const MedParams& M, const AntRec& A, const GeoM& g, float S,
-                                                float rho2, float Teh, float Tel, float qv) {
-  float uf;
-  const float eps = arrival_fast<KIND, SPLIT>(M, A, g, S, rho2, Teh, Tel, qv, 0.0f, uf);
-  if (uf < -eps || __fsub_rn(uf, eps) >= (float)M.n_bins) return kFastOut;
+// The bin that an FP32 arrival uf, off by at most eps, decides: uf - eps and uf +
+// eps (rounded; the one u |uf| that the bound keeps for it) must fall in one bin
+// of the window, or both before or both after it.  Their floors come from a
+// downward-rounded addition of 1.5 x 2^23, whose low bits then hold them: exact
+// below 2^22, and above or below that range the sum still sorts after or before
+// the window (as it does for an infinity; a NaN sorts after it, and deposits
+// nothing in the float-float form either).  Windows of more than 2^22 bins take
+// floorf (XU-pipe operations, as the conversion to an integer is).
+constexpr int kMagicBinBits = 0x4B400000;  // 1.5 x 2^23
+constexpr int kMagicBins = 1 << 22;
+__device__ __forceinline__ int decide_bin(int lo, int hi, int n_bins) {
+  const int k = lo == hi ? lo - kMagicBinBits : kFastUndecided;
+  return (hi < kMagicBinBits || lo >= kMagicBinBits + n_bins) ? kFastOut : k;
+}
+__device__ __forceinline__ int decide_bin_wide(float uf, float eps, int n_bins) {
+  if (uf < -eps || __fsub_rn(uf, eps) >= (float)n_bins) return kFastOut;
   const float k = floorf(uf);
   const float fr = __fsub_rn(uf, k);
   if (!(fr > eps && fr < __fsub_rn(1.0f, eps))) return kFastUndecided;  // also NaN
   return (int)k;
+}
+// the bins of a pair's two endpoints
+__device__ __forceinline__ void decide_bins(float2 uf, float2 eps, int n_bins, int& ka, int& kb) {
+  if (n_bins <= kMagicBins) {
+    const float2 magic = make_float2(12582912.0f, 12582912.0f);
+    const float2 lo = __fadd2_rd(sub_rn(uf, eps), magic), hi = __fadd2_rd(add_rn(uf, eps), magic);
+    ka = decide_bin(__float_as_int(lo.x), __float_as_int(hi.x), n_bins);
+    kb = decide_bin(__float_as_int(lo.y), __float_as_int(hi.y), n_bins);
+  } else {
+    ka = decide_bin_wide(uf.x, eps.x, n_bins);
+    kb = decide_bin_wide(uf.y, eps.y, n_bins);
+  }
 }
 
 // distance k + 1 - u from a float-float arrival u in bin k to the bin's upper
@@ -847,43 +907,73 @@ __device__ __forceinline__ bool bin_of(ff u, int n_bins, int& k, float& frac) {
 // rhat x (rhat x beta), D = 1 - n beta.rhat in a cancellation-free form:
 //   D = (1 - n|beta|) + n |w|^2 / (R (|beta| R + beta.d))   when beta.d >= 0
 // (the second term is n|beta|(1 - cos theta)); the direct form otherwise.
-struct FieldM {
-  float V[3];  // rhat x (rhat x beta) times R^2  (i.e. d x w)
-  float D;
-  float invR;
-  float bd;    // beta . d
-  float w[3];  // d x beta
+template <typename T>
+struct FieldT {
+  T V[3];  // rhat x (rhat x beta) times R^2  (i.e. d x w)
+  T D;
+  T invR;
+  T bd;    // beta . d
+  T w[3];  // d x beta
 };
+using FieldM = FieldT<float>;
 // Every step uses explicit-rounding intrinsics so the forward and the adjoint
 // kernels, which inline this in different contexts, take identical branch
 // decisions.
-__device__ __forceinline__ void field_mixed(const GeoM& g, float bx, float by, float bz, float bmag, float om_nb,
-                                            float n, FieldM& f) {
-  const float sx = g.s[0], sy = g.s[1], sz = g.s[2];
+template <typename T>
+__device__ __forceinline__ void field_mixed(const GeoT<T>& g, T bx, T by, T bz, T bmag, T om_nb, T n, FieldT<T>& f) {
+  const T sx = g.s[0], sy = g.s[1], sz = g.s[2];
   // w = d x beta from the FP32 part of d (the low parts, ~2^-24 |d|, change D by
   // ~1e-7 relative even near the Cherenkov angle, below the FP32 field arithmetic)
-  const float wx = __fmaf_rn(sy, bz, -__fmul_rn(sz, by));
-  const float wy = __fmaf_rn(sz, bx, -__fmul_rn(sx, bz));
-  const float wz = __fmaf_rn(sx, by, -__fmul_rn(sy, bx));
-  const float bd = __fmaf_rn(bx, sx, __fmaf_rn(by, sy, __fmul_rn(bz, sz)));
-  const float R = g.R0;
-  const float invR = g.y;
-  if (bd >= 0.0f) {
-    const float w2 = __fmaf_rn(wx, wx, __fmaf_rn(wy, wy, __fmul_rn(wz, wz)));
-    const float den = __fmul_rn(R, __fmaf_rn(bmag, R, bd));
-    f.D = __fadd_rn(om_nb, div_ap(__fmul_rn(n, w2), den));
-  } else {
-    f.D = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(n, bd), invR));
-  }
+  const T wx = fma_rn(sy, bz, neg(mul_rn(sz, by)));
+  const T wy = fma_rn(sz, bx, neg(mul_rn(sx, bz)));
+  const T wz = fma_rn(sx, by, neg(mul_rn(sy, bx)));
+  const T bd = fma_rn(bx, sx, fma_rn(by, sy, mul_rn(bz, sz)));
+  const T R = g.R0;
+  const T invR = g.y;
+  const T w2 = fma_rn(wx, wx, fma_rn(wy, wy, mul_rn(wz, wz)));
+  const T den = mul_rn(R, fma_rn(bmag, R, bd));
+  f.D = add_rn(om_nb, div_ap(mul_rn(n, w2), den));
+  if constexpr (!kUsualForm<T>)
+    if (!(bd >= 0.0f)) f.D = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(n, bd), invR));
   // d x w = d (d.beta) - beta R^2  ->  V R^2
-  f.V[0] = __fmaf_rn(sy, wz, -__fmul_rn(sz, wy));
-  f.V[1] = __fmaf_rn(sz, wx, -__fmul_rn(sx, wz));
-  f.V[2] = __fmaf_rn(sx, wy, -__fmul_rn(sy, wx));
+  f.V[0] = fma_rn(sy, wz, neg(mul_rn(sz, wy)));
+  f.V[1] = fma_rn(sz, wx, neg(mul_rn(sx, wz)));
+  f.V[2] = fma_rn(sx, wy, neg(mul_rn(sy, wx)));
   f.invR = invR;
   f.bd = bd;
   f.w[0] = wx;
   f.w[1] = wy;
   f.w[2] = wz;
+}
+
+// one half of a pair's geometry or field
+template <int J>
+__device__ __forceinline__ float half_of(float2 a) { return J == 0 ? a.x : a.y; }
+template <int J>
+__device__ __forceinline__ GeoM half_of(const GeoT<float2>& g) {
+  GeoM r;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    r.s[c] = half_of<J>(g.s[c]);
+    r.e[c] = half_of<J>(g.e[c]);
+  }
+  r.R0 = half_of<J>(g.R0);
+  r.R1 = half_of<J>(g.R1);
+  r.y = half_of<J>(g.y);
+  return r;
+}
+template <int J>
+__device__ __forceinline__ FieldM half_of(const FieldT<float2>& f) {
+  FieldM r;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    r.V[c] = half_of<J>(f.V[c]);
+    r.w[c] = half_of<J>(f.w[c]);
+  }
+  r.D = half_of<J>(f.D);
+  r.invR = half_of<J>(f.invR);
+  r.bd = half_of<J>(f.bd);
+  return r;
 }
 
 // D = 1 - n (beta . d)/R in float-float, for a refined geometry (R = R0 + R1)

@@ -208,6 +208,49 @@ struct ArrivalSink {
 // ---------------------------------------------------------------------------
 // forward
 // ---------------------------------------------------------------------------
+// What the main pass over one track sets aside, a bit per antenna of the tile:
+// whole pairs, and pairs with one or both endpoints undecided.  Almost every
+// warp holds a near-Cherenkov pair for every antenna, so appending to the queue
+// pair by pair ran its ~15 instructions for nearly each of them; a bit takes one.
+struct Aside {
+  uint32_t pair = 0, end0 = 0, end1 = 0;
+  __device__ __forceinline__ void add(int code, int ant) {
+    const uint32_t bit = 1u << ant;
+    if (code == kDeferPair) pair |= bit;
+    if (code & kDeferEnd0) end0 |= bit;
+    if (code & kDeferEnd1) end1 |= bit;
+  }
+};
+// The warp's set-aside pairs into the queue (track lane l): whole pairs from the
+// front, pairs with set-aside endpoints from the back; one shared-memory atomic
+// per warp and list reserves the places.  All lanes of the warp must call it.
+__device__ __forceinline__ void queue_aside(const Aside& s, int l, uint16_t* queue, int q_cap, int* q_cnt,
+                                            int* q_back) {
+  const int lane = threadIdx.x & 31;
+  uint32_t ends = s.end0 | s.end1, pairs = s.pair;
+  const int mine = __popc(pairs) | (__popc(ends) << 16);
+  int before = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, before, d);
+    if (lane >= d) before += v;
+  }
+  int base0 = 0, base1 = 0;
+  if (lane == 31) {
+    base0 = atomicAdd(q_cnt, before & 0xffff);
+    if (before >> 16) base1 = atomicAdd(q_back, before >> 16);
+  }
+  before -= mine;
+  int k = __shfl_sync(0xffffffffu, base0, 31) + (before & 0xffff);
+  int b = __shfl_sync(0xffffffffu, base1, 31) + (before >> 16);
+  for (; pairs; pairs &= pairs - 1) queue[k++] = (uint16_t)(l | ((__ffs(pairs) - 1) << 7));
+  for (; ends; ends &= ends - 1) {
+    const int ant = __ffs(ends) - 1;
+    const int code = ((s.end0 >> ant) & 1) * kDeferEnd0 | ((s.end1 >> ant) & 1) * kDeferEnd1;
+    queue[q_cap - 1 - b++] = (uint16_t)(l | (ant << 7) | (code << 10));
+  }
+}
+
 // Stream derived-track tiles [t_begin, t_end) through the two-slot TMA ring and
 // evaluate every (track, antenna) pair of the n_here antennas in ant_s, adding
 // deposits into the accumulator rows starting at acc_row0 (the row of ant_s[0]).
@@ -215,7 +258,7 @@ struct ArrivalSink {
 // mbarrier phase) and is advanced.  Returns false if a bounded wait gave up; the
 // CTA then has no copy in flight and must stop.
 template <class Ops>
-__device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* bar, const AntRec* ant_s,
+__device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* bar, const typename Ops::Ant* ant_s,
                              typename AccOf<typename Ops::acc_t>::type* acc_row0, int n_here,
                              const unsigned char* src, int64_t t_begin, int64_t t_end, int64_t& it,
                              const MedParams& M) {
@@ -252,24 +295,22 @@ __device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* 
   for (int64_t t = t_begin; t < t_end; ++t, ++it) {
     const int st = (int)(it & 1);
     const uint32_t parity = (uint32_t)((it >> 1) & 1);
-    const bool ok = mbar_wait_bounded(&bar[st], parity, M.wait_limit);
+    // one outcome for the warp: queue_aside's shuffles want every lane
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[st], parity, M.wait_limit));
     if (ok) {
       // one track per thread, held in registers, against every antenna of the tile
       for (int l = tid; l < kTileT; l += nthr) {
-        typename Ops::Track tr;
-        Ops::load(smem + st * L.stage_bytes, l, M, tr);
-        if (!Ops::live(tr)) continue;
+        typename Ops::MainTrack tr;
+        Ops::load_main(smem + st * L.stage_bytes, l, M, tr);
+        Aside aside;
+        if (Ops::live(tr))
 #pragma unroll 1
-        for (int ant = 0; ant < n_here; ++ant) {
-          GlobalSink<acc_t> sink{acc_row0 + (size_t)ant * row_stride, N};
-          const int code = Ops::pair_main(tr, Ops::load_ant(ant_s + ant), M, sink);
-          if constexpr (Ops::kDefers) {
-            if (code == kDeferPair)
-              queue[atomicAdd(&q_cnt[st], 1)] = (uint16_t)(l | (ant << 7));
-            else if (code != kDeferNone)
-              queue[L.q_cap - 1 - atomicAdd(&q_back[st], 1)] = (uint16_t)(l | (ant << 7) | (code << 10));
+          for (int ant = 0; ant < n_here; ++ant) {
+            GlobalSink<acc_t> sink{acc_row0 + (size_t)ant * row_stride, N};
+            const int code = Ops::pair_main(tr, ant_s + ant, M, sink);
+            if constexpr (Ops::kDefers) aside.add(code, ant);
           }
-        }
+        if constexpr (Ops::kDefers) queue_aside(aside, l, queue, L.q_cap, &q_cnt[st], &q_back[st]);
       }
     }
     if (__syncthreads_or(!ok)) {
@@ -361,7 +402,7 @@ __global__ void __launch_bounds__(kTileT, Ops::kMinBlocks) k_forward(const FwdAr
   extern __shared__ __align__(128) unsigned char smem[];
   const FwdLayout L = fwd_layout(Ops::kPrec, a.a_tile, Ops::kDefers);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.bar_off);
-  AntRec* ant_s = reinterpret_cast<AntRec*>(smem + L.ant_off);
+  typename Ops::Ant* ant_s = reinterpret_cast<typename Ops::Ant*>(smem + L.ant_off);
   int ant_tile;
   int64_t range;
   a.g.decode(blockIdx.x, ant_tile, range);
@@ -371,7 +412,7 @@ __global__ void __launch_bounds__(kTileT, Ops::kMinBlocks) k_forward(const FwdAr
   const int64_t t_end = min(t_begin + a.g.tiles_per_range, a.n_tiles);
   if (t_begin >= t_end || n_here <= 0) return;  // uniform over the CTA
   const int tid = threadIdx.x;
-  for (int i = tid; i < n_here; i += blockDim.x) ant_s[i] = a.ants[ant0 + i];
+  for (int i = tid; i < n_here; i += blockDim.x) Ops::stage_ant(ant_s + i, a.ants[ant0 + i]);
   if (tid == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -566,7 +607,7 @@ __global__ void __launch_bounds__(kTileT, Ops::kBwdMinBlocks) k_backward(const B
   const MedParams& M = a.M;
   const FwdLayout L = fwd_layout(Ops::kPrec, a.a_tile, Ops::kDefers);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.bar_off);
-  AntRec* ant_s = reinterpret_cast<AntRec*>(smem + L.ant_off);
+  typename Ops::Ant* ant_s = reinterpret_cast<typename Ops::Ant*>(smem + L.ant_off);
   uint16_t* queue = reinterpret_cast<uint16_t*>(smem + L.q_off);
   __shared__ acc_t sg[3 * kMaxATile + 1];  // antenna gradients of the tile, then dN0
   // set-aside work as in the forward kernel: whole pairs from the front of the
@@ -587,7 +628,7 @@ __global__ void __launch_bounds__(kTileT, Ops::kBwdMinBlocks) k_backward(const B
   const int N = M.n_bins;
   const acc4* G = static_cast<const acc4*>(a.G) + (size_t)ant0 * N;
   const PrefixFF* Gp = a.Gp ? a.Gp + (size_t)ant0 * (N + 1) : nullptr;
-  for (int i = tid; i < n_here; i += nthr) ant_s[i] = a.ants[ant0 + i];
+  for (int i = tid; i < n_here; i += nthr) Ops::stage_ant(ant_s + i, a.ants[ant0 + i]);
   for (int i = tid; i < 3 * n_here + 1; i += nthr) sg[i] = acc_t(0);
   const uint32_t bytes = (uint32_t)L.stage_bytes;
   const unsigned char* src = static_cast<const unsigned char*>(a.tiles);
@@ -613,30 +654,30 @@ __global__ void __launch_bounds__(kTileT, Ops::kBwdMinBlocks) k_backward(const B
     // every lane walks the antennas (dead slots included) so the warp reductions see all 32
     for (int l = tid; l < kTileT; l += nthr) {
       const int64_t i = t * kTileT + l;
-      typename Ops::Track tr;
-      Ops::load(stage, l, M, tr);
+      typename Ops::MainTrack tr;
+      Ops::load_main(stage, l, M, tr);
       const bool live = ok && i < a.n && Ops::live(tr);
-      acc_t tg[11];
-#pragma unroll
-      for (int k = 0; k < 11; ++k) tg[k] = acc_t(0);
+      typename Ops::MainGrad mg;
+      Ops::zero(mg);
+      Aside aside;
 #pragma unroll 1
       for (int ant = 0; ant < n_here; ++ant) {
         acc_t ga[3] = {0, 0, 0};
         const PrefixFF* Gp_a = Gp ? Gp + (size_t)ant * (N + 1) : nullptr;
         const int code =
-            live ? Ops::adj_main(tr, Ops::load_ant(ant_s + ant), M, G + (size_t)ant * N, Gp_a, tg, ga, dn_acc)
+            live ? Ops::adj_main(tr, ant_s + ant, M, G + (size_t)ant * N, Gp_a, mg, ga, dn_acc)
                  : kDeferNone;
-        if constexpr (Ops::kDefers) {
-          if (code == kDeferPair)
-            queue[atomicAdd(&q_cnt[st], 1)] = (uint16_t)(l | (ant << 7));
-          else if (code != kDeferNone)
-            queue[L.q_cap - 1 - atomicAdd(&q_back[st], 1)] = (uint16_t)(l | (ant << 7) | (code << 10));
-        }
+        if constexpr (Ops::kDefers) aside.add(code, ant);
         const int lane = tid & 31;
         const acc_t v = warp_sum3(ga[0], ga[1], ga[2], lane);  // x at lane 0, y at 8, z at 16
         if ((lane & 7) == 0 && lane < 24 && v != acc_t(0)) atomicAdd(&sg[3 * ant + (lane >> 3)], v);
       }
-      if (live) add_track_grads<acc_t>(a.out, i, tg);
+      if (live) {
+        acc_t tg[11];
+        Ops::collect(mg, tg);
+        add_track_grads<acc_t>(a.out, i, tg);
+      }
+      if constexpr (Ops::kDefers) queue_aside(aside, l, queue, L.q_cap, &q_cnt[st], &q_back[st]);
     }
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
@@ -746,13 +787,13 @@ cudaError_t launch_backward_ops(BwdArgs& a, const FwdShape& shape, int sm_count,
   auto k = k_backward<Ops>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kTileT, smem);
-  if (e != cudaSuccess) return e;
   FwdArgs f{a.tiles, a.n_tiles, a.ants, a.n_ant, a.a_tile, nullptr, a.err, FwdGrid{}, a.M};
   FwdShape one = shape;  // the L2 grouping covers one bin-major gradient, not the forward's accumulator copies
   one.replicas = 1;
-  const int64_t ctas = forward_grid(f, one, sm_count * (per_sm < 1 ? 1 : per_sm), sizeof(typename AccOf<typename Ops::acc_t>::type));
+  // (the antenna and N0 sums of a CTA are rounded over its track range, so the
+  // ranges follow a fixed count of resident CTAs, not what a build's registers give)
+  const int64_t ctas =
+      forward_grid(f, one, sm_count * Ops::kBwdGridBlocks, sizeof(typename AccOf<typename Ops::acc_t>::type));
   a.g = f.g;
   k<<<(unsigned)ctas, kTileT, smem, st>>>(a);
   return cudaGetLastError();

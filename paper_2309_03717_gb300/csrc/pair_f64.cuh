@@ -135,8 +135,11 @@ struct OpsF64 {
   static constexpr bool kDefers = FORM == C8R_ENDPOINT && !LIN;
   static constexpr bool kFastBins = false;
   static constexpr int kBwdMinBlocks = 2;
+  static constexpr int kBwdGridBlocks = 2;
   static constexpr int kAccRows = 1;      // no box deposits
 
+  using Ant = AntRec;
+  static __device__ __forceinline__ void stage_ant(AntRec* p, const AntRec& A) { *p = A; }
   static __device__ __forceinline__ AntRec load_ant(const AntRec* p) { return *p; }
 
   static __device__ __forceinline__ void load(const void* Tv, int l, const MedParams&, TrackD& t) {
@@ -145,6 +148,21 @@ struct OpsF64 {
     t.q = t.T[fd::Q * kTileT + l];
   }
   static __device__ __forceinline__ bool live(const TrackD& t) { return t.q != 0.0; }
+  using MainTrack = TrackD;
+  struct MainGrad {
+    double g[11];
+  };
+  static __device__ __forceinline__ void zero(MainGrad& m) {
+#pragma unroll
+    for (int k = 0; k < 11; ++k) m.g[k] = 0.0;
+  }
+  static __device__ __forceinline__ void collect(const MainGrad& m, double tg[11]) {
+#pragma unroll
+    for (int k = 0; k < 11; ++k) tg[k] = m.g[k];
+  }
+  static __device__ __forceinline__ void load_main(const void* Tv, int l, const MedParams& M, TrackD& t) {
+    load(Tv, l, M, t);
+  }
   template <class Sink>
   static __device__ __forceinline__ void pair(const TrackD& t, const AntRec& A, const MedParams& M, Sink& out) {
     if constexpr (FORM == C8R_ENDPOINT)
@@ -155,7 +173,8 @@ struct OpsF64 {
   // main pass: every pair but (kDefers) the near-Cherenkov ones, returned as
   // kDeferPair with nothing deposited; pair_deferred evaluates those in full
   template <class Sink>
-  static __device__ __forceinline__ int pair_main(const TrackD& t, const AntRec& A, const MedParams& M, Sink& out) {
+  static __device__ __forceinline__ int pair_main(const TrackD& t, const AntRec* p, const MedParams& M, Sink& out) {
+    const AntRec A = *p;
     if constexpr (kDefers) return endpoint(t.T, t.l, A, M, out, true);
     pair(t, A, M, out);
     return kDeferNone;
@@ -293,13 +312,14 @@ struct OpsF64 {
       zhs(T, l, A, M, out);
   }
 
-  static __device__ __forceinline__ int adj_main(const TrackD& tr, const AntRec& A, const MedParams& M,
-                                                 const Acc4D* G, const PrefixFF* Gp, double tg[11], double ga[3],
+  static __device__ __forceinline__ int adj_main(const TrackD& tr, const AntRec* p, const MedParams& M,
+                                                 const Acc4D* G, const PrefixFF* Gp, MainGrad& m, double ga[3],
                                                  double& dn) {
+    const AntRec A = *p;
     if constexpr (FORM == C8R_ZHS)
-      adj_zhs(tr, A, M, G, Gp, tg, ga, dn);
+      adj_zhs(tr, A, M, G, Gp, m.g, ga, dn);
     else
-      adj(tr, A, M, G, tg, ga, dn);
+      adj(tr, A, M, G, m.g, ga, dn);
     return kDeferNone;
   }
   static __device__ __forceinline__ void adj_deferred(const TrackD&, const AntRec&, const MedParams&, const Acc4D*,

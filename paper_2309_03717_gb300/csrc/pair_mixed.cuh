@@ -24,11 +24,9 @@ struct TrackM {
   float bx, by, bz, bmag;
   float amp;                     // q K/dt (Endpoint) or q K_A (t1-t0)/dt (ZHS); 0 = dropped
   float tau0h, tau0l, tau1h, tau1l, dtauh, dtaul;
-  float T0h, T0l, T1h, T1l;      // Endpoint, plain media: tau + k z at start and end (arrival_fast)
   // a flat antenna array (MedParams::flat, exponential medium): the quotient of
-  // the refractivity term, the same for every antenna, per track: FP32 at start
-  // and end (Endpoint, arrival_fast), float-float at the midpoint (ZHS)
-  float q0v, q1v, qmh, qml;
+  // the refractivity term at the midpoint, the same for every antenna
+  float qmh, qml;
   ZPart zm;                      // ZHS, flat array: the z part of the midpoint's d
   float E0h, E0l, E1h, E1l, Emh, Eml;
   float nm1_0, nm1_1, nm1_m;     // n - 1 at start, end, midpoint
@@ -49,12 +47,6 @@ __device__ __forceinline__ void load_track_mixed(const float* T, int l, const Me
   t.tau0h = TF(fm::TAU0H); t.tau0l = TF(fm::TAU0L);
   t.tau1h = TF(fm::TAU1H); t.tau1l = TF(fm::TAU1L);
   t.dtauh = TF(fm::DTAUH); t.dtaul = TF(fm::DTAUL);
-  if (FORM == C8R_ENDPOINT && (KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL)) {
-    // the shifted times of the FP32 arrival, once per track (k = n/(c dt) or 1/(c dt))
-    const float kh = KIND == C8R_UNIFORM ? M.s_h : M.kc_h, kl = KIND == C8R_UNIFORM ? M.s_l : M.kc_l;
-    shifted_time(t.tau0h, t.tau0l, t.z0, 0.0f, kh, kl, t.T0h, t.T0l);
-    shifted_time(t.tau1h, t.tau1l, t.z1, 0.0f, kh, kl, t.T1h, t.T1l);
-  }
   // n - 1 is formed directly (N0 E, or the uniform n - 1 rounded from FP64): as
   // (1 + x) - 1 in FP32 it would lose ~6e-8, comparable to D near Cherenkov
   t.E0h = t.E1h = t.Emh = 1.0f;
@@ -91,22 +83,68 @@ __device__ __forceinline__ void load_track_mixed(const float* T, int l, const Me
     two_sum(t.z0, t.z1, t.mz, t.mzl);
     t.mx *= 0.5f; t.mxl *= 0.5f; t.my *= 0.5f; t.myl *= 0.5f; t.mz *= 0.5f; t.mzl *= 0.5f;
   }
-  if constexpr (FLAT && KIND == C8R_EXPONENTIAL) {
+  if constexpr (FLAT && KIND == C8R_EXPONENTIAL && FORM == C8R_ZHS) {
     // the refractivity quotient against the array's altitude, formed as the
-    // per-pair arithmetic forms it (the altitude difference as geo_fast and
-    // geo_lite form it), so the values are the same
-    if constexpr (FORM == C8R_ENDPOINT) {
-      t.q0v = fast_quotient(M, M.flat_Eh, M.flat_El, __fadd_rn(M.flat_zh, -t.z0), t.E0h, t.E0l);
-      t.q1v = fast_quotient(M, M.flat_Eh, M.flat_El, __fadd_rn(M.flat_zh, -t.z1), t.E1h, t.E1l);
-    } else {
-      float dzh, dzl;
-      two_sum(M.flat_zh, -t.mz, dzh, dzl);
-      dzl = __fadd_rn(dzl, __fsub_rn(M.flat_zl, t.mzl));
-      refr_quotient(M, M.flat_Eh, M.flat_El, dzh, dzl, t.Emh, t.Eml, t.qmh, t.qml);
-      t.zm = z_part(dzh, dzl, t.bz);
-    }
+    // per-pair arithmetic forms it (the altitude difference as geo_lite forms
+    // it), so the values are the same
+    float dzh, dzl;
+    two_sum(M.flat_zh, -t.mz, dzh, dzl);
+    dzl = __fadd_rn(dzl, __fsub_rn(M.flat_zl, t.mzl));
+    refr_quotient(M, M.flat_Eh, M.flat_El, dzh, dzl, t.Emh, t.Eml, t.qmh, t.qml);
+    t.zm = z_part(dzh, dzl, t.bz);
   }
 }
+
+// a track for the main pass of the one-bin Endpoint kernels: its two endpoints
+// as pairs
+struct TrackE {
+  float2 x, y, z;        // FP32-exact endpoints
+  float2 Th, Tl;         // shifted times tau + k z (arrival_fast)
+  float2 Eh, El;         // exp(-z/H)
+  float2 q;              // flat antenna array: the refractivity quotient (MedParams::flat)
+  float2 om, n;          // 1 - n|beta|, n
+  float bx, by, bz, bmag;
+  float amp;             // q K/dt; 0 = dropped
+};
+
+template <int KIND, bool FLAT>
+__device__ __forceinline__ void load_track_endpoints(const float* T, int l, const MedParams& M, TrackE& t) {
+  t.amp = TF(fm::AMPE);
+  if (t.amp == 0.0f) return;  // filtered track or padding
+  t.x = make_float2(TF(fm::X0), TF(fm::X1));
+  t.y = make_float2(TF(fm::Y0), TF(fm::Y1));
+  t.z = make_float2(TF(fm::Z0), TF(fm::Z1));
+  t.bx = TF(fm::BX); t.by = TF(fm::BY); t.bz = TF(fm::BZ);
+  t.bmag = TF(fm::BMAG);
+  const float kh = KIND == C8R_UNIFORM ? M.s_h : M.kc_h, kl = KIND == C8R_UNIFORM ? M.s_l : M.kc_l;
+  shifted_time(TF(fm::TAU0H), TF(fm::TAU0L), t.z.x, 0.0f, kh, kl, t.Th.x, t.Tl.x);
+  shifted_time(TF(fm::TAU1H), TF(fm::TAU1L), t.z.y, 0.0f, kh, kl, t.Th.y, t.Tl.y);
+  float2 nm1 = bc<float2>(M.nm1f);
+  t.Eh = bc<float2>(1.0f);
+  if constexpr (KIND == C8R_EXPONENTIAL) {
+    t.Eh = make_float2(TF(fm::E0H), TF(fm::E1H));
+    t.El = make_float2(TF(fm::E0L), TF(fm::E1L));
+    nm1 = mul_rn(bc<float2>(M.N0f), t.Eh);
+  }
+  // 1 - n|beta| = (1 - |beta|) - (n - 1)|beta|
+  t.om = sub_rn(bc<float2>(TF(fm::OMB)), mul_rn(nm1, bc<float2>(t.bmag)));
+  t.n = add_rn(bc<float2>(1.0f), nm1);
+  // the quotient against the array's altitude, as the per-pair arithmetic forms
+  // it (the altitude difference as geo_fast forms it), so the same values
+  if constexpr (FLAT) {
+    t.q.x = fast_quotient(M, M.flat_Eh, M.flat_El, __fsub_rn(M.flat_zh, t.z.x), t.Eh.x, t.El.x);
+    t.q.y = fast_quotient(M, M.flat_Eh, M.flat_El, __fsub_rn(M.flat_zh, t.z.y), t.Eh.y, t.El.y);
+  }
+}
+
+// an antenna in shared memory for those kernels: what the main pass takes is
+// stored twice, as operands for pairs (four 16-byte loads), the rest follows
+struct alignas(16) AntE {
+  float2 x, y, z, Th, Tl, Eh, El;
+  float fb_abs, fb_rel_v;
+  float xl, yl, zl, tauh, taul, pad[3];
+};
+static_assert(sizeof(AntE) == sizeof(AntRec), "fwd_layout reckons with one antenna record size");
 
 // geometry shared by the forward and the adjoint Endpoint evaluation
 struct EndpointEvalM {
@@ -334,28 +372,62 @@ struct OpsMixed {
       FLAT && KIND == C8R_EXPONENTIAL && ((kFastBins && !SPLIT) || FORM == C8R_ZHS);
   // adjoint CTAs (128 threads) per SM the registers are set for (the linear
   // Endpoint adjoint carries the slide of each deposit as well)
-  static constexpr int kBwdMinBlocks = (LIN && FORM == C8R_ENDPOINT) ? 4 : 6;
+  static constexpr int kBwdMinBlocks = (LIN && FORM == C8R_ENDPOINT) ? 4 : (kFastBins ? 5 : 6);
+  // resident CTAs per SM that the adjoint's track ranges are cut for
+  static constexpr int kBwdGridBlocks = (LIN && FORM == C8R_ENDPOINT) ? 4 : 6;
   // ZHS: a second accumulator row holds the edges of box deposits
   static constexpr int kAccRows = FORM == C8R_ZHS ? 2 : 1;
 
-  // the float-float part of an antenna record, as three 16-byte shared-memory
-  // loads and one 8-byte load (the shifted time; loads whose fields a pass
-  // does not use are dropped by the compiler)
-  static __device__ __forceinline__ AntRec load_ant(const AntRec* p) {
-    const float4* f = reinterpret_cast<const float4*>(&p->xh);
-    const float4 a = f[0], b = f[1], c = f[2];
-    const float2 T = *reinterpret_cast<const float2*>(&p->Tah);
+  // the antenna record that the forward and adjoint kernels hold in shared memory
+  using Ant = std::conditional_t<kFastBins, AntE, AntRec>;
+  static __device__ __forceinline__ void stage_ant(Ant* p, const AntRec& A) {
+    if constexpr (kFastBins) {
+      AntE e;
+      e.x = bc<float2>(A.xh); e.y = bc<float2>(A.yh); e.z = bc<float2>(A.zh);
+      e.Th = bc<float2>(A.Tah); e.Tl = bc<float2>(A.Tal);
+      e.Eh = bc<float2>(A.Eah); e.El = bc<float2>(A.Eal);
+      e.fb_abs = A.fb_abs; e.fb_rel_v = A.fb_rel_v;
+      e.xl = A.xl; e.yl = A.yl; e.zl = A.zl; e.tauh = A.tauh; e.taul = A.taul;
+      e.pad[0] = e.pad[1] = e.pad[2] = 0.0f;
+      *p = e;
+    } else {
+      *p = A;
+    }
+  }
+  // the float-float part of an antenna record (loads whose fields a pass does
+  // not use are dropped by the compiler)
+  static __device__ __forceinline__ AntRec load_ant(const Ant* p) {
     AntRec r;
-    r.xh = a.x; r.yh = a.y; r.zh = a.z; r.xl = a.w;
-    r.yl = b.x; r.zl = b.y; r.tauh = b.z; r.taul = b.w;
-    r.Eah = c.x; r.Eal = c.y; r.fb_abs = c.z; r.fb_rel_v = c.w;
-    r.Tah = T.x; r.Tal = T.y;
+    if constexpr (kFastBins) {
+      r.xh = p->x.x; r.yh = p->y.x; r.zh = p->z.x;
+      r.xl = p->xl; r.yl = p->yl; r.zl = p->zl;
+      r.tauh = p->tauh; r.taul = p->taul;
+      r.Eah = p->Eh.x; r.Eal = p->El.x;
+      r.Tah = p->Th.x; r.Tal = p->Tl.x;
+      r.fb_abs = p->fb_abs; r.fb_rel_v = p->fb_rel_v;
+    } else {
+      // three 16-byte loads
+      const float4* f = reinterpret_cast<const float4*>(&p->xh);
+      const float4 a = f[0], b = f[1], c = f[2];
+      r.xh = a.x; r.yh = a.y; r.zh = a.z; r.xl = a.w;
+      r.yl = b.x; r.zl = b.y; r.tauh = b.z; r.taul = b.w;
+      r.Eah = c.x; r.Eal = c.y;
+    }
     return r;
   }
 
   static __device__ __forceinline__ void load(const void* Tv, int l, const MedParams& M, TrackM& t) {
     load_track_mixed<FORM, KIND, kFlat>(static_cast<const float*>(Tv), l, M, t);
   }
+  // the track as the main passes hold it
+  using MainTrack = std::conditional_t<kFastBins, TrackE, TrackM>;
+  static __device__ __forceinline__ void load_main(const void* Tv, int l, const MedParams& M, MainTrack& t) {
+    if constexpr (kFastBins)
+      load_track_endpoints<KIND, kFlat>(static_cast<const float*>(Tv), l, M, t);
+    else
+      load(Tv, l, M, t);
+  }
+  static __device__ __forceinline__ bool live(const TrackE& t) { return t.amp != 0.0f; }
   static __device__ __forceinline__ bool live(const TrackM& t) { return t.amp != 0.0f; }
 
   // -------------------------------------------------------------------------
@@ -542,21 +614,58 @@ struct OpsMixed {
     if (kb <= ke) out.dep_box(kb, ke, Mx * invW, My * invW, Mz * invW);
   }
 
-  // the bins of both endpoints from the FP32 arrival (kFastBins) in the form
-  // of x = R - w this kernel is compiled for
-  static __device__ __forceinline__ void fast_bins(const TrackM& t, const AntRec& A, const MedParams& M,
-                                                   const GeoM& g0, const GeoM& g1, float S0, float S1, float P0,
-                                                   float P1, int& ka, int& kb) {
-    float qa = 0.0f, qb = 0.0f;
-    if constexpr (kFlat) {
-      qa = t.q0v;
-      qb = t.q1v;
-    } else if constexpr (KIND == C8R_EXPONENTIAL) {
-      qa = fast_quotient(M, A.Eah, A.Eal, g0.s[2], t.E0h, t.E0l);
-      qb = fast_quotient(M, A.Eah, A.Eal, g1.s[2], t.E1h, t.E1l);
+  // one endpoint of a pair in which some condition of the usual forms fails: its
+  // arrival, bound and Doppler factor with each form chosen
+  template <int J>
+  static __device__ __forceinline__ void endpoint_rare(const TrackE& t, const AntE& A, const MedParams& M,
+                                                       const GeoT<float2>& g2, float2 S, float2 P, float& uf,
+                                                       float& eps, float& D) {
+    const GeoM g = half_of<J>(g2);
+    float q = 0.0f;
+    if constexpr (kFlat)
+      q = half_of<J>(t.q);
+    else if constexpr (KIND == C8R_EXPONENTIAL)
+      q = fast_quotient(M, A.Eh.x, A.El.x, g.s[2], half_of<J>(t.Eh), half_of<J>(t.El));
+    eps = arrival_fast<KIND, kSplit>(M, g, half_of<J>(S), half_of<J>(P), half_of<J>(t.Th), half_of<J>(t.Tl), A.Th.x,
+                                     A.Tl.x, A.fb_abs, A.fb_rel_v, q, 0.0f, uf);
+    FieldM f;
+    field_mixed(g, t.bx, t.by, t.bz, t.bmag, half_of<J>(t.om), half_of<J>(t.n), f);
+    D = f.D;
+  }
+
+  // the geometry, the field and the bins (arrival_fast in the form this kernel
+  // is compiled for) of a pair's two endpoints; true for a near-Cherenkov pair.
+  // Both endpoints at once (float2): 291 -> 187 thread instructions per pair with
+  // the set-aside bits (Aside).  Measured, ms: 4e6 tracks x 1024 antennas at 60
+  // degrees 40.3 -> 36.9, 64 uneven showers 3.30 -> 3.03, the adjoint on 1e6
+  // tracks x 64 antennas 1.23 -> 0.96 (5 CTAs per SM; 1.20 with 6, 1.11 with 4);
+  // a vertical shower x 160 antennas, 5.65 -> 5.3 to 5.5, is bound by its
+  // reductions (3.8 without them and the set-aside work)
+  static __device__ __forceinline__ bool endpoints_main(const TrackE& t, const AntE& A, const MedParams& M,
+                                                        GeoT<float2>& g, FieldT<float2>& f, int& ka, int& kb) {
+    float2 S, P, uf, q = bc<float2>(0.0f);
+    geo_fast(A.x, A.y, A.z, t.x, t.y, t.z, g, S, P);
+    if constexpr (kFlat)
+      q = t.q;
+    else if constexpr (KIND == C8R_EXPONENTIAL)
+      q = fast_quotient(M, A.Eh, A.El, g.s[2], t.Eh, t.El);
+    float2 eps = arrival_fast<KIND, kSplit>(M, g, S, P, t.Th, t.Tl, A.Th, A.Tl, A.fb_abs, A.fb_rel_v, q, 0.0f, uf);
+    field_mixed(g, bc<float2>(t.bx), bc<float2>(t.by), bc<float2>(t.bz), bc<float2>(t.bmag), t.om, t.n, f);
+    // the usual forms: bd >= 0 (the Doppler factor); an altitude difference
+    // beyond 1e-3 H, tested at 1.001e-3 H so that no rounding lets one through
+    // (the refractivity quotient); an emission point above the antenna (the
+    // split form)
+    bool usual = fminf(f.bd.x, f.bd.y) >= 0.0f;
+    if constexpr (kSplit)
+      usual = usual && fmaxf(g.s[2].x, g.s[2].y) < (KIND == C8R_EXPONENTIAL ? M.dz_series : 0.0f);
+    else if constexpr (KIND == C8R_EXPONENTIAL && !kFlat)
+      usual = usual && fminf(fabsf(g.s[2].x), fabsf(g.s[2].y)) > -M.dz_series;
+    if (!usual) {
+      endpoint_rare<0>(t, A, M, g, S, P, uf.x, eps.x, f.D.x);
+      endpoint_rare<1>(t, A, M, g, S, P, uf.y, eps.y, f.D.y);
     }
-    ka = arrival_bin_fast<KIND, kSplit>(M, A, g0, S0, P0, t.T0h, t.T0l, qa);
-    kb = arrival_bin_fast<KIND, kSplit>(M, A, g1, S1, P1, t.T1h, t.T1l, qb);
+    decide_bins(uf, eps, M.n_bins, ka, kb);
+    return !(fminf(fabsf(f.D.x), fabsf(f.D.y)) >= M.eps_C);
   }
 
   // main pass: every pair except (Endpoint) the near-Cherenkov ones, for which
@@ -564,34 +673,29 @@ struct OpsMixed {
   // whose bin the FP32 arrival leaves open, returned as kDeferEnd0/kDeferEnd1
   // bits after the other endpoint's deposit
   template <class Sink>
-  static __device__ __forceinline__ int pair_main(const TrackM& t, const AntRec& A, const MedParams& M, Sink& out) {
+  static __device__ __forceinline__ int pair_main(const MainTrack& t, const Ant* p, const MedParams& M, Sink& out) {
     if constexpr (kFastBins) {
-      GeoM g0, g1;
-      float S0, S1, P0, P1;
-      geo_fast(A, t.x0, t.y0, t.z0, g0, S0, P0);
-      geo_fast(A, t.x1, t.y1, t.z1, g1, S1, P1);
-      if (g0.R0 == 0.0f || g1.R0 == 0.0f) return kDeferNone;  // an emission point on the antenna
+      GeoT<float2> g;
+      FieldT<float2> f;
       int ka, kb;
-      fast_bins(t, A, M, g0, g1, S0, S1, P0, P1, ka, kb);
-      FieldM f0, f1;
-      field_mixed(g0, t.bx, t.by, t.bz, t.bmag, t.om0, __fadd_rn(1.0f, t.nm1_0), f0);
-      field_mixed(g1, t.bx, t.by, t.bz, t.bmag, t.om1, __fadd_rn(1.0f, t.nm1_1), f1);
-      if (!(fminf(fabsf(f0.D), fabsf(f1.D)) >= M.eps_C)) return kDeferPair;
-      const bool ina = ka >= 0, inb = kb >= 0;  // decided and inside the window
-      const float amp = t.amp;
-      const float c0 = div_ap(amp, f0.D * g0.R0) * (f0.invR * f0.invR);
-      const float c1 = div_ap(-amp, f1.D * g1.R0) * (f1.invR * f1.invR);
+      const bool near = endpoints_main(t, *p, M, g, f, ka, kb);
+      // decided and inside the window; no branch for near pairs, which almost
+      // every warp holds one of
+      const bool ina = ka >= 0 && !near, inb = kb >= 0 && !near;
+      const float2 c = mul_rn(div_ap(make_float2(t.amp, -t.amp), mul_rn(f.D, g.R0)), mul_rn(f.invR, f.invR));
       // both deposits in one bin add in registers (one reduction); otherwise
       // one each.  One code path for both kinds of lane: the start's deposit
       // carries the end's when they share the bin (the end's weight 0 else)
-      const bool same = ina && inb && ka == kb;
-      const float c1s = same ? c1 : 0.0f;
+      const bool same = ina && ka == kb;
+      const float c1s = same ? c.y : 0.0f;
+      const float2 dx = mul_rn(c, f.V[0]), dy = mul_rn(c, f.V[1]), dz = mul_rn(c, f.V[2]);
       if (ina)
-        out.dep(ka, __fmaf_rn(c1s, f1.V[0], c0 * f0.V[0]), __fmaf_rn(c1s, f1.V[1], c0 * f0.V[1]),
-                __fmaf_rn(c1s, f1.V[2], c0 * f0.V[2]));
-      if (inb && !same) out.dep(kb, c1 * f1.V[0], c1 * f1.V[1], c1 * f1.V[2]);
-      return (ka == kFastUndecided ? kDeferEnd0 : 0) | (kb == kFastUndecided ? kDeferEnd1 : 0);
+        out.dep(ka, __fmaf_rn(c1s, f.V[0].y, dx.x), __fmaf_rn(c1s, f.V[1].y, dy.x), __fmaf_rn(c1s, f.V[2].y, dz.x));
+      if (inb && !same) out.dep(kb, dx.y, dy.y, dz.y);
+      const int ends = (ka == kFastUndecided ? kDeferEnd0 : 0) | (kb == kFastUndecided ? kDeferEnd1 : 0);
+      return near ? kDeferPair : ends;
     } else if constexpr (FORM == C8R_ENDPOINT) {
+      const AntRec A = load_ant(p);
       EndpointEvalM e;
       if (!endpoint_fields<KIND>(t, A, M, e)) return kDeferNone;
       if (endpoint_near_cherenkov(e, M)) return kDeferPair;
@@ -599,7 +703,7 @@ struct OpsMixed {
       endpoint_deposit(t, e, M, out);
       return kDeferNone;
     } else {
-      zhs(t, A, M, out);
+      zhs(t, load_ant(p), M, out);
       return kDeferNone;
     }
   }
@@ -645,7 +749,7 @@ struct OpsMixed {
       }
       const float om = __fsub_rn(TF(fm::OMB), __fmul_rn(nm1, bmag));
       FieldM f;
-      field_mixed(g, bx, by, bz, bmag, om, __fadd_rn(1.0f, nm1), f);
+      field_mixed<float>(g, bx, by, bz, bmag, om, __fadd_rn(1.0f, nm1), f);
       // midpoint time (t0 + t1)/(2 dt), float-float, as load_track_mixed forms
       // it, shifted by k z_m at the exact midpoint height z_m = (z0 + z1)/2
       float tmh, tml;
@@ -659,10 +763,11 @@ struct OpsMixed {
       float Tmh, Tml;
       shifted_time(tmh, tml, 0.5f * zmh, 0.5f * zml, kh, kl, Tmh, Tml);
       float uf;
-      const float qv = KIND == C8R_EXPONENTIAL ? fast_quotient(M, A.Eah, A.Eal, g.s[2], Eh, El) : 0.0f;
+      const float qv = KIND == C8R_EXPONENTIAL ? fast_quotient<float>(M, A.Eah, A.Eal, g.s[2], Eh, El) : 0.0f;
       // the kernel's arrival form (either is exact to its own bound; one form
       // for every lane keeps the warp on one path)
-      const float eps_a = arrival_fast<KIND, kSplit>(M, A, g, S, rho2, Tmh, Tml, qv, 3.0f, uf);
+      const float eps_a =
+          arrival_fast<KIND, kSplit, float>(M, g, S, rho2, Tmh, Tml, A.Tah, A.Tal, A.fb_abs, A.fb_rel_v, qv, 3.0f, uf);
       const float eps_u = __fmaf_rn(2.0f * u * kh, L1, eps_a);
       const float dtau = TF(fm::DTAUH);
       const float aD = fabsf(f.D);
@@ -804,58 +909,110 @@ struct OpsMixed {
     dn += dLdopt * rg.dF_dN0;
   }
 
-  // chain rule of one one-bin Endpoint deposit (endpoint J, bin held fixed,
-  // dL/dtrace g4 at its bin) into the track gradients tg (positions of endpoint
-  // J, beta), the antenna gradient ga and dL/dN0
-  template <int J>
-  static __device__ __forceinline__ void adj_end(const GeoM& g, const FieldM& f, float nm1, float E, float kappa,
-                                                 const float4 g4, const MedParams& M, float tg[11], float ga[3],
-                                                 float& dn) {
-    const float dNdz_fac = (KIND == C8R_EXPONENTIAL) ? -M.N0f * M.invH_h : 0.0f;
-    const float gv[3] = {g4.x, g4.y, g4.z};
-    float dd[3], db[3], dns;
-    deposit_grad(g, f, 1.0f + nm1, gv, kappa, dd, db, dns);
+  // a track's gradients while its main pass runs: for the one-bin Endpoint
+  // kernels the positions of both endpoints as pairs, and beta with a sum per
+  // endpoint (the deposits do not depend on the times); otherwise the eleven
+  // gradients themselves
+  struct GradE {
+    float2 pos[3], beta[3];
+  };
+  struct GradPlain {
+    float g[11];
+  };
+  using MainGrad = std::conditional_t<kFastBins, GradE, GradPlain>;
+  static __device__ __forceinline__ void zero(MainGrad& m) {
+    if constexpr (kFastBins) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      tg[3 * J + c] -= dd[c];
-      ga[c] += dd[c];
-      tg[8 + c] += db[c];
+      for (int c = 0; c < 3; ++c) m.pos[c] = m.beta[c] = bc<float2>(0.0f);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 11; ++k) m.g[k] = 0.0f;
     }
-    tg[3 * J + 2] += dns * dNdz_fac * E;
-    dn += dns * E;
+  }
+  static __device__ __forceinline__ void collect(const MainGrad& m, float tg[11]) {
+    if constexpr (kFastBins) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        tg[c] = m.pos[c].x;
+        tg[3 + c] = m.pos[c].y;
+        tg[8 + c] = m.beta[c].x + m.beta[c].y;
+      }
+      tg[6] = tg[7] = 0.0f;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 11; ++k) tg[k] = m.g[k];
+    }
+  }
+
+  // chain rule of a pair's two one-bin Endpoint deposits +/- amp V/(D R) (bins
+  // held fixed, dL/dtrace ga and gb at them, zero for an endpoint without one):
+  // deposit_adjoint on both endpoints at once
+  static __device__ __forceinline__ void adj_ends(const GeoT<float2>& g, const FieldT<float2>& f, const TrackE& t,
+                                                  const float4 ga4, const float4 gb4, const MedParams& M, GradE& m,
+                                                  float ga[3], float& dn) {
+    const float2 G[3] = {make_float2(ga4.x, gb4.x), make_float2(ga4.y, gb4.y), make_float2(ga4.z, gb4.z)};
+    const float2 iR = f.invR, i2 = mul_rn(iR, iR), one = bc<float2>(1.0f);
+    // 1/D and 1/R with a Newton step, as good as rounded once: the approximate
+    // ones are off to one side by up to a bit, which the sums over all pairs
+    // would keep
+    float2 iD = rcp_ap(f.D), nR = iR;
+    iD = fma_rn(fma_rn(neg(f.D), iD, one), iD, iD);
+    nR = fma_rn(fma_rn(neg(g.R0), nR, one), nR, nR);
+    float2 rh[3], V[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      rh[k] = mul_rn(g.s[k], iR);
+      V[k] = mul_rn(f.V[k], i2);
+    }
+    const float2 c = mul_rn(f.bd, iR);
+    const float2 gV = fma_rn(G[2], V[2], fma_rn(G[0], V[0], mul_rn(G[1], V[1])));
+    const float2 rg = fma_rn(rh[2], G[2], fma_rn(rh[0], G[0], mul_rn(rh[1], G[1])));
+    const float2 f2 = mul_rn(mul_rn(make_float2(t.amp, -t.amp), iD), nR), f1 = mul_rn(f2, nR);
+    const float2 p = mul_rn(f2, fma_rn(mul_rn(gV, t.n), iD, rg)), q = neg(f2);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      // dl/dd = f1 x, x = c (g - rhat rg) - rg V - gV (n V/D + rhat); the order
+      // of these roundings is deposit_adjoint's as compiled, so that the two
+      // agree bit for bit (the set-aside pairs take that one)
+      const float2 x = fma_rn(neg(gV), fma_rn(mul_rn(t.n, V[k]), iD, rh[k]),
+                              fma_rn(c, fma_rn(neg(rh[k]), rg, G[k]), mul_rn(neg(rg), V[k])));
+      m.pos[k] = fma_rn(neg(f1), x, m.pos[k]);
+      ga[k] = __fmaf_rn(f1.y, x.y, __fmaf_rn(f1.x, x.x, ga[k]));
+      // dl/dbeta = f2 [(rg + gV n/D) rhat - g]
+      m.beta[k] = add_rn(m.beta[k], fma_rn(p, rh[k], mul_rn(q, G[k])));
+    }
+    const float2 dns = mul_rn(mul_rn(mul_rn(f2, gV), c), iD);  // dl/dn
+    if constexpr (KIND == C8R_EXPONENTIAL)
+      m.pos[2] = fma_rn(mul_rn(dns, bc<float2>(-M.N0f * M.invH_h)), t.Eh, m.pos[2]);
+    dn = __fmaf_rn(dns.y, t.Eh.y, __fmaf_rn(dns.x, t.Eh.x, dn));
   }
 
   // adjoint main pass: every pair except (Endpoint) the near-Cherenkov ones, for
   // which it adds nothing and returns kDeferPair, and (kFastBins) the endpoints
   // whose bin the FP32 arrival leaves open (kDeferEnd0/kDeferEnd1 bits), after
   // the other endpoint's part
-  static __device__ __forceinline__ int adj_main(const TrackM& t, const AntRec& A, const MedParams& M,
-                                                 const float4* G, const PrefixFF* Gp, float tg[11], float ga[3],
+  static __device__ __forceinline__ int adj_main(const MainTrack& t, const Ant* p, const MedParams& M,
+                                                 const float4* G, const PrefixFF* Gp, MainGrad& m, float ga[3],
                                                  float& dn) {
     if constexpr (FORM == C8R_ZHS) {
-      adj_zhs(t, A, M, G, Gp, tg, ga, dn);
+      adj_zhs(t, load_ant(p), M, G, Gp, m.g, ga, dn);
       return kDeferNone;
     } else if constexpr (kFastBins) {
-      GeoM g0, g1;
-      float S0, S1, P0, P1;
-      geo_fast(A, t.x0, t.y0, t.z0, g0, S0, P0);
-      geo_fast(A, t.x1, t.y1, t.z1, g1, S1, P1);
-      if (g0.R0 == 0.0f || g1.R0 == 0.0f) return kDeferNone;
-      FieldM f0, f1;
-      field_mixed(g0, t.bx, t.by, t.bz, t.bmag, t.om0, __fadd_rn(1.0f, t.nm1_0), f0);
-      field_mixed(g1, t.bx, t.by, t.bz, t.bmag, t.om1, __fadd_rn(1.0f, t.nm1_1), f1);
-      if (!(fminf(fabsf(f0.D), fabsf(f1.D)) >= M.eps_C)) return kDeferPair;
+      GeoT<float2> g;
+      FieldT<float2> f;
       int ka, kb;
-      fast_bins(t, A, M, g0, g1, S0, S1, P0, P1, ka, kb);
-      if (ka >= 0) adj_end<0>(g0, f0, t.nm1_0, t.E0h, t.amp, G[ka], M, tg, ga, dn);
-      if (kb >= 0) adj_end<1>(g1, f1, t.nm1_1, t.E1h, -t.amp, G[kb], M, tg, ga, dn);
+      if (endpoints_main(t, *p, M, g, f, ka, kb)) return kDeferPair;
+      const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      const float4 g0 = ka >= 0 ? G[ka] : zero, g1 = kb >= 0 ? G[kb] : zero;
+      if (ka >= 0 || kb >= 0) adj_ends(g, f, t, g0, g1, M, m, ga, dn);
       return (ka == kFastUndecided ? kDeferEnd0 : 0) | (kb == kFastUndecided ? kDeferEnd1 : 0);
     } else {
+      const AntRec A = load_ant(p);
       EndpointEvalM e;
       if (!endpoint_fields<KIND>(t, A, M, e)) return kDeferNone;
       if (endpoint_near_cherenkov(e, M)) return kDeferPair;
       endpoint_arrivals<KIND>(t, A, M, e);
-      adj_deposits(t, e, M, G, tg, ga, dn);
+      adj_deposits(t, e, M, G, m.g, ga, dn);
       return kDeferNone;
     }
   }

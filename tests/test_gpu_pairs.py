@@ -1,0 +1,70 @@
+"""The one-bin Endpoint kernels evaluate a pair's two endpoints together and
+redo the rare pair (an emission point near the antenna's altitude or below it,
+an antenna behind the track) half by half.  Antennas spread through the shower's
+own heights make those pairs common, next to usual ones; track counts around the
+128-track tile and antenna counts around the 32-antenna tile.  Traces and
+adjoint against the oracle at the mixed bar (1e-4 relative L2)."""
+import numpy as np
+import pytest
+
+import oracle
+from _util import built_lib, drop_tracks, oracle_arrivals, oracle_traces, rel_l2, to_device, unambiguous
+from paper_2309_03717_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+TOL = 1e-4
+UNIFORM = {"kind": "uniform", "n": 1.000292}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    built_lib()
+
+
+def among_the_tracks(n, n_ant, medium):
+    """A shower and n_ant antennas 60-460 m from its axis at heights from below to above its tracks."""
+    w = synth.workload(1, n_tracks=n + 60, n_ant=n_ant)
+    w["n_bins"], w["medium"] = 2048, medium or w["medium"]
+    tracks = synth.workload_tracks(w)
+    r = np.linspace(60.0, 460.0, n_ant)
+    a = 2.4 * np.arange(n_ant)
+    z = np.quantile(tracks["z0"], np.linspace(0.0, 1.0, n_ant + 2)[1:-1]).astype(np.float64)
+    w["ant_xyz"] = np.stack([r * np.cos(a), r * np.sin(a), z], 1)
+    zero = np.zeros(n_ant)
+    _, u0 = oracle_arrivals(tracks, w["ant_xyz"], zero, 1, w["dt_ns"], w["medium"], "endpoint")
+    w["t_start_ns"] = np.median(u0.reshape(n + 60, n_ant, 2)[..., 0], axis=0) * w["dt_ns"] - 200.0
+    keep = unambiguous(tracks, w["ant_xyz"], w["t_start_ns"], w["n_bins"], w["dt_ns"], w["medium"], "endpoint")
+    tracks = {f: x[:n] for f, x in drop_tracks(tracks, keep).items()}
+    assert len(tracks["x0"]) == n
+    return w, {f: np.ascontiguousarray(x) for f, x in tracks.items()}
+
+
+@pytest.mark.parametrize("form", ["split", "direct"])
+@pytest.mark.parametrize("medium", [None, UNIFORM])
+@pytest.mark.parametrize("n,n_ant", [(1, 1), (127, 31), (128, 32), (129, 33), (700, 5)])
+def test_traces_and_adjoint_with_antennas_among_the_tracks(n, n_ant, medium, form):
+    from paper_2309_03717_gb300 import c8r
+    w, tracks = among_the_tracks(n, n_ant, medium)
+    p = c8r.RadioProcess(w["medium"], w["ant_xyz"], w["t_start_ns"], w["n_bins"], w["dt_ns"], "endpoint", "mixed")
+    p.set_arrival_form(form)
+    dev = to_device(tracks)
+    p.push(dev)
+    ref, kept = oracle_traces(tracks, w["ant_xyz"], w["t_start_ns"], w["n_bins"], w["dt_ns"], w["medium"], "endpoint")
+    assert kept == n
+    assert rel_l2(p.traces().cpu().numpy(), ref) <= TOL
+    G = torch.from_numpy(np.random.default_rng(n).normal(size=ref.shape).astype(np.float32)).cuda()
+    tg = {f: torch.zeros(n, dtype=torch.float32, device="cuda") for f in c8r.GRAD_FIELDS}
+    ag = torch.zeros((n_ant, 3), dtype=torch.float64, device="cuda")
+    dn = torch.zeros(1, dtype=torch.float64, device="cuda")
+    c8r.c8r_backward(p.ctx, dev, G, tg, ag, dn)
+    got = np.stack([tg[f].double().cpu().numpy() for f in c8r.GRAD_FIELDS], axis=1)
+    p.close()
+    tg_ref, ag_ref, _ = oracle.backward(oracle.tracks_from_ns(tracks), w["ant_xyz"], w["t_start_ns"] * 1e-9,
+                                        w["n_bins"], w["dt_ns"] * 1e-9, w["medium"], G.double().cpu().numpy())
+    assert rel_l2(got[:, 0:6], tg_ref[:, 0:6]) <= TOL
+    assert rel_l2(got[:, 8:11], tg_ref[:, 8:11]) <= TOL
+    assert rel_l2(ag.cpu().numpy(), ag_ref) <= TOL
