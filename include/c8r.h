@@ -181,8 +181,8 @@ int c8r_set_medium_spherical(c8r_ctx* ctx, double N0, double scale_height_m, dou
  * zeroes) the context's trace accumulator, one (x, y, z) element per antenna and
  * bin, FP64 (C8R_FP64) or FP32 (C8R_MIXED), 32 or 16 bytes per element.  Mixed
  * ZHS keeps a second row per antenna (box edges), and the mixed path keeps 1 to
- * 16 copies of the whole accumulator, more for fewer antennas (up to 96 MB in
- * all), which the fetch sums; a push uses as many of them as its tracks pay for.  Replaces
+ * 16 copies of the whole accumulator, more for fewer antennas (up to 192 MB
+ * in all), which the fetch sums; a push uses as many of them as its tracks pay for.  Replaces
  * any previous antenna set and discards its traces (a call with the same
  * n_ant, n_bins, dt_ns, formalism and precision keeps the device memory and
  * only replaces the table, so moving an array between steps is cheap).  EINVAL on n_ant < 1,

@@ -610,7 +610,7 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
   const bool lin = c->deposit == C8R_DEPOSIT_LINEAR;
   form_poll(c);
   FwdShape shape = c->shape;  // of this push: with the accumulator copies it uses
-  shape.replicas = push_replicas(shape.replicas, n, c->n_bins);
+  shape.replicas = push_replicas(shape.replicas, n, c->n_bins, acc_rows(c->precision, c->formalism));
   if (capturing(st)) c->copies_all = true;
   if (shape.replicas > c->copies_used) c->copies_used = shape.replicas;
   for (int64_t off = 0; off < n; off += chunk) {

@@ -112,12 +112,12 @@ __global__ void __launch_bounds__(256) k_batch_votes(const float* tiles, const V
 }
 
 template <class Ops>
-__global__ void __launch_bounds__(kTileT, Ops::kMinBlocks) k_batch(const BatchArgs a) {
+__global__ void __launch_bounds__(Ops::kFwdThreads, Ops::kMinBlocks) k_batch(const BatchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   const MedParams& M = a.M;
   const FwdLayout L = fwd_layout(Ops::kPrec, a.a_tile, Ops::kDefers);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.bar_off);
-  typename Ops::Ant* ant_s = reinterpret_cast<typename Ops::Ant*>(smem + L.ant_off);
+  typename Ops::FwdAnt* ant_s = reinterpret_cast<typename Ops::FwdAnt*>(smem + L.ant_off);
   __shared__ int s_item;
   const int tid = threadIdx.x, nthr = blockDim.x;
   if (tid == 0) {
@@ -155,7 +155,7 @@ int batch_blocks_per_sm(int a_tile) {
   auto k = k_batch<Ops>;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 1;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kTileT, smem) != cudaSuccess) return 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Ops::kFwdThreads, smem) != cudaSuccess) return 1;
   return per_sm < 1 ? 1 : per_sm;
 }
 
@@ -165,7 +165,7 @@ cudaError_t launch_batch_ops(const BatchArgs& a, int sm_count, cudaStream_t st) 
   const size_t smem = fwd_layout(C8R_MIXED, a.a_tile, Ops::kDefers).total;
   auto k = k_batch<Ops>;
   const int per_sm = batch_blocks_per_sm<Ops>(a.a_tile);
-  k<<<sm_count * per_sm, kTileT, smem, st>>>(a);
+  k<<<sm_count * per_sm, Ops::kFwdThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -200,23 +200,28 @@ constexpr bool kUsualForm = std::is_same<T, float2>::value;
 // Knuth (TwoSum) and Dekker / the FMA form (TwoProd).  Intrinsics pin the
 // rounding of every step; nothing here may be contracted or reassociated.
 // ---------------------------------------------------------------------------
-struct ff {
-  float h, l;
+template <typename T>
+struct ffT {
+  T h, l;
 };
+using ff = ffT<float>;
 
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+template <typename T>
+__device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
+  s = add_rn(a, b);
+  const T bb = sub_rn(s, a);
+  e = add_rn(sub_rn(a, sub_rn(s, bb)), sub_rn(b, bb));
 }
-__device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
-  p = __fmul_rn(a, b);
-  e = __fmaf_rn(a, b, -p);
+template <typename T>
+__device__ __forceinline__ void two_prod(T a, T b, T& p, T& e) {
+  p = mul_rn(a, b);
+  e = fma_rn(a, b, neg(p));
 }
 // Dekker's Fast2Sum: exact when the exponent of a is at least that of b
-__device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  e = __fsub_rn(b, __fsub_rn(s, a));
+template <typename T>
+__device__ __forceinline__ void fast_two_sum(T a, T b, T& s, T& e) {
+  s = add_rn(a, b);
+  e = sub_rn(b, sub_rn(s, a));
 }
 
 // ---------------------------------------------------------------------------
@@ -523,146 +528,145 @@ __device__ __forceinline__ void geo_lite(const AntRec& A, float px, float py, fl
 // the z part of d = a - p that every antenna of a flat array (one altitude)
 // shares: d_z as float-float and the products of it that geo_refine and
 // doppler_ff form, formed once per point as they form them (so the same values)
-struct ZPart {
-  float sh, sl;  // d_z = sh + sl (geo_lite's s[2], e[2])
-  float qh, ql;  // sh^2, exact
-  float se;      // fl(sh sl)
-  float bh, bl;  // b_z sh, exact
-  float be;      // fl(b_z sl)
+template <typename T>
+struct ZPartT {
+  T sh, sl;  // d_z = sh + sl (geo_lite's s[2], e[2])
+  T qh, ql;  // sh^2, exact
+  T se;      // fl(sh sl)
+  T bh, bl;  // b_z sh, exact
+  T be;      // fl(b_z sl)
 };
-__device__ __forceinline__ ZPart z_part(float sh, float sl, float bz) {
-  ZPart z;
+using ZPart = ZPartT<float>;
+template <typename T>
+__device__ __forceinline__ ZPartT<T> z_part(T sh, T sl, T bz) {
+  ZPartT<T> z;
   z.sh = sh;
   z.sl = sl;
   two_prod(sh, sh, z.qh, z.ql);
-  z.se = __fmul_rn(sh, sl);
+  z.se = mul_rn(sh, sl);
   two_prod(bz, sh, z.bh, z.bl);
-  z.be = __fmul_rn(bz, sl);
+  z.be = mul_rn(bz, sl);
   return z;
 }
 
-// geo_lite of a float-float point whose z part comes from ZPart
-__device__ __forceinline__ void geo_lite(const AntRec& A, float pxh, float pyh, float pxl, float pyl, const ZPart& z,
-                                         GeoM& g) {
-  two_sum(A.xh, -pxh, g.s[0], g.e[0]);
-  two_sum(A.yh, -pyh, g.s[1], g.e[1]);
+// geo_lite of a float-float point whose z part comes from ZPart; the antenna's
+// x and y as float-float
+template <typename T>
+__device__ __forceinline__ void geo_lite(T axh, T ayh, T axl, T ayl, T pxh, T pyh, T pxl, T pyl, const ZPartT<T>& z,
+                                         GeoT<T>& g) {
+  two_sum(axh, neg(pxh), g.s[0], g.e[0]);
+  two_sum(ayh, neg(pyh), g.s[1], g.e[1]);
   g.s[2] = z.sh;
   g.e[2] = z.sl;
-  g.e[0] = __fadd_rn(g.e[0], __fsub_rn(A.xl, pxl));
-  g.e[1] = __fadd_rn(g.e[1], __fsub_rn(A.yl, pyl));
-  const float S = __fmaf_rn(g.s[2], g.s[2], __fmaf_rn(g.s[0], g.s[0], __fmul_rn(g.s[1], g.s[1])));
+  g.e[0] = add_rn(g.e[0], sub_rn(axl, pxl));
+  g.e[1] = add_rn(g.e[1], sub_rn(ayl, pyl));
+  const T S = fma_rn(g.s[2], g.s[2], fma_rn(g.s[0], g.s[0], mul_rn(g.s[1], g.s[1])));
   g.y = rsqrt_ap(S);
-  g.R0 = __fmul_rn(S, g.y);
-  g.R1 = 0.0f;
+  g.R0 = mul_rn(S, g.y);
+  g.R1 = bc<T>(0.0f);
 }
 
 // R from the exact squares of d's components (p2 + q2 = s_z^2 and se =
 // fl(s_z e_z) given)
-__device__ __forceinline__ void geo_refine(GeoM& g, float p2, float q2, float se) {
-  float p0, q0, p1, q1;
+template <typename T>
+__device__ __forceinline__ void geo_refine(GeoT<T>& g, T p2, T q2, T se) {
+  T p0, q0, p1, q1;
   two_prod(g.s[0], g.s[0], p0, q0);
   two_prod(g.s[1], g.s[1], p1, q1);
-  float S1, E1, S2, E2;
+  T S1, E1, S2, E2;
   two_sum(p0, p1, S1, E1);
   two_sum(S1, p2, S2, E2);
-  const float cross = __fmaf_rn(g.s[0], g.e[0], __fmaf_rn(g.s[1], g.e[1], se));
-  const float lo = __fadd_rn(__fadd_rn(__fadd_rn(q0, q1), __fadd_rn(q2, E1)), __fadd_rn(E2, __fmul_rn(2.0f, cross)));
-  float rq, rqe;
+  const T cross = fma_rn(g.s[0], g.e[0], fma_rn(g.s[1], g.e[1], se));
+  const T lo = add_rn(add_rn(add_rn(q0, q1), add_rn(q2, E1)), add_rn(E2, mul_rn(bc<T>(2.0f), cross)));
+  T rq, rqe;
   two_prod(g.R0, g.R0, rq, rqe);
-  const float rho = __fadd_rn(__fsub_rn(__fsub_rn(S2, rq), rqe), lo);
-  g.R1 = __fmul_rn(__fmul_rn(rho, 0.5f), g.y);
+  const T rho = add_rn(sub_rn(sub_rn(S2, rq), rqe), lo);
+  g.R1 = mul_rn(mul_rn(rho, bc<T>(0.5f)), g.y);
 }
-__device__ __forceinline__ void geo_refine(GeoM& g) {
-  float p2, q2;
+template <typename T>
+__device__ __forceinline__ void geo_refine(GeoT<T>& g) {
+  T p2, q2;
   two_prod(g.s[2], g.s[2], p2, q2);
-  geo_refine(g, p2, q2, __fmul_rn(g.s[2], g.e[2]));
+  geo_refine(g, p2, q2, mul_rn(g.s[2], g.e[2]));
 }
-__device__ __forceinline__ void geo_refine(GeoM& g, const ZPart& z) { geo_refine(g, z.qh, z.ql, z.se); }
-
-__device__ __forceinline__ void geo_mixed(const AntRec& A, float pxh, float pyh, float pzh, float pxl, float pyl,
-                                          float pzl, GeoM& g) {
-  geo_lite(A, pxh, pyh, pzh, pxl, pyl, pzl, g);
-  geo_refine(g);
+template <typename T>
+__device__ __forceinline__ void geo_refine(GeoT<T>& g, const ZPartT<T>& z) {
+  geo_refine(g, z.qh, z.ql, z.se);
 }
 
 // (E_e - E_a)/dz in float-float, the quotient of the refractivity term of the
 // exponential medium, dz = dzh + dzl the altitude difference a - e: the FP32
 // quotient corrected once from the exact residual, or for |dz/H| <= 1e-3 the
 // series (E_e/H)(1 + f), f = -x/2 + x^2/6 - x^3/24, x = dz/H
-__device__ __forceinline__ void refr_quotient(const MedParams& M, float Eah, float Eal, float dzh, float dzl,
-                                              float Eeh, float Eel, float& q0, float& q1) {
-  const float x = __fmul_rn(dzh, M.invH_h);
-  if (fabsf(x) > 1e-3f) {
-    float Qh, Ql;
-    two_sum(Eeh, -Eah, Qh, Ql);
-    Ql = __fadd_rn(Ql, __fsub_rn(Eel, Eal));
-    q0 = div_ap(Qh, dzh);
-    float ph, pl;
-    two_prod(q0, dzh, ph, pl);
-    const float r = __fsub_rn(__fadd_rn(__fsub_rn(__fsub_rn(Qh, ph), pl), Ql), __fmul_rn(q0, dzl));
-    q1 = div_ap(r, dzh);
-  } else {
-    const float f = __fmul_rn(x, __fmaf_rn(x, __fmaf_rn(x, -1.0f / 24.0f, 1.0f / 6.0f), -0.5f));
-    float eh, el;
-    two_prod(Eeh, M.invH_h, eh, el);
-    el = __fmaf_rn(Eeh, M.invH_l, __fmaf_rn(Eel, M.invH_h, el));
-    // (eh + el)(1 + f)
-    float g0, g1;
-    two_sum(eh, __fmul_rn(eh, f), g0, g1);
-    q0 = g0;
-    q1 = __fadd_rn(g1, __fmaf_rn(el, f, el));
+template <typename T>
+__device__ __forceinline__ void refr_quotient(const MedParams& M, T Eah, T Eal, T dzh, T dzl, T Eeh, T Eel, T& q0,
+                                              T& q1) {
+  if constexpr (!kUsualForm<T>) {
+    const float x = __fmul_rn(dzh, M.invH_h);
+    if (!(fabsf(x) > 1e-3f)) {
+      const float f = __fmul_rn(x, __fmaf_rn(x, __fmaf_rn(x, -1.0f / 24.0f, 1.0f / 6.0f), -0.5f));
+      float eh, el;
+      two_prod(Eeh, M.invH_h, eh, el);
+      el = __fmaf_rn(Eeh, M.invH_l, __fmaf_rn(Eel, M.invH_h, el));
+      // (eh + el)(1 + f)
+      float g0, g1;
+      two_sum(eh, __fmul_rn(eh, f), g0, g1);
+      q0 = g0;
+      q1 = __fadd_rn(g1, __fmaf_rn(el, f, el));
+      return;
+    }
   }
+  T Qh, Ql;
+  two_sum(Eeh, neg(Eah), Qh, Ql);
+  Ql = add_rn(Ql, sub_rn(Eel, Eal));
+  const T r = rcp_ap(dzh);
+  q0 = mul_rn(Qh, r);
+  T ph, pl;
+  two_prod(q0, dzh, ph, pl);
+  q1 = mul_rn(sub_rn(add_rn(sub_rn(sub_rn(Qh, ph), pl), Ql), mul_rn(q0, dzl)), r);
 }
 
 // arrival position u = (t_e - t_ref)/dt + n_avg R / (c dt) in bins, float-float,
 // with the refractivity quotient (q0, q1) given (exponential media; ignored in
 // the uniform one).  tau_e = t_e/dt and the antenna's tau = t_ref/dt come in
 // float-float.  KIND: the medium kind (a template argument, so each kernel
-// carries only its own medium's arithmetic; it equals M.kind).  `dop` (curved
-// rays only): the ray's optical path minus the straight line's, m
-template <int KIND>
-__device__ __forceinline__ ff arrival_mixed_q(const MedParams& M, const AntRec& A, const GeoM& g, float tauh,
-                                              float taul, float q0, float q1, float dop = 0.0f) {
-  float ts, te;
-  two_sum(tauh, -A.tauh, ts, te);
-  te = __fadd_rn(te, __fsub_rn(taul, A.taul));
-  float sh = (KIND == C8R_UNIFORM) ? M.s_h : M.kc_h;
-  float sl = (KIND == C8R_UNIFORM) ? M.s_l : M.kc_l;
-  float p, pe;
+// carries only its own medium's arithmetic; it equals M.kind).  `corr` (curved
+// rays, spherical Earth): the optical path minus the flat straight line's, m
+template <int KIND, typename T>
+__device__ __forceinline__ ffT<T> arrival_mixed_q(const MedParams& M, T atauh, T ataul, const GeoT<T>& g, T tauh, T taul,
+                                                  T q0, T q1, T corr = bc<T>(0.0f)) {
+  T ts, te;
+  two_sum(tauh, neg(atauh), ts, te);
+  te = add_rn(te, sub_rn(taul, ataul));
+  const T sh = bc<T>((KIND == C8R_UNIFORM) ? M.s_h : M.kc_h);
+  const T sl = bc<T>((KIND == C8R_UNIFORM) ? M.s_l : M.kc_l);
+  T p, pe;
   two_prod(g.R0, sh, p, pe);
-  pe = __fmaf_rn(g.R0, sl, __fmaf_rn(g.R1, sh, pe));
+  pe = fma_rn(g.R0, sl, fma_rn(g.R1, sh, pe));
   if constexpr (KIND != C8R_UNIFORM) {
     // refractivity term (n_avg - 1) R/(c dt) = N0 H/(c dt) * (E_e - E_a)/dz * R
-    float w, we;
+    T w, we;
     two_prod(q0, g.R0, w, we);
-    we = __fmaf_rn(q0, g.R1, __fmaf_rn(q1, g.R0, we));
-    float v, ve;
-    two_prod(w, M.cN_h, v, ve);
-    ve = __fmaf_rn(w, M.cN_l, __fmaf_rn(we, M.cN_h, ve));
-    float p2, pe2;
+    we = fma_rn(q0, g.R1, fma_rn(q1, g.R0, we));
+    T v, ve;
+    two_prod(w, bc<T>(M.cN_h), v, ve);
+    ve = fma_rn(w, bc<T>(M.cN_l), fma_rn(we, bc<T>(M.cN_h), ve));
+    T p2, pe2;
     fast_two_sum(p, v, p2, pe2);  // |v| = (n_avg - 1)|p| < |p|
     p = p2;
-    pe = __fadd_rn(pe, __fadd_rn(pe2, ve));
-    if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL) {
-      // curvature correction (~1e-3 of the refractivity term, FP32 is enough)
-      const float cs = __fmul_rn(
-          sphere_path_correction<float>(A.xh, A.yh, A.zh, g.s[0], g.s[1], g.s[2], g.R0, M.N0f, M.invH_h, M.RE_f),
-          M.kc_h);
-      fast_two_sum(p, cs, p2, pe2);
+    pe = add_rn(pe, add_rn(pe2, ve));
+    if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL || KIND == C8R_EXPONENTIAL_RAY) {
+      // the small change of the optical path in bins (the sphere's curvature,
+      // ~1e-3 of the refractivity term; the ray's time saved, <~1 bin): FP32 is enough
+      fast_two_sum(p, mul_rn(corr, bc<T>(M.kc_h)), p2, pe2);
       p = p2;
-      pe = __fadd_rn(pe, pe2);
-    }
-    if constexpr (KIND == C8R_EXPONENTIAL_RAY) {
-      // the ray's time saved against the straight line (<~1 bin; FP32 is enough)
-      fast_two_sum(p, __fmul_rn(dop, M.kc_h), p2, pe2);
-      p = p2;
-      pe = __fadd_rn(pe, pe2);
+      pe = add_rn(pe, pe2);
     }
   }
-  float uh, ue;
+  T uh, ue;
   two_sum(ts, p, uh, ue);
-  ue = __fadd_rn(ue, __fadd_rn(te, pe));
-  return ff{uh, ue};
+  ue = add_rn(ue, add_rn(te, pe));
+  return ffT<T>{uh, ue};
 }
 
 // the same with the quotient formed here, from the emission point's E_e =
@@ -672,7 +676,9 @@ __device__ __forceinline__ ff arrival_mixed(const MedParams& M, const AntRec& A,
                                             float Eeh, float Eel, float dop = 0.0f) {
   float q0 = 0.0f, q1 = 0.0f;
   if constexpr (KIND != C8R_UNIFORM) refr_quotient(M, A.Eah, A.Eal, g.s[2], g.e[2], Eeh, Eel, q0, q1);
-  return arrival_mixed_q<KIND>(M, A, g, tauh, taul, q0, q1, dop);
+  if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL)
+    dop = sphere_path_correction<float>(A.xh, A.yh, A.zh, g.s[0], g.s[1], g.s[2], g.R0, M.N0f, M.invH_h, M.RE_f);
+  return arrival_mixed_q<KIND>(M, A.tauh, A.taul, g, tauh, taul, q0, q1, dop);
 }
 
 // bin index of a float-float arrival, clamped to [-1, n_bins]: -1 stands for
@@ -898,9 +904,27 @@ __device__ __forceinline__ float gap_to_next_edge(ff u, int k) {
   return __fsub_rn(__fsub_rn((float)(k + 1), u.h), u.l);
 }
 
-__device__ __forceinline__ bool bin_of(ff u, int n_bins, int& k, float& frac) {
-  k = bin_raw(u, n_bins, frac);
-  return k >= 0 && k < n_bins;
+// The bins and fractions of two float-float arrivals as bin_raw has them, for
+// windows of at most kMagicBins / 2 bins: floors from rounded-down sums as in
+// decide_bins, of the high part and then of the fraction with the low part.
+// Arrivals outside the window give any index outside it.
+__device__ __forceinline__ void bins_of(ffT<float2> u, int n_bins, int& kx, int& ky, float2& kf, float2& frac) {
+  const float2 magic = make_float2(12582912.0f, 12582912.0f);
+  // a margin for the low part, as in bin_raw (fmaxf and fminf drop a NaN, to
+  // outside); far outside, where the low part can be any size, it is dropped
+  const float top = (float)n_bins + 128.0f;
+  const float2 h = make_float2(fminf(fmaxf(u.h.x, -128.0f), top), fminf(fmaxf(u.h.y, -128.0f), top));
+  const float2 l = make_float2(h.x == u.h.x ? u.l.x : 0.0f, h.y == u.h.y ? u.l.y : 0.0f);
+  const float2 t = __fadd2_rd(h, magic);
+  const float2 k0 = sub_rn(t, magic);
+  const float2 f = add_rn(sub_rn(h, k0), l);
+  const float2 t1 = __fadd2_rd(f, magic);
+  const float2 df = sub_rn(t1, magic);
+  kf = add_rn(k0, df);
+  frac = sub_rn(f, df);
+  constexpr unsigned two = 2u * (unsigned)kMagicBinBits;
+  kx = (int)(__float_as_uint(t.x) + __float_as_uint(t1.x) - two);
+  ky = (int)(__float_as_uint(t.y) + __float_as_uint(t1.y) - two);
 }
 
 // field part at one emission point (FP32): w = d x beta, V = (d x w)/R^2 =
@@ -982,44 +1006,46 @@ __device__ __forceinline__ FieldM half_of(const FieldT<float2>& f) {
 // half-width reaches ~10^2 bins, so D must be good to ~1e-9 absolute, which the
 // FP32 form of field_mixed (good to ~1e-7 relative) is not for |D| of order 1.
 // (p2 + q2 = b_z s_z exactly and bze = fl(b_z e_z) given)
-__device__ __forceinline__ ff doppler_ff(const GeoM& g, float bx, float by, float p2, float q2, float bze,
-                                         float nm1) {
+template <typename T>
+__device__ __forceinline__ ffT<T> doppler_ff(const GeoT<T>& g, T bx, T by, T p2, T q2, T bze, T nm1) {
   // beta . d with d = s + e exact: exact products of the high parts, summed
   // with TwoSum; the low parts and the rounding errors in FP32
-  float p0, q0, p1, q1;
+  T p0, q0, p1, q1;
   two_prod(bx, g.s[0], p0, q0);
   two_prod(by, g.s[1], p1, q1);
-  float S1, E1, S2, E2;
+  T S1, E1, S2, E2;
   two_sum(p0, p1, S1, E1);
   two_sum(S1, p2, S2, E2);
-  const float be = __fmaf_rn(bx, g.e[0], __fmaf_rn(by, g.e[1], bze));
-  const float lo = __fadd_rn(__fadd_rn(__fadd_rn(q0, q1), __fadd_rn(q2, E1)), __fadd_rn(E2, be));
+  const T be = fma_rn(bx, g.e[0], fma_rn(by, g.e[1], bze));
+  const T lo = add_rn(add_rn(add_rn(q0, q1), add_rn(q2, E1)), add_rn(E2, be));
   // q = (beta . d)/R: FP32 quotient, then one correction from the exact residual
-  const float qh = __fmul_rn(S2, g.y);
-  float ph, pl;
+  const T qh = mul_rn(S2, g.y);
+  T ph, pl;
   two_prod(qh, g.R0, ph, pl);
-  const float r = __fsub_rn(__fadd_rn(__fsub_rn(__fsub_rn(S2, ph), pl), lo), __fmul_rn(qh, g.R1));
-  const float ql = __fmul_rn(r, g.y);
+  const T r = sub_rn(add_rn(sub_rn(sub_rn(S2, ph), pl), lo), mul_rn(qh, g.R1));
+  const T ql = mul_rn(r, g.y);
   // n q = q + (n - 1) q, then D = 1 - n q
-  float nh, nl;
-  two_sum(qh, __fmul_rn(nm1, qh), nh, nl);
-  nl = __fadd_rn(nl, ql);
-  float dh, dl;
-  two_sum(1.0f, -nh, dh, dl);
-  dl = __fsub_rn(dl, nl);
+  T nh, nl;
+  two_sum(qh, mul_rn(nm1, qh), nh, nl);
+  nl = add_rn(nl, ql);
+  T dh, dl;
+  two_sum(bc<T>(1.0f), neg(nh), dh, dl);
+  dl = sub_rn(dl, nl);
   // renormalise, so that the sign of D is the sign of D.h (near D = 0 the high
   // part alone can be 0 or of the other sign)
-  ff D;
-  D.h = __fadd_rn(dh, dl);
-  D.l = __fsub_rn(dl, __fsub_rn(D.h, dh));
+  ffT<T> D;
+  D.h = add_rn(dh, dl);
+  D.l = sub_rn(dl, sub_rn(D.h, dh));
   return D;
 }
-__device__ __forceinline__ ff doppler_ff(const GeoM& g, float bx, float by, float bz, float nm1) {
-  float p2, q2;
+template <typename T>
+__device__ __forceinline__ ffT<T> doppler_ff(const GeoT<T>& g, T bx, T by, T bz, T nm1) {
+  T p2, q2;
   two_prod(bz, g.s[2], p2, q2);
-  return doppler_ff(g, bx, by, p2, q2, __fmul_rn(bz, g.e[2]), nm1);
+  return doppler_ff(g, bx, by, p2, q2, mul_rn(bz, g.e[2]), nm1);
 }
-__device__ __forceinline__ ff doppler_ff(const GeoM& g, float bx, float by, const ZPart& z, float nm1) {
+template <typename T>
+__device__ __forceinline__ ffT<T> doppler_ff(const GeoT<T>& g, T bx, T by, const ZPartT<T>& z, T nm1) {
   return doppler_ff(g, bx, by, z.bh, z.bl, z.be, nm1);
 }
 

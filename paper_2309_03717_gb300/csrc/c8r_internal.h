@@ -29,45 +29,47 @@ inline size_t acc_elem_bytes(int precision) { return precision == C8R_FP64 ? 32 
 inline int acc_rows(int precision, int formalism) { return precision == C8R_MIXED && formalism == C8R_ZHS ? 2 : 1; }
 // copies of the accumulator the forward kernel spreads its reductions over (CTA
 // range r adds into copy r % replicas; the fetch sums them).  Most reductions go
-// into the few bins per antenna that the pulse arrives in, and with many CTAs on
-// one antenna tile at a time those bins' addresses become the bottleneck: on 4e6
-// tracks of a vertical shower x 160 antennas the Endpoint kernel took 7.8 ms with
-// one copy, 5.7 / 5.48 / 5.49 with 2 / 4 / 8, and 5.4 with no reductions at all.
-// A copy costs its bytes once to zero and once to read per fetch, so few tracks
-// take few copies.  Measured (us per push and fetch, 4096 bins, 1 / 4 / 16
-// copies): Endpoint, 8 antennas, 1e6 tracks 646 / 224 / 152, 64 antennas 1123 /
-// 752 / 625, 160 antennas 1749 / 1412 / 1422, 512 antennas x 3e5 1303 / 1310 /
-// 1310; ZHS, 8 antennas 576 / 257 / 213, 160 antennas 1955 / 1552 / 1552 (the
-// budget allows 4); linear deposit, 64 antennas 2487 / 1612 / 1242.  With 3e4
-// tracks: Endpoint, 64 antennas 76 / 61 / 64, ZHS, 160 antennas 141 / 120 / 121.
+// into the few bins per antenna that the pulse arrives in, a few lines of L2
+// each, and the slices that hold more of those lines become the bottleneck (the
+// busiest ran at twice the mean with 4 copies).  4e6 tracks of a vertical shower x
+// 160 antennas, Endpoint, ms with 1 / 2 / 4 / 8 / 16 copies: 7.8 / 5.7 / 5.15 /
+// 4.71 / 4.74; ZHS, 2e7 tracks, 4 / 8 / 16: 26.5 / 24.7 / 24.8.  A copy costs its
+// bytes once to zero and once to read per fetch, so few tracks take few copies.
+// Us per push and fetch with 1 / 4 / 16 copies (4096 bins): Endpoint, 8 antennas,
+// 1e6 tracks 646 / 224 / 152, 64 antennas 1123 / 752 / 625, 512 antennas x 3e5
+// 1303 / 1310 / 1310; ZHS, 8 antennas 576 / 257 / 213; linear deposit, 64 antennas
+// 2487 / 1612 / 1242.  With 3e4 tracks, Endpoint, 64 antennas 76 / 61 / 64.
 //
 // the batched launch: its many showers' antenna tiles spread the CTAs, so 2
 // copies for ZHS and 1 for Endpoint
 inline int acc_replicas(int precision, int formalism) { return acc_rows(precision, formalism) == 2 ? 2 : 1; }
-// bytes of L2 that the accumulator rows in use at a time may take (forward_grid
-// groups the antenna tiles by it)
-constexpr size_t kAccL2Budget = (size_t)96 << 20;
+// bytes of the accumulator rows in use at a time (forward_grid groups the
+// antenna tiles by it) and of all copies.  Above L2's 129 MB: the bins that the
+// pulses reach, a small part of the rows, are what has to stay there
+constexpr size_t kAccBudget = (size_t)192 << 20;
 // the most copies a context uses (its accumulator is allocated for this many):
-// one per 29 resident CTAs of an antenna tile (6 CTAs per SM), at most 16 and
-// within the L2 budget, as a power of two.  29 is where the measurements above
-// part: 456 CTAs per tile (64 antennas) gain from 8 copies on, 182 (160
-// antennas) up to 4, 57 (512 antennas) not at all
+// one per 22 resident CTAs of an antenna tile (6 CTAs per SM), at most 16 and
+// within the budget, as a power of two, and one below 64 CTAs.  That is where the
+// measurements above part: 456 CTAs per tile (64 antennas) gain up to 16 copies,
+// 182 (160 antennas) up to 8, 57 (512 antennas) none (linear deposit, 1e5 tracks:
+// 906 us with 1, 920 with 2)
 inline int acc_replicas(int precision, int formalism, int n_ant, int n_bins, int a_tile, int sm_count) {
   if (precision != C8R_MIXED) return 1;
   const int64_t ant_tiles = (n_ant + a_tile - 1) / a_tile;
-  const int64_t want = (int64_t)sm_count * 6 / (ant_tiles > 0 ? ant_tiles : 1) / 29;
+  const int64_t per_tile = (int64_t)sm_count * 6 / (ant_tiles > 0 ? ant_tiles : 1);
+  const int64_t want = per_tile < 64 ? 1 : per_tile / 22;
   const size_t one = (size_t)n_ant * n_bins * 16 * acc_rows(precision, formalism);
-  const int64_t fit = (int64_t)(kAccL2Budget / (one > 0 ? one : 1));
+  const int64_t fit = (int64_t)(kAccBudget / (one > 0 ? one : 1));
   int r = 1;
   while (r < 16 && r * 2 <= want && r * 2 <= fit) r *= 2;
   return r;
 }
-// the copies that a push of n tracks uses, of the `most` allocated: a track per
-// bin and copy at least, where the cost of a copy (about 32 bytes per bin and
-// antenna) falls below what it takes off the reductions of the tracks
-inline int push_replicas(int most, int64_t n, int n_bins) {
+// the copies that a push of n tracks uses, of the `most` allocated: two tracks per
+// bin, row and copy at least, where the cost of a copy (about 32 bytes per bin,
+// row and antenna) falls below what it takes off the reductions of the tracks
+inline int push_replicas(int most, int64_t n, int n_bins, int rows) {
   int r = 1;
-  while (r * 2 <= most && (int64_t)r * 2 * n_bins <= n) r *= 2;
+  while (r * 2 <= most && (int64_t)r * 4 * n_bins * rows <= n) r *= 2;
   return r;
 }
 // accumulator [replicas][n_ant][rows][n_bins] -> traces [n_ant][3][n_bins]: the

@@ -258,7 +258,7 @@ __device__ __forceinline__ void queue_aside(const Aside& s, int l, uint16_t* que
 // mbarrier phase) and is advanced.  Returns false if a bounded wait gave up; the
 // CTA then has no copy in flight and must stop.
 template <class Ops>
-__device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* bar, const typename Ops::Ant* ant_s,
+__device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* bar, const typename Ops::FwdAnt* ant_s,
                              typename AccOf<typename Ops::acc_t>::type* acc_row0, int n_here,
                              const unsigned char* src, int64_t t_begin, int64_t t_end, int64_t& it,
                              const MedParams& M) {
@@ -298,16 +298,16 @@ __device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* 
     // one outcome for the warp: queue_aside's shuffles want every lane
     const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[st], parity, M.wait_limit));
     if (ok) {
-      // one track per thread, held in registers, against every antenna of the tile
-      for (int l = tid; l < kTileT; l += nthr) {
-        typename Ops::MainTrack tr;
-        Ops::load_main(smem + st * L.stage_bytes, l, M, tr);
+      // one track per thread (or two), held in registers, against every antenna of the tile
+      for (int l = tid; l < Ops::kFwdThreads; l += nthr) {
+        typename Ops::FwdTrack tr;
+        Ops::load_fwd(smem + st * L.stage_bytes, l, M, tr);
         Aside aside;
         if (Ops::live(tr))
 #pragma unroll 1
           for (int ant = 0; ant < n_here; ++ant) {
             GlobalSink<acc_t> sink{acc_row0 + (size_t)ant * row_stride, N};
-            const int code = Ops::pair_main(tr, ant_s + ant, M, sink);
+            const int code = Ops::pair_main(tr, ant_s + ant, smem + st * L.stage_bytes, l, M, sink);
             if constexpr (Ops::kDefers) aside.add(code, ant);
           }
         if constexpr (Ops::kDefers) queue_aside(aside, l, queue, L.q_cap, &q_cnt[st], &q_back[st]);
@@ -396,13 +396,13 @@ __device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* 
 }
 
 template <class Ops>
-__global__ void __launch_bounds__(kTileT, Ops::kMinBlocks) k_forward(const FwdArgs a) {
+__global__ void __launch_bounds__(Ops::kFwdThreads, Ops::kMinBlocks) k_forward(const FwdArgs a) {
   using acc_t = typename Ops::acc_t;
   using acc4 = typename AccOf<acc_t>::type;
   extern __shared__ __align__(128) unsigned char smem[];
   const FwdLayout L = fwd_layout(Ops::kPrec, a.a_tile, Ops::kDefers);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.bar_off);
-  typename Ops::Ant* ant_s = reinterpret_cast<typename Ops::Ant*>(smem + L.ant_off);
+  typename Ops::FwdAnt* ant_s = reinterpret_cast<typename Ops::FwdAnt*>(smem + L.ant_off);
   int ant_tile;
   int64_t range;
   a.g.decode(blockIdx.x, ant_tile, range);
@@ -436,13 +436,13 @@ inline int forward_threads(int a_tile) {
 // grid of the forward launch: about `waves` full waves of resident CTAs (a whole
 // number of them when the antenna tiles allow, so no wave runs part-empty);
 // antenna tiles grouped so that one block's accumulator rows take at most
-// kAccL2Budget bytes
+// kAccBudget bytes
 inline int64_t forward_grid(FwdArgs& a, const FwdShape& shape, int resident, size_t acc_elem_bytes) {
   FwdGrid& g = a.g;
   g.ant_tiles = (a.n_ant + shape.a_tile - 1) / shape.a_tile;
   // an antenna tile's rows in every copy of the accumulator
   const size_t tile_bytes = (size_t)shape.a_tile * a.M.n_bins * acc_elem_bytes * (shape.replicas > 1 ? shape.replicas : 1);
-  int tpb = (int)(kAccL2Budget / (tile_bytes > 0 ? tile_bytes : 1));
+  int tpb = (int)(kAccBudget / (tile_bytes > 0 ? tile_bytes : 1));
   g.tiles_per_block = tpb < 1 ? 1 : (tpb > g.ant_tiles ? g.ant_tiles : tpb);
   int64_t target = (int64_t)shape.waves * resident;
   int64_t ranges = (target + g.ant_tiles - 1) / g.ant_tiles;
@@ -470,7 +470,7 @@ cudaError_t launch_forward_ops(const FwdArgs& a, int64_t ctas, cudaStream_t st) 
   auto k = k_forward<Ops>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<(unsigned)ctas, kTileT, smem, st>>>(a);
+  k<<<(unsigned)ctas, Ops::kFwdThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -480,7 +480,7 @@ int forward_blocks_per_sm(int a_tile) {
   int n = 0;
   const size_t smem = fwd_layout(Ops::kPrec, a_tile, Ops::kDefers).total;
   cudaFuncSetAttribute(k_forward<Ops>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_forward<Ops>, kTileT, smem) != cudaSuccess) n = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_forward<Ops>, Ops::kFwdThreads, smem) != cudaSuccess) n = 1;
   return n < 1 ? 1 : n;
 }
 

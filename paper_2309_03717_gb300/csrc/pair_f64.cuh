@@ -149,6 +149,12 @@ struct OpsF64 {
   }
   static __device__ __forceinline__ bool live(const TrackD& t) { return t.q != 0.0; }
   using MainTrack = TrackD;
+  using FwdTrack = TrackD;
+  using FwdAnt = AntRec;
+  static constexpr int kFwdThreads = kTileT;
+  static __device__ __forceinline__ void load_fwd(const void* Tv, int l, const MedParams& M, TrackD& t) {
+    load(Tv, l, M, t);
+  }
   struct MainGrad {
     double g[11];
   };
@@ -173,7 +179,8 @@ struct OpsF64 {
   // main pass: every pair but (kDefers) the near-Cherenkov ones, returned as
   // kDeferPair with nothing deposited; pair_deferred evaluates those in full
   template <class Sink>
-  static __device__ __forceinline__ int pair_main(const TrackD& t, const AntRec* p, const MedParams& M, Sink& out) {
+  static __device__ __forceinline__ int pair_main(const TrackD& t, const AntRec* p, const void*, int, const MedParams& M,
+                                                  Sink& out) {
     const AntRec A = *p;
     if constexpr (kDefers) return endpoint(t.T, t.l, A, M, out, true);
     pair(t, A, M, out);

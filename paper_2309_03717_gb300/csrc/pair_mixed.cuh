@@ -146,6 +146,67 @@ struct alignas(16) AntE {
 };
 static_assert(sizeof(AntE) == sizeof(AntRec), "fwd_layout reckons with one antenna record size");
 
+// two tracks for the forward pass of the ZHS kernels, halves x and y; the
+// midpoint of each
+struct TrackZ {
+  float2 mx, mxl, my, myl, mz, mzl;   // position, float-float
+  float2 bx, by, bz, nm1;
+  float2 tmh, tml, dtauh, dtaul;      // (t0 + t1)/(2 dt), (t1 - t0)/dt
+  float2 Eh, El;                      // exp(-z/H); a flat antenna array: the refractivity quotient instead
+  ZPartT<float2> zm;                  // flat antenna array: the z part of d
+  float2 amp;                         // -q K_A (t1 - t0)/dt
+  bool live;
+};
+
+template <int KIND, bool FLAT>
+__device__ __forceinline__ void load_track_pair(const float* T, int l, const MedParams& M, TrackZ& t) {
+  auto ld = [&](int f) { return *reinterpret_cast<const float2*>(T + f * kTileT + 2 * l); };
+  const float2 keep = ld(fm::AMPE);
+  t.live = keep.x != 0.0f || keep.y != 0.0f;
+  if (!t.live) return;
+  t.amp = neg(ld(fm::AMPZ));
+  const float2 half = bc<float2>(0.5f);
+  two_sum(ld(fm::X0), ld(fm::X1), t.mx, t.mxl);
+  two_sum(ld(fm::Y0), ld(fm::Y1), t.my, t.myl);
+  two_sum(ld(fm::Z0), ld(fm::Z1), t.mz, t.mzl);
+  t.mx = mul_rn(t.mx, half); t.mxl = mul_rn(t.mxl, half);
+  t.my = mul_rn(t.my, half); t.myl = mul_rn(t.myl, half);
+  t.mz = mul_rn(t.mz, half); t.mzl = mul_rn(t.mzl, half);
+  t.bx = ld(fm::BX); t.by = ld(fm::BY); t.bz = ld(fm::BZ);
+  two_sum(ld(fm::TAU0H), ld(fm::TAU1H), t.tmh, t.tml);
+  t.tml = add_rn(t.tml, add_rn(ld(fm::TAU0L), ld(fm::TAU1L)));
+  t.tmh = mul_rn(t.tmh, half);
+  t.tml = mul_rn(t.tml, half);
+  // a filtered track or padding next to a live one: an arrival far before every
+  // window, so that it deposits nothing
+  if (keep.x == 0.0f) t.tmh.x = -1e30f;
+  if (keep.y == 0.0f) t.tmh.y = -1e30f;
+  t.dtauh = ld(fm::DTAUH); t.dtaul = ld(fm::DTAUL);
+  t.nm1 = bc<float2>(M.nm1f);
+  if constexpr (KIND != C8R_UNIFORM) {
+    t.Eh = ld(fm::EMH); t.El = ld(fm::EML);
+    t.nm1 = mul_rn(bc<float2>(M.N0f), t.Eh);
+  }
+  if constexpr (FLAT) {
+    // per track as the per-pair arithmetic forms it, so the same values
+    float2 dzh, dzl, q0, q1;
+    two_sum(bc<float2>(M.flat_zh), neg(t.mz), dzh, dzl);
+    dzl = add_rn(dzl, sub_rn(bc<float2>(M.flat_zl), t.mzl));
+    refr_quotient(M, M.flat_Eh, M.flat_El, dzh.x, dzl.x, t.Eh.x, t.El.x, q0.x, q1.x);
+    refr_quotient(M, M.flat_Eh, M.flat_El, dzh.y, dzl.y, t.Eh.y, t.El.y, q0.y, q1.y);
+    t.zm = z_part(dzh, dzl, t.bz);
+    t.Eh = q0;
+    t.El = q1;
+  }
+}
+
+// an antenna in shared memory for those kernels, each value twice
+struct alignas(16) AntZ {
+  float2 x, y, xl, yl, tauh, taul, z, zl, Eh, El;
+  float pad[4];
+};
+static_assert(sizeof(AntZ) == sizeof(AntRec), "fwd_layout reckons with one antenna record size");
+
 // geometry shared by the forward and the adjoint Endpoint evaluation
 struct EndpointEvalM {
   GeoM g0, g1, gm;
@@ -353,6 +414,10 @@ struct OpsMixed {
   // for the float-float arrival after the main pass
   static constexpr bool kFastBins =
       FORM == C8R_ENDPOINT && !LIN && (KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL);
+  // ZHS in those media: the forward kernel evaluates two tracks at a time
+  static constexpr bool kTwoTracks =
+      FORM == C8R_ZHS && (KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL);
+  static constexpr int kFwdThreads = kTwoTracks ? kTileT / 2 : kTileT;
   // the form of x = R - w in the FP32 arrival (arrival_fast): the split one
   // for lines of sight near the vertical, the direct one otherwise.  Either is
   // exact to its own bound; the host picks the kernel per launch from the
@@ -379,7 +444,25 @@ struct OpsMixed {
   static constexpr int kAccRows = FORM == C8R_ZHS ? 2 : 1;
 
   // the antenna record that the forward and adjoint kernels hold in shared memory
+  using FwdAnt = std::conditional_t<kTwoTracks, AntZ, std::conditional_t<kFastBins, AntE, AntRec>>;
   using Ant = std::conditional_t<kFastBins, AntE, AntRec>;
+  static __device__ __forceinline__ void stage_ant(AntZ* p, const AntRec& A) {
+    AntZ z;
+    z.x = bc<float2>(A.xh); z.y = bc<float2>(A.yh); z.z = bc<float2>(A.zh);
+    z.xl = bc<float2>(A.xl); z.yl = bc<float2>(A.yl); z.zl = bc<float2>(A.zl);
+    z.tauh = bc<float2>(A.tauh); z.taul = bc<float2>(A.taul);
+    z.Eh = bc<float2>(A.Eah); z.El = bc<float2>(A.Eal);
+    z.pad[0] = z.pad[1] = z.pad[2] = z.pad[3] = 0.0f;
+    *p = z;
+  }
+  static __device__ __forceinline__ AntRec load_ant(const AntZ* p) {
+    AntRec r;
+    r.xh = p->x.x; r.yh = p->y.x; r.zh = p->z.x;
+    r.xl = p->xl.x; r.yl = p->yl.x; r.zl = p->zl.x;
+    r.tauh = p->tauh.x; r.taul = p->taul.x;
+    r.Eah = p->Eh.x; r.Eal = p->El.x;
+    return r;
+  }
   static __device__ __forceinline__ void stage_ant(Ant* p, const AntRec& A) {
     if constexpr (kFastBins) {
       AntE e;
@@ -428,6 +511,15 @@ struct OpsMixed {
       load(Tv, l, M, t);
   }
   static __device__ __forceinline__ bool live(const TrackE& t) { return t.amp != 0.0f; }
+  static __device__ __forceinline__ bool live(const TrackZ& t) { return t.live; }
+  // what a thread of the forward main pass holds: a track, or two of them
+  using FwdTrack = std::conditional_t<kTwoTracks, TrackZ, MainTrack>;
+  static __device__ __forceinline__ void load_fwd(const void* Tv, int l, const MedParams& M, FwdTrack& t) {
+    if constexpr (kTwoTracks)
+      load_track_pair<KIND, kFlat>(static_cast<const float*>(Tv), l, M, t);
+    else
+      load_main(Tv, l, M, t);
+  }
   static __device__ __forceinline__ bool live(const TrackM& t) { return t.amp != 0.0f; }
 
   // -------------------------------------------------------------------------
@@ -531,7 +623,7 @@ struct OpsMixed {
     const int N = M.n_bins;
     GeoM gm;
     if constexpr (kFlat)
-      geo_lite(A, t.mx, t.my, t.mxl, t.myl, t.zm, gm);
+      geo_lite(A.xh, A.yh, A.xl, A.yl, t.mx, t.my, t.mxl, t.myl, t.zm, gm);
     else
       geo_lite(A, t.mx, t.my, t.mz, t.mxl, t.myl, t.mzl, gm);
     if (gm.R0 == 0.0f) return;
@@ -547,7 +639,7 @@ struct OpsMixed {
     ff um, aD;
     if constexpr (kFlat) {
       geo_refine(gm, t.zm);
-      um = arrival_mixed_q<KIND>(M, A, gm, t.tmh, t.tml, t.qmh, t.qml, dop);
+      um = arrival_mixed_q<KIND>(M, A.tauh, A.taul, gm, t.tmh, t.tml, t.qmh, t.qml, dop);
       aD = doppler_ff(gm, t.bx, t.by, t.zm, t.nm1_m);
     } else {
       geo_refine(gm);
@@ -576,42 +668,122 @@ struct OpsMixed {
     const int khi = bin_raw(uhi, N, fhi);
     out.rec(klo == khi ? 2 : 3, ulo, uhi);
     if constexpr (LIN) {
-      // reading LD: the tent weights averaged over the interval
-      float slo, shi;
-      const int Jlo = lin_cell(ulo, N, slo);
-      const int Jhi = lin_cell(uhi, N, shi);
-      if (Jlo == Jhi) {
-        // inside one cell the tents are linear: the tent at the middle
-        dep_lin(out, N, Jlo, 0.5f * (slo + shi), Mx, My, Mz);
-        return;
-      }
-      const float invW = div_ap(1.0f, 2.0f * hh);
-      const LinEnds z = lin_ends(Jlo, slo, Jhi, shi, invW);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (i < z.n && z.k[i] >= 0 && z.k[i] < N) out.dep(z.k[i], Mx * z.w[i], My * z.w[i], Mz * z.w[i]);
-      const int kb = Jlo + 1 < 0 ? 0 : Jlo + 1;
-      const int ke = Jhi - 2 > N - 1 ? N - 1 : Jhi - 2;
-      if (kb <= ke) out.dep_box(kb, ke, Mx * invW, My * invW, Mz * invW);
-      return;
+      zhs_deposit_lin(ulo, uhi, hh, Mx, My, Mz, N, out);
+    } else {
+      const float invW = div_ap(1.0f, 2.0f * hh);  // 1 / interval length in bins (unused when in one bin)
+      zhs_deposit(klo, khi, klo == khi ? 1.0f : gap_to_next_edge(ulo, klo) * invW, fhi * invW, invW, Mx, My, Mz, N, out);
     }
-    // the interval's first bin takes the whole deposit (an interval inside one
-    // bin: weight 1, M x 1 = M exactly) or the share it covers, in one
-    // reduction either way, so that lanes of both kinds take one path
-    const bool one = klo == khi;
-    const float invW = div_ap(1.0f, 2.0f * hh);  // 1 / interval length in bins (unused when one)
-    const float wlo = one ? 1.0f : gap_to_next_edge(ulo, klo) * invW;
-    if (klo >= 0 && klo < N && wlo > 0.0f) out.dep(klo, Mx * wlo, My * wlo, Mz * wlo);
-    if (one) return;
-    // the partly covered last bin
-    if (khi >= 0 && khi < N) {
-      const float w = fhi * invW;
-      if (w > 0.0f) out.dep(khi, Mx * w, My * w, Mz * w);
-    }
-    // the whole bins in between (inside the window) all receive M / W
+  }
+
+  // the deposits of an evaluated ZHS interval [ulo, uhi] (bins klo, khi; M the
+  // whole deposit, invW = 1/W): the first bin takes it all (an interval inside
+  // one bin: weight 1, M x 1 = M exactly) or the share it covers, in one
+  // reduction either way, so that lanes of both kinds take one path; the partly
+  // covered last bin; and the whole bins in between, which all receive M / W
+  template <class Sink>
+  static __device__ __forceinline__ void zhs_deposit(int klo, int khi, float wlo, float whi, float invW, float Mx,
+                                                     float My, float Mz, int N, Sink& out) {
+    if ((unsigned)klo < (unsigned)N && wlo > 0.0f) out.dep(klo, Mx * wlo, My * wlo, Mz * wlo);
+    if (klo == khi) return;
+    if ((unsigned)khi < (unsigned)N && whi > 0.0f) out.dep(khi, Mx * whi, My * whi, Mz * whi);
     const int kb = klo + 1 < 0 ? 0 : klo + 1;
     const int ke = khi - 1 > N - 1 ? N - 1 : khi - 1;
     if (kb <= ke) out.dep_box(kb, ke, Mx * invW, My * invW, Mz * invW);
+  }
+  // the same for the linear deposit (reading LD): the tent weights averaged over
+  // the interval
+  template <class Sink>
+  static __device__ __forceinline__ void zhs_deposit_lin(ff ulo, ff uhi, float hh, float Mx, float My, float Mz, int N,
+                                                         Sink& out) {
+    float slo, shi;
+    const int Jlo = lin_cell(ulo, N, slo);
+    const int Jhi = lin_cell(uhi, N, shi);
+    if (Jlo == Jhi) {
+      // inside one cell the tents are linear: the tent at the middle
+      dep_lin(out, N, Jlo, 0.5f * (slo + shi), Mx, My, Mz);
+      return;
+    }
+    const float invW = div_ap(1.0f, 2.0f * hh);
+    const LinEnds z = lin_ends(Jlo, slo, Jhi, shi, invW);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i < z.n && z.k[i] >= 0 && z.k[i] < N) out.dep(z.k[i], Mx * z.w[i], My * z.w[i], Mz * z.w[i]);
+    const int kb = Jlo + 1 < 0 ? 0 : Jlo + 1;
+    const int ke = Jhi - 2 > N - 1 ? N - 1 : Jhi - 2;
+    if (kb <= ke) out.dep_box(kb, ke, Mx * invW, My * invW, Mz * invW);
+  }
+
+  // ZHS of two tracks against one antenna, the arithmetic of `zhs` in both halves
+  // (float2): 302 -> 170 warp instructions per 32 pairs.  Bound by the FP32 pipe
+  // (63 % of its cycles, the float-float sums) and, for a vertical shower on few
+  // antennas, by its reductions.  Measured with the accumulator copies, ms: 2e7
+  // tracks x 160 antennas 29.4 -> 25.6; 3e5 tracks x 512 antennas 1.61 -> 1.47;
+  // false when a half needs another form of it (the altitude difference
+  // within 1e-3 H, or a window too long for bins_of), with nothing deposited
+  template <class Sink>
+  static __device__ __forceinline__ bool zhs_two(const TrackZ& t, const AntZ& A, const MedParams& M, Sink& out) {
+    const int N = M.n_bins;
+    if (!LIN && N > kMagicBins / 2) return false;
+    GeoT<float2> g;
+    ffT<float2> um, aD;
+    if constexpr (kFlat) {
+      geo_lite(A.x, A.y, A.xl, A.yl, t.mx, t.my, t.mxl, t.myl, t.zm, g);
+      geo_refine(g, t.zm);
+      um = arrival_mixed_q<KIND>(M, A.tauh, A.taul, g, t.tmh, t.tml, t.Eh, t.El);
+      aD = doppler_ff(g, t.bx, t.by, t.zm, t.nm1);
+    } else {
+      float2 dzh, dzl, q0 = bc<float2>(0.0f), q1 = q0;
+      two_sum(A.z, neg(t.mz), dzh, dzl);
+      dzl = add_rn(dzl, sub_rn(A.zl, t.mzl));
+      if constexpr (KIND == C8R_EXPONENTIAL) {
+        if (!(fminf(fabsf(dzh.x), fabsf(dzh.y)) > -M.dz_series)) return false;
+        refr_quotient(M, A.Eh, A.El, dzh, dzl, t.Eh, t.El, q0, q1);
+      }
+      const ZPartT<float2> z = z_part(dzh, dzl, t.bz);
+      geo_lite(A.x, A.y, A.xl, A.yl, t.mx, t.my, t.mxl, t.myl, z, g);
+      geo_refine(g, z);
+      um = arrival_mixed_q<KIND>(M, A.tauh, A.taul, g, t.tmh, t.tml, q0, q1);
+      aD = doppler_ff(g, t.bx, t.by, z, t.nm1);
+    }
+    // |D|: D renormalised, so its sign is that of the high part
+    if (aD.h.x < 0.0f) aD.l.x = -aD.l.x;
+    if (aD.h.y < 0.0f) aD.l.y = -aD.l.y;
+    aD.h = abs_of(aD.h);
+    float2 hh, hl;  // |D| (t1 - t0)/(2 dt), float-float
+    two_prod(aD.h, t.dtauh, hh, hl);
+    hl = fma_rn(aD.h, t.dtaul, fma_rn(aD.l, t.dtauh, hl));
+    const float2 half = bc<float2>(0.5f);
+    hh = mul_rn(hh, half);
+    hl = mul_rn(hl, half);
+    ffT<float2> ulo, uhi;
+    two_sum(um.h, neg(hh), ulo.h, ulo.l);
+    ulo.l = add_rn(ulo.l, sub_rn(um.l, hl));
+    two_sum(um.h, hh, uhi.h, uhi.l);
+    uhi.l = add_rn(uhi.l, add_rn(um.l, hl));
+    // the deposit A beta_perp/R = -A V, V R^2 = d x (d x beta)
+    const float2 wx = fma_rn(g.s[1], t.bz, neg(mul_rn(g.s[2], t.by)));
+    const float2 wy = fma_rn(g.s[2], t.bx, neg(mul_rn(g.s[0], t.bz)));
+    const float2 wz = fma_rn(g.s[0], t.by, neg(mul_rn(g.s[1], t.bx)));
+    const float2 s = mul_rn(mul_rn(t.amp, mul_rn(g.y, g.y)), g.y);
+    const float2 Mx = mul_rn(s, fma_rn(g.s[1], wz, neg(mul_rn(g.s[2], wy))));
+    const float2 My = mul_rn(s, fma_rn(g.s[2], wx, neg(mul_rn(g.s[0], wz))));
+    const float2 Mz = mul_rn(s, fma_rn(g.s[0], wy, neg(mul_rn(g.s[1], wx))));
+    if constexpr (LIN) {
+      zhs_deposit_lin(ff{ulo.h.x, ulo.l.x}, ff{uhi.h.x, uhi.l.x}, hh.x, Mx.x, My.x, Mz.x, N, out);
+      zhs_deposit_lin(ff{ulo.h.y, ulo.l.y}, ff{uhi.h.y, uhi.l.y}, hh.y, Mx.y, My.y, Mz.y, N, out);
+    } else {
+      int klox, kloy, khix, khiy;
+      float2 klo, khi, flo, fhi;
+      bins_of(ulo, N, klox, kloy, klo, flo);
+      bins_of(uhi, N, khix, khiy, khi, fhi);
+      const float2 invW = rcp_ap(mul_rn(bc<float2>(2.0f), hh));  // 1 / interval length in bins
+      // gap_to_next_edge
+      const float2 gap = sub_rn(sub_rn(add_rn(klo, bc<float2>(1.0f)), ulo.h), ulo.l);
+      const float2 wlo = mul_rn(gap, invW), whi = mul_rn(fhi, invW);
+      zhs_deposit(klox, khix, klox == khix ? 1.0f : wlo.x, whi.x, invW.x, Mx.x, My.x, Mz.x, N, out);
+      zhs_deposit(kloy, khiy, kloy == khiy ? 1.0f : wlo.y, whi.y, invW.y, Mx.y, My.y, Mz.y, N, out);
+    }
+    return true;
   }
 
   // one endpoint of a pair in which some condition of the usual forms fails: its
@@ -673,8 +845,20 @@ struct OpsMixed {
   // whose bin the FP32 arrival leaves open, returned as kDeferEnd0/kDeferEnd1
   // bits after the other endpoint's deposit
   template <class Sink>
-  static __device__ __forceinline__ int pair_main(const MainTrack& t, const Ant* p, const MedParams& M, Sink& out) {
-    if constexpr (kFastBins) {
+  static __device__ __forceinline__ int pair_main(const FwdTrack& t, const FwdAnt* p, const void* Tv, int l,
+                                                  const MedParams& M, Sink& out) {
+    if constexpr (kTwoTracks) {
+      if (!zhs_two(t, *p, M, out)) {
+        // one half at a time, from the staged tile
+        const AntRec A = load_ant(p);
+        for (int h = 0; h < 2; ++h) {
+          TrackM one;
+          load(Tv, 2 * l + h, M, one);
+          if (live(one)) zhs(one, A, M, out);
+        }
+      }
+      return kDeferNone;
+    } else if constexpr (kFastBins) {
       GeoT<float2> g;
       FieldT<float2> f;
       int ka, kb;
@@ -1106,7 +1290,7 @@ struct OpsMixed {
     const int N = M.n_bins;
     GeoM gm;
     if constexpr (kFlat)
-      geo_lite(A, t.mx, t.my, t.mxl, t.myl, t.zm, gm);
+      geo_lite(A.xh, A.yh, A.xl, A.yl, t.mx, t.my, t.mxl, t.myl, t.zm, gm);
     else
       geo_lite(A, t.mx, t.my, t.mz, t.mxl, t.myl, t.mzl, gm);
     if (gm.R0 == 0.0f) return;
@@ -1115,7 +1299,7 @@ struct OpsMixed {
     ff um, aD;
     if constexpr (kFlat) {
       geo_refine(gm, t.zm);
-      um = arrival_mixed_q<KIND>(M, A, gm, t.tmh, t.tml, t.qmh, t.qml);
+      um = arrival_mixed_q<KIND>(M, A.tauh, A.taul, gm, t.tmh, t.tml, t.qmh, t.qml);
       aD = doppler_ff(gm, t.bx, t.by, t.zm, t.nm1_m);
     } else {
       geo_refine(gm);

@@ -1,6 +1,7 @@
-"""The one-bin Endpoint kernels evaluate a pair's two endpoints together and
-redo the rare pair (an emission point near the antenna's altitude or below it,
-an antenna behind the track) half by half.  Antennas spread through the shower's
+"""The one-bin Endpoint kernels evaluate a pair's two endpoints together, the
+ZHS forward kernels two tracks, and both redo the rare pair (an emission point
+near the antenna's altitude or below it, an antenna behind the track) half by
+half.  Antennas spread through the shower's
 own heights make those pairs common, next to usual ones; track counts around the
 128-track tile and antenna counts around the 32-antenna tile.  Traces and
 adjoint against the oracle at the mixed bar (1e-4 relative L2)."""
@@ -68,3 +69,24 @@ def test_traces_and_adjoint_with_antennas_among_the_tracks(n, n_ant, medium, for
     assert rel_l2(got[:, 0:6], tg_ref[:, 0:6]) <= TOL
     assert rel_l2(got[:, 8:11], tg_ref[:, 8:11]) <= TOL
     assert rel_l2(ag.cpu().numpy(), ag_ref) <= TOL
+
+
+@pytest.mark.parametrize("deposit", ["bin", "linear"])
+@pytest.mark.parametrize("medium", [None, UNIFORM])
+@pytest.mark.parametrize("n,n_ant,n_bins", [(1, 1, 2048), (2, 3, 7), (127, 31, 2048), (129, 33, 2048), (700, 5, 1),
+                                            (33, 2, (1 << 21) + 5)])
+def test_zhs_traces_with_antennas_among_the_tracks(n, n_ant, n_bins, medium, deposit):
+    from paper_2309_03717_gb300 import c8r
+    w, tracks = among_the_tracks(n, n_ant, medium)
+    if n_bins < 2048:
+        w["t_start_ns"] = w["t_start_ns"] + 200.0  # around the arrivals
+    tracks["q"][n // 2 :: 7] = 0.0  # filtered tracks next to kept ones
+    p = c8r.RadioProcess(w["medium"], w["ant_xyz"], w["t_start_ns"], n_bins, w["dt_ns"], "zhs", "mixed",
+                         deposit=deposit)
+    p.push(to_device(tracks))
+    got = p.traces().cpu().numpy()
+    p.close()
+    ref, _ = oracle.forward(oracle.tracks_from_ns(tracks), w["ant_xyz"], w["t_start_ns"] * 1e-9, n_bins,
+                            w["dt_ns"] * 1e-9, w["medium"], oracle.ZHS,
+                            deposit=oracle.DEPOSIT_LINEAR if deposit == "linear" else oracle.DEPOSIT_BIN)
+    assert rel_l2(got, ref) <= TOL
