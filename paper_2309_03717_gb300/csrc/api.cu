@@ -59,6 +59,7 @@ void fill_medium(MedParams& M, int kind, double n_or_N0, double H, int n_bins, d
   M.n_bins = n_bins;
   M.wait_limit = kWaitLimit;
   M.dt_ns = dt_ns;
+  M.inv_dt = 1.0 / dt_ns;
   M.inv_c_ns = 1.0 / kCns;
   M.eps_Cd = eps_C;
   M.eps_C = (float)eps_C;
@@ -139,6 +140,8 @@ void set_flat_array(MedParams& M, const double* pos_xyz, int n_ant) {
   const double E = std::exp(-z / M.H);
   M.flat_Eh = (float)E;
   M.flat_El = (float)(E - (double)M.flat_Eh);
+  M.flat_z = z;
+  M.flat_E = E;
 }
 
 void set_form_centroid(MedParams& M, const double* pos_xyz, int n_ant) {
@@ -550,7 +553,7 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   c->shape.a_tile = want < n_ant ? want : n_ant;
   c->shape.waves = c->user_waves > 0 ? c->user_waves : kDefaultWaves;
   c->trace_bytes = (size_t)n_ant * 3 * n_bins * (precision == C8R_FP64 ? 8 : 4);
-  c->acc_bytes = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(precision, formalism);
+  c->acc_bytes = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(formalism);
   c->shape.replicas = acc_replicas(precision, formalism, n_ant, n_bins, c->shape.a_tile, c->sm_count);
   c->acc_bytes *= c->shape.replicas;
   c->copies_used = 1;
@@ -609,8 +612,11 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
   if ((r = ensure_tiles(c, chunk)) != C8R_OK) return r;
   const bool lin = c->deposit == C8R_DEPOSIT_LINEAR;
   form_poll(c);
-  FwdShape shape = c->shape;  // of this push: with the accumulator copies it uses
-  shape.replicas = push_replicas(shape.replicas, n, c->n_bins, acc_rows(c->precision, c->formalism));
+  FwdShape shape = c->shape;  // of this push: its antenna tile and the accumulator copies it uses
+  if (c->user_a_tile == 0)
+    shape.a_tile = push_a_tile(shape.a_tile, (chunk + kTileT - 1) / kTileT, c->n_ant, c->precision, c->formalism,
+                               c->sm_count);
+  shape.replicas = push_replicas(shape.replicas, n, c->n_bins, acc_rows(c->formalism));
   if (capturing(st)) c->copies_all = true;
   if (shape.replicas > c->copies_used) c->copies_used = shape.replicas;
   for (int64_t off = 0; off < n; off += chunk) {
@@ -655,7 +661,7 @@ static cudaError_t fetch_acc(c8r_ctx* c, void* dst, bool clear, cudaStream_t st)
   const int n = copies_in_use(c, st);
   const bool fused = clear && c->acc_bytes / c->shape.replicas * n <= kFusedClear;
   cudaError_t e = launch_acc_to_traces(c->precision, c->d_acc, c->n_ant, c->n_bins,
-                                       acc_rows(c->precision, c->formalism), dst, false, fused, st, n);
+                                       acc_rows(c->formalism), dst, false, fused, st, n);
   if (e == cudaSuccess && fused) c->copies_used = 1;
   if (e == cudaSuccess && clear && !fused) e = zero_acc(c, st);
   return e;

@@ -351,7 +351,7 @@ int enqueue_ingest(c8r_batch* b, const TrackPtrs& tp, cudaStream_t st) {
 // (the split-form group, then the direct-form group, one launch each, each
 // with its own item counter: d_counter[0] and d_counter[3])
 int enqueue_kernel(c8r_batch* b, int n_items_limit, cudaStream_t st) {
-  const int rows = acc_rows(C8R_MIXED, b->formalism);
+  const int rows = acc_rows(b->formalism);
   const int n = std::min(b->n_items, n_items_limit);
   const int ns = std::min(b->n_items_split, n);
   const int first[2] = {0, ns}, count[2] = {ns, n - ns};
@@ -379,7 +379,7 @@ int enqueue(c8r_batch* b, const TrackPtrs& tp, float* out, int n_items_limit, cu
   if (r != C8R_OK) return r;
   if (out) {
     cudaError_t e = launch_acc_to_traces(C8R_MIXED, b->d_acc, b->total_ant, b->M.n_bins,
-                                         acc_rows(C8R_MIXED, b->formalism), out, true, false, st, b->replicas);
+                                         acc_rows(b->formalism), out, true, false, st, b->replicas);
     if (e != cudaSuccess) return bfail(b, C8R_ECUDA, std::string("batch fetch: ") + cudaGetErrorString(e));
   }
   return C8R_OK;
@@ -567,8 +567,8 @@ int c8r_batch_create(c8r_batch** out, int device, const c8r_batch_desc* d, int k
     *out = b;
     return C8R_ECUDA;
   }
-  b->replicas = acc_replicas(C8R_MIXED, b->formalism);
-  b->acc_bytes = (size_t)b->total_ant * b->M.n_bins * sizeof(float4) * acc_rows(C8R_MIXED, b->formalism) *
+  b->replicas = acc_replicas(b->formalism);
+  b->acc_bytes = (size_t)b->total_ant * b->M.n_bins * sizeof(float4) * acc_rows(b->formalism) *
                  b->replicas;
   if (dev_malloc(&b->d_acc, b->acc_bytes) != cudaSuccess) {
     cudaGetLastError();

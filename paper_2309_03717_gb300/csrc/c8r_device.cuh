@@ -91,7 +91,7 @@ struct MedParams {
   double n;              // uniform index
   double N0, H, invH;    // exponential
   double R_E;            // spherical: Earth radius (m)
-  double dt_ns;
+  double dt_ns, inv_dt;  // bin width and its reciprocal (per ns)
   double inv_c_ns;       // 1 / c in ns/m
   double eps_Cd;         // near-Cherenkov threshold (FP64 path)
   // float-float constants of the mixed path
@@ -121,6 +121,7 @@ struct MedParams {
   // track (OpsMixed::kFlat)
   int flat;
   float flat_zh, flat_zl, flat_Eh, flat_El;
+  double flat_z, flat_E;  // the same for the FP64 path
 };
 
 // ---------------------------------------------------------------------------

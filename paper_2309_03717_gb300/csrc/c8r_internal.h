@@ -25,8 +25,8 @@ struct TrackPtrs {
 size_t tile_bytes(int precision);
 // bytes of one accumulator element (one bin of one antenna: x, y, z, pad)
 inline size_t acc_elem_bytes(int precision) { return precision == C8R_FP64 ? 32 : 16; }
-// accumulator rows per antenna: the mixed ZHS path adds a row of box edges
-inline int acc_rows(int precision, int formalism) { return precision == C8R_MIXED && formalism == C8R_ZHS ? 2 : 1; }
+// accumulator rows per antenna: ZHS adds a row of box edges
+inline int acc_rows(int formalism) { return formalism == C8R_ZHS ? 2 : 1; }
 // copies of the accumulator the forward kernel spreads its reductions over (CTA
 // range r adds into copy r % replicas; the fetch sums them).  Most reductions go
 // into the few bins per antenna that the pulse arrives in, a few lines of L2
@@ -42,7 +42,7 @@ inline int acc_rows(int precision, int formalism) { return precision == C8R_MIXE
 //
 // the batched launch: its many showers' antenna tiles spread the CTAs, so 2
 // copies for ZHS and 1 for Endpoint
-inline int acc_replicas(int precision, int formalism) { return acc_rows(precision, formalism) == 2 ? 2 : 1; }
+inline int acc_replicas(int formalism) { return acc_rows(formalism) == 2 ? 2 : 1; }
 // bytes of the accumulator rows in use at a time (forward_grid groups the
 // antenna tiles by it) and of all copies.  Above L2's 129 MB: the bins that the
 // pulses reach, a small part of the rows, are what has to stay there
@@ -58,7 +58,7 @@ inline int acc_replicas(int precision, int formalism, int n_ant, int n_bins, int
   const int64_t ant_tiles = (n_ant + a_tile - 1) / a_tile;
   const int64_t per_tile = (int64_t)sm_count * 6 / (ant_tiles > 0 ? ant_tiles : 1);
   const int64_t want = per_tile < 64 ? 1 : per_tile / 22;
-  const size_t one = (size_t)n_ant * n_bins * 16 * acc_rows(precision, formalism);
+  const size_t one = (size_t)n_ant * n_bins * 16 * acc_rows(formalism);
   const int64_t fit = (int64_t)(kAccBudget / (one > 0 ? one : 1));
   int r = 1;
   while (r < 16 && r * 2 <= want && r * 2 <= fit) r *= 2;
@@ -71,6 +71,27 @@ inline int push_replicas(int most, int64_t n, int n_bins, int rows) {
   int r = 1;
   while (r * 2 <= most && (int64_t)r * 4 * n_bins * rows <= n) r *= 2;
   return r;
+}
+// antennas per CTA of a forward launch over n_tiles track tiles, `a_tile` at
+// most.  A CTA walks its antennas one after the other, so few CTAs with many
+// antennas leave the device waiting for the last of them, and each CTA costs its
+// set-up and the per-track preparation once more: the tile is halved until the
+// launch has enough CTAs per SM (14; 28 of the ZHS kernels' 64 threads), down to
+// 4 antennas (FP64, where a pair takes longest: 2, or 1 below one CTA per SM).
+// Measured, us per push with 32 / 16 / 8 / 4 / 2 antennas: Endpoint, 64 antennas x
+// 3e4 tracks 55 / 46 / 40 / 40 / 50, 160 x 3e4 69 / 60 / 62 / 75 / 102, 160 x 3e3
+// 28 / 24 / 23 / 23 / 24; ZHS, 160 x 3e4 99 / 78 / 75 / 74 / 72; FP64 Endpoint, 16
+// antennas x 1e5 - / 530 / 362 / 342 / 367, 64 x 3e3 134 / 77 / 73 / 61 / 67; FP64
+// ZHS, 8 antennas x 1e5 - / - / 416 / 261 / 193
+inline int push_a_tile(int a_tile, int64_t n_tiles, int n_ant, int precision, int formalism, int sm_count) {
+  const bool f64 = precision == C8R_FP64;
+  const int64_t enough = (int64_t)sm_count * (!f64 && formalism == C8R_ZHS ? 28 : 14);
+  const int least = f64 ? 2 : 4;
+  auto ctas = [&](int a) { return n_tiles * ((n_ant + a - 1) / a); };
+  int a = a_tile;
+  while (a > least && ctas(a) < enough) a = (a + 1) / 2 > least ? (a + 1) / 2 : least;
+  if (f64 && a == least && ctas(a) < sm_count) a = 1;
+  return a;
 }
 // accumulator [replicas][n_ant][rows][n_bins] -> traces [n_ant][3][n_bins]: the
 // copies are summed; with rows == 2 the second row (box edges) is integrated over

@@ -173,6 +173,16 @@ struct GlobalSink<double> {
     atomicAdd(&row[k].y, y);
     atomicAdd(&row[k].z, z);
   }
+  // the same vector into bins k0..k1, as GlobalSink<float> adds it
+  __device__ __forceinline__ void dep_box(int k0, int k1, double x, double y, double z) {
+    if (k1 - k0 < 2) {
+      dep(k0, x, y, z);
+      if (k1 > k0) dep(k1, x, y, z);
+      return;
+    }
+    dep(n + k0, x, y, z);
+    if (k1 + 1 < n) dep(n + k1 + 1, -x, -y, -z);
+  }
   __device__ __forceinline__ void rec(int, ff, ff) {}
   __device__ __forceinline__ void rec(int, double, double) {}
 };
@@ -186,6 +196,7 @@ struct ArrivalSink {
   __device__ __forceinline__ void dep(int, float, float, float) {}
   __device__ __forceinline__ void dep(int, double, double, double) {}
   __device__ __forceinline__ void dep_box(int, int, float, float, float) {}
+  __device__ __forceinline__ void dep_box(int, int, double, double, double) {}
   __device__ __forceinline__ void rec(int b, ff ua, ff ub) {
     float fa, fb;
     int ka = bin_raw(ua, N, fa), kb = bin_raw(ub, N, fb);

@@ -15,6 +15,13 @@ cudaError_t launch_forward_f64(int formalism, bool lin, const void* tiles, int64
 cudaError_t launch_arrivals_f64(int formalism, const void* tiles, int64_t n, const AntRec* ants, int n_ant,
                                 const MedParams& M, int32_t* branch, int32_t* bin, float* frac, cudaStream_t st) {
   const unsigned blocks = (unsigned)((n * (int64_t)n_ant + 255) / 256);
+  if (plain_medium(M)) {
+    if (formalism == C8R_ENDPOINT)
+      k_arrivals<OpsF64Plain<C8R_ENDPOINT>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin, frac);
+    else
+      k_arrivals<OpsF64Plain<C8R_ZHS>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin, frac);
+    return cudaGetLastError();
+  }
   if (formalism == C8R_ENDPOINT)
     k_arrivals<OpsF64<C8R_ENDPOINT>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin, frac);
   else

@@ -137,54 +137,79 @@ constexpr int kFetchBins = 4;
 constexpr int kFetchCluster = 8;
 static_assert(kScanT / 32 == 8 && kFetchCluster == 8, "sum_before8 takes eight totals");
 
-// From eight float-float totals of three components (t[c][q]), the sum of the
-// first `n` (before) and of all (tot), in every lane of the warp: lane 8c + q
-// takes one total and three shuffles add them
-__device__ __forceinline__ void sum_before8(const ff (*t)[8], int n, ff before[3], ff tot[3]) {
+// the running sums of the fetch: float-float for the mixed path (on the FP32
+// pipe; FP64 runs at 1/64 of its rate here), FP64 for the FP64 path
+__device__ __forceinline__ double ff_sum(double a, double b) { return a + b; }
+__device__ __forceinline__ double ff_add_f(double a, double b) { return a + b; }
+__device__ __forceinline__ float rounded(ff a) { return __fadd_rn(a.h, a.l); }
+__device__ __forceinline__ double rounded(double a) { return a; }
+__device__ __forceinline__ ff from_lane(ff a, int l) {
+  return ff{__shfl_sync(0xffffffffu, a.h, l), __shfl_sync(0xffffffffu, a.l, l)};
+}
+__device__ __forceinline__ double from_lane(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+template <typename T>
+struct SumOf;
+template <>
+struct SumOf<float> {
+  using type = ff;
+};
+template <>
+struct SumOf<double> {
+  using type = double;
+};
+
+// From eight totals of three components (t[c][q]), the sum of the first `n`
+// (before) and of all (tot), in every lane of the warp: lane 8c + q takes one
+// total and three shuffles add them
+template <class S>
+__device__ __forceinline__ void sum_before8(const S (*t)[8], int n, S before[3], S tot[3]) {
   const int lane = threadIdx.x & 31, q = lane & 7;
-  ff all = lane < 24 ? t[lane >> 3][q] : ff{0.0f, 0.0f};
-  ff pre = q < n ? all : ff{0.0f, 0.0f};
+  S all = lane < 24 ? t[lane >> 3][q] : S{};
+  S pre = q < n ? all : S{};
 #pragma unroll
   for (int d = 1; d < 8; d <<= 1) {
-    all = ff_sum(all, ff{__shfl_xor_sync(0xffffffffu, all.h, d), __shfl_xor_sync(0xffffffffu, all.l, d)});
-    pre = ff_sum(pre, ff{__shfl_xor_sync(0xffffffffu, pre.h, d), __shfl_xor_sync(0xffffffffu, pre.l, d)});
+    all = ff_sum(all, from_lane(all, lane ^ d));
+    pre = ff_sum(pre, from_lane(pre, lane ^ d));
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    before[c] = ff{__shfl_sync(0xffffffffu, pre.h, 8 * c), __shfl_sync(0xffffffffu, pre.l, 8 * c)};
-    tot[c] = ff{__shfl_sync(0xffffffffu, all.h, 8 * c), __shfl_sync(0xffffffffu, all.l, 8 * c)};
+    before[c] = from_lane(pre, 8 * c);
+    tot[c] = from_lane(all, 8 * c);
   }
 }
 
-__global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(float4* acc, int n_bins, float* out, bool add,
-                                                               bool clear, int replicas, int64_t stride) {
+template <typename T>
+__global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(typename AccOf<T>::type* acc, int n_bins, T* out,
+                                                               bool add, bool clear, int replicas, int64_t stride) {
   namespace cg = cooperative_groups;
+  using S = typename SumOf<T>::type;
+  using acc4 = typename AccOf<T>::type;
   const cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank(), n_cta = (int)cluster.num_blocks();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __shared__ ff warp_tot[3][kScanT / 32];
-  __shared__ ff cta_tot[2][3][kFetchCluster];  // the cluster's totals, of this round and the next
-  if (threadIdx.x < 6 * kFetchCluster) cta_tot[0][0][threadIdx.x] = ff{0.0f, 0.0f};  // absent CTAs count as zero
+  __shared__ S warp_tot[3][kScanT / 32];
+  __shared__ S cta_tot[2][3][kFetchCluster];  // the cluster's totals, of this round and the next
+  if (threadIdx.x < 6 * kFetchCluster) cta_tot[0][0][threadIdx.x] = S{};  // absent CTAs count as zero
   cluster.sync();
   const int a = blockIdx.x / n_cta;
-  float4* direct = acc + (size_t)a * 2 * n_bins;
-  float* o = out + (size_t)a * 3 * n_bins;
-  ff carry[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+  acc4* direct = acc + (size_t)a * 2 * n_bins;
+  T* o = out + (size_t)a * 3 * n_bins;
+  S carry[3] = {S{}, S{}, S{}};
   int buf = 0;
   for (int64_t base = 0; base < n_bins; base += (int64_t)n_cta * kScanT * kFetchBins, buf ^= 1) {
     const int64_t k0 = base + ((int64_t)rank * kScanT + threadIdx.x) * kFetchBins;
-    ff e[kFetchBins][3], d[kFetchBins][3];
+    S e[kFetchBins][3], d[kFetchBins][3];
 #pragma unroll
     for (int b = 0; b < kFetchBins; ++b)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) e[b][c] = d[b][c] = ff{0.0f, 0.0f};
+      for (int c = 0; c < 3; ++c) e[b][c] = d[b][c] = S{};
 #pragma unroll 2
     for (int r = 0; r < replicas; ++r) {
 #pragma unroll
       for (int b = 0; b < kFetchBins; ++b) {
         if (k0 + b >= n_bins) continue;
-        const float4* p = direct + k0 + b + r * stride;
-        const float4 u = p[0], w = p[n_bins];
+        const acc4* p = direct + k0 + b + r * stride;
+        const acc4 u = p[0], w = p[n_bins];
         d[b][0] = ff_add_f(d[b][0], u.x);
         d[b][1] = ff_add_f(d[b][1], u.y);
         d[b][2] = ff_add_f(d[b][2], u.z);
@@ -194,7 +219,7 @@ __global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(float4* acc, int 
       }
     }
     if (clear) {
-      const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      const acc4 zero{T(0), T(0), T(0), T(0)};
       for (int r = 0; r < replicas; ++r)
 #pragma unroll
         for (int b = 0; b < kFetchBins; ++b)
@@ -202,23 +227,23 @@ __global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(float4* acc, int 
     }
     // the edges before this thread's bins: of the lanes before it, of the warps
     // before its own, and of the CTAs before its own
-    ff lanes[3];
+    S lanes[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      ff inc = e[0][c];
+      S inc = e[0][c];
 #pragma unroll
       for (int b = 1; b < kFetchBins; ++b) inc = ff_sum(inc, e[b][c]);
 #pragma unroll
       for (int s = 1; s < 32; s <<= 1) {
-        const ff u{__shfl_up_sync(0xffffffffu, inc.h, s), __shfl_up_sync(0xffffffffu, inc.l, s)};
+        const S u = from_lane(inc, lane >= s ? lane - s : lane);
         if (lane >= s) inc = ff_sum(inc, u);
       }
       if (lane == 31) warp_tot[c][wid] = inc;
-      lanes[c] = ff{__shfl_up_sync(0xffffffffu, inc.h, 1), __shfl_up_sync(0xffffffffu, inc.l, 1)};
-      if (lane == 0) lanes[c] = ff{0.0f, 0.0f};
+      lanes[c] = from_lane(inc, lane > 0 ? lane - 1 : 0);
+      if (lane == 0) lanes[c] = S{};
     }
     __syncthreads();
-    ff run[3], tot[3];
+    S run[3], tot[3];
     sum_before8(warp_tot, wid, run, tot);
 #pragma unroll
     for (int c = 0; c < 3; ++c) run[c] = ff_sum(run[c], lanes[c]);
@@ -226,12 +251,12 @@ __global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(float4* acc, int 
       // every CTA's totals to every CTA; two buffers, so that a round's totals
       // are not overwritten before the slowest CTA has read them
       if (threadIdx.x < n_cta) {
-        ff(*peer)[3][kFetchCluster] = cluster.map_shared_rank(cta_tot, threadIdx.x);
+        S(*peer)[3][kFetchCluster] = cluster.map_shared_rank(cta_tot, threadIdx.x);
 #pragma unroll
         for (int c = 0; c < 3; ++c) peer[buf][c][rank] = tot[c];
       }
       cluster.sync();
-      ff before[3];
+      S before[3];
       sum_before8(cta_tot[buf], rank, before, tot);
 #pragma unroll
       for (int c = 0; c < 3; ++c) run[c] = ff_sum(before[c], run[c]);
@@ -249,9 +274,8 @@ __global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(float4* acc, int 
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         run[c] = ff_sum(run[c], e[b][c]);
-        const ff s = ff_sum(run[c], d[b][c]);
-        const float x = __fadd_rn(s.h, s.l);
-        float* q = o + (size_t)c * n_bins + k0 + b;
+        const T x = rounded(ff_sum(run[c], d[b][c]));
+        T* q = o + (size_t)c * n_bins + k0 + b;
         *q = add ? *q + x : x;
       }
     }
@@ -290,8 +314,11 @@ cudaError_t launch_acc_to_traces(int precision, void* acc, int n_ant, int n_bins
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_acc_scan_to_traces, static_cast<float4*>(acc), n_bins, static_cast<float*>(out),
-                              add, clear, replicas, stride);
+    if (precision == C8R_FP64)
+      return cudaLaunchKernelEx(&cfg, k_acc_scan_to_traces<double>, static_cast<Acc4D*>(acc), n_bins,
+                                static_cast<double*>(out), add, clear, replicas, stride);
+    return cudaLaunchKernelEx(&cfg, k_acc_scan_to_traces<float>, static_cast<float4*>(acc), n_bins,
+                              static_cast<float*>(out), add, clear, replicas, stride);
   }
   if (precision == C8R_FP64) {
     k_acc_to_traces_f64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(static_cast<Acc4D*>(acc), n, n_bins,

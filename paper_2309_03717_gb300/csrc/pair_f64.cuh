@@ -136,7 +136,7 @@ struct OpsF64 {
   static constexpr bool kFastBins = false;
   static constexpr int kBwdMinBlocks = 2;
   static constexpr int kBwdGridBlocks = 2;
-  static constexpr int kAccRows = 1;      // no box deposits
+  static constexpr int kAccRows = FORM == C8R_ZHS ? 2 : 1;  // as the plain media's kernels (OpsF64Plain)
 
   using Ant = AntRec;
   static __device__ __forceinline__ void stage_ant(AntRec* p, const AntRec& A) { *p = A; }
@@ -654,7 +654,260 @@ struct OpsF64 {
   }
 };
 
+// ---------------------------------------------------------------------------
+// The forward pass and the arrival listing in the plain media (uniform,
+// exponential) with the one-bin deposit.  Bound by the FP64 pipe, which on this
+// part runs at 1/64 of the FP32 rate, so the arithmetic is arranged for few FP64
+// operations: one reciprocal square root and two reciprocals per emission point
+// in place of a square root and five quotients, fused multiply-adds, what
+// depends on the track alone formed once per track and held in registers, bins
+// from the low word of a rounded-down sum.  About 90 -> 42 FP64 operations per
+// emission point; and a ZHS interval's whole bins go in as a box (two edges)
+// rather than bin by bin.  Measured, ms: 1e5 tracks x 16 antennas Endpoint in the
+// uniform medium 0.92 -> 0.49, 1e5 x 160 ZHS in the exponential one 6.2 -> 2.3;
+// errors against a 64-bit evaluation in plain torch unchanged (1e-12, 8e-12).
+// ---------------------------------------------------------------------------
+// 1/sqrt(x) and 1/x for normal x: the hardware's approximation (20 bits or more)
+// and one third-order step (Householder's iteration: the residual e = 1 - x y^2
+// or 1 - x r is of order 2^-20, and what is left is of order e^3)
+__device__ __forceinline__ double rsqrt_f64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+  return __fma_rn(__fma_rn(e, 0.375, 0.5), __dmul_rn(y, e), y);
+}
+__device__ __forceinline__ double rcp_f64(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = __fma_rn(-x, r, 1.0);
+  return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+
+// floor of an arrival position and its bin: k inside the window, or -1.  1.5 x
+// 2^52 added with rounding down leaves floor(u) in the low word for |u| < 2^31;
+// the high word tells whether it is one of 0 .. 2^32 - 1
+struct FloorD {
+  double k;
+  int bin;
+};
+__device__ __forceinline__ FloorD floor_bin(double u, int n_bins) {
+  const double magic = 6755399441055744.0;
+  const double t = __dadd_rd(u, magic);
+  const int lo = __double2loint(t);
+  return FloorD{__dsub_rn(t, magic),
+                __double2hiint(t) == 0x43380000 && (unsigned)lo < (unsigned)n_bins ? lo : -1};
+}
+
+template <int FORM>
+struct OpsF64Plain {
+  using acc_t = double;
+  static constexpr int kPrec = C8R_FP64;
+  static constexpr int kTileBytes = kTileBytesF64;
+  static constexpr int kMinBlocks = 4;
+  static constexpr int kFwdThreads = kTileT;
+  static constexpr bool kDefers = FORM == C8R_ENDPOINT;  // near-Cherenkov pairs, as OpsF64
+  static constexpr bool kFastBins = false;
+  static constexpr int kAccRows = FORM == C8R_ZHS ? 2 : 1;  // ZHS: box edges in the second row
+
+  // an emission point of the track
+  struct Point {
+    double x, y, z, t;
+    double n;  // refractive index
+    double E;  // exp(-z/H)
+    double r;  // n_avg - 1 where every antenna has the same (uniform medium, flat array)
+  };
+  struct FwdTrack {
+    Point p[FORM == C8R_ENDPOINT ? 2 : 1];  // start and end, or the midpoint
+    double bx, by, bz;
+    double amp;  // q K/dt, or q K_A (t1 - t0)/dt
+    double hw;   // ZHS: (t1 - t0)/(2 dt)
+  };
+  using FwdAnt = AntRec;
+  using Ant = AntRec;
+  static __device__ __forceinline__ void stage_ant(AntRec* p, const AntRec& A) { *p = A; }
+  static __device__ __forceinline__ AntRec load_ant(const AntRec* p) { return *p; }
+
+  // n_avg - 1 of the path from altitude z_e to z_a, dz = z_a - z_e, in the
+  // exponential medium (the series within 1e-3 H)
+  static __device__ __forceinline__ double refr(const MedParams& M, double Ea, double Ee, double dz) {
+    const double x = __dmul_rn(dz, M.invH);
+    double ratio;
+    if (fabs(x) > 1e-3)
+      ratio = __dmul_rn(__dsub_rn(Ee, Ea), rcp_f64(x));
+    else
+      ratio = Ee * (1.0 + x * (-0.5 + x * (1.0 / 6.0 + x * (-1.0 / 24.0 + x * (1.0 / 120.0)))));
+    return __dmul_rn(M.N0, ratio);
+  }
+  static __device__ __forceinline__ void point(const MedParams& M, double x, double y, double z, double t, double E,
+                                               Point& p) {
+    p.x = x;
+    p.y = y;
+    p.z = z;
+    p.t = t;
+    p.E = E;
+    p.r = M.n - 1.0;
+    p.n = M.n;
+    if (M.kind != C8R_UNIFORM) p.n = __fma_rn(M.N0, E, 1.0);
+    if (M.flat) p.r = refr(M, M.flat_E, E, __dsub_rn(M.flat_z, z));
+  }
+  static __device__ __forceinline__ void load_fwd(const void* Tv, int l, const MedParams& M, FwdTrack& t) {
+    const double* T = static_cast<const double*>(Tv);
+    const double q = TF(fd::Q);
+    t.amp = q;
+    if (q == 0.0) return;
+    t.bx = TF(fd::BX);
+    t.by = TF(fd::BY);
+    t.bz = TF(fd::BZ);
+    if constexpr (FORM == C8R_ENDPOINT) {
+      t.amp = q * (kKendpoint / (M.dt_ns * 1e-9));
+      point(M, TF(fd::X0), TF(fd::Y0), TF(fd::Z0), TF(fd::T0), TF(fd::E0), t.p[0]);
+      point(M, TF(fd::X1), TF(fd::Y1), TF(fd::Z1), TF(fd::T1), TF(fd::E1), t.p[1]);
+    } else {
+      const double dte = TF(fd::T1) - TF(fd::T0);
+      t.hw = 0.5 * dte * M.inv_dt;
+      t.amp = q * kKzhs * dte * M.inv_dt;
+      midpoint(Tv, l, M, t.p[0]);
+    }
+  }
+  static __device__ __forceinline__ void midpoint(const void* Tv, int l, const MedParams& M, Point& p) {
+    const double* T = static_cast<const double*>(Tv);
+    point(M, 0.5 * (TF(fd::X0) + TF(fd::X1)), 0.5 * (TF(fd::Y0) + TF(fd::Y1)), 0.5 * (TF(fd::Z0) + TF(fd::Z1)),
+          0.5 * (TF(fd::T0) + TF(fd::T1)), TF(fd::EM), p);
+  }
+  static __device__ __forceinline__ bool live(const FwdTrack& t) { return t.amp != 0.0; }
+
+  // propagator and field: rhat, V = rhat (rhat.beta) - beta, D, 1/R and the
+  // arrival position u; false when the emission point sits on the antenna
+  struct Eval {
+    double V[3], D, iR, u;
+  };
+  static __device__ __forceinline__ bool eval(const FwdTrack& t, const Point& p, const AntRec& A, const MedParams& M,
+                                              Eval& e) {
+    const double dx = __dsub_rn(A.x, p.x), dy = __dsub_rn(A.y, p.y), dz = __dsub_rn(A.z, p.z);
+    const double S = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
+    if (!(S >= 2.2250738585072014e-308)) return false;
+    e.iR = rsqrt_f64(S);
+    double R = __dmul_rn(S, e.iR);
+    R = __fma_rn(__fma_rn(-R, R, S), __dmul_rn(0.5, e.iR), R);
+    const double rx = __dmul_rn(dx, e.iR), ry = __dmul_rn(dy, e.iR), rz = __dmul_rn(dz, e.iR);
+    const double c = __fma_rn(t.bz, rz, __fma_rn(t.by, ry, __dmul_rn(t.bx, rx)));
+    e.V[0] = __fma_rn(c, rx, -t.bx);
+    e.V[1] = __fma_rn(c, ry, -t.by);
+    e.V[2] = __fma_rn(c, rz, -t.bz);
+    e.D = __fma_rn(-p.n, c, 1.0);
+    double r = p.r;
+    if (M.kind != C8R_UNIFORM && !M.flat) r = refr(M, A.Ea, p.E, dz);
+    e.u = __dmul_rn(__fma_rn(__fma_rn(r, R, R), M.inv_c_ns, __dsub_rn(p.t, A.t_ref)), M.inv_dt);
+    return true;
+  }
+
+  template <class Sink>
+  static __device__ __forceinline__ int pair_main(const FwdTrack& t, const AntRec* pa, const void*, int,
+                                                  const MedParams& M, Sink& out) {
+    const AntRec& A = *pa;
+    const int N = M.n_bins;
+    if constexpr (FORM == C8R_ENDPOINT) {
+      Eval e0, e1;
+      if (!eval(t, t.p[0], A, M, e0) || !eval(t, t.p[1], A, M, e1)) return kDeferNone;
+      if (!(fmin(fabs(e0.D), fabs(e1.D)) >= M.eps_Cd)) return kDeferPair;
+      out.rec(0, e0.u, e1.u);
+      const int ka = floor_bin(e0.u, N).bin, kb = floor_bin(e1.u, N).bin;
+      const double s0 = __dmul_rn(__dmul_rn(t.amp, e0.iR), rcp_f64(e0.D));
+      const double s1 = -__dmul_rn(__dmul_rn(t.amp, e1.iR), rcp_f64(e1.D));
+      // both in one bin: added in registers
+      const bool same = ka >= 0 && ka == kb;
+      if (same) {
+        out.dep(ka, __fma_rn(s1, e1.V[0], s0 * e0.V[0]), __fma_rn(s1, e1.V[1], s0 * e0.V[1]),
+                __fma_rn(s1, e1.V[2], s0 * e0.V[2]));
+      } else {
+        if (ka >= 0) out.dep(ka, s0 * e0.V[0], s0 * e0.V[1], s0 * e0.V[2]);
+        if (kb >= 0) out.dep(kb, s1 * e1.V[0], s1 * e1.V[1], s1 * e1.V[2]);
+      }
+    } else {
+      Eval e;
+      if (!eval(t, t.p[0], A, M, e)) return kDeferNone;
+      const double h = __dmul_rn(fabs(e.D), t.hw);
+      const double u_lo = __dsub_rn(e.u, h), u_hi = __dadd_rn(e.u, h);
+      const FloorD lo = floor_bin(u_lo, N), hi = floor_bin(u_hi, N);
+      const bool one = lo.k == hi.k;
+      out.rec(one ? 2 : 3, u_lo, u_hi);
+      const double s = -__dmul_rn(t.amp, e.iR);  // beta_perp = -V
+      const double invW = one ? 1.0 : rcp_f64(__dadd_rn(h, h));
+      // the share of the interval in its first bin (all of it when it has one),
+      // in its last, and 1/W in each whole bin between
+      if (lo.bin >= 0) {
+        const double w = one ? s : s * (__dsub_rn(lo.k + 1.0, u_lo) * invW);
+        out.dep(lo.bin, w * e.V[0], w * e.V[1], w * e.V[2]);
+      }
+      if (one) return kDeferNone;
+      if (hi.bin >= 0) {
+        const double w = s * (__dsub_rn(u_hi, hi.k) * invW);
+        out.dep(hi.bin, w * e.V[0], w * e.V[1], w * e.V[2]);
+      }
+      const double kb = fmax(lo.k + 1.0, 0.0), ke = fmin(hi.k - 1.0, (double)(N - 1));
+      if (kb <= ke) {
+        const double w = s * invW;
+        out.dep_box((int)kb, (int)ke, w * e.V[0], w * e.V[1], w * e.V[2]);
+      }
+    }
+    return kDeferNone;
+  }
+
+  // a near-Cherenkov Endpoint pair (reading C): the midpoint and its linearised
+  // arrivals
+  template <class Sink>
+  static __device__ __forceinline__ void near_pair(const void* Tv, int l, const AntRec& A, const MedParams& M,
+                                                   Sink& out) {
+    const double* T = static_cast<const double*>(Tv);
+    const int N = M.n_bins;
+    FwdTrack t;
+    t.bx = TF(fd::BX);
+    t.by = TF(fd::BY);
+    t.bz = TF(fd::BZ);
+    midpoint(Tv, l, M, t.p[0]);
+    Eval e;
+    if (!eval(t, t.p[0], A, M, e)) return;
+    const double h = e.D * (0.5 * (TF(fd::T1) - TF(fd::T0)) * M.inv_dt);
+    const double ua = e.u - h, ub = e.u + h;
+    out.rec(1, ua, ub);
+    const FloorD a = floor_bin(ua, N), b = floor_bin(ub, N);
+    if (a.k == b.k) return;  // both linearised arrivals in one bin: zero
+    const double s = TF(fd::Q) * (kKendpoint / (M.dt_ns * 1e-9)) * e.iR * rcp_f64(e.D);
+    if (a.bin >= 0) out.dep(a.bin, s * e.V[0], s * e.V[1], s * e.V[2]);
+    if (b.bin >= 0) out.dep(b.bin, -s * e.V[0], -s * e.V[1], -s * e.V[2]);
+  }
+  // set-aside pairs come with the staged tile and the lane
+  struct Track {
+    const void* T;
+    int l;
+  };
+  static __device__ __forceinline__ void load(const void* Tv, int l, const MedParams&, Track& t) {
+    t.T = Tv;
+    t.l = l;
+  }
+  template <class Sink>
+  static __device__ __forceinline__ void pair_deferred(const Track& t, const AntRec& A, const MedParams& M,
+                                                       Sink& out) {
+    if constexpr (kDefers) near_pair(t.T, t.l, A, M, out);
+  }
+  template <class Sink>
+  static __device__ __forceinline__ void end_deferred(const void*, int, const AntRec&, const MedParams&, Sink&, int) {}
+  static __device__ __forceinline__ bool near_zero_fast(const void*, int, const AntRec&, const MedParams&) {
+    return false;
+  }
+  // one pair from a tile (the arrival listing)
+  template <class Sink>
+  static __device__ __forceinline__ void fwd(const void* Tv, int l, const AntRec& A, const MedParams& M, Sink& out) {
+    FwdTrack t;
+    load_fwd(Tv, l, M, t);
+    if (live(t) && pair_main(t, &A, Tv, l, M, out) == kDeferPair) near_pair(Tv, l, A, M, out);
+  }
+};
+
 #undef TF
+
+// uniform or flat exponential: the medium of OpsF64Plain
+inline bool plain_medium(const MedParams& M) { return M.kind == C8R_UNIFORM || M.kind == C8R_EXPONENTIAL; }
 
 // forward and adjoint launches for one deposit shape
 template <bool LIN>
@@ -668,6 +921,9 @@ cudaError_t forward_f64(int formalism, const void* tiles, int64_t n_tiles, const
         forward_grid(a, shape, sm_count * forward_blocks_per_sm<O>(shape.a_tile), sizeof(Acc4D) * O::kAccRows);
     return launch_forward_ops<O>(a, ctas, st);
   };
+  if constexpr (!LIN) {
+    if (plain_medium(M)) return formalism == C8R_ENDPOINT ? go(OpsF64Plain<C8R_ENDPOINT>{}) : go(OpsF64Plain<C8R_ZHS>{});
+  }
   return formalism == C8R_ENDPOINT ? go(OpsF64<C8R_ENDPOINT, LIN>{}) : go(OpsF64<C8R_ZHS, LIN>{});
 }
 
