@@ -147,7 +147,8 @@ def _check(ctx, rc):
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current stream's handle without building a Stream object
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(stream.cuda_stream)
 
 
@@ -165,11 +166,7 @@ def tracks_struct(tracks: dict) -> c8r_tracks:
             raise ValueError("track fields must be contiguous CUDA tensors of one dtype and length")
     if dt not in (torch.float32, torch.float64):
         raise ValueError("track dtype must be float32 or float64")
-    s = c8r_tracks()
-    s.dtype = C8R_F64 if dt == torch.float64 else C8R_F32
-    for f, t in zip(TRACK_FIELDS, ts):
-        setattr(s, f, t.data_ptr())
-    return s
+    return c8r_tracks(C8R_F64 if dt == torch.float64 else C8R_F32, *[t.data_ptr() for t in ts])
 
 
 # ---------------------------------------------------------------------------
@@ -484,9 +481,12 @@ class RadioTraces(torch.autograd.Function):
         process = ctx.process
         gdt = torch.float64 if process.precision == "fp64" else torch.float32
         n = tracks["x0"].numel()
-        tg = {f: torch.zeros(n, dtype=gdt, device=process.device) for f in GRAD_FIELDS}
-        ag = torch.zeros((process.n_ant, 3), dtype=torch.float64, device=process.device)
-        dn = torch.zeros(1, dtype=torch.float64, device=process.device)
+        # the gradients as rows of two zeroed buffers (a fill per gradient is what
+        # a small step would wait for), each row on a 256-byte boundary
+        rows = torch.zeros((len(GRAD_FIELDS), (n + 63) // 64 * 64), dtype=gdt, device=process.device)
+        tg = {f: r[:n] for f, r in zip(GRAD_FIELDS, rows.unbind(0))}
+        sums = torch.zeros(3 * process.n_ant + 1, dtype=torch.float64, device=process.device)
+        ag, dn = sums[:-1].view(process.n_ant, 3), sums[-1:]
         g = grad_out.to(process.trace_dtype).contiguous()
         c8r_backward(process.ctx, tracks, g, tg, ag, dn)
         grads = [tg[f].to(tracks[f].dtype) for f in GRAD_FIELDS] + [torch.zeros_like(tracks["q"])]

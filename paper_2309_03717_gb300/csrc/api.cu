@@ -208,6 +208,7 @@ struct c8r_ctx {
   unsigned long long* h_form = nullptr;  // pinned: [kept tracks, seen from above]
   cudaEvent_t ev_form = nullptr;
   bool form_pending = false;
+  int form_pushes = 0, form_next = 1;    // pushes counted, and the push after which the votes are read next
   int64_t pushed = 0;
   cudaStream_t last_stream = nullptr;
   FwdShape shape{1, 8};
@@ -263,9 +264,15 @@ void form_poll(c8r_ctx* c) {
 }
 
 void form_fetch(c8r_ctx* c, cudaStream_t st) {
-  if (c->form_mode != C8R_FORM_AUTO || c->form_pending || !c->h_form || !c->ev_form || c->precision != C8R_MIXED)
+  // only the one-bin Endpoint kernels of the plain media come in two forms
+  if (c->form_mode != C8R_FORM_AUTO || c->form_pending || !c->h_form || !c->ev_form || c->precision != C8R_MIXED ||
+      c->formalism != C8R_ENDPOINT || c->deposit != C8R_DEPOSIT_BIN ||
+      (c->med_kind != C8R_UNIFORM && c->med_kind != C8R_EXPONENTIAL))
     return;
-  if (capturing(st)) return;
+  // the counts go on over all pushes, so they are read after the first, second,
+  // fourth, ... and then every 16th push (a read costs a small push 4 us)
+  if (capturing(st) || ++c->form_pushes < c->form_next) return;
+  c->form_next = c->form_pushes + (c->form_pushes < 16 ? c->form_pushes : 16);
   if (cudaMemcpyAsync(c->h_form, c->d_kept + 1, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st) !=
           cudaSuccess ||
       cudaEventRecord(c->ev_form, st) != cudaSuccess) {
@@ -293,6 +300,8 @@ cudaError_t zero_acc(c8r_ctx* c, cudaStream_t st) {
 void form_reset(c8r_ctx* c) {
   if (c->form_pending) cudaEventSynchronize(c->ev_form);
   c->form_pending = false;
+  c->form_pushes = 0;
+  c->form_next = 1;
   cudaMemset(c->d_kept + 1, 0, 2 * sizeof(unsigned long long));
   c->split = c->form_mode != C8R_FORM_DIRECT;
 }

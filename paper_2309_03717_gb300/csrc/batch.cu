@@ -151,12 +151,7 @@ __global__ void __launch_bounds__(Ops::kFwdThreads, Ops::kMinBlocks) k_batch(con
 // resident CTAs per SM of the batch kernel for antenna tiles of a_tile
 template <class Ops>
 int batch_blocks_per_sm(int a_tile) {
-  const size_t smem = fwd_layout(C8R_MIXED, a_tile, Ops::kDefers).total;
-  auto k = k_batch<Ops>;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 1;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, Ops::kFwdThreads, smem) != cudaSuccess) return 1;
-  return per_sm < 1 ? 1 : per_sm;
+  return resident_per_sm<Ops>(k_batch<Ops>, a_tile);
 }
 
 // persistent grid: every CTA that fits on the device at once

@@ -21,6 +21,7 @@
 // reductions are fire-and-forget.
 #pragma once
 
+#include <atomic>
 #include <type_traits>
 
 #include "c8r_internal.h"
@@ -475,24 +476,39 @@ inline int64_t forward_grid(FwdArgs& a, const FwdShape& shape, int resident, siz
   return (int64_t)g.ant_tiles * g.ranges;
 }
 
-template <class Ops>
-cudaError_t launch_forward_ops(const FwdArgs& a, int64_t ctas, cudaStream_t st) {
-  const size_t smem = fwd_layout(Ops::kPrec, a.a_tile, Ops::kDefers).total;
-  auto k = k_forward<Ops>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k<<<(unsigned)ctas, Ops::kFwdThreads, smem, st>>>(a);
-  return cudaGetLastError();
+// Once per kernel and device: the shared memory it may take (that of the largest
+// antenna tile), and its resident CTAs per SM for each antenna tile.  Asking the
+// runtime for both on every push took 3 us of the 20 of a small one.
+constexpr int kMaxDevices = 64;
+template <class Ops, class K>
+int resident_per_sm(K kernel, int a_tile) {
+  static std::atomic<int> known[kMaxDevices][kMaxATile + 1];
+  int dev = 0;
+  const bool cached = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices;
+  int n = cached ? known[dev][a_tile].load(std::memory_order_relaxed) : 0;
+  if (n > 0) return n;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)fwd_layout(Ops::kPrec, kMaxATile, Ops::kDefers).total);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, Ops::kFwdThreads,
+                                                    fwd_layout(Ops::kPrec, a_tile, Ops::kDefers).total) != cudaSuccess)
+    return 1;
+  n = n < 1 ? 1 : n;
+  if (cached) known[dev][a_tile].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // resident CTAs of the forward kernel per SM
 template <class Ops>
 int forward_blocks_per_sm(int a_tile) {
-  int n = 0;
-  const size_t smem = fwd_layout(Ops::kPrec, a_tile, Ops::kDefers).total;
-  cudaFuncSetAttribute(k_forward<Ops>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_forward<Ops>, Ops::kFwdThreads, smem) != cudaSuccess) n = 1;
-  return n < 1 ? 1 : n;
+  return resident_per_sm<Ops>(k_forward<Ops>, a_tile);
+}
+
+// (after forward_blocks_per_sm, which sets the kernel's shared-memory limit)
+template <class Ops>
+cudaError_t launch_forward_ops(const FwdArgs& a, int64_t ctas, cudaStream_t st) {
+  const size_t smem = fwd_layout(Ops::kPrec, a.a_tile, Ops::kDefers).total;
+  k_forward<Ops><<<(unsigned)ctas, Ops::kFwdThreads, smem, st>>>(a);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
