@@ -88,6 +88,7 @@ void fill_medium(MedParams& M, int kind, double n_or_N0, double H, int n_bins, d
     M.nf = 1.0f;
     M.R_E = earth_radius;
     M.RE_f = (float)earth_radius;
+    M.RE_k = earth_radius > 0.0 ? (float)(H / earth_radius) : 0.0f;
   }
 }
 
@@ -129,10 +130,14 @@ void fill_antenna(AntRec& r, double x, double y, double z, double t_ref_ns, cons
 
 void set_flat_array(MedParams& M, const double* pos_xyz, int n_ant) {
   M.flat = 0;
-  if (M.kind != C8R_EXPONENTIAL || n_ant <= 0) return;
+  if (M.kind == C8R_UNIFORM || n_ant <= 0) return;
   const double z = pos_xyz[2];
-  for (int a = 1; a < n_ant; ++a)
-    if (pos_xyz[3 * (size_t)a + 2] != z) return;
+  for (int a = 0; a < n_ant; ++a) {
+    const double* p = pos_xyz + 3 * (size_t)a;
+    if (p[2] != z) return;
+    // spherical Earth: the range of the curvature's series (PathZ)
+    if (M.kind == C8R_EXPONENTIAL_SPHERICAL && !(p[0] * p[0] + p[1] * p[1] < 0.01 * 2.0 * (M.R_E + z) * M.H)) return;
+  }
   // split as fill_antenna splits the antennas' z and exp(-z/H)
   M.flat = 1;
   M.flat_zh = (float)z;

@@ -105,6 +105,7 @@ struct MedParams {
   float kzhs;            // K_A of the ZHS amplitude
   float nm1f;            // uniform: n - 1 formed in FP64, then rounded (never (1 + x) - 1 in FP32)
   float RE_f;            // spherical: Earth radius (m)
+  float RE_k;            // spherical: H / Earth radius
   float eps_C;           // near-Cherenkov threshold
   float dz_series;       // exponential: -1.001e-3 H, the altitude difference from where the quotient's series may apply
   uint32_t wait_limit;   // polls of a bounded wait on a staged track tile before it gives up
@@ -115,7 +116,7 @@ struct MedParams {
   float cen_x, cen_y, cen_z;
   int split;
   // a flat antenna array (every antenna at one altitude z_a, exponential
-  // medium): z_a and exp(-z_a/H) as float-float, the same values the antenna
+  // media; spherical Earth: and within 32 km of the origin, PathZ): z_a and exp(-z_a/H) as float-float, the same values the antenna
   // records hold, so that the quotient (E_e - E_a)/(z_a - z_e) of the
   // refractivity term, the same for every antenna, can be formed once per
   // track (OpsMixed::kFlat)

@@ -83,7 +83,7 @@ __device__ __forceinline__ void load_track_mixed(const float* T, int l, const Me
     two_sum(t.z0, t.z1, t.mz, t.mzl);
     t.mx *= 0.5f; t.mxl *= 0.5f; t.my *= 0.5f; t.myl *= 0.5f; t.mz *= 0.5f; t.mzl *= 0.5f;
   }
-  if constexpr (FLAT && KIND == C8R_EXPONENTIAL && FORM == C8R_ZHS) {
+  if constexpr (FLAT && KIND != C8R_UNIFORM && FORM == C8R_ZHS) {
     // the refractivity quotient against the array's altitude, formed as the
     // per-pair arithmetic forms it (the altitude difference as geo_lite forms
     // it), so the values are the same
@@ -146,9 +146,134 @@ struct alignas(16) AntE {
 };
 static_assert(sizeof(AntE) == sizeof(AntRec), "fwd_layout reckons with one antenna record size");
 
+// What the spherical-Earth and curved-ray propagators need of a track for a flat
+// antenna array, where the path's heights and the refractivity along it are the
+// same for every antenna (two tracks, halves x and y).  Per pair and node the
+// quadratures took an exponential, a root and a quotient (sphere) or six roots
+// and quotients (rays) on the XU pipe; these take none.  ZHS, ms: 2.5e5 tracks x
+// 1024 antennas over a sphere 4.43 -> 3.21, x 256 antennas along rays 1.69 -> 0.82
+// (6 CTAs of 64 threads per SM; 7 and 8, with 128 registers: 3.45, 3.50 and 0.82,
+// 0.84).
+template <int KIND>
+struct PathZ {};
+
+// Spherical Earth: the curvature part of the optical path (sphere_path_correction),
+//   N0 R sum_j w_j E_j (exp(-d_j/H) - 1),  E_j = exp(-z_j/H), d_j the altitude
+//   excess of node j at the distance y_j^(1/2) from the vertical through the
+//   origin.  With x_j = y_j h_j, h_j = 1/(2 (z_j + R_E) H), and k = H/(2 R_E), d_j/H =
+//   x_j (1 - k x_j + ...) and the bracket is -x_j [1 - x_j (k + 1/2) + x_j^2 (k + 1/6)]
+//   up to x^3/24 of it: 4e-8 for x_j < 0.01, which holds within 32 km of the origin
+//   (antennas: checked by the host, tracks: `small`).  Per track: w_j E_j h_j, and
+//   h as a linear function along the path for the bracket.
+template <>
+struct PathZ<C8R_EXPONENTIAL_SPHERICAL> {
+  float2 weh[kSphNodes];
+  float2 h0, h1;
+  bool small;
+  __device__ __forceinline__ void set(const MedParams& M, float2 mx, float2 my, float2 mz, float2 dz) {
+    const float inv2H = 0.5f * M.invH_h;
+    h0 = make_float2(div_ap(inv2H, M.RE_f + M.flat_zh), div_ap(inv2H, M.RE_f + M.flat_zh));
+    h1 = make_float2(div_ap(inv2H, M.RE_f + mz.x) - h0.x, div_ap(inv2H, M.RE_f + mz.y) - h0.y);
+    const float2 y = fma_rn(mx, mx, mul_rn(my, my));
+    small = fmaxf(y.x * h0.x, y.y * h0.y) < 0.01f;
+#pragma unroll
+    for (int j = 0; j < kSphNodes; ++j) {
+      const float f = 1.0f - (float)kSphSigma[j];
+      const float2 z = fma_rn(bc<float2>(-f), dz, bc<float2>(M.flat_zh));
+      const float w = (float)kSphWeight[j] * inv2H;
+      weh[j] = make_float2(div_ap(w * exp_ap(-z.x * M.invH_h), M.RE_f + z.x),
+                           div_ap(w * exp_ap(-z.y * M.invH_h), M.RE_f + z.y));
+    }
+  }
+  // the change of the optical path to the antenna at (ax, ay), m
+  __device__ __forceinline__ float2 path(const MedParams& M, float2 ax, float2 ay, const GeoT<float2>& g) const {
+    const float k = 0.5f * M.RE_k;
+    float2 sum = bc<float2>(0.0f);
+#pragma unroll
+    for (int j = 0; j < kSphNodes; ++j) {
+      const float f = 1.0f - (float)kSphSigma[j];
+      const float2 x = fma_rn(bc<float2>(-f), g.s[0], ax), y = fma_rn(bc<float2>(-f), g.s[1], ay);
+      const float2 r2 = fma_rn(x, x, mul_rn(y, y));
+      const float2 xj = mul_rn(r2, fma_rn(bc<float2>(f), h1, h0));
+      const float2 p = fma_rn(xj, fma_rn(xj, bc<float2>(k + 1.0f / 6.0f), bc<float2>(-k - 0.5f)), bc<float2>(1.0f));
+      sum = fma_rn(mul_rn(weh[j], r2), p, sum);
+    }
+    return mul_rn(mul_rn(bc<float2>(-M.N0f), g.R0), sum);
+  }
+};
+
+// Curved rays (ray_fix): with a_j = 1/n_j at the Gauss-Legendre nodes, abar their
+// weighted mean, b_j = a_j/abar - 1 (~1e-4), B_k = sum_j w_j b_j^k and T = tan of the
+// straight line's angle from the vertical, the ray's constant is p = S (1 + t)/abar,
+// and expanding the end-point condition and Fermat's time saved in b (a series in
+// T^2 b, carried to b^4) gives
+//   t = -(3/2) T^2 B2 - (1/2) T^2 (1 + 5 T^2) B3,
+//   path change = -(R T^2/abar) [B2/2 + (T^2 - 1) B3/2 + (4 - 3 T^2 + 5 T^4) B4/8 -
+//                 (9/8) T^4 B2^2],
+//   C Q at x_e = e (1 + T^2 e/2 + T^4 e^2/2),  e = t + (1 + t) b_e.
+// The rest is of order (T^2 b)^3 of these: below 1e-7 for T^2 b < 4e-3, the pairs
+// taken here (zenith angles to ~78 degrees in air).  Everything but T^2 is a
+// property of the track; b is formed from r_j = nu_j/n_j without cancellation.
+template <>
+struct PathZ<C8R_EXPONENTIAL_RAY> {
+  float2 inv_abar, B2, B3, B4, be, bmax, inv_dz2;
+  __device__ __forceinline__ void set(const MedParams& M, float2 nu_e, float2 dz) {
+    float2 r[kSphNodes], mean = bc<float2>(0.0f);
+#pragma unroll
+    for (int j = 0; j < kSphNodes; ++j) {
+      const float c = -(float)kSphSigma[j] * M.invH_h;
+      const float2 nu = mul_rn(nu_e, make_float2(exp_ap(c * dz.x), exp_ap(c * dz.y)));
+      r[j] = mul_rn(nu, rcp_ap(add_rn(bc<float2>(1.0f), nu)));
+      mean = fma_rn(bc<float2>((float)kSphWeight[j]), r[j], mean);
+    }
+    inv_abar = rcp_ap(sub_rn(bc<float2>(1.0f), mean));
+    B2 = B3 = B4 = bc<float2>(0.0f);
+#pragma unroll
+    for (int j = 0; j < kSphNodes; ++j) {
+      const float2 b = mul_rn(sub_rn(mean, r[j]), inv_abar), b2 = mul_rn(b, b);
+      const float2 w = bc<float2>((float)kSphWeight[j]);
+      B2 = fma_rn(w, b2, B2);
+      B3 = fma_rn(w, mul_rn(b2, b), B3);
+      B4 = fma_rn(w, mul_rn(b2, b2), B4);
+    }
+    be = mul_rn(sub_rn(mean, mul_rn(nu_e, rcp_ap(add_rn(bc<float2>(1.0f), nu_e)))), inv_abar);
+    // b at the antenna's end
+    const float2 nu_a = mul_rn(nu_e, make_float2(exp_ap(-M.invH_h * dz.x), exp_ap(-M.invH_h * dz.y)));
+    const float2 ba = mul_rn(sub_rn(mean, mul_rn(nu_a, rcp_ap(add_rn(bc<float2>(1.0f), nu_a)))), inv_abar);
+    bmax = make_float2(fmaxf(fabsf(be.x), fabsf(ba.x)), fmaxf(fabsf(be.y), fabsf(ba.y)));
+    inv_dz2 = rcp_ap(mul_rn(dz, dz));
+  }
+  // the change of the optical path (m) and the turn of the direction at x_e (the
+  // change of R rhat); false for pairs outside the series' range
+  __device__ __forceinline__ bool path(const GeoT<float2>& g, float2& dop, float2 turn[3]) const {
+    const float2 T2 = mul_rn(fma_rn(g.s[0], g.s[0], mul_rn(g.s[1], g.s[1])), inv_dz2);
+    const float2 q = mul_rn(T2, bmax);
+    if (!(fmaxf(q.x, q.y) < 4e-3f) || !(fmaxf(T2.x, T2.y) < 1e5f)) return false;
+    const float2 half = bc<float2>(0.5f);
+    const float2 hT = mul_rn(half, T2);
+    const float2 t = neg(mul_rn(hT, fma_rn(bc<float2>(3.0f), B2, mul_rn(B3, fma_rn(bc<float2>(5.0f), T2, bc<float2>(1.0f))))));
+    const float2 c4 = fma_rn(T2, fma_rn(T2, bc<float2>(0.625f), bc<float2>(-0.375f)), half);
+    float2 v = fma_rn(half, B2, mul_rn(B3, fma_rn(half, T2, bc<float2>(-0.5f))));
+    v = fma_rn(c4, B4, v);
+    const float2 TB = mul_rn(T2, B2);
+    v = fma_rn(mul_rn(bc<float2>(-1.125f), TB), TB, v);
+    dop = neg(mul_rn(mul_rn(mul_rn(g.R0, T2), inv_abar), v));
+    const float2 e = fma_rn(t, be, add_rn(t, be));
+    // sin(turn) = T cq, cos(turn) - 1 = -(T cq)^2/2 to a relative 1e-8
+    const float2 cq = mul_rn(e, fma_rn(mul_rn(hT, e), fma_rn(T2, e, bc<float2>(1.0f)), bc<float2>(1.0f)));
+    const float2 cm = neg(mul_rn(mul_rn(hT, cq), cq));
+    const float2 f = add_rn(cm, cq);
+    turn[0] = mul_rn(f, g.s[0]);
+    turn[1] = mul_rn(f, g.s[1]);
+    turn[2] = mul_rn(fma_rn(neg(T2), cq, cm), g.s[2]);
+    return true;
+  }
+};
+
 // two tracks for the forward pass of the ZHS kernels, halves x and y; the
 // midpoint of each
-struct TrackZ {
+template <int KIND>
+struct TrackZ : PathZ<KIND> {
   float2 mx, mxl, my, myl, mz, mzl;   // position, float-float
   float2 bx, by, bz, nm1;
   float2 tmh, tml, dtauh, dtaul;      // (t0 + t1)/(2 dt), (t1 - t0)/dt
@@ -159,7 +284,7 @@ struct TrackZ {
 };
 
 template <int KIND, bool FLAT>
-__device__ __forceinline__ void load_track_pair(const float* T, int l, const MedParams& M, TrackZ& t) {
+__device__ __forceinline__ void load_track_pair(const float* T, int l, const MedParams& M, TrackZ<KIND>& t) {
   auto ld = [&](int f) { return *reinterpret_cast<const float2*>(T + f * kTileT + 2 * l); };
   const float2 keep = ld(fm::AMPE);
   t.live = keep.x != 0.0f || keep.y != 0.0f;
@@ -187,6 +312,11 @@ __device__ __forceinline__ void load_track_pair(const float* T, int l, const Med
     t.Eh = ld(fm::EMH); t.El = ld(fm::EML);
     t.nm1 = mul_rn(bc<float2>(M.N0f), t.Eh);
   }
+  if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL) {
+    // n - 1 at the midpoint over the sphere, as load_track_mixed has it
+    t.nm1.x *= expf(-sphere_excess(t.mx.x, t.my.x, t.mz.x, M.RE_f) * M.invH_h);
+    t.nm1.y *= expf(-sphere_excess(t.mx.y, t.my.y, t.mz.y, M.RE_f) * M.invH_h);
+  }
   if constexpr (FLAT) {
     // per track as the per-pair arithmetic forms it, so the same values
     float2 dzh, dzl, q0, q1;
@@ -197,6 +327,8 @@ __device__ __forceinline__ void load_track_pair(const float* T, int l, const Med
     t.zm = z_part(dzh, dzl, t.bz);
     t.Eh = q0;
     t.El = q1;
+    if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL) t.set(M, t.mx, t.my, t.mz, dzh);
+    if constexpr (KIND == C8R_EXPONENTIAL_RAY) t.set(M, t.nm1, dzh);
   }
 }
 
@@ -235,13 +367,14 @@ __device__ __forceinline__ void ray_turn_mixed(GeoM& g, float nu_e, float bx, fl
 }
 
 // D in float-float plus a small FP32 change, renormalised
-__device__ __forceinline__ ff ff_add_small(ff D, float d) {
-  float h, l;
+template <typename T>
+__device__ __forceinline__ ffT<T> ff_add_small(ffT<T> D, T d) {
+  T h, l;
   two_sum(D.h, d, h, l);
-  l = __fadd_rn(l, D.l);
-  ff r;
-  r.h = __fadd_rn(h, l);
-  r.l = __fsub_rn(l, __fsub_rn(r.h, h));
+  l = add_rn(l, D.l);
+  ffT<T> r;
+  r.h = add_rn(h, l);
+  r.l = sub_rn(l, sub_rn(r.h, h));
   return r;
 }
 
@@ -404,7 +537,7 @@ struct OpsMixed {
   // 5 CTAs has no spills and is 1.6 % faster than at 6)
   static constexpr int kMinBlocks =
       FORM == C8R_ENDPOINT ? (KIND == C8R_EXPONENTIAL_RAY ? 4 : (KIND == C8R_EXPONENTIAL_SPHERICAL ? 5 : 6))
-                           : (KIND == C8R_EXPONENTIAL_RAY ? 6 : 8);
+                           : (KIND == C8R_EXPONENTIAL_RAY || (KIND == C8R_EXPONENTIAL_SPHERICAL && FLAT) ? 6 : 8);
   // Endpoint: the near-Cherenkov pairs (a minority, spread over most warps)
   // are set aside by the main pass and evaluated together afterwards
   static constexpr bool kDefers = FORM == C8R_ENDPOINT;
@@ -414,9 +547,9 @@ struct OpsMixed {
   // for the float-float arrival after the main pass
   static constexpr bool kFastBins =
       FORM == C8R_ENDPOINT && !LIN && (KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL);
-  // ZHS in those media: the forward kernel evaluates two tracks at a time
-  static constexpr bool kTwoTracks =
-      FORM == C8R_ZHS && (KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL);
+  // ZHS in those media, and in the others for a flat array: the forward kernel
+  // evaluates two tracks at a time
+  static constexpr bool kTwoTracks = FORM == C8R_ZHS && (KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL || FLAT);
   static constexpr int kFwdThreads = kTwoTracks ? kTileT / 2 : kTileT;
   // the form of x = R - w in the FP32 arrival (arrival_fast): the split one
   // for lines of sight near the vertical, the direct one otherwise.  Either is
@@ -434,7 +567,7 @@ struct OpsMixed {
   // the Endpoint and then the ZHS process on the same tracks.  The split-form
   // Endpoint kernel keeps the quotient per pair (within 0.3 % either way)
   static constexpr bool kFlat =
-      FLAT && KIND == C8R_EXPONENTIAL && ((kFastBins && !SPLIT) || FORM == C8R_ZHS);
+      FLAT && KIND != C8R_UNIFORM && ((kFastBins && !SPLIT) || FORM == C8R_ZHS);
   // adjoint CTAs (128 threads) per SM the registers are set for (the linear
   // Endpoint adjoint carries the slide of each deposit as well)
   static constexpr int kBwdMinBlocks = (LIN && FORM == C8R_ENDPOINT) ? 4 : (kFastBins ? 5 : 6);
@@ -511,9 +644,9 @@ struct OpsMixed {
       load(Tv, l, M, t);
   }
   static __device__ __forceinline__ bool live(const TrackE& t) { return t.amp != 0.0f; }
-  static __device__ __forceinline__ bool live(const TrackZ& t) { return t.live; }
+  static __device__ __forceinline__ bool live(const TrackZ<KIND>& t) { return t.live; }
   // what a thread of the forward main pass holds: a track, or two of them
-  using FwdTrack = std::conditional_t<kTwoTracks, TrackZ, MainTrack>;
+  using FwdTrack = std::conditional_t<kTwoTracks, TrackZ<KIND>, MainTrack>;
   static __device__ __forceinline__ void load_fwd(const void* Tv, int l, const MedParams& M, FwdTrack& t) {
     if constexpr (kTwoTracks)
       load_track_pair<KIND, kFlat>(static_cast<const float*>(Tv), l, M, t);
@@ -639,6 +772,8 @@ struct OpsMixed {
     ff um, aD;
     if constexpr (kFlat) {
       geo_refine(gm, t.zm);
+      if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL)
+        dop = sphere_path_correction<float>(A.xh, A.yh, A.zh, gm.s[0], gm.s[1], gm.s[2], gm.R0, M.N0f, M.invH_h, M.RE_f);
       um = arrival_mixed_q<KIND>(M, A.tauh, A.taul, gm, t.tmh, t.tml, t.qmh, t.qml, dop);
       aD = doppler_ff(gm, t.bx, t.by, t.zm, t.nm1_m);
     } else {
@@ -721,16 +856,31 @@ struct OpsMixed {
   // false when a half needs another form of it (the altitude difference
   // within 1e-3 H, or a window too long for bins_of), with nothing deposited
   template <class Sink>
-  static __device__ __forceinline__ bool zhs_two(const TrackZ& t, const AntZ& A, const MedParams& M, Sink& out) {
+  static __device__ __forceinline__ bool zhs_two(const TrackZ<KIND>& t, const AntZ& A, const MedParams& M, Sink& out) {
     const int N = M.n_bins;
     if (!LIN && N > kMagicBins / 2) return false;
     GeoT<float2> g;
     ffT<float2> um, aD;
     if constexpr (kFlat) {
       geo_lite(A.x, A.y, A.xl, A.yl, t.mx, t.my, t.mxl, t.myl, t.zm, g);
+      float2 corr = bc<float2>(0.0f), turn[3];
+      if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL) {
+        if (!t.small) return false;
+        corr = t.path(M, A.x, A.y, g);
+      }
+      if constexpr (KIND == C8R_EXPONENTIAL_RAY) {
+        if (!t.path(g, corr, turn)) return false;
+      }
       geo_refine(g, t.zm);
-      um = arrival_mixed_q<KIND>(M, A.tauh, A.taul, g, t.tmh, t.tml, t.Eh, t.El);
+      um = arrival_mixed_q<KIND>(M, A.tauh, A.taul, g, t.tmh, t.tml, t.Eh, t.El, corr);
       aD = doppler_ff(g, t.bx, t.by, t.zm, t.nm1);
+      if constexpr (KIND == C8R_EXPONENTIAL_RAY) {
+        // the field along the ray, and the change of D that the turn makes
+        const float2 bt = fma_rn(t.bx, turn[0], fma_rn(t.by, turn[1], mul_rn(t.bz, turn[2])));
+        aD = ff_add_small(aD, neg(mul_rn(mul_rn(add_rn(bc<float2>(1.0f), t.nm1), bt), g.y)));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) g.s[c] = add_rn(g.s[c], turn[c]);
+      }
     } else {
       float2 dzh, dzl, q0 = bc<float2>(0.0f), q1 = q0;
       two_sum(A.z, neg(t.mz), dzh, dzl);
@@ -1636,9 +1786,11 @@ cudaError_t forward_mixed(int formalism, const void* tiles, int64_t n_tiles, con
   const bool ex = M.kind == C8R_EXPONENTIAL;
   if (M.kind == C8R_EXPONENTIAL_SPHERICAL)
     return formalism == C8R_ENDPOINT ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_SPHERICAL, LIN>{})
+           : M.flat                  ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_SPHERICAL, LIN, false, true>{})
                                      : go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_SPHERICAL, LIN>{});
   if (M.kind == C8R_EXPONENTIAL_RAY)
     return formalism == C8R_ENDPOINT ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_RAY, LIN>{})
+           : M.flat                  ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, LIN, false, true>{})
                                      : go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, LIN>{});
   if constexpr (!LIN) {
     // the one-bin Endpoint kernels come in both arrival forms (M.split) and,

@@ -90,3 +90,42 @@ def test_zhs_traces_with_antennas_among_the_tracks(n, n_ant, n_bins, medium, dep
                             w["dt_ns"] * 1e-9, w["medium"], oracle.ZHS,
                             deposit=oracle.DEPOSIT_LINEAR if deposit == "linear" else oracle.DEPOSIT_BIN)
     assert rel_l2(got, ref) <= TOL
+
+
+HEAVY = [{"kind": "exponential_spherical", "N0": 3.25e-4, "H": 8000.0, "R_E": 6.371e6},
+         {"kind": "exponential_ray", "N0": 3.25e-4, "H": 8000.0},
+         {"kind": "exponential_ray", "N0": 5e-3, "H": 2000.0}]
+
+
+@pytest.mark.parametrize("deposit", ["bin", "linear"])
+@pytest.mark.parametrize("medium", HEAVY)
+@pytest.mark.parametrize("reach,z", [(400.0, 0.0), (12_000.0, 120.0), (60_000.0, 0.0), (3_000.0, None)])
+def test_zhs_over_a_sphere_and_along_rays(reach, z, medium, deposit):
+    """Flat arrays take the propagators' series in the pairs where those hold
+    (steep lines of sight, sites within 32 km), the quadrature elsewhere: sites
+    from the shower axis out to where only the latter is left, and uneven ground
+    (z None), where no pair takes the series."""
+    from paper_2309_03717_gb300 import c8r
+    n, n_ant = 301, 33
+    w = synth.workload(1, n_tracks=n, n_ant=n_ant)
+    tracks = synth.workload_tracks(w)
+    tracks["q"][5::11] = 0.0  # filtered tracks next to kept ones
+    x = np.concatenate([[0.0], np.geomspace(reach / 1000.0, reach, n_ant - 1)])
+    heights = np.linspace(0.0, 200.0, n_ant) if z is None else np.full(n_ant, z)
+    ant = np.stack([x, 0.3 * x, heights], 1)
+    _, u0 = oracle_arrivals(tracks, ant, np.zeros(n_ant), 1, w["dt_ns"], medium, "zhs")
+    t_start = np.median(u0.reshape(n, n_ant, 2)[..., 0], axis=0) * w["dt_ns"] - 200.0
+    # (in the steep atmosphere no direct ray reaches the farthest sites: no start time there)
+    ant, t_start = ant[np.isfinite(t_start)], t_start[np.isfinite(t_start)]
+    n_ant = len(ant)
+    assert n_ant >= 25
+    p = c8r.RadioProcess(medium, ant, t_start, 2048, w["dt_ns"], "zhs", "mixed", deposit=deposit)
+    p.push(to_device(tracks))
+    got = p.traces().cpu().numpy()
+    p.close()
+    ref, _ = oracle.forward(oracle.tracks_from_ns(tracks), ant, t_start * 1e-9, 2048, w["dt_ns"] * 1e-9, medium,
+                            oracle.ZHS,
+                            deposit=oracle.DEPOSIT_LINEAR if deposit == "linear" else oracle.DEPOSIT_BIN)
+    for a in range(n_ant):
+        if np.abs(ref[a]).max() > 0:
+            assert rel_l2(got[a], ref[a]) <= TOL, a
