@@ -237,6 +237,10 @@ int c8r_set_launch_shape(c8r_ctx* ctx, int a_tile, int waves, int64_t chunk_trac
  * the counts are copied back asynchronously, and later pushes and adjoints use
  * the split form when at least half of the tracks counted do (the split form
  * until a count has arrived; c8r_set_antennas with a new layout starts over).
+ * There, when the trace start times follow a plane front 30 degrees or more off
+ * the vertical, both give way to a third form with the front's direction in the
+ * place of the vertical (x = R minus the distance along it), unless the counts
+ * contradict that direction.
  * Other precisions, media and deposits ignore the setting.  EINVAL for another
  * value. */
 int c8r_set_arrival_form(c8r_ctx* ctx, int form);

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(Ops::kFwdThreads, Ops::kMinBlocks) k_batch(con
     const int idx = s_item;
     if (idx < 0 || idx >= a.n_items) break;
     const WorkItem w = a.items[idx];
-    for (int i = tid; i < w.n_here; i += nthr) Ops::stage_ant(ant_s + i, a.ants[w.ant0 + i]);
+    for (int i = tid; i < w.n_here; i += nthr) Ops::stage_ant(ant_s + i, a.ants[w.ant0 + i], M);
     __syncthreads();
     float4* acc = a.acc + (size_t)(idx % a.replicas) * a.replica_stride + (size_t)w.ant0 * M.n_bins * Ops::kAccRows;
     if (!stream_range<Ops>(smem, L, bar, ant_s, acc, w.n_here,
@@ -167,14 +167,14 @@ cudaError_t launch_batch_ops(const BatchArgs& a, int sm_count, cudaStream_t st) 
 template <class F>
 auto with_batch_ops(int formalism, int kind, bool split, bool flat, F f) {
   const bool ex = kind == C8R_EXPONENTIAL;
-  // the arrival form of the one-bin Endpoint kernel (OpsMixed::kSplit) and, for
+  // the arrival form of the one-bin Endpoint kernel (OpsMixed::kAF) and, for
   // the direct form, the flat-array kernel of the exponential medium
   // (OpsMixed::kFlat)
   if (formalism == C8R_ENDPOINT) {
     if (!ex)
-      return split ? f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, true>{}) : f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
-    if (split) return f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, true>{});
-    return flat ? f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, false, true>{})
+      return split ? f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{}) : f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
+    if (split) return f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{});
+    return flat ? f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{})
                 : f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>{});
   }
   return ex ? f(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL>{}) : f(OpsMixed<C8R_ZHS, C8R_UNIFORM>{});

@@ -115,6 +115,11 @@ struct MedParams {
   // count (1: the split form of x = R - w)
   float cen_x, cen_y, cen_z;
   int split;
+  // the axis form of the FP32 arrival, taken when axis != 0 (arrival_fast): the
+  // axis, an FP32 vector of unit length up to rounding, and k/|ax| ax (k = n/(c dt)
+  // or 1/(c dt)) as float-float
+  int axis;
+  float ax[3], kax_h[3], kax_l[3];
   // a flat antenna array (every antenna at one altitude z_a, exponential
   // media; spherical Earth: and within 32 km of the origin, PathZ): z_a and exp(-z_a/H) as float-float, the same values the antenna
   // records hold, so that the quotient (E_e - E_a)/(z_a - z_e) of the
@@ -777,6 +782,31 @@ __device__ __forceinline__ int bin_raw(ff u, int n_bins, float& frac) {
 // per pair).  On a shower inclined by 60 degrees x is about R/2 and the direct
 // form holds the bound near that of an arrival rounded in FP32 throughout.
 // ---------------------------------------------------------------------------
+// Along an axis (kFormAxis).  The vertical split carries over to any direction A:
+// with w = -(d . A)/|A| and x = R - w = |d x A|^2/(|A| (|A| R - d . A)), T = tau + k
+// (position . A)/|A|.  A shower's lines of sight all lie near its axis, so x and
+// its error stay small for inclined showers too, where the direct form rounds
+// terms of k R.  A is an FP32 vector taken exactly; its length, 1 within 3u, enters
+// T through k/|A| and is dropped from x (9u x at most).  The errors, where w >= 0:
+//   s: |delta| <= u R (2-norm), and x changes with d at |d/R + A| = sqrt(2x/R), so
+//     u sqrt(2 x R); a_l: at most 2 |a_l|, as above;
+//   c = fl(s x A): each component off by u |s_j A_k| + u |c_i|, u (R + rho) in 2-norm,
+//     rho = |c|, rho^2 = x (2R - x) <= 2 x R; it moves x = rho^2/(R + w) by at most
+//     2 rho u (R + rho)/R <= 4 u rho;
+//   together at most 5.5 u sqrt(2 x R) <= 5.5 u (8 x + R/16), an arithmetic mean;
+//   rho^2 3u, R0 6u R, w 3u R and the denominator's rounding u (R + w >= R), the
+//     quotient 4u and |A| 9u: 26u x;
+//   q, Td, v, uf as in the split form.
+// The bound used is u (2.25 |Td| + 72 q + 22 |v| + 3.25 |uf| + 0.375 k R) + fb_rel_v |v|
+// + fb_abs with 16 u^2 |T_a| of the axis' T_a (2 + 26 + 44 and 0.344 derived).  Where w <
+// 0 (a line of sight beyond 90 degrees from the axis) x = fl(R0 - w), and 10 k R in
+// place of 0.375 k R covers R0's and w's errors.  q_extra, for a geometry whose d is
+// off by q_extra/1.5 times the above, adds u q_extra (8 q + k R/16).  On showers at 12 to
+// 75 degrees 0.4 % of the in-window endpoints are left undecided at 0.2 ns per bin,
+// against 0.3 to 12 % (split) and 2 to 7 % (direct); the worst error was 0.11 of the
+// bound (test_fp32_axis_bound).
+enum : int { kFormDirect = 0, kFormSplit = 1, kFormAxis = 2 };
+
 constexpr int kFastOut = -1;        // the arrival lies outside the window: no deposit
 constexpr int kFastUndecided = -2;  // an edge lies within the bound: the float-float arrival decides
 
@@ -807,6 +837,28 @@ __device__ __forceinline__ void shifted_time(float tauh, float taul, float zh, f
   fast_two_sum(s, e2, Th, Tl);
 }
 
+// T = tau + k (p . A)/|A| as float-float for a position p given as float-float
+__device__ __forceinline__ void axis_time(const MedParams& M, float tauh, float taul, const float ph[3],
+                                          const float pl[3], float& Th, float& Tl) {
+  float h = tauh, l = taul;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float p, e, s, e2;
+    two_prod(ph[c], M.kax_h[c], p, e);
+    e = __fmaf_rn(ph[c], M.kax_l[c], __fmaf_rn(pl[c], M.kax_h[c], e));
+    two_sum(h, p, s, e2);
+    l = __fadd_rn(l, __fadd_rn(e, e2));
+    h = s;
+  }
+  fast_two_sum(h, l, Th, Tl);
+}
+
+// w = -(d . A) of the axis form
+template <typename T>
+__device__ __forceinline__ T axis_w(const MedParams& M, const GeoT<T>& g) {
+  return neg(fma_rn(g.s[0], bc<T>(M.ax[0]), fma_rn(g.s[1], bc<T>(M.ax[1]), mul_rn(g.s[2], bc<T>(M.ax[2])))));
+}
+
 // the FP32 quotient (E_e - E_a)/dz of the refractivity term for the FP32
 // arrival (exponential medium); dz = s_z, the FP32 a_h - p of the emission
 // point (the same for every antenna of a flat array); for |dz/H| <= 1e-3 its
@@ -825,10 +877,10 @@ __device__ __forceinline__ T fast_quotient(const MedParams& M, T Eah, T Eal, T s
 
 // The FP32 arrival uf of the emission point of g (S = |d|^2, rho2 = d_x^2 +
 // d_y^2, T_e = Teh + Tel, the antenna's T_a = Tah + Tal and bound constants, qv
-// the refractivity quotient of fast_quotient) and its error bound, returned; SPLIT picks the form of x; q_extra adds a term
+// the refractivity quotient of fast_quotient) and its error bound, returned; AF picks the form of x; q_extra adds a term
 // u * q_extra * k x for geometry whose d carries more than the one rounding of
 // a_h - p (the midpoint)
-template <int KIND, bool SPLIT, typename T>
+template <int KIND, int AF, typename T>
 __device__ __forceinline__ T arrival_fast(const MedParams& M, const GeoT<T>& g, T S, T rho2, T Teh, T Tel, T Tah, T Tal,
                                           float fb_abs, float fb_rel_v, T qv, float q_extra, T& uf_out) {
   static_assert(KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL, "plain straight-line media only");
@@ -836,11 +888,24 @@ __device__ __forceinline__ T arrival_fast(const MedParams& M, const GeoT<T>& g, 
   // R' = sqrt(S) rounded once (the direct form), or the unrefined R0 (the
   // split form, whose x is small: R enters it only through its denominator)
   T R = g.R0;
-  if constexpr (!SPLIT) R = fma_rn(fma_rn(neg(g.R0), g.R0, S), mul_rn(bc<T>(0.5f), g.y), g.R0);
+  if constexpr (AF == kFormDirect) R = fma_rn(fma_rn(neg(g.R0), g.R0, S), mul_rn(bc<T>(0.5f), g.y), g.R0);
   // x = R - w, w = z_e - z_a = -s_z
   const T sz = g.s[2];
   T x;
-  if constexpr (SPLIT) {
+  float kR = AF == kFormAxis ? 0.375f : 2.5f;
+  if constexpr (AF == kFormAxis) {
+    const T a0 = bc<T>(M.ax[0]), a1 = bc<T>(M.ax[1]), a2 = bc<T>(M.ax[2]);
+    const T cx = fma_rn(g.s[1], a2, neg(mul_rn(sz, a1))), cy = fma_rn(sz, a0, neg(mul_rn(g.s[0], a2))),
+            cz = fma_rn(g.s[0], a1, neg(mul_rn(g.s[1], a0)));
+    const T w = axis_w(M, g);
+    x = div_ap(fma_rn(cx, cx, fma_rn(cy, cy, mul_rn(cz, cz))), add_rn(R, w));
+    kR = __fmaf_rn(q_extra, 0.0625f, kR);
+    if constexpr (!kUsualForm<T>)
+      if (!(w >= 0.0f)) {
+        x = __fsub_rn(R, w);
+        kR = 10.0f;
+      }
+  } else if constexpr (AF == kFormSplit) {
     x = div_ap(rho2, sub_rn(R, sz));
     if constexpr (!kUsualForm<T>) x = sz < 0.0f ? x : __fadd_rn(R, sz);
   } else {
@@ -854,12 +919,13 @@ __device__ __forceinline__ T arrival_fast(const MedParams& M, const GeoT<T>& g, 
   const T uf = add_rn(add_rn(Td, q), v);
   uf_out = uf;
   const T tail = fma_rn(bc<T>(2.25f * u), abs_of(Td),
-                        fma_rn(bc<T>(__fmaf_rn(SPLIT ? 22.0f : 17.0f, u, fb_rel_v)), abs_of(v),
+                        fma_rn(bc<T>(__fmaf_rn(AF == kFormDirect ? 17.0f : 22.0f, u, fb_rel_v)), abs_of(v),
                                fma_rn(bc<T>(3.25f * u), abs_of(uf), bc<T>(fb_abs))));
-  if constexpr (SPLIT) {
+  if constexpr (AF == kFormSplit) {
     return fma_rn(bc<T>(__fmaf_rn(q_extra, u, 19.0f * u)), q, tail);
   } else {
-    return fma_rn(bc<T>(__fmaf_rn(q_extra, u, 6.25f * u)), q, fma_rn(bc<T>(__fmul_rn(2.5f * u, kh)), R, tail));
+    const float cq = AF == kFormAxis ? __fmaf_rn(q_extra, 8.0f * u, 72.0f * u) : __fmaf_rn(q_extra, u, 6.25f * u);
+    return fma_rn(bc<T>(cq), q, fma_rn(bc<T>(__fmul_rn(kR * u, kh)), R, tail));
   }
 }
 

@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(Ops::kFwdThreads, Ops::kMinBlocks) k_forward(c
   const int64_t t_end = min(t_begin + a.g.tiles_per_range, a.n_tiles);
   if (t_begin >= t_end || n_here <= 0) return;  // uniform over the CTA
   const int tid = threadIdx.x;
-  for (int i = tid; i < n_here; i += blockDim.x) Ops::stage_ant(ant_s + i, a.ants[ant0 + i]);
+  for (int i = tid; i < n_here; i += blockDim.x) Ops::stage_ant(ant_s + i, a.ants[ant0 + i], a.M);
   if (tid == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -655,7 +655,7 @@ __global__ void __launch_bounds__(kTileT, Ops::kBwdMinBlocks) k_backward(const B
   const int N = M.n_bins;
   const acc4* G = static_cast<const acc4*>(a.G) + (size_t)ant0 * N;
   const PrefixFF* Gp = a.Gp ? a.Gp + (size_t)ant0 * (N + 1) : nullptr;
-  for (int i = tid; i < n_here; i += nthr) Ops::stage_ant(ant_s + i, a.ants[ant0 + i]);
+  for (int i = tid; i < n_here; i += nthr) Ops::stage_ant(ant_s + i, a.ants[ant0 + i], a.M);
   for (int i = tid; i < 3 * n_here + 1; i += nthr) sg[i] = acc_t(0);
   const uint32_t bytes = (uint32_t)L.stage_bytes;
   const unsigned char* src = static_cast<const unsigned char*>(a.tiles);

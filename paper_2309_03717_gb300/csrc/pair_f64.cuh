@@ -139,7 +139,7 @@ struct OpsF64 {
   static constexpr int kAccRows = FORM == C8R_ZHS ? 2 : 1;  // as the plain media's kernels (OpsF64Plain)
 
   using Ant = AntRec;
-  static __device__ __forceinline__ void stage_ant(AntRec* p, const AntRec& A) { *p = A; }
+  static __device__ __forceinline__ void stage_ant(AntRec* p, const AntRec& A, const MedParams&) { *p = A; }
   static __device__ __forceinline__ AntRec load_ant(const AntRec* p) { return *p; }
 
   static __device__ __forceinline__ void load(const void* Tv, int l, const MedParams&, TrackD& t) {
@@ -724,7 +724,7 @@ struct OpsF64Plain {
   };
   using FwdAnt = AntRec;
   using Ant = AntRec;
-  static __device__ __forceinline__ void stage_ant(AntRec* p, const AntRec& A) { *p = A; }
+  static __device__ __forceinline__ void stage_ant(AntRec* p, const AntRec& A, const MedParams&) { *p = A; }
   static __device__ __forceinline__ AntRec load_ant(const AntRec* p) { return *p; }
 
   // n_avg - 1 of the path from altitude z_e to z_a, dz = z_a - z_e, in the

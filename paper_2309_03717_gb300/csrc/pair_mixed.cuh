@@ -107,7 +107,7 @@ struct TrackE {
   float amp;             // q K/dt; 0 = dropped
 };
 
-template <int KIND, bool FLAT>
+template <int KIND, int AF, bool FLAT>
 __device__ __forceinline__ void load_track_endpoints(const float* T, int l, const MedParams& M, TrackE& t) {
   t.amp = TF(fm::AMPE);
   if (t.amp == 0.0f) return;  // filtered track or padding
@@ -117,8 +117,14 @@ __device__ __forceinline__ void load_track_endpoints(const float* T, int l, cons
   t.bx = TF(fm::BX); t.by = TF(fm::BY); t.bz = TF(fm::BZ);
   t.bmag = TF(fm::BMAG);
   const float kh = KIND == C8R_UNIFORM ? M.s_h : M.kc_h, kl = KIND == C8R_UNIFORM ? M.s_l : M.kc_l;
-  shifted_time(TF(fm::TAU0H), TF(fm::TAU0L), t.z.x, 0.0f, kh, kl, t.Th.x, t.Tl.x);
-  shifted_time(TF(fm::TAU1H), TF(fm::TAU1L), t.z.y, 0.0f, kh, kl, t.Th.y, t.Tl.y);
+  if constexpr (AF == kFormAxis) {
+    const float p0[3] = {t.x.x, t.y.x, t.z.x}, p1[3] = {t.x.y, t.y.y, t.z.y}, low[3] = {0.0f, 0.0f, 0.0f};
+    axis_time(M, TF(fm::TAU0H), TF(fm::TAU0L), p0, low, t.Th.x, t.Tl.x);
+    axis_time(M, TF(fm::TAU1H), TF(fm::TAU1L), p1, low, t.Th.y, t.Tl.y);
+  } else {
+    shifted_time(TF(fm::TAU0H), TF(fm::TAU0L), t.z.x, 0.0f, kh, kl, t.Th.x, t.Tl.x);
+    shifted_time(TF(fm::TAU1H), TF(fm::TAU1L), t.z.y, 0.0f, kh, kl, t.Th.y, t.Tl.y);
+  }
   float2 nm1 = bc<float2>(M.nm1f);
   t.Eh = bc<float2>(1.0f);
   if constexpr (KIND == C8R_EXPONENTIAL) {
@@ -525,7 +531,7 @@ __device__ __forceinline__ LinEnds lin_ends(int Jlo, float slo, int Jhi, float s
   return z;
 }
 
-template <int FORM, int KIND, bool LIN = false, bool SPLIT = false, bool FLAT = false>
+template <int FORM, int KIND, bool LIN = false, int AF = kFormDirect, bool FLAT = false>
 struct OpsMixed {
   using acc_t = float;
   using Track = TrackM;
@@ -556,7 +562,7 @@ struct OpsMixed {
   // exact to its own bound; the host picks the kernel per launch from the
   // share of tracks that see the antenna array from above within 45 degrees
   // (counted by the ingest of earlier launches)
-  static constexpr bool kSplit = SPLIT && kFastBins;
+  static constexpr int kAF = kFastBins ? AF : kFormDirect;
   // a flat antenna array: the refractivity quotient per track, in the main pass
   // of the Endpoint forward kernel of the direct arrival form and in the ZHS
   // forward and adjoint kernels, which also take the z part of the midpoint's
@@ -567,7 +573,7 @@ struct OpsMixed {
   // the Endpoint and then the ZHS process on the same tracks.  The split-form
   // Endpoint kernel keeps the quotient per pair (within 0.3 % either way)
   static constexpr bool kFlat =
-      FLAT && KIND != C8R_UNIFORM && ((kFastBins && !SPLIT) || FORM == C8R_ZHS);
+      FLAT && KIND != C8R_UNIFORM && ((kFastBins && AF != kFormSplit) || FORM == C8R_ZHS);
   // adjoint CTAs (128 threads) per SM the registers are set for (the linear
   // Endpoint adjoint carries the slide of each deposit as well)
   static constexpr int kBwdMinBlocks = (LIN && FORM == C8R_ENDPOINT) ? 4 : (kFastBins ? 5 : 6);
@@ -579,7 +585,7 @@ struct OpsMixed {
   // the antenna record that the forward and adjoint kernels hold in shared memory
   using FwdAnt = std::conditional_t<kTwoTracks, AntZ, std::conditional_t<kFastBins, AntE, AntRec>>;
   using Ant = std::conditional_t<kFastBins, AntE, AntRec>;
-  static __device__ __forceinline__ void stage_ant(AntZ* p, const AntRec& A) {
+  static __device__ __forceinline__ void stage_ant(AntZ* p, const AntRec& A, const MedParams&) {
     AntZ z;
     z.x = bc<float2>(A.xh); z.y = bc<float2>(A.yh); z.z = bc<float2>(A.zh);
     z.xl = bc<float2>(A.xl); z.yl = bc<float2>(A.yl); z.zl = bc<float2>(A.zl);
@@ -596,7 +602,7 @@ struct OpsMixed {
     r.Eah = p->Eh.x; r.Eal = p->El.x;
     return r;
   }
-  static __device__ __forceinline__ void stage_ant(Ant* p, const AntRec& A) {
+  static __device__ __forceinline__ void stage_ant(Ant* p, const AntRec& A, const MedParams& M) {
     if constexpr (kFastBins) {
       AntE e;
       e.x = bc<float2>(A.xh); e.y = bc<float2>(A.yh); e.z = bc<float2>(A.zh);
@@ -605,6 +611,15 @@ struct OpsMixed {
       e.fb_abs = A.fb_abs; e.fb_rel_v = A.fb_rel_v;
       e.xl = A.xl; e.yl = A.yl; e.zl = A.zl; e.tauh = A.tauh; e.taul = A.taul;
       e.pad[0] = e.pad[1] = e.pad[2] = 0.0f;
+      if constexpr (kAF == kFormAxis) {
+        // the antenna's shifted time along the axis, and 16 u^2 of it for the bound
+        const float ph[3] = {A.xh, A.yh, A.zh}, pl[3] = {A.xl, A.yl, A.zl};
+        float Th, Tl;
+        axis_time(M, A.tauh, A.taul, ph, pl, Th, Tl);
+        e.Th = bc<float2>(Th);
+        e.Tl = bc<float2>(Tl);
+        e.fb_abs = __fmaf_rn(5.7e-14f, fabsf(Th), e.fb_abs);
+      }
       *p = e;
     } else {
       *p = A;
@@ -639,7 +654,7 @@ struct OpsMixed {
   using MainTrack = std::conditional_t<kFastBins, TrackE, TrackM>;
   static __device__ __forceinline__ void load_main(const void* Tv, int l, const MedParams& M, MainTrack& t) {
     if constexpr (kFastBins)
-      load_track_endpoints<KIND, kFlat>(static_cast<const float*>(Tv), l, M, t);
+      load_track_endpoints<KIND, kAF, kFlat>(static_cast<const float*>(Tv), l, M, t);
     else
       load(Tv, l, M, t);
   }
@@ -948,7 +963,7 @@ struct OpsMixed {
       q = half_of<J>(t.q);
     else if constexpr (KIND == C8R_EXPONENTIAL)
       q = fast_quotient(M, A.Eh.x, A.El.x, g.s[2], half_of<J>(t.Eh), half_of<J>(t.El));
-    eps = arrival_fast<KIND, kSplit>(M, g, half_of<J>(S), half_of<J>(P), half_of<J>(t.Th), half_of<J>(t.Tl), A.Th.x,
+    eps = arrival_fast<KIND, kAF>(M, g, half_of<J>(S), half_of<J>(P), half_of<J>(t.Th), half_of<J>(t.Tl), A.Th.x,
                                      A.Tl.x, A.fb_abs, A.fb_rel_v, q, 0.0f, uf);
     FieldM f;
     field_mixed(g, t.bx, t.by, t.bz, t.bmag, half_of<J>(t.om), half_of<J>(t.n), f);
@@ -971,14 +986,18 @@ struct OpsMixed {
       q = t.q;
     else if constexpr (KIND == C8R_EXPONENTIAL)
       q = fast_quotient(M, A.Eh, A.El, g.s[2], t.Eh, t.El);
-    float2 eps = arrival_fast<KIND, kSplit>(M, g, S, P, t.Th, t.Tl, A.Th, A.Tl, A.fb_abs, A.fb_rel_v, q, 0.0f, uf);
+    float2 eps = arrival_fast<KIND, kAF>(M, g, S, P, t.Th, t.Tl, A.Th, A.Tl, A.fb_abs, A.fb_rel_v, q, 0.0f, uf);
     field_mixed(g, bc<float2>(t.bx), bc<float2>(t.by), bc<float2>(t.bz), bc<float2>(t.bmag), t.om, t.n, f);
     // the usual forms: bd >= 0 (the Doppler factor); an altitude difference
     // beyond 1e-3 H, tested at 1.001e-3 H so that no rounding lets one through
     // (the refractivity quotient); an emission point above the antenna (the
-    // split form)
+    // split form); an antenna ahead of it along the axis (the axis form)
     bool usual = fminf(f.bd.x, f.bd.y) >= 0.0f;
-    if constexpr (kSplit)
+    if constexpr (kAF == kFormAxis) {
+      const float2 w = axis_w(M, g);
+      usual = usual && fminf(w.x, w.y) >= 0.0f;
+    }
+    if constexpr (kAF == kFormSplit)
       usual = usual && fmaxf(g.s[2].x, g.s[2].y) < (KIND == C8R_EXPONENTIAL ? M.dz_series : 0.0f);
     else if constexpr (KIND == C8R_EXPONENTIAL && !kFlat)
       usual = usual && fminf(fabsf(g.s[2].x), fabsf(g.s[2].y)) > -M.dz_series;
@@ -1095,13 +1114,21 @@ struct OpsMixed {
       two_sum(z0, z1, zmh, zml);
       const float kh = KIND == C8R_UNIFORM ? M.s_h : M.kc_h, kl = KIND == C8R_UNIFORM ? M.s_l : M.kc_l;
       float Tmh, Tml;
-      shifted_time(tmh, tml, 0.5f * zmh, 0.5f * zml, kh, kl, Tmh, Tml);
+      if constexpr (kAF == kFormAxis) {
+        float xmh, xml, ymh, yml;
+        two_sum(x0, x1, xmh, xml);
+        two_sum(y0, y1, ymh, yml);
+        const float ph[3] = {0.5f * xmh, 0.5f * ymh, 0.5f * zmh}, pl[3] = {0.5f * xml, 0.5f * yml, 0.5f * zml};
+        axis_time(M, tmh, tml, ph, pl, Tmh, Tml);
+      } else {
+        shifted_time(tmh, tml, 0.5f * zmh, 0.5f * zml, kh, kl, Tmh, Tml);
+      }
       float uf;
       const float qv = KIND == C8R_EXPONENTIAL ? fast_quotient<float>(M, A.Eah, A.Eal, g.s[2], Eh, El) : 0.0f;
       // the kernel's arrival form (either is exact to its own bound; one form
       // for every lane keeps the warp on one path)
       const float eps_a =
-          arrival_fast<KIND, kSplit, float>(M, g, S, rho2, Tmh, Tml, A.Tah, A.Tal, A.fb_abs, A.fb_rel_v, qv, 3.0f, uf);
+          arrival_fast<KIND, kAF, float>(M, g, S, rho2, Tmh, Tml, A.Tah, A.Tal, A.fb_abs, A.fb_rel_v, qv, 3.0f, uf);
       const float eps_u = __fmaf_rn(2.0f * u * kh, L1, eps_a);
       const float dtau = TF(fm::DTAUH);
       const float aD = fabsf(f.D);
@@ -1786,23 +1813,28 @@ cudaError_t forward_mixed(int formalism, const void* tiles, int64_t n_tiles, con
   const bool ex = M.kind == C8R_EXPONENTIAL;
   if (M.kind == C8R_EXPONENTIAL_SPHERICAL)
     return formalism == C8R_ENDPOINT ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_SPHERICAL, LIN>{})
-           : M.flat                  ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_SPHERICAL, LIN, false, true>{})
+           : M.flat                  ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_SPHERICAL, LIN, kFormDirect, true>{})
                                      : go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_SPHERICAL, LIN>{});
   if (M.kind == C8R_EXPONENTIAL_RAY)
     return formalism == C8R_ENDPOINT ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_RAY, LIN>{})
-           : M.flat                  ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, LIN, false, true>{})
+           : M.flat                  ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, LIN, kFormDirect, true>{})
                                      : go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, LIN>{});
   if constexpr (!LIN) {
-    // the one-bin Endpoint kernels come in both arrival forms (M.split) and,
-    // for the direct form in the exponential medium, for a flat antenna array
+    // the one-bin Endpoint kernels come in the arrival forms (M.axis, M.split)
+    // and, but for the split form, in the exponential medium for a flat antenna array
     // (M.flat, OpsMixed::kFlat)
     if (formalism == C8R_ENDPOINT) {
+      if (M.axis) {
+        if (!ex) return go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>{});
+        return M.flat ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis, true>{})
+                      : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis>{});
+      }
       if (!ex)
-        return M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, true>{})
-                       : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, false>{});
-      if (M.split) return go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, true>{});
-      return M.flat ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, false, true>{})
-                    : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, false>{});
+        return M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{})
+                       : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
+      if (M.split) return go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{});
+      return M.flat ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{})
+                    : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>{});
     }
   }
   if (formalism == C8R_ENDPOINT)
@@ -1810,7 +1842,7 @@ cudaError_t forward_mixed(int formalism, const void* tiles, int64_t n_tiles, con
   // ZHS in the exponential medium: for a flat array the kernel that forms the
   // midpoint's refractivity quotient and the z part of its d once per track
   // (OpsMixed::kFlat)
-  if (ex && M.flat) return go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, LIN, false, true>{});
+  if (ex && M.flat) return go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, LIN, kFormDirect, true>{});
   return ex ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, LIN>{}) : go(OpsMixed<C8R_ZHS, C8R_UNIFORM, LIN>{});
 }
 
@@ -1819,14 +1851,17 @@ cudaError_t backward_mixed(int formalism, BwdArgs& a, const FwdShape& shape, int
   const bool ex = a.M.kind == C8R_EXPONENTIAL;
   if (formalism == C8R_ZHS) {
     if (ex && a.M.flat)
-      return launch_backward_ops<OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, LIN, false, true>>(a, shape, sm_count, st);
+      return launch_backward_ops<OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, LIN, kFormDirect, true>>(a, shape, sm_count, st);
     return ex ? launch_backward_ops<OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, LIN>>(a, shape, sm_count, st)
               : launch_backward_ops<OpsMixed<C8R_ZHS, C8R_UNIFORM, LIN>>(a, shape, sm_count, st);
   }
   if constexpr (!LIN) {
+    if (a.M.axis)
+      return ex ? launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis>>(a, shape, sm_count, st)
+                : launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>>(a, shape, sm_count, st);
     if (a.M.split)
-      return ex ? launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, true>>(a, shape, sm_count, st)
-                : launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, true>>(a, shape, sm_count, st);
+      return ex ? launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>>(a, shape, sm_count, st)
+                : launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>>(a, shape, sm_count, st);
   }
   return ex ? launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, LIN>>(a, shape, sm_count, st)
             : launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, LIN>>(a, shape, sm_count, st);

@@ -129,3 +129,43 @@ def test_zhs_over_a_sphere_and_along_rays(reach, z, medium, deposit):
     for a in range(n_ant):
         if np.abs(ref[a]).max() > 0:
             assert rel_l2(got[a], ref[a]) <= TOL, a
+
+
+@pytest.mark.parametrize("medium", [None, UNIFORM])
+@pytest.mark.parametrize("zenith,hills,offset", [(35.0, 0.0, 0.0), (60.0, 0.0, 0.0), (60.0, 150.0, 0.0),
+                                                 (78.0, 0.0, 1.0e6), (50.0, 0.0, None)])
+def test_axis_form_gives_the_bins_of_the_others(zenith, hills, offset, medium):
+    """Windows placed along an inclined front: the automatic form (along the
+    front's axis) against the pinned direct one, traces and adjoint, which take
+    the same bins and so differ by the order of additions only.  Also with a time
+    origin 1e6 ns early, and (offset None) with antennas far up the axis, behind
+    most of the tracks."""
+    from paper_2309_03717_gb300 import c8r
+    n = 4001
+    tracks = synth.make_tracks(n, 31, zenith)
+    ant = synth.antennas_star(8, n_radii=9)[:67].copy()
+    ant[:, 2] = np.linspace(0.0, hills, len(ant))
+    if offset is None:
+        ant[::3] += 5000.0 * synth.shower_axis_up(zenith)
+    t_start = synth.trace_start_ns(ant, zenith)
+    if offset:
+        t_start = t_start + offset
+        for f in ("t0", "t1"):
+            tracks[f] = (tracks[f].astype(np.float64) + offset).astype(np.float32)
+    out = []
+    for form in ("auto", "direct"):
+        p = c8r.RadioProcess(medium or synth.AIR_EXPONENTIAL, ant, t_start, 4096, 0.2, "endpoint", "mixed")
+        p.set_arrival_form(form)
+        dev = to_device(tracks)
+        p.push(dev)
+        tr = p.traces().cpu().numpy()
+        G = torch.from_numpy(np.random.default_rng(3).normal(size=tr.shape).astype(np.float32)).cuda()
+        tg = {f: torch.zeros(n, dtype=torch.float32, device="cuda") for f in c8r.GRAD_FIELDS}
+        ag = torch.zeros((len(ant), 3), dtype=torch.float64, device="cuda")
+        dn = torch.zeros(1, dtype=torch.float64, device="cuda")
+        c8r.c8r_backward(p.ctx, dev, G, tg, ag, dn)
+        out.append((tr, np.stack([tg[f].cpu().numpy() for f in c8r.GRAD_FIELDS]), ag.cpu().numpy()))
+        p.close()
+    assert np.abs(out[1][0]).max() > 0
+    for a, d in zip(*out):
+        assert rel_l2(a, d) <= 2e-6
