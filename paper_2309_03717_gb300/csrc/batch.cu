@@ -167,16 +167,18 @@ cudaError_t launch_batch_ops(const BatchArgs& a, int sm_count, cudaStream_t st) 
 template <class F>
 auto with_batch_ops(int formalism, int kind, bool split, bool flat, F f) {
   const bool ex = kind == C8R_EXPONENTIAL;
-  // the arrival form of the one-bin Endpoint kernel (OpsMixed::kAF) and, for
-  // the direct form, the flat-array kernel of the exponential medium
-  // (OpsMixed::kFlat)
+  // the arrival form of the one-bin Endpoint kernel (OpsMixed::kAF) and the
+  // flat-array kernels of the exponential medium (OpsMixed::kFlat)
   if (formalism == C8R_ENDPOINT) {
     if (!ex)
       return split ? f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{}) : f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
-    if (split) return f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{});
+    if (split)
+      return flat ? f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit, true>{})
+                  : f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{});
     return flat ? f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{})
                 : f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>{});
   }
+  if (ex && flat) return f(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, false, kFormDirect, true>{});
   return ex ? f(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL>{}) : f(OpsMixed<C8R_ZHS, C8R_UNIFORM>{});
 }
 

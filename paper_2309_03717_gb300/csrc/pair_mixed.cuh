@@ -563,17 +563,16 @@ struct OpsMixed {
   // share of tracks that see the antenna array from above within 45 degrees
   // (counted by the ingest of earlier launches)
   static constexpr int kAF = kFastBins ? AF : kFormDirect;
-  // a flat antenna array: the refractivity quotient per track, in the main pass
-  // of the Endpoint forward kernel of the direct arrival form and in the ZHS
-  // forward and adjoint kernels, which also take the z part of the midpoint's
-  // d once per track (ZPart; the host picks the kernel, MedParams::flat).
-  // Measured: 47.96 -> 44.01 ms on 4e6 tracks of the 60-degree array
-  // (Endpoint); ZHS 31.96 -> 29.56 ms with the quotient and -> 28.50 ms with
-  // the z part as well, on the 2e7-track vertical shower in a step that runs
-  // the Endpoint and then the ZHS process on the same tracks.  The split-form
-  // Endpoint kernel keeps the quotient per pair (within 0.3 % either way)
-  static constexpr bool kFlat =
-      FLAT && KIND != C8R_UNIFORM && ((kFastBins && AF != kFormSplit) || FORM == C8R_ZHS);
+  // a flat antenna array: the refractivity quotient per track, in the one-bin
+  // Endpoint kernels and in the ZHS forward and adjoint kernels, which also take
+  // the z part of the midpoint's d once per track (ZPart; the host picks the
+  // kernel, MedParams::flat).  Both the per-pair quotient and its operands leave
+  // the pair's registers.  Endpoint, per-pair quotient -> per track: 4e6-track
+  // vertical shower x 160 antennas (split form) 4.71 -> 4.58 ms; adjoint on 1e6
+  // tracks x 64 antennas 963 -> 942 us (split), 1039 -> 988 (axis); 64 uneven
+  // showers in a batch 2.99 -> 2.96 ms.  ZHS, one track per thread, 2e7-track
+  // vertical shower: 31.96 -> 29.56 ms, and 28.50 with the z part as well
+  static constexpr bool kFlat = FLAT && KIND != C8R_UNIFORM && (kFastBins || FORM == C8R_ZHS);
   // adjoint CTAs (128 threads) per SM the registers are set for (the linear
   // Endpoint adjoint carries the slide of each deposit as well)
   static constexpr int kBwdMinBlocks = (LIN && FORM == C8R_ENDPOINT) ? 4 : (kFastBins ? 5 : 6);
@@ -1821,8 +1820,8 @@ cudaError_t forward_mixed(int formalism, const void* tiles, int64_t n_tiles, con
                                      : go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, LIN>{});
   if constexpr (!LIN) {
     // the one-bin Endpoint kernels come in the arrival forms (M.axis, M.split)
-    // and, but for the split form, in the exponential medium for a flat antenna array
-    // (M.flat, OpsMixed::kFlat)
+    // and, in the exponential medium, for a flat antenna array (M.flat,
+    // OpsMixed::kFlat)
     if (formalism == C8R_ENDPOINT) {
       if (M.axis) {
         if (!ex) return go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>{});
@@ -1832,7 +1831,9 @@ cudaError_t forward_mixed(int formalism, const void* tiles, int64_t n_tiles, con
       if (!ex)
         return M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{})
                        : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
-      if (M.split) return go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{});
+      if (M.split)
+        return M.flat ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit, true>{})
+                      : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{});
       return M.flat ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{})
                     : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>{});
     }
@@ -1856,12 +1857,17 @@ cudaError_t backward_mixed(int formalism, BwdArgs& a, const FwdShape& shape, int
               : launch_backward_ops<OpsMixed<C8R_ZHS, C8R_UNIFORM, LIN>>(a, shape, sm_count, st);
   }
   if constexpr (!LIN) {
+    auto go = [&](auto ops) { return launch_backward_ops<decltype(ops)>(a, shape, sm_count, st); };
+    if (ex && a.M.flat)
+      return a.M.axis    ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis, true>{})
+             : a.M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit, true>{})
+                         : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{});
     if (a.M.axis)
-      return ex ? launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis>>(a, shape, sm_count, st)
-                : launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>>(a, shape, sm_count, st);
+      return ex ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis>{})
+                : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>{});
     if (a.M.split)
-      return ex ? launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>>(a, shape, sm_count, st)
-                : launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>>(a, shape, sm_count, st);
+      return ex ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{})
+                : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{});
   }
   return ex ? launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, LIN>>(a, shape, sm_count, st)
             : launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, LIN>>(a, shape, sm_count, st);

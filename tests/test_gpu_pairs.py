@@ -71,6 +71,44 @@ def test_traces_and_adjoint_with_antennas_among_the_tracks(n, n_ant, medium, for
     assert rel_l2(ag.cpu().numpy(), ag_ref) <= TOL
 
 
+@pytest.mark.parametrize("form", ["split", "direct"])
+@pytest.mark.parametrize("n,n_ant,height", [(1, 1, 0.0), (129, 33, 0.0), (700, 5, None)])
+def test_flat_arrays_give_what_uneven_ones_do(n, n_ant, height, form):
+    """A flat array's kernels form the refractivity quotient per track; one more
+    antenna at another altitude (its dL/dtrace is zero) sends the same antennas
+    through the kernels that form it per pair.  Same bins and roundings: what is
+    left is the order of up to 2 x 700 additions, 1400 x 2^-24 at most of the sum
+    of magnitudes and its square root of them as a rule (2e-6).  Ground below the
+    tracks, and at their median height (None), where some quotients are series."""
+    from paper_2309_03717_gb300 import c8r
+    w, tracks = among_the_tracks(n, n_ant, None)
+    if height is None:
+        height = float(np.median(tracks["z0"]))
+    ant = w["ant_xyz"].copy()
+    ant[:, 2] = height
+    _, u0 = oracle_arrivals(tracks, ant, np.zeros(n_ant), 1, w["dt_ns"], w["medium"], "endpoint")
+    t_start = np.median(u0.reshape(n, n_ant, 2)[..., 0], axis=0) * w["dt_ns"] - 200.0
+    G = np.random.default_rng(n).normal(size=(n_ant + 1, 3, w["n_bins"])).astype(np.float32)
+    G[-1] = 0.0
+    dev, out = to_device(tracks), []
+    for extra in (0, 1):
+        k = n_ant + extra
+        p = c8r.RadioProcess(w["medium"], np.concatenate([ant, ant[:1] + [0.0, 0.0, 900.0]])[:k],
+                             np.concatenate([t_start, t_start[:1]])[:k], w["n_bins"], w["dt_ns"], "endpoint", "mixed")
+        p.set_arrival_form(form)
+        p.push(dev)
+        tg = {f: torch.zeros(n, dtype=torch.float32, device="cuda") for f in c8r.GRAD_FIELDS}
+        ag = torch.zeros((k, 3), dtype=torch.float64, device="cuda")
+        dn = torch.zeros(1, dtype=torch.float64, device="cuda")
+        c8r.c8r_backward(p.ctx, dev, torch.from_numpy(G[:k]).cuda(), tg, ag, dn)
+        out.append((p.traces().cpu().numpy()[:n_ant], ag.cpu().numpy()[:n_ant],
+                    np.stack([tg[f].double().cpu().numpy() for f in c8r.GRAD_FIELDS], axis=1)))
+        p.close()
+    for flat, uneven in zip(*out):
+        assert np.abs(uneven).max() > 0
+        assert rel_l2(flat, uneven) <= 2e-5
+
+
 @pytest.mark.parametrize("deposit", ["bin", "linear"])
 @pytest.mark.parametrize("medium", [None, UNIFORM])
 @pytest.mark.parametrize("n,n_ant,n_bins", [(1, 1, 2048), (2, 3, 7), (127, 31, 2048), (129, 33, 2048), (700, 5, 1),
