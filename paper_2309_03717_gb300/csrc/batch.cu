@@ -6,14 +6,15 @@
 // track tiles) and uploads the list, largest shower first and, inside a shower,
 // antenna tiles fastest (so the items in flight share track tiles in L2 and add
 // into one shower's accumulator rows); for the one-bin Endpoint evaluation the
-// showers are grouped by the form of their FP32 arrival (a vote per shower),
-// and each group gets a launch of its own.  A persistent grid of every CTA the
-// device holds pops items from a global atomic counter; for each item a CTA streams the item's
-// track tiles through the same TMA ring as the single-shower kernel and adds the
-// deposits into the batch accumulator.  The CTA polls a cancel word between
-// items.  Zeroing the accumulator, the ingest of all showers, the counter reset,
-// the persistent kernel and the conversion into the caller's trace layout are
-// captured once into a CUDA graph and replayed.  The tile shape (antennas per
+// showers are grouped by the form of their FP32 arrival (their windows' front and
+// a vote per shower), and each group gets a launch of its own, the groups side by
+// side.  A persistent grid of every CTA the device holds pops items from a global
+// atomic counter; for each item a CTA streams the item's track tiles
+// through the same TMA ring as the single-shower kernel and adds the deposits into
+// the batch accumulator.  The CTA polls a cancel word between items.  Zeroing the
+// accumulator, the ingest of all showers, the counter reset, the persistent
+// kernels and the conversion into the caller's trace layout are captured once into
+// a CUDA graph and replayed.  The tile shape (antennas per
 // CTA, track tiles per item) is picked by a small autotuner that times the
 // candidates on a subsample of the real work list and caches the choice.
 #include <algorithm>
@@ -36,6 +37,12 @@ struct WorkItem {
   int32_t n_here;   // antennas in this item
   int64_t t_begin;  // first derived-track tile
   int64_t t_end;
+  int64_t shower;   // whose axis an item of the axis form takes (BatchArgs::axes)
+};
+
+// the axis of a shower's windows for the axis form (MedParams::ax, kax_h, kax_l)
+struct ShowerAxis {
+  float ax[3], kax_h[3], kax_l[3];
 };
 
 struct BatchArgs {
@@ -51,6 +58,7 @@ struct BatchArgs {
   MedParams M;
   int replicas;            // accumulator copies: work item i adds into copy i % replicas
   int64_t replica_stride;  // elements per copy
+  const ShowerAxis* axes;  // [n_showers] (the axis form only)
 };
 
 // slot -> caller track index for the concatenated showers: shower s owns tiles
@@ -114,7 +122,6 @@ __global__ void __launch_bounds__(256) k_batch_votes(const float* tiles, const V
 template <class Ops>
 __global__ void __launch_bounds__(Ops::kFwdThreads, Ops::kMinBlocks) k_batch(const BatchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
-  const MedParams& M = a.M;
   const FwdLayout L = fwd_layout(Ops::kPrec, a.a_tile, Ops::kDefers);
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.bar_off);
   typename Ops::FwdAnt* ant_s = reinterpret_cast<typename Ops::FwdAnt*>(smem + L.ant_off);
@@ -136,6 +143,15 @@ __global__ void __launch_bounds__(Ops::kFwdThreads, Ops::kMinBlocks) k_batch(con
     const int idx = s_item;
     if (idx < 0 || idx >= a.n_items) break;
     const WorkItem w = a.items[idx];
+    MedParams M = a.M;
+    if constexpr (Ops::kAF == kFormAxis) {
+      const ShowerAxis x = a.axes[w.shower];
+      for (int c = 0; c < 3; ++c) {
+        M.ax[c] = x.ax[c];
+        M.kax_h[c] = x.kax_h[c];
+        M.kax_l[c] = x.kax_l[c];
+      }
+    }
     for (int i = tid; i < w.n_here; i += nthr) Ops::stage_ant(ant_s + i, a.ants[w.ant0 + i], M);
     __syncthreads();
     float4* acc = a.acc + (size_t)(idx % a.replicas) * a.replica_stride + (size_t)w.ant0 * M.n_bins * Ops::kAccRows;
@@ -165,14 +181,19 @@ cudaError_t launch_batch_ops(const BatchArgs& a, int sm_count, cudaStream_t st) 
 }
 
 template <class F>
-auto with_batch_ops(int formalism, int kind, bool split, bool flat, F f) {
+auto with_batch_ops(int formalism, int kind, int form, bool flat, F f) {
   const bool ex = kind == C8R_EXPONENTIAL;
   // the arrival form of the one-bin Endpoint kernel (OpsMixed::kAF) and the
   // flat-array kernels of the exponential medium (OpsMixed::kFlat)
   if (formalism == C8R_ENDPOINT) {
     if (!ex)
-      return split ? f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{}) : f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
-    if (split)
+      return form == kFormAxis    ? f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>{})
+             : form == kFormSplit ? f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{})
+                                  : f(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
+    if (form == kFormAxis)
+      return flat ? f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis, true>{})
+                  : f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis>{});
+    if (form == kFormSplit)
       return flat ? f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit, true>{})
                   : f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{});
     return flat ? f(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{})
@@ -182,13 +203,13 @@ auto with_batch_ops(int formalism, int kind, bool split, bool flat, F f) {
   return ex ? f(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL>{}) : f(OpsMixed<C8R_ZHS, C8R_UNIFORM>{});
 }
 
-cudaError_t launch_batch(const BatchArgs& a, int formalism, int sm_count, cudaStream_t st) {
-  return with_batch_ops(formalism, a.M.kind, a.M.split != 0, a.M.flat != 0,
+cudaError_t launch_batch(const BatchArgs& a, int formalism, int form, int sm_count, cudaStream_t st) {
+  return with_batch_ops(formalism, a.M.kind, form, a.M.flat != 0,
                         [&](auto ops) { return launch_batch_ops<decltype(ops)>(a, sm_count, st); });
 }
 
 int batch_resident(int formalism, int kind, int a_tile, int sm_count) {
-  return sm_count * with_batch_ops(formalism, kind, false, false,
+  return sm_count * with_batch_ops(formalism, kind, kFormDirect, false,
                                    [&](auto ops) { return batch_blocks_per_sm<decltype(ops)>(a_tile); });
 }
 
@@ -258,17 +279,24 @@ struct c8r_batch {
   int* d_counter = nullptr;
   int* d_cancel = nullptr;
   int* d_err = nullptr;
-  // the arrival form of each shower (Endpoint, one-bin: MedParams::split);
-  // the work list holds the split-form showers' items first, n_items_split of
-  // them, then the direct-form showers', each group run by its own launch
-  std::vector<char> shower_split;
-  int n_items_split = 0;
+  // the arrival form of each shower (Endpoint, one-bin; kFormSplit until the
+  // votes are in); the work list holds the items of each form one after the other
+  // (kForms), up to item group_end[g], each group run by its own launch
+  std::vector<char> shower_form;
+  int group_end[3] = {0, 0, 0};
+  // the axis of each shower's windows, where they follow an inclined front
+  // (window_axis; axis_up_z 0 elsewhere)
+  std::vector<double> axis_up_z;
+  ShowerAxis* d_axes = nullptr;
   std::vector<float> cen;  // per shower: antenna centroid (x, y, z)
   float4* d_acc = nullptr;  // [replicas][total_ant][rows][n_bins] accumulator
   size_t acc_bytes = 0;
   int replicas = 1;
   cudaStream_t cap_stream = nullptr;  // graph capture (the caller's stream may be the legacy default stream)
   cudaStream_t aux_stream = nullptr;  // non-blocking: cancel word updates while a batch runs
+  // the groups of showers after the first (enqueue_kernel)
+  cudaStream_t side_stream[2] = {};
+  cudaEvent_t ev_fork = nullptr, ev_join[2] = {};
   bool tuned = false;
   TuneChoice choice{4, 64};
   // graph bound to (tracks, out) of its capture
@@ -285,21 +313,26 @@ int bfail(c8r_batch* b, int code, const std::string& m) {
   return code;
 }
 
-// the work list: the split-form showers first, then the direct-form ones (their
-// count of items in *n_split), each group largest shower first
-std::vector<WorkItem> make_items(const c8r_batch* b, int a_tile, int64_t tpi, int* n_split = nullptr) {
+// the arrival forms in the order of their groups in the work list
+constexpr int kForms[3] = {kFormSplit, kFormAxis, kFormDirect};
+int group_of(const c8r_batch* b, int s) {
+  const int form = b->shower_form.empty() ? kFormSplit : b->shower_form[s];
+  return form == kFormSplit ? 0 : (form == kFormAxis ? 1 : 2);
+}
+
+// the work list: the showers grouped by form (the end of each group in
+// b->group_end), each group largest shower first
+std::vector<WorkItem> make_items(c8r_batch* b, int a_tile, int64_t tpi) {
   std::vector<int> order(b->n_showers);
   for (int s = 0; s < b->n_showers; ++s) order[s] = s;
-  auto split_of = [&](int s) { return b->shower_split.empty() || b->shower_split[s]; };
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-    if (split_of(x) != split_of(y)) return split_of(x);
+    if (group_of(b, x) != group_of(b, y)) return group_of(b, x) < group_of(b, y);
     return b->n_tracks[x] * (int64_t)b->n_ant[x] > b->n_tracks[y] * (int64_t)b->n_ant[y];
   });
   std::vector<WorkItem> v;
-  if (n_split) *n_split = 0;
+  for (int& e : b->group_end) e = 0;
   for (int s : order) {
     const int64_t nt = b->tile_off[s + 1] - b->tile_off[s];
-    if (nt == 0) continue;
     for (int64_t r = 0; r < nt; r += tpi) {
       for (int a0 = 0; a0 < b->n_ant[s]; a0 += a_tile) {
         WorkItem w;
@@ -307,10 +340,11 @@ std::vector<WorkItem> make_items(const c8r_batch* b, int a_tile, int64_t tpi, in
         w.n_here = std::min(a_tile, b->n_ant[s] - a0);
         w.t_begin = b->tile_off[s] + r;
         w.t_end = b->tile_off[s] + std::min(nt, r + tpi);
+        w.shower = s;
         v.push_back(w);
       }
     }
-    if (n_split && split_of(s)) *n_split = (int)v.size();
+    for (int g = group_of(b, s); g < 3; ++g) b->group_end[g] = (int)v.size();
   }
   return v;
 }
@@ -344,27 +378,51 @@ int enqueue_ingest(c8r_batch* b, const TrackPtrs& tp, cudaStream_t st) {
   return C8R_OK;
 }
 
-// run the persistent kernel over the first n_items_limit items of the work list
-// (the split-form group, then the direct-form group, one launch each, each
-// with its own item counter: d_counter[0] and d_counter[3])
+// run the persistent kernel over the first n_items_limit items of the work list:
+// one launch per group of showers of one form, each with its own item counter
+// (d_counter[0], [3] and [4]).  The groups are independent, so those after the
+// first run on streams of their own between a fork and a join: their CTAs start
+// where the ones before run out of items, instead of after the last of them.
+// Showers of all zeniths to 65 degrees: a group for the axis form in the place of
+// the direct one takes the set-aside arrivals of the inclined showers from 2-7 %
+// to 0.4 %.  1e11 pairs/s, one group after the other without the axis form / with
+// it / side by side: 64 showers of 1e5 to 1e7 tracks 1.066 / 1.15 / 1.21; a tenth
+// of the tracks 1.098 / 1.12 / 1.215; up to 1e5 tracks, with the fetch, ms 2.97 /
+// 3.02 / 2.88
 int enqueue_kernel(c8r_batch* b, int n_items_limit, cudaStream_t st) {
   const int rows = acc_rows(b->formalism);
   const int n = std::min(b->n_items, n_items_limit);
-  const int ns = std::min(b->n_items_split, n);
-  const int first[2] = {0, ns}, count[2] = {ns, n - ns};
-  for (int g = 0; g < 2; ++g) {
-    if (count[g] <= 0) continue;
-    int* counter = b->d_counter + (g == 0 ? 0 : 3);
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-    if (e != cudaSuccess) return bfail(b, C8R_ECUDA, std::string("batch counter: ") + cudaGetErrorString(e));
-    BatchArgs a{b->d_tiles, b->d_items + first[g], count[g], b->d_ants, b->d_acc, counter,
+  cudaError_t e = cudaMemsetAsync(b->d_counter, 0, sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counter + 3, 0, 2 * sizeof(int), st);
+  if (e == cudaSuccess) e = cudaEventRecord(b->ev_fork, st);
+  int first = 0, used = 0;
+  bool joins[2] = {false, false};
+  for (int g = 0; g < 3 && e == cudaSuccess; ++g) {
+    const int end = std::min(b->group_end[g], n);
+    if (end <= first) continue;
+    BatchArgs a{b->d_tiles, b->d_items + first, end - first, b->d_ants, b->d_acc,
+                b->d_counter + (g == 0 ? 0 : 2 + g),
                 b->d_cancel, b->d_err, b->choice.a_tile, b->M, b->replicas,
-                (int64_t)b->total_ant * b->M.n_bins * rows};
+                (int64_t)b->total_ant * b->M.n_bins * rows, b->d_axes};
     a.M.wait_limit = current_wait_limit();
-    a.M.split = g == 0 ? 1 : 0;
-    e = launch_batch(a, b->formalism, b->sm_count, st);
-    if (e != cudaSuccess) return bfail(b, C8R_ECUDA, std::string("batch launch: ") + cudaGetErrorString(e));
+    first = end;
+    const int side = used++ - 1;  // the first group runs on st itself
+    if (side < 0) {
+      e = launch_batch(a, b->formalism, kForms[g], b->sm_count, st);
+      continue;
+    }
+    e = cudaStreamWaitEvent(b->side_stream[side], b->ev_fork, 0);
+    if (e != cudaSuccess) break;
+    joins[side] = true;
+    e = launch_batch(a, b->formalism, kForms[g], b->sm_count, b->side_stream[side]);
   }
+  for (int i = 0; i < 2; ++i) {
+    if (!joins[i]) continue;
+    const cudaError_t r = cudaEventRecord(b->ev_join[i], b->side_stream[i]);
+    const cudaError_t w = cudaStreamWaitEvent(st, b->ev_join[i], 0);
+    if (e == cudaSuccess) e = r != cudaSuccess ? r : w;
+  }
+  if (e != cudaSuccess) return bfail(b, C8R_ECUDA, std::string("batch launch: ") + cudaGetErrorString(e));
   return C8R_OK;
 }
 
@@ -383,13 +441,15 @@ int enqueue(c8r_batch* b, const TrackPtrs& tp, float* out, int n_items_limit, cu
 }
 
 // the arrival form of each shower's one-bin Endpoint evaluation
-// (MedParams::split) from its votes (k_batch_votes on the ingested tiles): the
-// split form when at least half of the tracks counted see the shower's antenna
-// centroid from above within 45 degrees.  Once per batch, before the first
+// from its votes (k_batch_votes on the ingested tiles): the split form when at
+// least half of the tracks counted see the shower's antenna centroid from above
+// within 45 degrees, else the direct one, and the axis form in the place of either
+// when the shower's windows follow an inclined front that the votes do not speak
+// against (as form_apply has it for one shower).  Once per batch, before the first
 // run: one ingest, the vote kernel (its counts written into the accumulator,
 // which every run zeroes first), a synchronous read.
 int choose_forms(c8r_batch* b, const TrackPtrs& tp, cudaStream_t st) {
-  b->shower_split.assign(b->n_showers, 1);
+  b->shower_form.assign(b->n_showers, (char)kFormSplit);
   BatchMap map{b->d_tile_off, b->d_track_off, b->d_n_tracks, b->n_showers};
   cudaError_t e =
       launch_ingest_map(C8R_MIXED, tp, map, b->total_tiles * kTileT, b->d_tiles, b->M, nullptr, st);
@@ -409,8 +469,12 @@ int choose_forms(c8r_batch* b, const TrackPtrs& tp, cudaStream_t st) {
     e = cudaMemcpyAsync(h.data(), counts, sizeof(unsigned) * h.size(), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return bfail(b, C8R_ECUDA, std::string("batch form votes: ") + cudaGetErrorString(e));
-  for (int s = 0; s < b->n_showers; ++s)
-    if (h[2 * s] > 0) b->shower_split[s] = 2 * (size_t)h[2 * s + 1] >= h[2 * s] ? 1 : 0;
+  for (int s = 0; s < b->n_showers; ++s) {
+    if (h[2 * s] == 0) continue;
+    const bool split = 2 * (size_t)h[2 * s + 1] >= h[2 * s];
+    const bool axis = b->axis_up_z[s] > 0.0 && split == (b->axis_up_z[s] > 0.7071);
+    b->shower_form[s] = (char)(axis ? kFormAxis : (split ? kFormSplit : kFormDirect));
+  }
   return C8R_OK;
 }
 
@@ -420,14 +484,14 @@ int autotune(c8r_batch* b, const TrackPtrs& tp, cudaStream_t st) {
     if (r != C8R_OK) return r;
   }
   char keybuf[160];
-  std::snprintf(keybuf, sizeof keybuf, "batch3:N%d:f%d:m%d:sm%d:P%lld", b->M.n_bins, b->formalism, b->M.kind,
+  std::snprintf(keybuf, sizeof keybuf, "batch4:N%d:f%d:m%d:sm%d:P%lld", b->M.n_bins, b->formalism, b->M.kind,
                 b->sm_count, (long long)(b->total_pairs >> 26));
   const std::string key = keybuf;
   TuneChoice best{};
   if (tune_lookup(key, best) && best.a_tile <= kMaxATile) {
     b->choice = best;
     b->tuned = true;
-    return upload_items(b, make_items(b, best.a_tile, best.tiles_per_item, &b->n_items_split));
+    return upload_items(b, make_items(b, best.a_tile, best.tiles_per_item));
   }
   std::vector<TuneChoice> cands;
   for (int at : {8, 16, 32})
@@ -443,7 +507,7 @@ int autotune(c8r_batch* b, const TrackPtrs& tp, cudaStream_t st) {
   if (r != C8R_OK) return r;
   for (const TuneChoice& c : cands) {
     b->choice = c;
-    std::vector<WorkItem> v = make_items(b, c.a_tile, c.tiles_per_item, &b->n_items_split);
+    std::vector<WorkItem> v = make_items(b, c.a_tile, c.tiles_per_item);
     const int min_items = 4 * batch_resident(b->formalism, b->M.kind, c.a_tile, b->sm_count);
     int lim = 0;
     double pairs = 0;
@@ -475,7 +539,7 @@ int autotune(c8r_batch* b, const TrackPtrs& tp, cudaStream_t st) {
   int status = kErrNone;
   if (cudaMemcpy(&status, b->d_err, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess && status == kErrNone)
     tune_store(key, best);
-  return upload_items(b, make_items(b, best.a_tile, best.tiles_per_item, &b->n_items_split));
+  return upload_items(b, make_items(b, best.a_tile, best.tiles_per_item));
 }
 
 }  // namespace
@@ -521,13 +585,28 @@ int c8r_batch_create(c8r_batch** out, int device, const c8r_batch_desc* d, int k
   }
   b->total_tiles = b->tile_off[d->n_showers];
   set_flat_array(b->M, d->pos_xyz, b->total_ant);
-  b->M.split = 1;
+  b->axis_up_z.assign(b->n_showers, 0.0);
+  std::vector<ShowerAxis> axes(b->n_showers);
   b->cen.assign(3 * (size_t)b->n_showers, 0.0f);
   for (int s = 0; s < b->n_showers; ++s) {
     double c[3] = {0.0, 0.0, 0.0};
     for (int a = 0; a < b->n_ant[s]; ++a)
       for (int k = 0; k < 3; ++k) c[k] += d->pos_xyz[3 * (size_t)(b->ant_off[s] + a) + k];
     for (int k = 0; k < 3; ++k) b->cen[3 * (size_t)s + k] = (float)(c[k] / b->n_ant[s]);
+  }
+  for (int s = 0; s < b->n_showers; ++s) {
+    const size_t a0 = (size_t)b->ant_off[s];
+    double up[3];
+    axes[s] = ShowerAxis{};
+    if (!window_axis(d->pos_xyz + 3 * a0, d->t_start_ns + a0, b->n_ant[s], up)) continue;
+    MedParams m = b->M;
+    set_axis(m, up);
+    for (int k = 0; k < 3; ++k) {
+      axes[s].ax[k] = m.ax[k];
+      axes[s].kax_h[k] = m.kax_h[k];
+      axes[s].kax_l[k] = m.kax_l[k];
+    }
+    b->axis_up_z[s] = up[2];
   }
   std::vector<AntRec> recs(b->total_ant);
   for (int a = 0; a < b->total_ant; ++a) {
@@ -539,6 +618,8 @@ int c8r_batch_create(c8r_batch** out, int device, const c8r_batch_desc* d, int k
   cudaError_t e = dev_malloc(&b->d_ants, sizeof(AntRec) * recs.size());
   if (e == cudaSuccess) e = cudaMemcpy(b->d_ants, recs.data(), sizeof(AntRec) * recs.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && b->total_tiles > 0) e = dev_malloc(&b->d_tiles, (size_t)b->total_tiles * kTileBytesMixed);
+  if (e == cudaSuccess) e = dev_malloc(&b->d_axes, sizeof(ShowerAxis) * axes.size());
+  if (e == cudaSuccess) e = cudaMemcpy(b->d_axes, axes.data(), sizeof(ShowerAxis) * axes.size(), cudaMemcpyHostToDevice);
   const size_t sb = sizeof(int64_t) * (b->n_showers + 1);
   if (e == cudaSuccess) e = dev_malloc(&b->d_tile_off, sb);
   if (e == cudaSuccess) e = dev_malloc(&b->d_track_off, sb);
@@ -559,7 +640,12 @@ int c8r_batch_create(c8r_batch** out, int device, const c8r_batch_desc* d, int k
   b->d_cancel = b->d_counter + 1;
   b->d_err = b->d_counter + 2;
   if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&b->aux_stream, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaStreamCreateWithFlags(&b->aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&b->side_stream[0], cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&b->side_stream[1], cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&b->ev_join[0], cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&b->ev_join[1], cudaEventDisableTiming) != cudaSuccess) {
     b->err = "stream creation failed";
     *out = b;
     return C8R_ECUDA;
@@ -576,7 +662,7 @@ int c8r_batch_create(c8r_batch** out, int device, const c8r_batch_desc* d, int k
   }
   b->choice = {8, tpi_for(b, 8, 8)};
   *out = b;
-  return upload_items(b, make_items(b, b->choice.a_tile, b->choice.tiles_per_item, &b->n_items_split));
+  return upload_items(b, make_items(b, b->choice.a_tile, b->choice.tiles_per_item));
 }
 
 void c8r_batch_destroy(c8r_batch* b) {
@@ -591,9 +677,14 @@ void c8r_batch_destroy(c8r_batch* b) {
   cudaFree(b->d_n_tracks);
   cudaFree(b->d_items);
   cudaFree(b->d_counter);
+  cudaFree(b->d_axes);
   cudaFree(b->d_acc);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
   if (b->aux_stream) cudaStreamDestroy(b->aux_stream);
+  for (cudaStream_t s : b->side_stream)
+    if (s) cudaStreamDestroy(s);
+  for (cudaEvent_t e : {b->ev_fork, b->ev_join[0], b->ev_join[1]})
+    if (e) cudaEventDestroy(e);
   delete b;
 }
 

@@ -169,5 +169,9 @@ void set_form_centroid(MedParams& M, const double* pos_xyz, int n_ant);
 // MedParams::flat and its altitude terms: set when the medium is one of the
 // exponential atmospheres and every antenna has the same z (exactly)
 void set_flat_array(MedParams& M, const double* pos_xyz, int n_ant);
+// the direction of the inclined front that the trace windows follow, if they
+// do, and the axis form's constants for it (MedParams::ax, kax_*)
+bool window_axis(const double* pos_xyz, const double* t_start_ns, int n_ant, double up[3]);
+void set_axis(MedParams& M, const double up[3]);
 
 }  // namespace c8r

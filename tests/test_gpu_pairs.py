@@ -207,3 +207,41 @@ def test_axis_form_gives_the_bins_of_the_others(zenith, hills, offset, medium):
     assert np.abs(out[1][0]).max() > 0
     for a, d in zip(*out):
         assert rel_l2(a, d) <= 2e-6
+
+
+@pytest.mark.parametrize("medium", [synth.AIR_EXPONENTIAL, UNIFORM])
+@pytest.mark.parametrize("hills", [0.0, 150.0])
+def test_batch_groups_showers_by_arrival_form(hills, medium):
+    """Showers from the vertical to 75 degrees in one batch, each with the axis
+    of its own windows, an empty one, and one whose windows open together, so
+    that no front orders them: every shower's traces as its own process in the
+    direct form gives them, to the order of the additions."""
+    from paper_2309_03717_gb300 import c8r
+    showers, tracks = [], []
+    for k, (zenith, n) in enumerate([(75.0, 700), (0.0, 129), (50.0, 1), (60.0, 0), (35.0, 3000), (70.0, 1500)]):
+        ant = synth.antennas_star(8, n_radii=5)[: 5 + 7 * k].copy()
+        ant[:, 2] = np.linspace(0.0, hills, len(ant))
+        t_start = synth.trace_start_ns(ant, zenith)
+        if k == 5:
+            t_start = np.full(len(ant), t_start.min())
+        showers.append({"n_tracks": n, "ant_xyz": ant, "t_start_ns": t_start})
+        tracks.append({f: x[:n] for f, x in synth.make_tracks(max(n, 1), 50 + k, zenith).items()})
+    b = c8r.Batch(showers, medium, 8192, 0.2, "endpoint")
+    out = b.new_output()
+    b.run(to_device({f: np.concatenate([t[f] for t in tracks]) for f in synth.FIELDS}), out)
+    b.sync()
+    got, off = out.cpu().numpy(), 0
+    b.close()
+    for s, t in zip(showers, tracks):
+        k = len(s["ant_xyz"])
+        if s["n_tracks"]:
+            p = c8r.RadioProcess(medium, s["ant_xyz"], s["t_start_ns"], 8192, 0.2, "endpoint", "mixed")
+            p.set_arrival_form("direct")
+            p.push(to_device(t))
+            ref = p.traces().cpu().numpy()
+            p.close()
+            assert np.abs(ref).max() > 0
+            assert rel_l2(got[off:off + k], ref) <= 2e-6
+        else:
+            assert not got[off:off + k].any()
+        off += k
