@@ -664,6 +664,14 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   c->trace_bytes = (size_t)n_ant * 3 * n_bins * (precision == C8R_FP64 ? 8 : 4);
   c->acc_bytes = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(formalism);
   c->shape.replicas = acc_replicas(precision, formalism, n_ant, n_bins, c->shape.a_tile, c->sm_count);
+  // the copies are there for speed alone: on a device that is nearly full they
+  // do not keep the first one from being allocated
+  size_t mem_free = 0, mem_total = 0;
+  if (c->shape.replicas > 1 && cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) {
+    cudaGetLastError();
+    mem_free = 0;
+  }
+  while (c->shape.replicas > 1 && c->acc_bytes * c->shape.replicas > mem_free / 4) c->shape.replicas /= 2;
   c->acc_bytes *= c->shape.replicas;
   c->copies_used = 1;
   c->copies_all = false;
