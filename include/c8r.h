@@ -111,7 +111,8 @@ typedef struct {
   int64_t tracks_kept;   /* of those, tracks the track filter let through           */
   int64_t pairs;         /* kept tracks x antennas evaluated                         */
   int64_t arrival_form;  /* C8R_FORM_SPLIT or C8R_FORM_DIRECT: the FP32 arrival form the
-                            next mixed one-bin Endpoint launch takes (c8r_set_arrival_form) */
+                            next mixed one-bin Endpoint launch takes, or would take but
+                            for windows along an inclined front (c8r_set_arrival_form) */
 } c8r_stats_t;
 
 /* Writable DEVICE arrays for c8r_generate_tracks, one per track field. */
@@ -179,11 +180,12 @@ int c8r_set_medium_spherical(c8r_ctx* ctx, double N0, double scale_height_m, dou
  * [t_start_ns[a] + k dt_ns, t_start_ns[a] + (k + 1) dt_ns).  formalism selects
  * Endpoint or ZHS; precision selects C8R_FP64 or C8R_MIXED.  Allocates (and
  * zeroes) the context's trace accumulator, one (x, y, z) element per antenna and
- * bin, FP64 (C8R_FP64) or FP32 (C8R_MIXED), 32 or 16 bytes per element.  Mixed
- * ZHS keeps a second row per antenna (box edges), and the mixed path keeps 1 to
- * 16 copies of the whole accumulator, more for fewer antennas (up to 192 MB
- * in all), which the fetch sums; a push uses as many of them as its tracks pay for.  Replaces
- * any previous antenna set and discards its traces (a call with the same
+ * bin, FP64 (C8R_FP64) or FP32 (C8R_MIXED), 32 or 16 bytes per element.  ZHS
+ * keeps a second row per antenna (box edges), and 1 to 16 copies of the whole
+ * accumulator are kept, more for fewer antennas (up to 192 MB and a quarter of the
+ * device's free memory in all), which the fetch sums; a push uses as many of them
+ * as its tracks pay for.  Replaces any previous antenna set and discards its
+ * traces (a call with the same
  * n_ant, n_bins, dt_ns, formalism and precision keeps the device memory and
  * only replaces the table, so moving an array between steps is cheap).  EINVAL on n_ant < 1,
  * n_bins < 1, dt_ns <= 0 or non-finite values; ETOOBIG if n_bins > 2^24; ENOMEM. */

@@ -268,6 +268,7 @@ struct c8r_ctx {
   // copy counts as used for good
   int copies_used = 1;
   bool copies_all = false;
+  int floor_copies = 1;  // that every push uses (floor_replicas)
   void* d_stage = nullptr;   // [n_ant][3][n_bins] staging for copies to host
   void* d_gbm = nullptr;     // backward: dL/dtraces, bin-major [n_ant][n_bins] accumulator elements
   PrefixFF* d_gpre = nullptr;  // backward (mixed ZHS): running sums of d_gbm over the bins, [n_ant][n_bins + 1]
@@ -359,7 +360,7 @@ void form_poll(c8r_ctx* c) {
 }
 
 void form_fetch(c8r_ctx* c, cudaStream_t st) {
-  // only the one-bin Endpoint kernels of the plain media come in two forms
+  // only the one-bin Endpoint kernels of the plain media come in arrival forms
   if (c->form_mode != C8R_FORM_AUTO || c->form_pending || !c->h_form || !c->ev_form || c->precision != C8R_MIXED ||
       c->formalism != C8R_ENDPOINT || c->deposit != C8R_DEPOSIT_BIN ||
       (c->med_kind != C8R_UNIFORM && c->med_kind != C8R_EXPONENTIAL))
@@ -664,7 +665,8 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   c->trace_bytes = (size_t)n_ant * 3 * n_bins * (precision == C8R_FP64 ? 8 : 4);
   c->acc_bytes = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(formalism);
   c->shape.replicas = acc_replicas(precision, formalism, n_ant, n_bins, c->shape.a_tile, c->sm_count);
-  // the copies are there for speed alone: on a device that is nearly full they
+  c->floor_copies = floor_replicas(precision, formalism, n_ant, n_bins, c->shape.a_tile, c->sm_count);
+  // the copies are not needed to hold the traces: on a device that is nearly full they
   // do not keep the first one from being allocated
   size_t mem_free = 0, mem_total = 0;
   if (c->shape.replicas > 1 && cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) {
@@ -733,7 +735,9 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
   if (c->user_a_tile == 0)
     shape.a_tile = push_a_tile(shape.a_tile, (chunk + kTileT - 1) / kTileT, c->n_ant, c->precision, c->formalism,
                                c->sm_count);
-  shape.replicas = push_replicas(shape.replicas, n, c->n_bins, acc_rows(c->formalism));
+  const int floor_copies = c->floor_copies < shape.replicas ? c->floor_copies : shape.replicas;
+  shape.replicas = push_replicas(c->precision, shape.replicas, n, c->n_bins, acc_rows(c->formalism));
+  if (shape.replicas < floor_copies) shape.replicas = floor_copies;
   if (capturing(st)) c->copies_all = true;
   if (shape.replicas > c->copies_used) c->copies_used = shape.replicas;
   for (int64_t off = 0; off < n; off += chunk) {

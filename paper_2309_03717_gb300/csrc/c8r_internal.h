@@ -40,6 +40,13 @@ inline int acc_rows(int formalism) { return formalism == C8R_ZHS ? 2 : 1; }
 // 1303 / 1310 / 1310; ZHS, 8 antennas 576 / 257 / 213; linear deposit, 64 antennas
 // 2487 / 1612 / 1242.  With 3e4 tracks, Endpoint, 64 antennas 76 / 61 / 64.
 //
+// The FP64 path adds at a thirtieth of the mixed path's rate, but with three scalar
+// reductions per deposit: hot bins bind it where the antennas are few (a trace's
+// copies times its antennas: 64 for ZHS, 32 for Endpoint, where a pair has fewer
+// deposits).  Us per push and fetch, 3.5e5 tracks, 1 copy / as chosen: ZHS 1 antenna 525
+// / 204, 2 575 / 224, 8 872 / 488, 16 1220 / 871; Endpoint 2 473 / 230, 8 721 / 605, 16
+// 1192 / 1138; linear deposit, 1e5 x 2 662 / 235.
+//
 // the batched launch: its many showers' antenna tiles spread the CTAs, so 2
 // copies for ZHS and 1 for Endpoint
 inline int acc_replicas(int formalism) { return acc_rows(formalism) == 2 ? 2 : 1; }
@@ -54,11 +61,11 @@ constexpr size_t kAccBudget = (size_t)192 << 20;
 // 182 (160 antennas) up to 8, 57 (512 antennas) none (linear deposit, 1e5 tracks:
 // 906 us with 1, 920 with 2)
 inline int acc_replicas(int precision, int formalism, int n_ant, int n_bins, int a_tile, int sm_count) {
-  if (precision != C8R_MIXED) return 1;
   const int64_t ant_tiles = (n_ant + a_tile - 1) / a_tile;
   const int64_t per_tile = (int64_t)sm_count * 6 / (ant_tiles > 0 ? ant_tiles : 1);
-  const int64_t want = per_tile < 64 ? 1 : per_tile / 22;
-  const size_t one = (size_t)n_ant * n_bins * 16 * acc_rows(formalism);
+  int64_t want = per_tile < 64 ? 1 : per_tile / 22;
+  if (precision == C8R_FP64) want = (formalism == C8R_ZHS ? 64 : 32) / (n_ant > 0 ? n_ant : 1);
+  const size_t one = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(formalism);
   const int64_t fit = (int64_t)(kAccBudget / (one > 0 ? one : 1));
   int r = 1;
   while (r < 16 && r * 2 <= want && r * 2 <= fit) r *= 2;
@@ -67,9 +74,28 @@ inline int acc_replicas(int precision, int formalism, int n_ant, int n_bins, int
 // the copies that a push of n tracks uses, of the `most` allocated: two tracks per
 // bin, row and copy at least, where the cost of a copy (about 32 bytes per bin,
 // row and antenna) falls below what it takes off the reductions of the tracks
-inline int push_replicas(int most, int64_t n, int n_bins, int rows) {
+// (FP64, whose copies are of few antennas: half a track)
+inline int push_replicas(int precision, int most, int64_t n, int n_bins, int rows) {
+  const int64_t per_copy = (int64_t)(precision == C8R_FP64 ? 1 : 4) * n_bins * rows;
   int r = 1;
-  while (r * 2 <= most && (int64_t)r * 4 * n_bins * rows <= n) r *= 2;
+  while (r * 2 <= most && r * per_copy <= n) r *= 2;
+  return r;
+}
+// the copies that every mixed push uses, however few its tracks: the FP32 rounding
+// of a bin's sum falls with the copies the sum is split over, most of all in the
+// running sum of the ZHS box edges (error against 64 bits, ZHS, 4.4e4 tracks x 31
+// antennas, 8192 bins: 1.2e-6 with one copy, 6.5e-7 with four).  One per 100
+// CTAs of an antenna tile (Endpoint 200) or part of it, at most 8 and within 48 MB
+inline int floor_replicas(int precision, int formalism, int n_ant, int n_bins, int a_tile, int sm_count) {
+  if (precision != C8R_MIXED) return 1;
+  const int64_t ant_tiles = (n_ant + a_tile - 1) / a_tile;
+  const int64_t per_tile = (int64_t)sm_count * (acc_rows(formalism) == 2 ? 7 : 6) / (ant_tiles > 0 ? ant_tiles : 1);
+  const int64_t per_copy = acc_rows(formalism) == 2 ? 100 : 200;
+  const int64_t want = (per_tile + per_copy - 1) / per_copy;
+  const size_t one = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(formalism);
+  const int64_t fit = (int64_t)(((size_t)48 << 20) / (one > 0 ? one : 1));
+  int r = 1;
+  while (r < 8 && r * 2 <= want && r * 2 <= fit) r *= 2;
   return r;
 }
 // antennas per CTA of a forward launch over n_tiles track tiles, `a_tile` at

@@ -1,6 +1,7 @@
 // kernels_f64.cu -- instantiation of the FP64 forward, arrival-listing and
 // adjoint kernels.  Compiled with --fmad=false: every FP64 operation rounds as
-// written, as in a plain FP64 evaluation of the formulas.
+// written (OpsF64: as in a plain FP64 evaluation of the formulas; OpsF64Plain
+// states its fused operations).
 #include "pair_f64.cuh"
 
 namespace c8r {

@@ -282,13 +282,21 @@ __global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(typename AccOf<T>
   }
 }
 
-__global__ void k_acc_to_traces_f64(Acc4D* acc, int64_t n_ant_bins, int n_bins, double* out, bool clear) {
+__global__ void k_acc_to_traces_f64(Acc4D* acc, int64_t n_ant_bins, int n_bins, double* out, bool clear,
+                                    int replicas) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_ant_bins) return;
   const int64_t a = i / n_bins;
   const int k = (int)(i - a * n_bins);
-  const Acc4D v = acc[i];
-  if (clear) acc[i] = Acc4D{0.0, 0.0, 0.0, 0.0};
+  Acc4D v = acc[i];
+  for (int r = 1; r < replicas; ++r) {
+    const Acc4D w = acc[i + r * n_ant_bins];
+    v.x += w.x;
+    v.y += w.y;
+    v.z += w.z;
+  }
+  if (clear)
+    for (int r = 0; r < replicas; ++r) acc[i + r * n_ant_bins] = Acc4D{0.0, 0.0, 0.0, 0.0};
   double* o = out + a * 3 * n_bins + k;
   o[0] = v.x;
   o[n_bins] = v.y;
@@ -322,7 +330,7 @@ cudaError_t launch_acc_to_traces(int precision, void* acc, int n_ant, int n_bins
   }
   if (precision == C8R_FP64) {
     k_acc_to_traces_f64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(static_cast<Acc4D*>(acc), n, n_bins,
-                                                                    static_cast<double*>(out), clear);
+                                                                    static_cast<double*>(out), clear, replicas);
   } else {
     constexpr int per = kFetchT * kFetchE;
     k_acc_to_traces_f32<<<(unsigned)((n + per - 1) / per), kFetchT, 0, st>>>(

@@ -664,8 +664,10 @@ struct OpsF64 {
 // from the low word of a rounded-down sum.  About 90 -> 42 FP64 operations per
 // emission point; and a ZHS interval's whole bins go in as a box (two edges)
 // rather than bin by bin.  Measured, ms: 1e5 tracks x 16 antennas Endpoint in the
-// uniform medium 0.92 -> 0.49, 1e5 x 160 ZHS in the exponential one 6.2 -> 2.3;
-// errors against a 64-bit evaluation in plain torch unchanged (1e-12, 8e-12).
+// uniform medium 0.92 -> 0.49 (0.32 with push_a_tile's tiles), 1e5 x 160 ZHS in the
+// exponential one 6.2 -> 2.3.  Error of an Endpoint deposit against an 80-bit
+// evaluation (emulated on 2e5 tracks, three antennas, 0 and 50 degrees): 3.9e-14 to
+// 5.3e-14 -> 3.0e-14 to 4.4e-14 relative, since a fused operation rounds once.
 // ---------------------------------------------------------------------------
 // 1/sqrt(x) and 1/x for normal x: the hardware's approximation (20 bits or more)
 // and one third-order step (Householder's iteration: the residual e = 1 - x y^2
@@ -917,6 +919,8 @@ cudaError_t forward_f64(int formalism, const void* tiles, int64_t n_tiles, const
   FwdArgs a{tiles, n_tiles, ants, n_ant, shape.a_tile, acc, err, FwdGrid{}, M};
   auto go = [&](auto ops) {
     using O = decltype(ops);
+    a.replicas = shape.replicas > 1 ? shape.replicas : 1;
+    a.replica_stride = (int64_t)n_ant * M.n_bins * O::kAccRows;
     const int64_t ctas =
         forward_grid(a, shape, sm_count * forward_blocks_per_sm<O>(shape.a_tile), sizeof(Acc4D) * O::kAccRows);
     return launch_forward_ops<O>(a, ctas, st);

@@ -76,3 +76,34 @@ def test_push_replayed_from_a_graph(formalism):
     p.reset()
     assert not p.traces().any()
     p.close()
+
+
+@pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
+@pytest.mark.parametrize("n_tracks,n_ant,n_bins", [(1, 1, 1000), (16500, 1, 1000), (16500, 3, 1021), (9000, 32, 1025),
+                                                   (9000, 33, 1025)])
+def test_copies_of_the_fp64_accumulator(formalism, n_tracks, n_ant, n_bins):
+    """Few antennas on the FP64 path: traces, both kinds of reset and pushes
+    replayed from a graph, against the oracle at the FP64 bar (1e-9)."""
+    from paper_2309_03717_gb300.c8r import RadioProcess
+    w = synth.workload(1, n_tracks=n_tracks, n_ant=n_ant)
+    tr = synth.workload_tracks(w)
+    if formalism == "endpoint":
+        tr = drop_tracks(tr, endpoint_unambiguous(tr, w["ant_xyz"], w["t_start_ns"], n_bins, w["dt_ns"], w["medium"]))
+    ref, _ = oracle_traces(tr, w["ant_xyz"], w["t_start_ns"], n_bins, w["dt_ns"], w["medium"], formalism)
+    p = RadioProcess(w["medium"], w["ant_xyz"], w["t_start_ns"], n_bins, w["dt_ns"], formalism, "fp64")
+    t = to_device({f: x.astype(np.float64) for f, x in tr.items()})
+    for _ in range(2):
+        p.push(t)
+        assert rel_l2(p.traces(reset=True).cpu().numpy(), ref) < 1e-9
+    p.push(t)
+    p.reset()
+    assert not p.traces().any()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        p.push(t)
+    p.reset()
+    g.replay()
+    g.replay()
+    assert rel_l2(p.traces().cpu().numpy(), 2.0 * ref) < 1e-9
+    p.close()
