@@ -1362,6 +1362,10 @@ struct OpsMixed {
       FieldT<float2> f;
       int ka, kb;
       if (endpoints_main(t, *p, M, g, f, ka, kb)) return kDeferPair;
+      // an endpoint on the antenna, or too far away for FP32: R, and with it the
+      // half's field and gradients, are NaN, which a zero dL/dtrace would not keep
+      // out of the sums.  The other endpoint is left to the pass after this one
+      if (!(g.R0.x + g.R0.y > 0.0f)) return (ka != kFastOut ? kDeferEnd0 : 0) | (kb != kFastOut ? kDeferEnd1 : 0);
       const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       const float4 g0 = ka >= 0 ? G[ka] : zero, g1 = kb >= 0 ? G[kb] : zero;
       if (ka >= 0 || kb >= 0) adj_ends(g, f, t, g0, g1, M, m, ga, dn);
