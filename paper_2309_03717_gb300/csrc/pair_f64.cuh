@@ -800,6 +800,12 @@ struct OpsF64Plain {
     double r = p.r;
     if (M.kind != C8R_UNIFORM && !M.flat) r = refr(M, A.Ea, p.E, dz);
     e.u = __dmul_rn(__fma_rn(__fma_rn(r, R, R), M.inv_c_ns, __dsub_rn(p.t, A.t_ref)), M.inv_dt);
+    // |d|^2 overflows: the roots above are NaN.  The signal arrives after every
+    // window (tested on the high word, off the FP64 pipe)
+    if (__double2hiint(S) == 0x7ff00000) {
+      e.D = 1.0;
+      e.u = S;
+    }
     return true;
   }
 

@@ -1,0 +1,92 @@
+"""Arrivals within rounding of a bin edge: the forward pass, the arrival listing
+and the adjoint form them by the same arithmetic, so they put every deposit in the
+same bin, wherever a rounding leaves it.  One track and many antennas, each with a
+window that opens a whole number of bins before the track's arrival there (the
+oracle's, in FP64), so that about half of the arrivals fall on either side."""
+import numpy as np
+import pytest
+
+from _util import built_lib, oracle_arrivals, to_device
+from paper_2309_03717_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+UNIFORM = {"kind": "uniform", "n": 1.000292}
+SPHERE = {"kind": "exponential_spherical", "N0": 3.25e-4, "H": 8000.0, "R_E": 6.371e6}
+RAY = {"kind": "exponential_ray", "N0": 3.25e-4, "H": 8000.0}
+K = 40  # the bin whose lower edge the arrivals lie on
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    built_lib()
+
+
+def on_the_edge(formalism, medium, hills, dt, n_ant, dtype):
+    """A 4 m track 3 km up and n_ant antennas, the first arrival of each on edge K."""
+    rng = np.random.default_rng(11)
+    b = np.array([0.02, 0.01, -0.999])
+    x0 = np.array([30.0, -20.0, 3000.0])
+    t0 = 7.0 / 0.299792458
+    t1 = t0 + 4.0 / (np.linalg.norm(b) * 0.299792458)
+    x1 = x0 + 4.0 * b / np.linalg.norm(b)
+    vals = [*x0, *x1, t0, t1, *b, -1.0]
+    tracks = {f: np.array([v], dtype) for f, v in zip(synth.FIELDS, vals)}
+    r, a = rng.uniform(700.0, 1500.0, n_ant), rng.uniform(0.0, 2.0 * np.pi, n_ant)
+    ant = np.stack([r * np.cos(a), r * np.sin(a), rng.uniform(0.0, 1.0, n_ant) * hills], 1)
+    exact = {f: x.astype(np.float64) for f, x in tracks.items()}
+    br, u = oracle_arrivals(exact, ant, np.zeros(n_ant), 1, dt, medium, formalism)
+    u = u.reshape(n_ant, 2)
+    assert (br.ravel() == (0 if formalism == "endpoint" else 3)).all()
+    assert (np.abs(u[:, 1] - u[:, 0]) > 3.0).all()
+    return tracks, ant, (u.min(1) - K) * dt, int(np.argmin(u[0]))
+
+
+def forward_listing_adjoint(formalism, precision, medium, hills, dt, adjoint=True):
+    from paper_2309_03717_gb300 import c8r
+    n_ant, N = 1500, 512
+    dtype = np.float64 if precision == "fp64" else np.float32
+    tracks, ant, t_start, first = on_the_edge(formalism, medium, hills, dt, n_ant, dtype)
+    dev = to_device(tracks)
+    p = c8r.RadioProcess(medium, ant, t_start, N, dt, formalism, precision)
+    p.push(dev)
+    tr = p.traces().cpu().numpy()
+    _, bins, frac = p.arrivals(dev)
+    bins, frac = bins.cpu().numpy()[0, :, first], frac.cpu().numpy()[0, :, first]
+    ag = None
+    if adjoint:
+        # dL/dtrace in bin K - 1 only: an antenna has a gradient when its deposit is there
+        G = torch.zeros((n_ant, 3, N), dtype=p.trace_dtype, device="cuda")
+        G[:, :, K - 1] = torch.tensor([1.0, -2.0, 3.0], dtype=p.trace_dtype, device="cuda") * 1e9
+        gdt = torch.float64 if precision == "fp64" else torch.float32
+        tg = {f: torch.zeros(1, dtype=gdt, device="cuda") for f in c8r.GRAD_FIELDS}
+        ag = torch.zeros((n_ant, 3), dtype=torch.float64, device="cuda")
+        dn = torch.zeros(1, dtype=torch.float64, device="cuda")
+        c8r.c8r_backward(p.ctx, dev, G, tg, ag, dn)
+        ag = ag.cpu().numpy()
+    p.close()
+    below = np.abs(tr[:, :, K - 1]).max(1) > 0
+    assert 0.02 < below.mean() < 0.98  # both sides of the edge are reached
+    return tr, below, bins, frac, ag
+
+
+@pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
+@pytest.mark.parametrize("medium", [synth.AIR_EXPONENTIAL, UNIFORM])
+@pytest.mark.parametrize("hills", [0.0, 150.0])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_forward_listing_and_adjoint_agree(precision, hills, medium, formalism):
+    _, below, bins, _, ag = forward_listing_adjoint(formalism, precision, medium, hills, 0.05)
+    assert np.array_equal(bins == K - 1, below)
+    assert np.array_equal(np.abs(ag).max(1) > 0, below)
+
+
+@pytest.mark.parametrize("medium", [SPHERE, RAY])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
+@pytest.mark.parametrize("hills", [0.0, 150.0])
+def test_forward_and_listing_agree_in_the_costlier_media(hills, formalism, precision, medium):
+    _, below, bins, _, _ = forward_listing_adjoint(formalism, precision, medium, hills, 0.05, adjoint=False)
+    assert np.array_equal(bins == K - 1, below)

@@ -1,6 +1,7 @@
 """Pairs whose geometry has no finite form: an antenna exactly on a track's endpoint
-(R = 0).  Such an endpoint deposits nothing; everything else stays finite and as it
-is without it."""
+(R = 0), and an emission point so far away that the square of its distance
+overflows.  Such an endpoint deposits nothing; everything else stays finite and as
+it is without it."""
 import numpy as np
 import pytest
 
@@ -76,3 +77,35 @@ def test_antenna_on_a_track_end(end, hills, medium, form):
     for f in got:
         assert np.isfinite(got[f]).all(), f
         assert np.abs(got[f] - ref[f]).max() <= 600 * 2.0 ** -24 * np.abs(ref[f]).max(), f
+
+
+@pytest.mark.parametrize("medium", [synth.AIR_EXPONENTIAL, UNIFORM])
+@pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
+@pytest.mark.parametrize("hills", [0.0, 150.0])
+def test_fp64_emission_point_whose_distance_overflows(hills, formalism, medium):
+    """Tracks at 1e200 m pass the track filter; they arrive after every window."""
+    from paper_2309_03717_gb300 import c8r
+    n = 200
+    tracks = {f: x.astype(np.float64) for f, x in synth.make_tracks(n, 31, 0.0).items()}
+    ant = synth.antennas_star(8, n_radii=2)[:9].copy()
+    ant[:, 2] = np.linspace(0.0, hills, len(ant))
+    t_start = synth.trace_start_ns(ant, 0.0)
+    out = []
+    for far in (False, True):
+        t = {f: x.copy() for f, x in tracks.items()}
+        if far:
+            t["x0"][::7] = 1.0e200
+            t["x1"][::7] = 1.1e200
+        else:
+            t["q"][::7] = 0.0
+        p = c8r.RadioProcess(medium, ant, t_start, 1024, 0.2, formalism, "fp64")
+        dev = to_device(t)
+        p.push(dev)
+        assert p.stats()["tracks_kept"] == (n if far else n - len(t["q"][::7]))
+        out.append(p.traces().cpu().numpy())
+        if far:
+            _, bins, _ = p.arrivals(dev)
+            assert (bins[::7] == 1024).all()
+        p.close()
+    assert np.abs(out[0]).max() > 0 and np.isfinite(out[1]).all()
+    assert np.abs(out[1] - out[0]).max() <= 1e-12 * np.abs(out[0]).max()
