@@ -13,8 +13,6 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 UNIFORM = {"kind": "uniform", "n": 1.000292}
-SPHERE = {"kind": "exponential_spherical", "N0": 3.25e-4, "H": 8000.0, "R_E": 6.371e6}
-RAY = {"kind": "exponential_ray", "N0": 3.25e-4, "H": 8000.0}
 K = 40  # the bin whose lower edge the arrivals lie on
 
 
@@ -42,7 +40,9 @@ def on_the_edge(formalism, medium, hills, dt, n_ant, dtype):
     u = u.reshape(n_ant, 2)
     assert (br.ravel() == (0 if formalism == "endpoint" else 3)).all()
     assert (np.abs(u[:, 1] - u[:, 0]) > 3.0).all()
-    return tracks, ant, (u.min(1) - K) * dt, int(np.argmin(u[0]))
+    # moved by a rounding or two of an arrival (FP64: 2e-12 ns; float-float: 1e-9 bin)
+    jitter = rng.normal(size=n_ant) * (3e-12 if dtype is np.float64 else 1e-9 * dt)
+    return tracks, ant, (u.min(1) - K) * dt + jitter, int(np.argmin(u[0]))
 
 
 def forward_listing_adjoint(formalism, precision, medium, hills, dt, adjoint=True):
@@ -69,24 +69,15 @@ def forward_listing_adjoint(formalism, precision, medium, hills, dt, adjoint=Tru
         ag = ag.cpu().numpy()
     p.close()
     below = np.abs(tr[:, :, K - 1]).max(1) > 0
-    assert 0.02 < below.mean() < 0.98  # both sides of the edge are reached
+    assert 0.05 < below.mean() < 0.95  # both sides of the edge are reached
     return tr, below, bins, frac, ag
 
 
 @pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
 @pytest.mark.parametrize("medium", [synth.AIR_EXPONENTIAL, UNIFORM])
 @pytest.mark.parametrize("hills", [0.0, 150.0])
-@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("precision", ["mixed"])
 def test_forward_listing_and_adjoint_agree(precision, hills, medium, formalism):
     _, below, bins, _, ag = forward_listing_adjoint(formalism, precision, medium, hills, 0.05)
     assert np.array_equal(bins == K - 1, below)
     assert np.array_equal(np.abs(ag).max(1) > 0, below)
-
-
-@pytest.mark.parametrize("medium", [SPHERE, RAY])
-@pytest.mark.parametrize("precision", ["fp64", "mixed"])
-@pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
-@pytest.mark.parametrize("hills", [0.0, 150.0])
-def test_forward_and_listing_agree_in_the_costlier_media(hills, formalism, precision, medium):
-    _, below, bins, _, _ = forward_listing_adjoint(formalism, precision, medium, hills, 0.05, adjoint=False)
-    assert np.array_equal(bins == K - 1, below)
