@@ -169,8 +169,9 @@ __device__ __forceinline__ float exp_ap(float x) {
 // (counted on this part), while the FP32 pipe's rate per value stays the same.
 // One exception, whatever -fmad says: the assembler makes one fused operation of
 // a packed product that goes into packed sums only, which it never does with the
-// plain ones.  So where such a sum decides a bin or a branch, which other kernels
-// form from plain values, it is written as the fused operation for both.
+// plain ones.  Where such a sum decides a bin that other kernels form from plain
+// values, mul_apart keeps the product rounded: two plain multiplications, an
+// issue slot more.
 // The pair kernels are bound by issue, so the per-pair arithmetic is written
 // once for T = float or float2 and the main passes run it on pairs: a pair's
 // two endpoints (Endpoint).  Comparisons and the approximate reciprocals take
@@ -188,6 +189,10 @@ __device__ __forceinline__ float2 add_rn(float2 a, float2 b) { return __fadd2_rn
 __device__ __forceinline__ float2 sub_rn(float2 a, float2 b) { return __fadd2_rn(a, neg(b)); }
 __device__ __forceinline__ float2 mul_rn(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma_rn(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float mul_apart(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float2 mul_apart(float2 a, float2 b) {
+  return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
+}
 __device__ __forceinline__ float2 rsqrt_ap(float2 x) { return make_float2(rsqrt_ap(x.x), rsqrt_ap(x.y)); }
 __device__ __forceinline__ float2 rcp_ap(float2 x) { return make_float2(rcp_ap(x.x), rcp_ap(x.y)); }
 __device__ __forceinline__ float2 div_ap(float2 a, float2 b) { return __fmul2_rn(a, rcp_ap(b)); }
@@ -223,13 +228,6 @@ __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
   const T bb = sub_rn(s, a);
   e = add_rn(sub_rn(a, sub_rn(s, bb)), sub_rn(b, bb));
 }
-// a + b c: two_sum with the product in its sums unrounded (fused operations)
-template <typename T>
-__device__ __forceinline__ void two_sum_prod(T a, T b, T c, T& s, T& e) {
-  s = fma_rn(b, c, a);
-  const T bb = sub_rn(s, a);
-  e = add_rn(sub_rn(a, sub_rn(s, bb)), fma_rn(b, c, neg(bb)));
-}
 template <typename T>
 __device__ __forceinline__ void two_prod(T a, T b, T& p, T& e) {
   p = mul_rn(a, b);
@@ -240,12 +238,6 @@ template <typename T>
 __device__ __forceinline__ void fast_two_sum(T a, T b, T& s, T& e) {
   s = add_rn(a, b);
   e = sub_rn(b, sub_rn(s, a));
-}
-// the same for a + b c, |b c| < |a|
-template <typename T>
-__device__ __forceinline__ void fast_two_sum_prod(T a, T b, T c, T& s, T& e) {
-  s = fma_rn(b, c, a);
-  e = fma_rn(b, c, neg(sub_rn(s, a)));
 }
 
 // ---------------------------------------------------------------------------
@@ -682,7 +674,7 @@ __device__ __forceinline__ ffT<T> arrival_mixed_q(const MedParams& M, T atauh, T
     if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL || KIND == C8R_EXPONENTIAL_RAY) {
       // the small change of the optical path in bins (the sphere's curvature,
       // ~1e-3 of the refractivity term; the ray's time saved, <~1 bin): FP32 is enough
-      fast_two_sum_prod(p, corr, bc<T>(M.kc_h), p2, pe2);
+      fast_two_sum(p, mul_apart(corr, bc<T>(M.kc_h)), p2, pe2);
       p = p2;
       pe = add_rn(pe, pe2);
     }
@@ -1041,7 +1033,12 @@ __device__ __forceinline__ void field_mixed(const GeoT<T>& g, T bx, T by, T bz, 
   const T invR = g.y;
   const T w2 = fma_rn(wx, wx, fma_rn(wy, wy, mul_rn(wz, wz)));
   const T den = mul_rn(R, fma_rn(bmag, R, bd));
-  f.D = fma_rn(mul_rn(n, w2), rcp_ap(den), om_nb);
+  // (fused in pairs, which the assembler would do by itself: written out so that
+  // every main pass takes the same near-Cherenkov decisions)
+  if constexpr (kUsualForm<T>)
+    f.D = fma_rn(mul_rn(n, w2), rcp_ap(den), om_nb);
+  else
+    f.D = add_rn(om_nb, div_ap(mul_rn(n, w2), den));
   if constexpr (!kUsualForm<T>)
     if (!(bd >= 0.0f)) f.D = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(n, bd), invR));
   // d x w = d (d.beta) - beta R^2  ->  V R^2
@@ -1111,7 +1108,7 @@ __device__ __forceinline__ ffT<T> doppler_ff(const GeoT<T>& g, T bx, T by, T p2,
   const T ql = mul_rn(r, g.y);
   // n q = q + (n - 1) q, then D = 1 - n q
   T nh, nl;
-  two_sum_prod(qh, nm1, qh, nh, nl);
+  two_sum(qh, mul_apart(nm1, qh), nh, nl);
   nl = add_rn(nl, ql);
   T dh, dl;
   two_sum(bc<T>(1.0f), neg(nh), dh, dl);
