@@ -210,8 +210,9 @@ struct ArrivalSink {
   __device__ __forceinline__ void rec(int b, double ua, double ub) {
     double ka = floor(ua), kb = floor(ub);
     branch[j] = b;
-    bin[2 * j] = ka < 0.0 ? -1 : (ka >= (double)N ? N : (int)ka);
-    bin[2 * j + 1] = kb < 0.0 ? -1 : (kb >= (double)N ? N : (int)kb);
+    // (NaN, where the squared distance overflows, as after the window)
+    bin[2 * j] = ka < 0.0 ? -1 : (ka < (double)N ? (int)ka : N);
+    bin[2 * j + 1] = kb < 0.0 ? -1 : (kb < (double)N ? (int)kb : N);
     frac[2 * j] = (float)(ua - ka);
     frac[2 * j + 1] = (float)(ub - kb);
   }

@@ -800,12 +800,6 @@ struct OpsF64Plain {
     double r = p.r;
     if (M.kind != C8R_UNIFORM && !M.flat) r = refr(M, A.Ea, p.E, dz);
     e.u = __dmul_rn(__fma_rn(__fma_rn(r, R, R), M.inv_c_ns, __dsub_rn(p.t, A.t_ref)), M.inv_dt);
-    // |d|^2 overflows: the roots above are NaN.  The signal arrives after every
-    // window (tested on the high word, off the FP64 pipe)
-    if (__double2hiint(S) == 0x7ff00000) {
-      e.D = 1.0;
-      e.u = S;
-    }
     return true;
   }
 
@@ -837,7 +831,9 @@ struct OpsF64Plain {
       const double h = __dmul_rn(fabs(e.D), t.hw);
       const double u_lo = __dsub_rn(e.u, h), u_hi = __dadd_rn(e.u, h);
       const FloorD lo = floor_bin(u_lo, N), hi = floor_bin(u_hi, N);
-      const bool one = lo.k == hi.k;
+      // (also when |d|^2 overflows: u is NaN then, in no bin, and an interval of it
+      // must not go in as a box)
+      const bool one = !(lo.k < hi.k);
       out.rec(one ? 2 : 3, u_lo, u_hi);
       const double s = -__dmul_rn(t.amp, e.iR);  // beta_perp = -V
       const double invW = one ? 1.0 : rcp_f64(__dadd_rn(h, h));
