@@ -156,6 +156,12 @@ __device__ __forceinline__ float rcp_ap(float x) {
   return r;
 }
 __device__ __forceinline__ float div_ap(float a, float b) { return __fmul_rn(a, rcp_ap(b)); }
+// the smaller, or NaN if either is
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 __device__ __forceinline__ float exp_ap(float x) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__fmul_rn(x, 1.44269504088896341f)));
@@ -169,8 +175,8 @@ __device__ __forceinline__ float exp_ap(float x) {
 // (counted on this part), while the FP32 pipe's rate per value stays the same.
 // One exception, whatever -fmad says: the assembler makes one fused operation of
 // a packed product that goes into packed sums only, which it never does with the
-// plain ones.  Where such a sum decides a bin that other kernels form from plain
-// values, mul_apart keeps the product rounded: two plain multiplications, an
+// plain ones.  Where such a sum decides a bin or a branch that other kernels form from
+// plain values, mul_apart keeps the product rounded: two plain multiplications, an
 // issue slot more.
 // The pair kernels are bound by issue, so the per-pair arithmetic is written
 // once for T = float or float2 and the main passes run it on pairs: a pair's
@@ -1033,12 +1039,7 @@ __device__ __forceinline__ void field_mixed(const GeoT<T>& g, T bx, T by, T bz, 
   const T invR = g.y;
   const T w2 = fma_rn(wx, wx, fma_rn(wy, wy, mul_rn(wz, wz)));
   const T den = mul_rn(R, fma_rn(bmag, R, bd));
-  // (fused in pairs, which the assembler would do by itself: written out so that
-  // every main pass takes the same near-Cherenkov decisions)
-  if constexpr (kUsualForm<T>)
-    f.D = fma_rn(mul_rn(n, w2), rcp_ap(den), om_nb);
-  else
-    f.D = add_rn(om_nb, div_ap(mul_rn(n, w2), den));
+  f.D = add_rn(om_nb, mul_apart(mul_rn(n, w2), rcp_ap(den)));
   if constexpr (!kUsualForm<T>)
     if (!(bd >= 0.0f)) f.D = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(n, bd), invR));
   // d x w = d (d.beta) - beta R^2  ->  V R^2

@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(kTileT, Ops::kBwdMinBlocks) k_backward(const B
           if constexpr (Ops::kFastBins) {
             // a pair settled as zero has no adjoint either
             exact = false;
-            if (!Ops::near_zero_fast(stage, l, A, M)) {
+            if (!Ops::template near_zero_fast<true>(stage, l, A, M)) {
               const int k = atomicAdd(&q_exact, 1);
               if (k < kCap) list[kCap + k] = (uint16_t)(e & 0xfff);
             }
@@ -776,8 +776,9 @@ __global__ void __launch_bounds__(kTileT, Ops::kBwdMinBlocks) k_backward(const B
         const int l = e & (kTileT - 1), ant = (e >> 7) & (kMaxATile - 1);
         const AntRec A = Ops::load_ant(ant_s + ant);
         acc_t ga[3] = {0, 0, 0};
-        if (q < nA) {
-          Ops::adj_end_deferred(stage, l, A, M, G + (size_t)ant * N, a.out, t * kTileT + l, ga, dn_acc, kDeferEnd1);
+        const int end = q < nA ? (int)kDeferEnd1 : Ops::lone_end(stage, l, A, M);
+        if (end) {
+          Ops::adj_end_deferred(stage, l, A, M, G + (size_t)ant * N, a.out, t * kTileT + l, ga, dn_acc, end);
         } else {
           typename Ops::Track tr;
           Ops::load(stage, l, M, tr);

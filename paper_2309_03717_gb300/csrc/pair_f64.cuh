@@ -193,6 +193,7 @@ struct OpsF64 {
   }
   template <class Sink>
   static __device__ __forceinline__ void end_deferred(const void*, int, const AntRec&, const MedParams&, Sink&, int) {}
+  template <bool ADJ = false>
   static __device__ __forceinline__ bool near_zero_fast(const void*, int, const AntRec&, const MedParams&) {
     return false;
   }
@@ -329,6 +330,7 @@ struct OpsF64 {
       adj(tr, A, M, G, m.g, ga, dn);
     return kDeferNone;
   }
+  static __device__ __forceinline__ int lone_end(const void*, int, const AntRec&, const MedParams&) { return 0; }
   static __device__ __forceinline__ void adj_deferred(const TrackD&, const AntRec&, const MedParams&, const Acc4D*,
                                                       const PrefixFF*, double*, double*, double&) {}
   static __device__ __forceinline__ void adj_end_deferred(const void*, int, const AntRec&, const MedParams&,

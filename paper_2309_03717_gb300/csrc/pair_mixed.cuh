@@ -971,12 +971,16 @@ struct OpsMixed {
 
   // the geometry, the field and the bins (arrival_fast in the form this kernel
   // is compiled for) of a pair's two endpoints; true for a near-Cherenkov pair.
+  // An endpoint without a geometry (on the antenna, |d| = 0, or out of FP32's range)
+  // has D = NaN and no bin.  The forward pass leaves it at that; the adjoint (ADJ)
+  // sets the pair aside with the near ones (lone_end), to keep 0 x NaN out of its sums.
   // Both endpoints at once (float2): 291 -> 187 thread instructions per pair with
   // the set-aside bits (Aside).  Measured, ms: 4e6 tracks x 1024 antennas at 60
   // degrees 40.3 -> 36.9, 64 uneven showers 3.30 -> 3.03, the adjoint on 1e6
   // tracks x 64 antennas 1.23 -> 0.96 (5 CTAs per SM; 1.20 with 6, 1.11 with 4);
   // a vertical shower x 160 antennas, 5.65 -> 5.3 to 5.5, is bound by its
   // reductions (3.8 without them and the set-aside work)
+  template <bool ADJ = false>
   static __device__ __forceinline__ bool endpoints_main(const TrackE& t, const AntE& A, const MedParams& M,
                                                         GeoT<float2>& g, FieldT<float2>& f, int& ka, int& kb) {
     float2 S, P, uf, q = bc<float2>(0.0f);
@@ -1005,7 +1009,8 @@ struct OpsMixed {
       endpoint_rare<1>(t, A, M, g, S, P, uf.y, eps.y, f.D.y);
     }
     decide_bins(uf, eps, M.n_bins, ka, kb);
-    return !(fminf(fabsf(f.D.x), fabsf(f.D.y)) >= M.eps_C);
+    const float d0 = fabsf(f.D.x), d1 = fabsf(f.D.y);
+    return !((ADJ ? min_nan(d0, d1) : fminf(d0, d1)) >= M.eps_C);
   }
 
   // main pass: every pair except (Endpoint) the near-Cherenkov ones, for which
@@ -1073,6 +1078,7 @@ struct OpsMixed {
   // more roundings on the interval ends.  True when the pair is decided to be
   // zero, false when the float-float evaluation must run (about 4 % of the
   // near-Cherenkov pairs of a shower).
+  template <bool ADJ = false>
   static __device__ __forceinline__ bool near_zero_fast(const void* Tv, int l, const AntRec& A, const MedParams& M) {
     if constexpr (kFastBins) {
       constexpr float u = 5.9604644775390625e-8f;  // 2^-24
@@ -1081,6 +1087,10 @@ struct OpsMixed {
       const float x1 = TF(fm::X1), y1 = TF(fm::Y1), z1 = TF(fm::Z1);
       const float a0x = __fadd_rn(A.xh, -x0), a0y = __fadd_rn(A.yh, -y0), a0z = __fadd_rn(A.zh, -z0);
       const float a1x = __fadd_rn(A.xh, -x1), a1y = __fadd_rn(A.yh, -y1), a1z = __fadd_rn(A.zh, -z1);
+      // (adjoint) an endpoint on the antenna: not this form
+      if constexpr (ADJ) {
+        if (on_antenna(a0x, a0y, a0z) || on_antenna(a1x, a1y, a1z)) return false;
+      }
       GeoM g;
       g.s[0] = 0.5f * __fadd_rn(a0x, a1x);
       g.s[1] = 0.5f * __fadd_rn(a0y, a1y);
@@ -1347,6 +1357,35 @@ struct OpsMixed {
     dn = __fmaf_rn(dns.y, t.Eh.y, __fmaf_rn(dns.x, t.Eh.x, dn));
   }
 
+  // a squared distance of zero, also from components whose squares are denormal
+  static __device__ __forceinline__ bool on_antenna(float x, float y, float z) {
+    constexpr float none = 1.1e-19f;
+    return fabsf(x) < none && fabsf(y) < none && fabsf(z) < none;
+  }
+  // of a pair that the adjoint's main pass set aside whole: the one endpoint with a
+  // geometry where the other has none and that one is not near the Cherenkov angle
+  // (kDeferEnd0 or kDeferEnd1), or 0
+  static __device__ __forceinline__ int lone_end(const void* Tv, int l, const AntRec& A, const MedParams& M) {
+    if constexpr (kFastBins) {
+      const float* T = static_cast<const float*>(Tv);
+      GeoM g0, g1;
+      geo_lite(A, TF(fm::X0), TF(fm::Y0), TF(fm::Z0), g0);
+      geo_lite(A, TF(fm::X1), TF(fm::Y1), TF(fm::Z1), g1);
+      if (g0.R0 + g1.R0 > 0.0f) return 0;
+      const int end = g0.R0 > 0.0f ? kDeferEnd0 : kDeferEnd1;
+      const GeoM& g = end == kDeferEnd0 ? g0 : g1;
+      const float bmag = TF(fm::BMAG);
+      float nm1 = M.nm1f;
+      if (KIND != C8R_UNIFORM) nm1 = __fmul_rn(M.N0f, end == kDeferEnd0 ? TF(fm::E0H) : TF(fm::E1H));
+      FieldM f;
+      field_mixed<float>(g, TF(fm::BX), TF(fm::BY), TF(fm::BZ), bmag, __fsub_rn(TF(fm::OMB), __fmul_rn(nm1, bmag)),
+                         __fadd_rn(1.0f, nm1), f);
+      return fabsf(f.D) >= M.eps_C ? end : 0;
+    } else {
+      return 0;
+    }
+  }
+
   // adjoint main pass: every pair except (Endpoint) the near-Cherenkov ones, for
   // which it adds nothing and returns kDeferPair, and (kFastBins) the endpoints
   // whose bin the FP32 arrival leaves open (kDeferEnd0/kDeferEnd1 bits), after
@@ -1361,11 +1400,7 @@ struct OpsMixed {
       GeoT<float2> g;
       FieldT<float2> f;
       int ka, kb;
-      if (endpoints_main(t, *p, M, g, f, ka, kb)) return kDeferPair;
-      // an endpoint on the antenna, or too far away for FP32: R, and with it the
-      // half's field and gradients, are NaN, which a zero dL/dtrace would not keep
-      // out of the sums.  The other endpoint is left to the pass after this one
-      if (!(g.R0.x + g.R0.y > 0.0f)) return (ka != kFastOut ? kDeferEnd0 : 0) | (kb != kFastOut ? kDeferEnd1 : 0);
+      if (endpoints_main<true>(t, *p, M, g, f, ka, kb)) return kDeferPair;
       const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       const float4 g0 = ka >= 0 ? G[ka] : zero, g1 = kb >= 0 ? G[kb] : zero;
       if (ka >= 0 || kb >= 0) adj_ends(g, f, t, g0, g1, M, m, ga, dn);
