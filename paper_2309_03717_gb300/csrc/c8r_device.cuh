@@ -987,9 +987,11 @@ __device__ __forceinline__ float gap_to_next_edge(ff u, int k) {
   return __fsub_rn(__fsub_rn((float)(k + 1), u.h), u.l);
 }
 
-// The bins and fractions of two float-float arrivals as bin_raw has them, for
-// windows of at most kMagicBins / 2 bins: floors from rounded-down sums as in
-// decide_bins, of the high part and then of the fraction with the low part.
+// The bins and fractions of two float-float arrivals as bin_raw has them: floors
+// from rounded-down sums as in decide_bins, of the high part and then of the
+// fraction with the low part.  Beyond 2^22 the first sum's spacing is 2, and the
+// second floor takes what is left.  The index comes from the sums' low bits for
+// windows of at most kMagicBins / 2 bins, by conversion for longer ones (XU pipe).
 // Arrivals outside the window give any index outside it.
 __device__ __forceinline__ void bins_of(ffT<float2> u, int n_bins, int& kx, int& ky, float2& kf, float2& frac) {
   const float2 magic = make_float2(12582912.0f, 12582912.0f);
@@ -1005,9 +1007,14 @@ __device__ __forceinline__ void bins_of(ffT<float2> u, int n_bins, int& kx, int&
   const float2 df = sub_rn(t1, magic);
   kf = add_rn(k0, df);
   frac = sub_rn(f, df);
-  constexpr unsigned two = 2u * (unsigned)kMagicBinBits;
-  kx = (int)(__float_as_uint(t.x) + __float_as_uint(t1.x) - two);
-  ky = (int)(__float_as_uint(t.y) + __float_as_uint(t1.y) - two);
+  if (n_bins <= kMagicBins / 2) {
+    constexpr unsigned two = 2u * (unsigned)kMagicBinBits;
+    kx = (int)(__float_as_uint(t.x) + __float_as_uint(t1.x) - two);
+    ky = (int)(__float_as_uint(t.y) + __float_as_uint(t1.y) - two);
+  } else {
+    kx = __float2int_rn(kf.x);
+    ky = __float2int_rn(kf.y);
+  }
 }
 
 // field part at one emission point (FP32): w = d x beta, V = (d x w)/R^2 =

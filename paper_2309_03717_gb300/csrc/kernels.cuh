@@ -143,6 +143,7 @@ template <typename T>
 struct GlobalSink;
 template <>
 struct GlobalSink<float> {
+  static constexpr bool kRecords = false;
   // accumulator of one antenna: n bins, followed (formalisms that add boxes) by
   // n bins of box edges, which the fetch integrates over the bins
   float4* row;
@@ -189,16 +190,19 @@ struct GlobalSink<double> {
 };
 
 struct ArrivalSink {
+  static constexpr bool kRecords = true;
   int32_t* branch;
   int32_t* bin;
   float* frac;
   int64_t j;
   int N;
+  bool off = false;  // records nothing (a pair's neighbour)
   __device__ __forceinline__ void dep(int, float, float, float) {}
   __device__ __forceinline__ void dep(int, double, double, double) {}
   __device__ __forceinline__ void dep_box(int, int, float, float, float) {}
   __device__ __forceinline__ void dep_box(int, int, double, double, double) {}
   __device__ __forceinline__ void rec(int b, ff ua, ff ub) {
+    if (off) return;
     float fa, fb;
     int ka = bin_raw(ua, N, fa), kb = bin_raw(ub, N, fb);
     branch[j] = b;

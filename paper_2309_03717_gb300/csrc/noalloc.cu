@@ -44,6 +44,7 @@ std::once_flag g_na_once[kNaMaxDevices];
 
 // deposits straight into the caller's traces [n_ant][3][n_bins]
 struct TraceSink {
+  static constexpr bool kRecords = false;
   float* tr;  // traces of one antenna
   int N;
   __device__ __forceinline__ void dep(int k, float x, float y, float z) {

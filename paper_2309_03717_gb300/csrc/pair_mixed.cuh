@@ -359,16 +359,19 @@ struct EndpointEvalM {
 // the field arithmetic; the straight geometry stays with the arrival time and
 // the amplitude's R) and return the ray's optical-path change and the change of
 // D = 1 - n beta.rhat that the turn makes
-__device__ __forceinline__ void ray_turn_mixed(GeoM& g, float nu_e, float bx, float by, float bz, const MedParams& M,
-                                               float& dop, float& dD) {
+__device__ __forceinline__ float ray_turn(const GeoM& g, float nu_e, const MedParams& M, float t[3]) {
   const float dx = g.s[0], dy = g.s[1], dz = g.s[2], R = g.R0;
   const RayFix<float> r = ray_fix<float, 1>(dx * dx + dy * dy, dz, R, nu_e, M.invH_h);
-  float t[3];
   ray_turn_vector<float>(dx, dy, dz, R, r.Q, t);
+  return r.dop;
+}
+__device__ __forceinline__ void ray_turn_mixed(GeoM& g, float nu_e, float bx, float by, float bz, const MedParams& M,
+                                               float& dop, float& dD) {
+  float t[3];
+  dop = ray_turn(g, nu_e, M, t);
   g.s[0] = __fadd_rn(g.s[0], t[0]);
   g.s[1] = __fadd_rn(g.s[1], t[1]);
   g.s[2] = __fadd_rn(g.s[2], t[2]);
-  dop = r.dop;
   dD = -(1.0f + nu_e) * (bx * t[0] + by * t[1] + bz * t[2]) * g.y;
 }
 
@@ -863,27 +866,39 @@ struct OpsMixed {
   }
 
   // ZHS of two tracks against one antenna, the arithmetic of `zhs` in both halves
-  // (float2): 302 -> 170 warp instructions per 32 pairs.  Bound by the FP32 pipe
-  // (63 % of its cycles, the float-float sums) and, for a vertical shower on few
-  // antennas, by its reductions.  Measured with the accumulator copies, ms: 2e7
-  // tracks x 160 antennas 29.4 -> 25.6; 3e5 tracks x 512 antennas 1.61 -> 1.47;
-  // false when a half needs another form of it (the altitude difference
-  // within 1e-3 H, or a window too long for bins_of), with nothing deposited
+  // (float2), with a sink for each: 302 -> 170 warp instructions per 32 pairs.
+  // Bound by the FP32 pipe (63 % of its cycles, the float-float sums) and, for a
+  // vertical shower on few antennas, by its reductions.  Measured with the
+  // accumulator copies, ms: 2e7 tracks x 160 antennas 29.4 -> 25.6; 3e5 tracks x 512
+  // antennas 1.61 -> 1.47.  What has a rarer form takes it half by half, and only
+  // that part of the arithmetic does: the quotient's series (the altitude
+  // difference within 1e-3 H) and the propagator's quadrature where the series of
+  // PathZ does not hold.
   template <class Sink>
-  static __device__ __forceinline__ bool zhs_two(const TrackZ<KIND>& t, const AntZ& A, const MedParams& M, Sink& out) {
+  static __device__ __forceinline__ void zhs_two(const TrackZ<KIND>& t, const AntZ& A, const MedParams& M, Sink& outx,
+                                                 Sink& outy) {
     const int N = M.n_bins;
-    if (!LIN && N > kMagicBins / 2) return false;
     GeoT<float2> g;
     ffT<float2> um, aD;
     if constexpr (kFlat) {
       geo_lite(A.x, A.y, A.xl, A.yl, t.mx, t.my, t.mxl, t.myl, t.zm, g);
       float2 corr = bc<float2>(0.0f), turn[3];
       if constexpr (KIND == C8R_EXPONENTIAL_SPHERICAL) {
-        if (!t.small) return false;
-        corr = t.path(M, A.x, A.y, g);
+        if (t.small) {
+          corr = t.path(M, A.x, A.y, g);
+        } else {
+          corr.x = sphere_half<0>(A, M, g);
+          corr.y = sphere_half<1>(A, M, g);
+        }
       }
       if constexpr (KIND == C8R_EXPONENTIAL_RAY) {
-        if (!t.path(g, corr, turn)) return false;
+        if (!t.path(g, corr, turn)) {
+          float tx[3], ty[3];
+          corr.x = ray_turn(half_of<0>(g), t.nm1.x, M, tx);
+          corr.y = ray_turn(half_of<1>(g), t.nm1.y, M, ty);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) turn[c] = make_float2(tx[c], ty[c]);
+        }
       }
       geo_refine(g, t.zm);
       um = arrival_mixed_q<KIND>(M, A.tauh, A.taul, g, t.tmh, t.tml, t.Eh, t.El, corr);
@@ -900,8 +915,12 @@ struct OpsMixed {
       two_sum(A.z, neg(t.mz), dzh, dzl);
       dzl = add_rn(dzl, sub_rn(A.zl, t.mzl));
       if constexpr (KIND == C8R_EXPONENTIAL) {
-        if (!(fminf(fabsf(dzh.x), fabsf(dzh.y)) > -M.dz_series)) return false;
-        refr_quotient(M, A.Eh, A.El, dzh, dzl, t.Eh, t.El, q0, q1);
+        if (fminf(fabsf(dzh.x), fabsf(dzh.y)) > -M.dz_series) {
+          refr_quotient(M, A.Eh, A.El, dzh, dzl, t.Eh, t.El, q0, q1);
+        } else {
+          refr_quotient(M, A.Eh.x, A.El.x, dzh.x, dzl.x, t.Eh.x, t.El.x, q0.x, q1.x);
+          refr_quotient(M, A.Eh.y, A.El.y, dzh.y, dzl.y, t.Eh.y, t.El.y, q0.y, q1.y);
+        }
       }
       const ZPartT<float2> z = z_part(dzh, dzl, t.bz);
       geo_lite(A.x, A.y, A.xl, A.yl, t.mx, t.my, t.mxl, t.myl, z, g);
@@ -932,22 +951,34 @@ struct OpsMixed {
     const float2 Mx = mul_rn(s, fma_rn(g.s[1], wz, neg(mul_rn(g.s[2], wy))));
     const float2 My = mul_rn(s, fma_rn(g.s[2], wx, neg(mul_rn(g.s[0], wz))));
     const float2 Mz = mul_rn(s, fma_rn(g.s[0], wy, neg(mul_rn(g.s[1], wx))));
+    const ff lox{ulo.h.x, ulo.l.x}, loy{ulo.h.y, ulo.l.y}, hix{uhi.h.x, uhi.l.x}, hiy{uhi.h.y, uhi.l.y};
+    if constexpr (Sink::kRecords) {
+      float f;
+      outx.rec(bin_raw(lox, N, f) == bin_raw(hix, N, f) ? 2 : 3, lox, hix);
+      outy.rec(bin_raw(loy, N, f) == bin_raw(hiy, N, f) ? 2 : 3, loy, hiy);
+      return;
+    }
     if constexpr (LIN) {
-      zhs_deposit_lin(ff{ulo.h.x, ulo.l.x}, ff{uhi.h.x, uhi.l.x}, hh.x, Mx.x, My.x, Mz.x, N, out);
-      zhs_deposit_lin(ff{ulo.h.y, ulo.l.y}, ff{uhi.h.y, uhi.l.y}, hh.y, Mx.y, My.y, Mz.y, N, out);
+      zhs_deposit_lin(lox, hix, hh.x, Mx.x, My.x, Mz.x, N, outx);
+      zhs_deposit_lin(loy, hiy, hh.y, Mx.y, My.y, Mz.y, N, outy);
     } else {
+      const float2 invW = rcp_ap(mul_rn(bc<float2>(2.0f), hh));  // 1 / interval length in bins
       int klox, kloy, khix, khiy;
       float2 klo, khi, flo, fhi;
       bins_of(ulo, N, klox, kloy, klo, flo);
       bins_of(uhi, N, khix, khiy, khi, fhi);
-      const float2 invW = rcp_ap(mul_rn(bc<float2>(2.0f), hh));  // 1 / interval length in bins
       // gap_to_next_edge
       const float2 gap = sub_rn(sub_rn(add_rn(klo, bc<float2>(1.0f)), ulo.h), ulo.l);
       const float2 wlo = mul_rn(gap, invW), whi = mul_rn(fhi, invW);
-      zhs_deposit(klox, khix, klox == khix ? 1.0f : wlo.x, whi.x, invW.x, Mx.x, My.x, Mz.x, N, out);
-      zhs_deposit(kloy, khiy, kloy == khiy ? 1.0f : wlo.y, whi.y, invW.y, Mx.y, My.y, Mz.y, N, out);
+      zhs_deposit(klox, khix, klox == khix ? 1.0f : wlo.x, whi.x, invW.x, Mx.x, My.x, Mz.x, N, outx);
+      zhs_deposit(kloy, khiy, kloy == khiy ? 1.0f : wlo.y, whi.y, invW.y, Mx.y, My.y, Mz.y, N, outy);
     }
-    return true;
+  }
+  // the curvature quadrature of one half
+  template <int J>
+  static __device__ __forceinline__ float sphere_half(const AntZ& A, const MedParams& M, const GeoT<float2>& g) {
+    return sphere_path_correction<float>(A.x.x, A.y.x, A.z.x, half_of<J>(g.s[0]), half_of<J>(g.s[1]),
+                                         half_of<J>(g.s[2]), half_of<J>(g.R0), M.N0f, M.invH_h, M.RE_f);
   }
 
   // one endpoint of a pair in which some condition of the usual forms fails: its
@@ -1021,15 +1052,7 @@ struct OpsMixed {
   static __device__ __forceinline__ int pair_main(const FwdTrack& t, const FwdAnt* p, const void* Tv, int l,
                                                   const MedParams& M, Sink& out) {
     if constexpr (kTwoTracks) {
-      if (!zhs_two(t, *p, M, out)) {
-        // one half at a time, from the staged tile
-        const AntRec A = load_ant(p);
-        for (int h = 0; h < 2; ++h) {
-          TrackM one;
-          load(Tv, 2 * l + h, M, one);
-          if (live(one)) zhs(one, A, M, out);
-        }
-      }
+      zhs_two(t, *p, M, out, out);
       return kDeferNone;
     } else if constexpr (kFastBins) {
       GeoT<float2> g;
@@ -1213,7 +1236,45 @@ struct OpsMixed {
     }
   }
 
-  // one pair from a staged tile (the arrival listing uses this)
+  // one pair from a staged tile, for the arrival listing: as the forward kernel
+  // has it, the track with its neighbour where that takes two at a time
+  template <class Sink>
+  static __device__ __forceinline__ void list(const void* Tv, int l, const AntRec& A, const MedParams& M, Sink& out) {
+    if constexpr (kTwoTracks) {
+      TrackZ<KIND> t;
+      load_fwd(Tv, l / 2, M, t);
+      if (static_cast<const float*>(Tv)[fm::AMPE * kTileT + l] == 0.0f) return;
+      AntZ z;
+      stage_ant(&z, A, M);
+      Sink none = out;
+      none.off = true;
+      zhs_two(t, z, M, l & 1 ? none : out, l & 1 ? out : none);
+    } else if constexpr (kFastBins) {
+      // the main pass decides the near-Cherenkov pairs; which bin a pair's
+      // endpoints have does not depend on the way it takes there
+      TrackE te;
+      load_main(Tv, l, M, te);
+      if (!live(te)) return;
+      AntE ae;
+      stage_ant(&ae, A, M);
+      GeoT<float2> g;
+      FieldT<float2> f;
+      int ka, kb;
+      const bool near = endpoints_main(te, ae, M, g, f, ka, kb);
+      TrackM t;
+      load(Tv, l, M, t);
+      EndpointEvalM e;
+      if (!endpoint_fields<KIND>(t, A, M, e)) return;
+      if (!near)
+        endpoint_arrivals<KIND>(t, A, M, e);
+      else if (!endpoint_midpoint<KIND>(t, A, M, e))
+        return;
+      out.rec(e.branch, e.ua, e.ub);
+    } else {
+      fwd(Tv, l, A, M, out);
+    }
+  }
+  // one pair from a staged tile (the allocation-free pass uses this)
   template <class Sink>
   static __device__ __forceinline__ void fwd(const void* Tv, int l, const AntRec& A, const MedParams& M, Sink& out) {
     TrackM t;
