@@ -532,7 +532,10 @@ __global__ void __launch_bounds__(256) k_arrivals(const void* tiles, int64_t n, 
   const AntRec A = ants[a];
   ArrivalSink sink{branch, bin, frac, j, M.n_bins};
   const unsigned char* T = static_cast<const unsigned char*>(tiles) + (i / kTileT) * (int64_t)Ops::kTileBytes;
-  Ops::fwd(T, (int)(i % kTileT), A, M, sink);
+  if constexpr (Ops::kPrec == C8R_MIXED)
+    Ops::list(T, (int)(i % kTileT), A, M, sink);
+  else
+    Ops::fwd(T, (int)(i % kTileT), A, M, sink);
 }
 
 // ---------------------------------------------------------------------------

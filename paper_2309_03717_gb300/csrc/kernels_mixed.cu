@@ -431,41 +431,29 @@ cudaError_t launch_bin_running_sums(const void* g, int n_ant, int n_bins, Prefix
 cudaError_t launch_arrivals_mixed(int formalism, const void* tiles, int64_t n, const AntRec* ants, int n_ant,
                                   const MedParams& M, int32_t* branch, int32_t* bin, float* frac, cudaStream_t st) {
   const unsigned blocks = (unsigned)((n * (int64_t)n_ant + 255) / 256);
-  if (M.kind == C8R_EXPONENTIAL_RAY) {
-    if (formalism == C8R_ENDPOINT)
-      k_arrivals<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_RAY>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch,
-                                                                                     bin, frac);
-    else
-      k_arrivals<OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin,
-                                                                                frac);
+  auto go = [&](auto ops) {
+    k_arrivals<decltype(ops)><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin, frac);
     return cudaGetLastError();
-  }
-  if (M.kind == C8R_EXPONENTIAL_SPHERICAL) {
-    if (formalism == C8R_ENDPOINT)
-      k_arrivals<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_SPHERICAL>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M,
-                                                                                           branch, bin, frac);
-    else
-      k_arrivals<OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_SPHERICAL>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M,
-                                                                                      branch, bin, frac);
-    return cudaGetLastError();
-  }
-  const bool ex = M.kind == C8R_EXPONENTIAL;
+  };
+  // the kernels of forward_mixed (the arrival form and an Endpoint's flat array
+  // change nothing that is listed)
   if (formalism == C8R_ENDPOINT) {
-    if (ex)
-      k_arrivals<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch,
-                                                                                 bin, frac);
-    else
-      k_arrivals<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin,
-                                                                             frac);
-  } else {
-    if (ex)
-      k_arrivals<OpsMixed<C8R_ZHS, C8R_EXPONENTIAL>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin,
-                                                                            frac);
-    else
-      k_arrivals<OpsMixed<C8R_ZHS, C8R_UNIFORM>><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin,
-                                                                        frac);
+    if (M.kind == C8R_EXPONENTIAL_RAY) return go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_RAY>{});
+    if (M.kind == C8R_EXPONENTIAL_SPHERICAL) return go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_SPHERICAL>{});
+    return M.kind == C8R_EXPONENTIAL ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>{})
+                                     : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
   }
-  return cudaGetLastError();
+  if (M.flat) {
+    if (M.kind == C8R_EXPONENTIAL_RAY)
+      return go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, false, kFormDirect, true>{});
+    if (M.kind == C8R_EXPONENTIAL_SPHERICAL)
+      return go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_SPHERICAL, false, kFormDirect, true>{});
+    return go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, false, kFormDirect, true>{});
+  }
+  if (M.kind == C8R_EXPONENTIAL_RAY) return go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY>{});
+  if (M.kind == C8R_EXPONENTIAL_SPHERICAL) return go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_SPHERICAL>{});
+  return M.kind == C8R_EXPONENTIAL ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL>{})
+                                   : go(OpsMixed<C8R_ZHS, C8R_UNIFORM>{});
 }
 
 cudaError_t launch_backward_mixed(int formalism, bool lin, BwdArgs& a, const FwdShape& shape, int sm_count,

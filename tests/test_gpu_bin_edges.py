@@ -13,6 +13,8 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 UNIFORM = {"kind": "uniform", "n": 1.000292}
+SPHERE = {"kind": "exponential_spherical", "N0": 3.25e-4, "H": 8000.0, "R_E": 6.371e6}
+RAY = {"kind": "exponential_ray", "N0": 3.25e-4, "H": 8000.0}
 K = 40  # the bin whose lower edge the arrivals lie on
 
 
@@ -23,7 +25,7 @@ def _lib():
     built_lib()
 
 
-def on_the_edge(formalism, medium, hills, dt, n_ant, dtype):
+def on_the_edge(formalism, medium, hills, dt, n_ant, dtype, K=K, spread=1e-9):
     """A 4 m track 3 km up and n_ant antennas, the first arrival of each on edge K."""
     rng = np.random.default_rng(11)
     b = np.array([0.02, 0.01, -0.999])
@@ -40,22 +42,21 @@ def on_the_edge(formalism, medium, hills, dt, n_ant, dtype):
     u = u.reshape(n_ant, 2)
     assert (br.ravel() == (0 if formalism == "endpoint" else 3)).all()
     assert (np.abs(u[:, 1] - u[:, 0]) > 3.0).all()
-    # moved by a rounding or two of an arrival (FP64: 2e-12 ns; float-float: 1e-9 bin)
-    jitter = rng.normal(size=n_ant) * (3e-12 if dtype is np.float64 else 1e-9 * dt)
+    # moved by a rounding or two of an arrival (FP64: 2e-12 ns; float-float: `spread` bins)
+    jitter = rng.normal(size=n_ant) * (3e-12 if dtype is np.float64 else spread * dt)
     return tracks, ant, (u.min(1) - K) * dt + jitter, int(np.argmin(u[0]))
 
 
-def forward_listing_adjoint(formalism, precision, medium, hills, dt, adjoint=True):
+def forward_listing_adjoint(formalism, precision, medium, hills, dt, adjoint=True, n_ant=1500, N=512, K=K,
+                            spread=1e-9):
     from paper_2309_03717_gb300 import c8r
-    n_ant, N = 1500, 512
     dtype = np.float64 if precision == "fp64" else np.float32
-    tracks, ant, t_start, first = on_the_edge(formalism, medium, hills, dt, n_ant, dtype)
+    tracks, ant, t_start, first = on_the_edge(formalism, medium, hills, dt, n_ant, dtype, K, spread)
     dev = to_device(tracks)
     p = c8r.RadioProcess(medium, ant, t_start, N, dt, formalism, precision)
     p.push(dev)
-    tr = p.traces().cpu().numpy()
-    _, bins, frac = p.arrivals(dev)
-    bins, frac = bins.cpu().numpy()[0, :, first], frac.cpu().numpy()[0, :, first]
+    below = p.traces()[:, :, K - 1].abs().amax(1).cpu().numpy() > 0
+    bins = p.arrivals(dev)[1].cpu().numpy()[0, :, first]
     ag = None
     if adjoint:
         # dL/dtrace in bin K - 1 only: an antenna has a gradient when its deposit is there
@@ -68,9 +69,8 @@ def forward_listing_adjoint(formalism, precision, medium, hills, dt, adjoint=Tru
         c8r.c8r_backward(p.ctx, dev, G, tg, ag, dn)
         ag = ag.cpu().numpy()
     p.close()
-    below = np.abs(tr[:, :, K - 1]).max(1) > 0
     assert 0.05 < below.mean() < 0.95  # both sides of the edge are reached
-    return tr, below, bins, frac, ag
+    return below, bins, ag
 
 
 @pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
@@ -78,6 +78,25 @@ def forward_listing_adjoint(formalism, precision, medium, hills, dt, adjoint=Tru
 @pytest.mark.parametrize("hills", [0.0, 150.0])
 @pytest.mark.parametrize("precision", ["mixed"])
 def test_forward_listing_and_adjoint_agree(precision, hills, medium, formalism):
-    _, below, bins, _, ag = forward_listing_adjoint(formalism, precision, medium, hills, 0.05)
+    below, bins, ag = forward_listing_adjoint(formalism, precision, medium, hills, 0.05)
     assert np.array_equal(bins == K - 1, below)
     assert np.array_equal(np.abs(ag).max(1) > 0, below)
+
+
+@pytest.mark.parametrize("medium", [SPHERE, RAY])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
+@pytest.mark.parametrize("hills", [0.0, 150.0])
+def test_forward_and_listing_agree_in_the_costlier_media(hills, formalism, precision, medium):
+    below, bins, _ = forward_listing_adjoint(formalism, precision, medium, hills, 0.05, adjoint=False)
+    assert np.array_equal(bins == K - 1, below)
+
+
+@pytest.mark.parametrize("medium", [synth.AIR_EXPONENTIAL, SPHERE, UNIFORM])
+@pytest.mark.parametrize("N,K", [((1 << 21) + 300, (1 << 21) + 9), ((1 << 23) + 5, (1 << 23) - 90), (1 << 24, (1 << 24) - 95)])
+def test_long_windows(N, K, medium):
+    """Windows beyond 2^21 bins, where the FP32 spacing of an arrival reaches a bin:
+    a tent of bins in front of the window's end."""
+    below, bins, _ = forward_listing_adjoint("zhs", "mixed", medium, 0.0, 0.05, adjoint=False, n_ant=24, N=N, K=K,
+                                             spread=1e-6)
+    assert np.array_equal(bins == K - 1, below)
