@@ -100,3 +100,27 @@ def test_long_windows(N, K, medium):
     below, bins, _ = forward_listing_adjoint("zhs", "mixed", medium, 0.0, 0.05, adjoint=False, n_ant=24, N=N, K=K,
                                              spread=1e-6)
     assert np.array_equal(bins == K - 1, below)
+
+
+@pytest.mark.parametrize("medium", [SPHERE, RAY, synth.AIR_EXPONENTIAL, UNIFORM])
+@pytest.mark.parametrize("z", [0.0, 5.0])
+def test_a_filtered_neighbour_changes_no_arrival(z, medium):
+    """The ZHS kernels take tracks two at a time: the arrivals of one are the same
+    bit for bit whether the other passes the filter or not."""
+    from paper_2309_03717_gb300 import c8r
+    n = 257
+    ant = synth.antennas_star(8, n_radii=3)[:17].copy()
+    ant[:, 2] = z
+    tracks = synth.make_tracks(n, 31, 40.0)
+    p = c8r.RadioProcess(medium, ant, synth.trace_start_ns(ant, 40.0) - 100.0, 4096, 0.2, "zhs", "mixed")
+    want = [x.cpu().numpy() for x in p.arrivals(to_device(tracks))]
+    assert (want[1] >= 0).any()
+    for first in (0, 1):
+        t = {f: x.copy() for f, x in tracks.items()}
+        t["q"][1 - first::2] = 0.0
+        t["x0"][1 - first::2] = np.nan
+        got = [x.cpu().numpy() for x in p.arrivals(to_device(t))]
+        assert (got[0][1 - first::2] == -1).all()
+        for g, w in zip(got, want):
+            assert np.array_equal(g[first::2], w[first::2])
+    p.close()
