@@ -136,7 +136,9 @@ void set_flat_array(MedParams& M, const double* pos_xyz, int n_ant) {
     const double* p = pos_xyz + 3 * (size_t)a;
     if (p[2] != z) return;
     // spherical Earth: the range of the curvature's series (PathZ)
-    if (M.kind == C8R_EXPONENTIAL_SPHERICAL && !(p[0] * p[0] + p[1] * p[1] < 0.01 * 2.0 * (M.R_E + z) * M.H)) return;
+    if (M.kind == C8R_EXPONENTIAL_SPHERICAL &&
+        !(p[0] * p[0] + p[1] * p[1] < 0.01 * 2.0 * (M.R_E + z) * M.H && 250.0 * M.H < M.R_E))
+      return;
   }
   // split as fill_antenna splits the antennas' z and exp(-z/H)
   M.flat = 1;

@@ -121,7 +121,7 @@ struct MedParams {
   int axis;
   float ax[3], kax_h[3], kax_l[3];
   // a flat antenna array (every antenna at one altitude z_a, exponential
-  // media; spherical Earth: and within 32 km of the origin, PathZ): z_a and exp(-z_a/H) as float-float, the same values the antenna
+  // media; spherical Earth: and within the range of its series, PathZ): z_a and exp(-z_a/H) as float-float, the same values the antenna
   // records hold, so that the quotient (E_e - E_a)/(z_a - z_e) of the
   // refractivity term, the same for every antenna, can be formed once per
   // track (OpsMixed::kFlat)

@@ -170,7 +170,10 @@ struct PathZ {};
 //   x_j (1 - k x_j + ...) and the bracket is -x_j [1 - x_j (k + 1/2) + x_j^2 (k + 1/6)]
 //   up to x^3/24 of it: 4e-8 for x_j < 0.01, which holds within 32 km of the origin
 //   (antennas: checked by the host, tracks: `small`).  Per track: w_j E_j h_j, and
-//   h as a linear function along the path for the bracket.
+//   h as a linear function along the path for the bracket.  k is taken at the sphere's
+//   radius and 2 k^2 x^2 dropped: the host asks for H < R_E/250 (the Earth: R_E/800)
+//   and `small` for altitude differences below 3 % of the radius, which keep both
+//   and the linear h below 6e-7 of the correction.
 template <>
 struct PathZ<C8R_EXPONENTIAL_SPHERICAL> {
   float2 weh[kSphNodes];
@@ -181,7 +184,8 @@ struct PathZ<C8R_EXPONENTIAL_SPHERICAL> {
     h0 = make_float2(div_ap(inv2H, M.RE_f + M.flat_zh), div_ap(inv2H, M.RE_f + M.flat_zh));
     h1 = make_float2(div_ap(inv2H, M.RE_f + mz.x) - h0.x, div_ap(inv2H, M.RE_f + mz.y) - h0.y);
     const float2 y = fma_rn(mx, mx, mul_rn(my, my));
-    small = fmaxf(y.x * h0.x, y.y * h0.y) < 0.01f;
+    small = fmaxf(y.x * h0.x, y.y * h0.y) < 0.01f &&
+            fmaxf(fabsf(dz.x), fabsf(dz.y)) < 0.03f * (M.RE_f + M.flat_zh);
 #pragma unroll
     for (int j = 0; j < kSphNodes; ++j) {
       const float f = 1.0f - (float)kSphSigma[j];

@@ -1,7 +1,8 @@
 """The series of the curved-ray and spherical-Earth propagators for flat antenna
 arrays: on the host, the ray series in FP64 against the exact solve inside the range
 the kernels take it in (T^2 b < 4e-3 and b < 1e-2), and on the GPU the arrivals
-against the quadrature's in media where the range ends: dense and steep atmospheres."""
+against the quadrature's in media where the range ends: dense and steep atmospheres,
+small spheres."""
 import numpy as np
 import pytest
 
@@ -76,7 +77,7 @@ def test_ray_series_inside_its_range():
 
 RAYS = [{"kind": "exponential_ray", "N0": N0, "H": H} for N0, H in ((3.25e-4, 8000.0), (0.01, 2000.0), (0.3, 1000.0),
                                                                     (0.4, 77.0), (0.78, 100.0))]
-SPHERES = [{"kind": "exponential_spherical", "N0": 3.25e-4, "H": 8000.0, "R_E": R} for R in (6.371e6, 2.0e6)]
+SPHERES = [{"kind": "exponential_spherical", "N0": 3.25e-4, "H": 8000.0, "R_E": R} for R in (6.371e6, 2.0e6, 2.0e4, 5.0e3)]
 
 
 @pytest.mark.gpu
