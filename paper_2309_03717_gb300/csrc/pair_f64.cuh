@@ -119,6 +119,9 @@ struct TrackD {
   double q;
 };
 
+template <int FORM>
+struct OpsF64Plain;
+
 template <int FORM, bool LIN = false>
 struct OpsF64 {
   using acc_t = double;
@@ -148,7 +151,10 @@ struct OpsF64 {
     t.q = t.T[fd::Q * kTileT + l];
   }
   static __device__ __forceinline__ bool live(const TrackD& t) { return t.q != 0.0; }
-  using MainTrack = TrackD;
+  // the adjoint's main pass: with the one-bin deposit (plain media only) the track
+  // as the forward pass holds it
+  using Plain = OpsF64Plain<FORM>;
+  using MainTrack = std::conditional_t<LIN, TrackD, typename Plain::AdjTrack>;
   using FwdTrack = TrackD;
   using FwdAnt = AntRec;
   static constexpr int kFwdThreads = kTileT;
@@ -166,9 +172,17 @@ struct OpsF64 {
 #pragma unroll
     for (int k = 0; k < 11; ++k) tg[k] = m.g[k];
   }
-  static __device__ __forceinline__ void load_main(const void* Tv, int l, const MedParams& M, TrackD& t) {
-    load(Tv, l, M, t);
+  static __device__ __forceinline__ void load_main(const void* Tv, int l, const MedParams& M, MainTrack& t) {
+    if constexpr (LIN) {
+      load(Tv, l, M, t);
+    } else {
+      t.T = Tv;
+      t.l = l;
+      Plain::load_fwd(Tv, l, M, t.t);
+    }
   }
+  template <class T, class = decltype(T::t)>
+  static __device__ __forceinline__ bool live(const T& t) { return Plain::live(t.t); }
   template <class Sink>
   static __device__ __forceinline__ void pair(const TrackD& t, const AntRec& A, const MedParams& M, Sink& out) {
     if constexpr (FORM == C8R_ENDPOINT)
@@ -320,7 +334,7 @@ struct OpsF64 {
       zhs(T, l, A, M, out);
   }
 
-  static __device__ __forceinline__ int adj_main(const TrackD& tr, const AntRec* p, const MedParams& M,
+  static __device__ __forceinline__ int adj_main(const MainTrack& tr, const AntRec* p, const MedParams& M,
                                                  const Acc4D* G, const PrefixFF* Gp, MainGrad& m, double ga[3],
                                                  double& dn) {
     const AntRec A = *p;
@@ -338,32 +352,50 @@ struct OpsF64 {
                                                           double&, int) {}
 
   // ZHS adjoint (bins of the interval ends held fixed; see the mixed path for
-  // the formulas): in FP64, times in ns, positions in m
-  static __device__ __forceinline__ void adj_zhs(const TrackD& tr, const AntRec& A, const MedParams& M,
+  // the formulas): in FP64, times in ns, positions in m.  The geometry and the
+  // interval are the forward pass's own: with the one-bin deposit OpsF64Plain's, so
+  // that an arrival within rounding of an edge is in one bin for both
+  static __device__ __forceinline__ void adj_zhs(const MainTrack& tr, const AntRec& A, const MedParams& M,
                                                  const Acc4D* G, const PrefixFF*, double tg[11], double ga[3],
                                                  double& dn) {
-    const double* T = tr.T;
+    const double* T = static_cast<const double*>(tr.T);
     const int l = tr.l;
     const double q = TF(fd::Q);
     if (q == 0.0) return;
     const int N = M.n_bins;
     const double b[3] = {TF(fd::BX), TF(fd::BY), TF(fd::BZ)};
-    const double x0 = TF(fd::X0), y0 = TF(fd::Y0), z0 = TF(fd::Z0);
-    const double x1 = TF(fd::X1), y1 = TF(fd::Y1), z1 = TF(fd::Z1);
     const double t0 = TF(fd::T0), t1 = TF(fd::T1);
     const double Em = TF(fd::EM);
-    GeoD gm;
-    geo_f64(M, A, 0.5 * (x0 + x1), 0.5 * (y0 + y1), 0.5 * (z0 + z1), Em, gm);
-    if (gm.R == 0.0) return;
-    const double c = b[0] * gm.rh[0] + b[1] * gm.rh[1] + b[2] * gm.rh[2];
-    const double Dm = 1.0 - gm.n_src * c;
     const double dte = t1 - t0;
-    const double tm = 0.5 * (t0 + t1);
-    const double tarr_rel = (tm - A.t_ref) + gm.n_avg * gm.R * M.inv_c_ns;
-    const double half = fabs(Dm) * dte / 2.0;
     const double dt = M.dt_ns;
-    const double u_lo = (tarr_rel - half) / dt, u_hi = (tarr_rel + half) / dt;
-    const double k_lo = floor(u_lo), k_hi = floor(u_hi);
+    GeoD gm;
+    double c, Dm, u_lo, u_hi, k_lo, k_hi;
+    if constexpr (LIN) {
+      geo_f64(M, A, 0.5 * (TF(fd::X0) + TF(fd::X1)), 0.5 * (TF(fd::Y0) + TF(fd::Y1)),
+              0.5 * (TF(fd::Z0) + TF(fd::Z1)), Em, gm);
+      if (gm.R == 0.0) return;
+      c = b[0] * gm.rh[0] + b[1] * gm.rh[1] + b[2] * gm.rh[2];
+      Dm = 1.0 - gm.n_src * c;
+      const double tm = 0.5 * (t0 + t1);
+      const double tarr_rel = (tm - A.t_ref) + gm.n_avg * gm.R * M.inv_c_ns;
+      const double half = fabs(Dm) * dte / 2.0;
+      u_lo = (tarr_rel - half) / dt;
+      u_hi = (tarr_rel + half) / dt;
+      k_lo = floor(u_lo);
+      k_hi = floor(u_hi);
+    } else {
+      typename Plain::Eval e;
+      if (!Plain::eval(tr.t, tr.t.p[0], A, M, e)) return;
+      typename Plain::Interval v;
+      Plain::interval(tr.t, e, N, v);
+      Plain::geometry(tr.t.p[0], A, e, gm);
+      c = e.c;
+      Dm = e.D;
+      u_lo = v.u_lo;
+      u_hi = v.u_hi;
+      k_lo = v.lo.k;
+      k_hi = v.one ? v.lo.k : v.hi.k;
+    }
     const double KA = q * kKzhs;
     double Av[3];
     for (int k = 0; k < 3; ++k) Av[k] = KA * (b[k] - c * gm.rh[k]) * dte / (gm.R * dt);
@@ -586,79 +618,81 @@ struct OpsF64 {
     tg[7] += (0.5 * dLdum + dLd_dtau) / dt;
   }
 
-  static __device__ __forceinline__ void adj(const TrackD& tr, const AntRec& A, const MedParams& M,
+  static __device__ __forceinline__ void adj(const MainTrack& tr, const AntRec& A, const MedParams& M,
                                              const Acc4D* G, double tg[11], double ga[3], double& dn) {
     static_assert(FORM == C8R_ENDPOINT, "adjoint is defined for the Endpoint formalism");
-    const double* T = tr.T;
+    const double* T = static_cast<const double*>(tr.T);
     const int l = tr.l;
     const double q = TF(fd::Q);
     if (q == 0.0) return;
     const int N = M.n_bins;
-    EndpointEvalD e;
-    endpoint_eval_f64(T, l, A, M, e);
-    if (!e.valid) return;
     const double b[3] = {TF(fd::BX), TF(fd::BY), TF(fd::BZ)};
     const double K = q * kKendpoint;
     const double dt_s = M.dt_ns * 1e-9;
     if constexpr (LIN) {
-      adj_lin(T, l, e, b, K, dt_s, M, G, tg, ga, dn);
-      return;
-    }
-    const double ka = floor(e.ua), kb = floor(e.ub);
-    const bool ina = ka >= 0.0 && ka < (double)N, inb = kb >= 0.0 && kb < (double)N;
-    const bool expo = M.kind == C8R_EXPONENTIAL;
-    double dd[3], db[3], dns;
-    if (e.branch == 0) {
-      for (int j = 0; j < 2; ++j) {
-        const bool in = j == 0 ? ina : inb;
-        if (!in) continue;
-        const int k = (int)(j == 0 ? ka : kb);
-        const double gv[3] = {G[k].x, G[k].y, G[k].z};
-        const GeoD& g = j == 0 ? e.g0 : e.g1;
-        const double* V = j == 0 ? e.V0 : e.V1;
-        const double c = b[0] * g.rh[0] + b[1] * g.rh[1] + b[2] * g.rh[2];
-        deposit_adjoint<double>(g.rh, V, c, j == 0 ? e.D0 : e.D1, g.R, g.n_src, gv, (j == 0 ? K : -K) / dt_s, dd,
-                                db, dns);
-        const double E = j == 0 ? e.E0 : e.E1;
-        for (int cc = 0; cc < 3; ++cc) {
-          tg[3 * j + cc] -= dd[cc];
-          ga[cc] += dd[cc];
-          tg[8 + cc] += db[cc];
-        }
-        if (expo) {
-          tg[3 * j + 2] += dns * (-M.N0 * E / M.H);
-          dn += dns * E;
-        } else {
-          dn += dns;
-        }
-      }
-      return;
-    }
-    if (ka == kb) return;
-    double gv[3];
-    for (int cc = 0; cc < 3; ++cc)
-      gv[cc] = (ina ? (&G[(int)ka].x)[cc] : 0.0) - (inb ? (&G[(int)kb].x)[cc] : 0.0);
-    const double c = b[0] * e.gm.rh[0] + b[1] * e.gm.rh[1] + b[2] * e.gm.rh[2];
-    deposit_adjoint<double>(e.gm.rh, e.Vm, c, e.Dm, e.gm.R, e.gm.n_src, gv, K / dt_s, dd, db, dns);
-    for (int cc = 0; cc < 3; ++cc) {
-      tg[cc] -= 0.5 * dd[cc];
-      tg[3 + cc] -= 0.5 * dd[cc];
-      ga[cc] += dd[cc];
-      tg[8 + cc] += db[cc];
-    }
-    if (expo) {
-      tg[2] += 0.5 * dns * (-M.N0 * e.Em / M.H);
-      tg[5] += 0.5 * dns * (-M.N0 * e.Em / M.H);
-      dn += dns * e.Em;
+      EndpointEvalD e;
+      endpoint_eval_f64(T, l, A, M, e);
+      if (e.valid) adj_lin(T, l, e, b, K, dt_s, M, G, tg, ga, dn);
     } else {
-      dn += dns;
+      // the forward pass's own evaluation, as in adj_zhs
+      const bool expo = M.kind == C8R_EXPONENTIAL;
+      double dd[3], db[3], dns;
+      typename Plain::Eval e[2];
+      if (!Plain::eval(tr.t, tr.t.p[0], A, M, e[0]) || !Plain::eval(tr.t, tr.t.p[1], A, M, e[1])) return;
+      if (fmin(fabs(e[0].D), fabs(e[1].D)) >= M.eps_Cd) {
+        for (int j = 0; j < 2; ++j) {
+          const int k = Plain::bin(e[j].u, N);
+          if (k < 0) continue;
+          const double gv[3] = {G[k].x, G[k].y, G[k].z};
+          const typename Plain::Point& p = tr.t.p[j];
+          GeoD g;
+          Plain::geometry(p, A, e[j], g);
+          deposit_adjoint<double>(g.rh, e[j].V, e[j].c, e[j].D, g.R, p.n, gv, (j == 0 ? K : -K) / dt_s, dd, db, dns);
+          for (int cc = 0; cc < 3; ++cc) {
+            tg[3 * j + cc] -= dd[cc];
+            ga[cc] += dd[cc];
+            tg[8 + cc] += db[cc];
+          }
+          if (expo) {
+            tg[3 * j + 2] += dns * (-M.N0 * p.E / M.H);
+            dn += dns * p.E;
+          } else {
+            dn += dns;
+          }
+        }
+        return;
+      }
+      typename Plain::Point pm;
+      typename Plain::Eval em;
+      typename Plain::Near v;
+      if (!Plain::near_arrivals(tr.t, T, l, A, M, pm, em, v)) return;
+      if (v.a.k == v.b.k) return;
+      double gv[3];
+      for (int cc = 0; cc < 3; ++cc)
+        gv[cc] = (v.a.bin >= 0 ? (&G[v.a.bin].x)[cc] : 0.0) - (v.b.bin >= 0 ? (&G[v.b.bin].x)[cc] : 0.0);
+      GeoD g;
+      Plain::geometry(pm, A, em, g);
+      deposit_adjoint<double>(g.rh, em.V, em.c, em.D, g.R, pm.n, gv, K / dt_s, dd, db, dns);
+      for (int cc = 0; cc < 3; ++cc) {
+        tg[cc] -= 0.5 * dd[cc];
+        tg[3 + cc] -= 0.5 * dd[cc];
+        ga[cc] += dd[cc];
+        tg[8 + cc] += db[cc];
+      }
+      if (expo) {
+        tg[2] += 0.5 * dns * (-M.N0 * pm.E / M.H);
+        tg[5] += 0.5 * dns * (-M.N0 * pm.E / M.H);
+        dn += dns * pm.E;
+      } else {
+        dn += dns;
+      }
     }
   }
 };
 
 // ---------------------------------------------------------------------------
-// The forward pass and the arrival listing in the plain media (uniform,
-// exponential) with the one-bin deposit.  Bound by the FP64 pipe, which on this
+// The forward pass, the arrival listing and the adjoint's geometry and bins in the
+// plain media (uniform, exponential) with the one-bin deposit.  Bound by the FP64 pipe, which on this
 // part runs at 1/64 of the FP32 rate, so the arithmetic is arranged for few FP64
 // operations: one reciprocal square root and two reciprocals per emission point
 // in place of a square root and five quotients, fused multiply-adds, what
@@ -784,6 +818,13 @@ struct OpsF64Plain {
   // arrival position u; false when the emission point sits on the antenna
   struct Eval {
     double V[3], D, iR, u;
+    double rh[3], c, R;  // (the adjoint's)
+  };
+  // a track for the adjoint's main pass, with its place in the staged tile
+  struct AdjTrack {
+    FwdTrack t;
+    const void* T;
+    int l;
   };
   static __device__ __forceinline__ bool eval(const FwdTrack& t, const Point& p, const AntRec& A, const MedParams& M,
                                               Eval& e) {
@@ -795,6 +836,11 @@ struct OpsF64Plain {
     R = __fma_rn(__fma_rn(-R, R, S), __dmul_rn(0.5, e.iR), R);
     const double rx = __dmul_rn(dx, e.iR), ry = __dmul_rn(dy, e.iR), rz = __dmul_rn(dz, e.iR);
     const double c = __fma_rn(t.bz, rz, __fma_rn(t.by, ry, __dmul_rn(t.bx, rx)));
+    e.rh[0] = rx;
+    e.rh[1] = ry;
+    e.rh[2] = rz;
+    e.c = c;
+    e.R = R;
     e.V[0] = __fma_rn(c, rx, -t.bx);
     e.V[1] = __fma_rn(c, ry, -t.by);
     e.V[2] = __fma_rn(c, rz, -t.bz);
@@ -802,6 +848,49 @@ struct OpsF64Plain {
     double r = p.r;
     if (M.kind != C8R_UNIFORM && !M.flat) r = refr(M, A.Ea, p.E, dz);
     e.u = __dmul_rn(__fma_rn(__fma_rn(r, R, R), M.inv_c_ns, __dsub_rn(p.t, A.t_ref)), M.inv_dt);
+    return true;
+  }
+
+  // the geometry of an evaluated point as the adjoint's chain rule takes it
+  static __device__ __forceinline__ void geometry(const Point& p, const AntRec& A, const Eval& e, GeoD& g) {
+    g.d[0] = __dsub_rn(A.x, p.x);
+    g.d[1] = __dsub_rn(A.y, p.y);
+    g.d[2] = __dsub_rn(A.z, p.z);
+    g.R = e.R;
+    for (int k = 0; k < 3; ++k) g.rh[k] = e.rh[k];
+    g.n_src = p.n;
+  }
+  static __device__ __forceinline__ int bin(double u, int N) { return floor_bin(u, N).bin; }
+  // ZHS: the ends of the arrival interval and their bins; `one`: in one bin
+  struct Interval {
+    double u_lo, u_hi, h;
+    FloorD lo, hi;
+    bool one;
+  };
+  static __device__ __forceinline__ void interval(const FwdTrack& t, const Eval& e, int N, Interval& v) {
+    v.h = __dmul_rn(fabs(e.D), t.hw);
+    v.u_lo = __dsub_rn(e.u, v.h);
+    v.u_hi = __dadd_rn(e.u, v.h);
+    v.lo = floor_bin(v.u_lo, N);
+    v.hi = floor_bin(v.u_hi, N);
+    // (also when |d|^2 overflows: u is NaN then, in no bin, and an interval of it
+    // must not go in as a box)
+    v.one = !(v.lo.k < v.hi.k);
+  }
+  // the adjoint of a near-Cherenkov pair: the midpoint and the bins of its linearised
+  // arrivals by near_pair's operations (near_pair itself, built on this, took 0.7 %
+  // longer per push); false when the midpoint sits on the antenna
+  struct Near {
+    FloorD a, b;
+  };
+  static __device__ __forceinline__ bool near_arrivals(const FwdTrack& t, const void* Tv, int l, const AntRec& A,
+                                                       const MedParams& M, Point& p, Eval& e, Near& v) {
+    const double* T = static_cast<const double*>(Tv);
+    midpoint(Tv, l, M, p);
+    if (!eval(t, p, A, M, e)) return false;
+    const double h = e.D * (0.5 * (TF(fd::T1) - TF(fd::T0)) * M.inv_dt);
+    v.a = floor_bin(e.u - h, M.n_bins);
+    v.b = floor_bin(e.u + h, M.n_bins);
     return true;
   }
 
@@ -830,12 +919,11 @@ struct OpsF64Plain {
     } else {
       Eval e;
       if (!eval(t, t.p[0], A, M, e)) return kDeferNone;
-      const double h = __dmul_rn(fabs(e.D), t.hw);
-      const double u_lo = __dsub_rn(e.u, h), u_hi = __dadd_rn(e.u, h);
-      const FloorD lo = floor_bin(u_lo, N), hi = floor_bin(u_hi, N);
-      // (also when |d|^2 overflows: u is NaN then, in no bin, and an interval of it
-      // must not go in as a box)
-      const bool one = !(lo.k < hi.k);
+      Interval v;
+      interval(t, e, N, v);
+      const double u_lo = v.u_lo, u_hi = v.u_hi, h = v.h;
+      const FloorD lo = v.lo, hi = v.hi;
+      const bool one = v.one;
       out.rec(one ? 2 : 3, u_lo, u_hi);
       const double s = -__dmul_rn(t.amp, e.iR);  // beta_perp = -V
       const double invW = one ? 1.0 : rcp_f64(__dadd_rn(h, h));
@@ -865,11 +953,11 @@ struct OpsF64Plain {
   static __device__ __forceinline__ void near_pair(const void* Tv, int l, const AntRec& A, const MedParams& M,
                                                    Sink& out) {
     const double* T = static_cast<const double*>(Tv);
-    const int N = M.n_bins;
     FwdTrack t;
     t.bx = TF(fd::BX);
     t.by = TF(fd::BY);
     t.bz = TF(fd::BZ);
+    const int N = M.n_bins;
     midpoint(Tv, l, M, t.p[0]);
     Eval e;
     if (!eval(t, t.p[0], A, M, e)) return;

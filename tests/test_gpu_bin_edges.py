@@ -76,7 +76,7 @@ def forward_listing_adjoint(formalism, precision, medium, hills, dt, adjoint=Tru
 @pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
 @pytest.mark.parametrize("medium", [synth.AIR_EXPONENTIAL, UNIFORM])
 @pytest.mark.parametrize("hills", [0.0, 150.0])
-@pytest.mark.parametrize("precision", ["mixed"])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_forward_listing_and_adjoint_agree(precision, hills, medium, formalism):
     below, bins, ag = forward_listing_adjoint(formalism, precision, medium, hills, 0.05)
     assert np.array_equal(bins == K - 1, below)
