@@ -180,11 +180,13 @@ int c8r_set_medium_spherical(c8r_ctx* ctx, double N0, double scale_height_m, dou
  * [t_start_ns[a] + k dt_ns, t_start_ns[a] + (k + 1) dt_ns).  formalism selects
  * Endpoint or ZHS; precision selects C8R_FP64 or C8R_MIXED.  Allocates (and
  * zeroes) the context's trace accumulator, one (x, y, z) element per antenna and
- * bin, FP64 (C8R_FP64) or FP32 (C8R_MIXED), 32 or 16 bytes per element.  ZHS
- * keeps a second row per antenna (box edges), and 1 to 16 copies of the whole
+ * bin, FP64 (C8R_FP64) or FP32 (C8R_MIXED), 32 or 16 bytes per element.  Mixed
+ * ZHS keeps a second row per antenna (box edges), and 1 to 16 copies of the whole
  * accumulator are kept, more for fewer antennas (up to 192 MB and a quarter of the
  * device's free memory in all), which the fetch sums; a push uses as many of them
- * as its tracks pay for.  Replaces any previous antenna set and discards its
+ * as its tracks pay for.  FP64 ZHS allocates box edges of the accumulator's size at
+ * the first push that has a use for them (one-bin deposit in the uniform or flat
+ * exponential medium) where a quarter of the free memory holds them.  Replaces any previous antenna set and discards its
  * traces (a call with the same
  * n_ant, n_bins, dt_ns, formalism and precision keeps the device memory and
  * only replaces the table, so moving an array between steps is cheap).  EINVAL on n_ant < 1,

@@ -270,6 +270,10 @@ struct c8r_ctx {
   // copy counts as used for good
   int copies_used = 1;
   bool copies_all = false;
+  // FP64 ZHS: box edges, [copies][n_ant][n_bins], from the first push with boxes on
+  // where there is room, and whether they may hold any (as copies_used)
+  void* d_edges = nullptr;
+  bool edges_used = false, edges_refused = false;
   int floor_copies = 1;  // that every push uses (floor_replicas)
   void* d_stage = nullptr;   // [n_ant][3][n_bins] staging for copies to host
   void* d_gbm = nullptr;     // backward: dL/dtraces, bin-major [n_ant][n_bins] accumulator elements
@@ -385,13 +389,38 @@ int copies_in_use(c8r_ctx* c, cudaStream_t st) {
   if (capturing(st)) c->copies_all = true;
   return c->copies_all ? c->shape.replicas : c->copies_used;
 }
+// and its box edges, if they may hold any (after copies_in_use)
+void* edges_in_use(c8r_ctx* c) { return c->edges_used || c->copies_all ? c->d_edges : nullptr; }
 
 // zero the accumulator
 cudaError_t zero_acc(c8r_ctx* c, cudaStream_t st) {
   const int n = copies_in_use(c, st);
-  const cudaError_t e = cudaMemsetAsync(c->d_acc, 0, c->acc_bytes / c->shape.replicas * n, st);
-  if (e == cudaSuccess) c->copies_used = 1;
+  const size_t bytes = c->acc_bytes / c->shape.replicas * n;
+  cudaError_t e = cudaMemsetAsync(c->d_acc, 0, bytes, st);
+  if (e == cudaSuccess && edges_in_use(c)) e = cudaMemsetAsync(c->d_edges, 0, bytes, st);
+  if (e != cudaSuccess) return e;
+  c->copies_used = 1;
+  c->edges_used = false;
   return e;
+}
+
+// whether a push on st can add boxes by their edges: they take as much memory as
+// the accumulator, which on a device that is nearly full (a quarter of what is free,
+// as for its copies) the traces do not need.  Not from the middle of a capture, nor
+// once a captured fetch may be about that knows nothing of them
+bool ensure_edges(c8r_ctx* c, cudaStream_t st) {
+  if (c->d_edges || c->edges_refused || c->copies_all || capturing(st)) return c->d_edges != nullptr;
+  size_t mem_free = 0, mem_total = 0;
+  cudaError_t e = cudaMemGetInfo(&mem_free, &mem_total);
+  if (e == cudaSuccess && c->acc_bytes <= mem_free / 4) e = dev_malloc(&c->d_edges, c->acc_bytes);
+  if (e == cudaSuccess && c->d_edges) e = cudaMemsetAsync(c->d_edges, 0, c->acc_bytes, st);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    if (c->d_edges) cudaFree(c->d_edges);
+    c->d_edges = nullptr;
+  }
+  c->edges_refused = !c->d_edges;
+  return c->d_edges != nullptr;
 }
 
 // a new antenna layout or medium: earlier votes no longer apply
@@ -432,6 +461,9 @@ int rebuild_tables(c8r_ctx* c) {
 void free_antenna_state(c8r_ctx* c) {
   if (c->d_ants) cudaFree(c->d_ants);
   if (c->d_acc) cudaFree(c->d_acc);
+  if (c->d_edges) cudaFree(c->d_edges);
+  c->d_edges = nullptr;
+  c->edges_used = c->edges_refused = false;
   if (c->d_stage) cudaFree(c->d_stage);
   if (c->d_gbm) cudaFree(c->d_gbm);
   c->d_gbm = nullptr;
@@ -642,8 +674,10 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
     c->pos.assign(pos, pos + 3 * (size_t)n_ant);
     c->t_start.assign(t_start, t_start + n_ant);
     cudaError_t e = cudaMemset(c->d_acc, 0, c->acc_bytes);
+    if (e == cudaSuccess && c->d_edges) e = cudaMemset(c->d_edges, 0, c->acc_bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, "trace reset");
     c->copies_used = 1;
+    c->edges_used = false;
     c->pushed = 0;
     cudaMemset(c->d_kept, 0, sizeof(unsigned long long));
     return rebuild_tables(c);
@@ -665,7 +699,7 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   c->shape.a_tile = want < n_ant ? want : n_ant;
   c->shape.waves = c->user_waves > 0 ? c->user_waves : kDefaultWaves;
   c->trace_bytes = (size_t)n_ant * 3 * n_bins * (precision == C8R_FP64 ? 8 : 4);
-  c->acc_bytes = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(formalism);
+  c->acc_bytes = (size_t)n_ant * n_bins * acc_elem_bytes(precision) * acc_rows(precision, formalism);
   c->shape.replicas = acc_replicas(precision, formalism, n_ant, n_bins, c->shape.a_tile, c->sm_count);
   c->floor_copies = floor_replicas(precision, formalism, n_ant, n_bins, c->shape.a_tile, c->sm_count);
   // the copies are not needed to hold the traces: on a device that is nearly full they
@@ -738,7 +772,16 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
     shape.a_tile = push_a_tile(shape.a_tile, (chunk + kTileT - 1) / kTileT, c->n_ant, c->precision, c->formalism,
                                c->sm_count);
   const int floor_copies = c->floor_copies < shape.replicas ? c->floor_copies : shape.replicas;
-  shape.replicas = push_replicas(c->precision, shape.replicas, n, c->n_bins, acc_rows(c->formalism));
+  const bool boxes = c->precision == C8R_FP64 && c->formalism == C8R_ZHS && !lin &&
+                     (c->med_kind == C8R_UNIFORM || c->med_kind == C8R_EXPONENTIAL);
+  int rows = acc_rows(c->precision, c->formalism);
+  if (boxes && ensure_edges(c, st)) {
+    rows = 2;
+    shape.edge_off = (static_cast<char*>(c->d_edges) - static_cast<char*>(c->d_acc)) /
+                     (int64_t)acc_elem_bytes(C8R_FP64);
+    c->edges_used = true;
+  }
+  shape.replicas = push_replicas(c->precision, shape.replicas, n, c->n_bins, rows);
   if (shape.replicas < floor_copies) shape.replicas = floor_copies;
   if (capturing(st)) c->copies_all = true;
   if (shape.replicas > c->copies_used) c->copies_used = shape.replicas;
@@ -782,10 +825,14 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
 constexpr size_t kFusedClear = (size_t)4 << 20;
 static cudaError_t fetch_acc(c8r_ctx* c, void* dst, bool clear, cudaStream_t st) {
   const int n = copies_in_use(c, st);
-  const bool fused = clear && c->acc_bytes / c->shape.replicas * n <= kFusedClear;
+  void* edges = edges_in_use(c);
+  const bool fused = clear && c->acc_bytes / c->shape.replicas * n * (edges ? 2 : 1) <= kFusedClear;
   cudaError_t e = launch_acc_to_traces(c->precision, c->d_acc, c->n_ant, c->n_bins,
-                                       acc_rows(c->formalism), dst, false, fused, st, n);
-  if (e == cudaSuccess && fused) c->copies_used = 1;
+                                       acc_rows(c->precision, c->formalism), dst, false, fused, st, n, edges);
+  if (e == cudaSuccess && fused) {
+    c->copies_used = 1;
+    c->edges_used = false;
+  }
   if (e == cudaSuccess && clear && !fused) e = zero_acc(c, st);
   return e;
 }

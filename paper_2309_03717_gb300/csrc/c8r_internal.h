@@ -14,6 +14,7 @@ struct FwdShape {
   int a_tile;  // antennas per CTA: each thread holds one staged track and loops over them
   int waves;   // target number of waves (all CTAs resident at once) per launch
   int replicas = 1;  // copies of the accumulator (acc_replicas)
+  int64_t edge_off = 0;  // FP64: accumulator elements from a row to its box edges, 0 without them
 };
 
 // SoA track pointers of the caller, already offset to a chunk
@@ -25,8 +26,12 @@ struct TrackPtrs {
 size_t tile_bytes(int precision);
 // bytes of one accumulator element (one bin of one antenna: x, y, z, pad)
 inline size_t acc_elem_bytes(int precision) { return precision == C8R_FP64 ? 32 : 16; }
-// accumulator rows per antenna: ZHS adds a row of box edges
+// accumulator rows per antenna, box edges included (ZHS)
 inline int acc_rows(int formalism) { return formalism == C8R_ZHS ? 2 : 1; }
+// and of the accumulator itself: the FP64 path keeps the edges apart, in memory
+// that the first push with boxes allocates where there is room (only the one-bin
+// deposit of the plain media has boxes; without the edges they go in bin by bin)
+inline int acc_rows(int precision, int formalism) { return precision == C8R_MIXED ? acc_rows(formalism) : 1; }
 // copies of the accumulator the forward kernel spreads its reductions over (CTA
 // range r adds into copy r % replicas; the fetch sums them).  Most reductions go
 // into the few bins per antenna that the pulse arrives in, a few lines of L2
@@ -120,11 +125,12 @@ inline int push_a_tile(int a_tile, int64_t n_tiles, int n_ant, int precision, in
   return a;
 }
 // accumulator [replicas][n_ant][rows][n_bins] -> traces [n_ant][3][n_bins]: the
-// copies are summed; with rows == 2 the second row (box edges) is integrated over
-// the bins and added; add adds into out; clear zeroes the accumulator (the copies
-// given) as it is read.  FP32 only for add or replicas > 1
+// copies are summed; box edges (the second row with rows == 2, or `edges`
+// [replicas][n_ant][n_bins]) are integrated over the bins and added; add adds into
+// out (FP32 only); clear zeroes the accumulator and the edges (the copies given) as
+// they are read
 cudaError_t launch_acc_to_traces(int precision, void* acc, int n_ant, int n_bins, int rows, void* out, bool add,
-                                 bool clear, cudaStream_t st, int replicas = 1);
+                                 bool clear, cudaStream_t st, int replicas = 1, void* edges = nullptr);
 
 // dL/dtraces [n_ant][3][n_bins] -> bin-major [n_ant][n_bins] accumulator elements
 cudaError_t launch_traces_to_bin_major(int precision, const void* g, int n_ant, int n_bins, void* out,

@@ -108,6 +108,7 @@ struct FwdArgs {
   MedParams M;
   int replicas = 1;            // accumulator copies; CTA range r adds into copy r % replicas
   int64_t replica_stride = 0;  // accumulator elements per copy
+  int64_t edge_off = 0;        // FwdShape::edge_off
 };
 
 struct BwdArgs {
@@ -168,22 +169,24 @@ struct GlobalSink<float> {
 };
 template <>
 struct GlobalSink<double> {
+  static constexpr bool kRecords = false;
   Acc4D* row;
   int n;
-  __device__ __forceinline__ void dep(int k, double x, double y, double z) {
+  int64_t edge = 0;  // elements from the row to its box edges, 0: none kept
+  __device__ __forceinline__ void dep(int k, double x, double y, double z) const {
     atomicAdd(&row[k].x, x);
     atomicAdd(&row[k].y, y);
     atomicAdd(&row[k].z, z);
   }
-  // the same vector into bins k0..k1, as GlobalSink<float> adds it
+  // the same vector into bins k0..k1: as GlobalSink<float> adds it, or bin by bin
   __device__ __forceinline__ void dep_box(int k0, int k1, double x, double y, double z) {
-    if (k1 - k0 < 2) {
-      dep(k0, x, y, z);
-      if (k1 > k0) dep(k1, x, y, z);
+    if (k1 - k0 < 2 || edge == 0) {
+      for (int k = k0; k <= k1; ++k) dep(k, x, y, z);
       return;
     }
-    dep(n + k0, x, y, z);
-    if (k1 + 1 < n) dep(n + k1 + 1, -x, -y, -z);
+    const GlobalSink<double> e{row + edge, n};
+    e.dep(k0, x, y, z);
+    if (k1 + 1 < n) e.dep(k1 + 1, -x, -y, -z);
   }
   __device__ __forceinline__ void rec(int, ff, ff) {}
   __device__ __forceinline__ void rec(int, double, double) {}
@@ -278,7 +281,7 @@ template <class Ops>
 __device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* bar, const typename Ops::FwdAnt* ant_s,
                              typename AccOf<typename Ops::acc_t>::type* acc_row0, int n_here,
                              const unsigned char* src, int64_t t_begin, int64_t t_end, int64_t& it,
-                             const MedParams& M) {
+                             const MedParams& M, int64_t edge_off = 0) {
   using acc_t = typename Ops::acc_t;
   const int tid = threadIdx.x;
   const int nthr = blockDim.x;
@@ -324,6 +327,7 @@ __device__ bool stream_range(unsigned char* smem, const FwdLayout& L, uint64_t* 
 #pragma unroll 1
           for (int ant = 0; ant < n_here; ++ant) {
             GlobalSink<acc_t> sink{acc_row0 + (size_t)ant * row_stride, N};
+            if constexpr (Ops::kPrec == C8R_FP64) sink.edge = edge_off;
             const int code = Ops::pair_main(tr, ant_s + ant, smem + st * L.stage_bytes, l, M, sink);
             if constexpr (Ops::kDefers) aside.add(code, ant);
           }
@@ -440,7 +444,7 @@ __global__ void __launch_bounds__(Ops::kFwdThreads, Ops::kMinBlocks) k_forward(c
   acc4* row0 = static_cast<acc4*>(a.acc) + (size_t)ant0 * a.M.n_bins * Ops::kAccRows +
                (size_t)(range % a.replicas) * a.replica_stride;
   if (!stream_range<Ops>(smem, L, bar, ant_s, row0, n_here, static_cast<const unsigned char*>(a.tiles), t_begin,
-                         t_end, it, a.M)) {
+                         t_end, it, a.M, a.edge_off)) {
     if (tid == 0) atomicExch(a.err, kErrWaitTimeout);
   }
 }

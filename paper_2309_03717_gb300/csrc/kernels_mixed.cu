@@ -119,7 +119,7 @@ __device__ __forceinline__ void cta_exclusive_scan_ff3(const ff v[3], ff excl[3]
   }
 }
 
-// accumulator with a row of box edges [n_ant][2][n_bins] float4 -> traces:
+// accumulator and box edges, rows of n_bins elements `row` apart -> traces:
 // out[k] = direct[k] + sum_{j <= k} edge[j], each summed over the `replicas`
 // copies of the accumulator (`stride` elements apart; zeroed if `clear`).  A
 // cluster of up to kFetchCluster CTAs has an antenna, each CTA kScanT x kFetchBins
@@ -179,8 +179,10 @@ __device__ __forceinline__ void sum_before8(const S (*t)[8], int n, S before[3],
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(typename AccOf<T>::type* acc, int n_bins, T* out,
-                                                               bool add, bool clear, int replicas, int64_t stride) {
+__global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(typename AccOf<T>::type* acc,
+                                                               typename AccOf<T>::type* edges, int64_t row, int n_bins,
+                                                               T* out, bool add, bool clear, int replicas,
+                                                               int64_t stride) {
   namespace cg = cooperative_groups;
   using S = typename SumOf<T>::type;
   using acc4 = typename AccOf<T>::type;
@@ -192,7 +194,8 @@ __global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(typename AccOf<T>
   if (threadIdx.x < 6 * kFetchCluster) cta_tot[0][0][threadIdx.x] = S{};  // absent CTAs count as zero
   cluster.sync();
   const int a = blockIdx.x / n_cta;
-  acc4* direct = acc + (size_t)a * 2 * n_bins;
+  acc4* direct = acc + a * row;
+  acc4* edge = edges + a * row;
   T* o = out + (size_t)a * 3 * n_bins;
   S carry[3] = {S{}, S{}, S{}};
   int buf = 0;
@@ -208,8 +211,8 @@ __global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(typename AccOf<T>
 #pragma unroll
       for (int b = 0; b < kFetchBins; ++b) {
         if (k0 + b >= n_bins) continue;
-        const acc4* p = direct + k0 + b + r * stride;
-        const acc4 u = p[0], w = p[n_bins];
+        const int64_t i = k0 + b + r * stride;
+        const acc4 u = direct[i], w = edge[i];
         d[b][0] = ff_add_f(d[b][0], u.x);
         d[b][1] = ff_add_f(d[b][1], u.y);
         d[b][2] = ff_add_f(d[b][2], u.z);
@@ -223,7 +226,7 @@ __global__ void __launch_bounds__(kScanT) k_acc_scan_to_traces(typename AccOf<T>
       for (int r = 0; r < replicas; ++r)
 #pragma unroll
         for (int b = 0; b < kFetchBins; ++b)
-          if (k0 + b < n_bins) direct[k0 + b + r * stride] = direct[n_bins + k0 + b + r * stride] = zero;
+          if (k0 + b < n_bins) direct[k0 + b + r * stride] = edge[k0 + b + r * stride] = zero;
     }
     // the edges before this thread's bins: of the lanes before it, of the warps
     // before its own, and of the CTAs before its own
@@ -304,11 +307,11 @@ __global__ void k_acc_to_traces_f64(Acc4D* acc, int64_t n_ant_bins, int n_bins, 
 }
 
 cudaError_t launch_acc_to_traces(int precision, void* acc, int n_ant, int n_bins, int rows, void* out, bool add,
-                                 bool clear, cudaStream_t st, int replicas) {
+                                 bool clear, cudaStream_t st, int replicas, void* edges) {
   const int64_t n = (int64_t)n_ant * n_bins;
   if (n <= 0) return cudaSuccess;
   const int64_t stride = n * rows;  // accumulator elements per copy
-  if (rows == 2) {
+  if (rows == 2 || edges) {
     // a cluster of CTAs per antenna, as many as one round over the window needs
     int n_cta = 1;
     while (n_cta < kFetchCluster && n_cta * kScanT * kFetchBins < n_bins) n_cta *= 2;
@@ -322,11 +325,14 @@ cudaError_t launch_acc_to_traces(int precision, void* acc, int n_ant, int n_bins
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    const int64_t row = (int64_t)n_bins * rows;
     if (precision == C8R_FP64)
-      return cudaLaunchKernelEx(&cfg, k_acc_scan_to_traces<double>, static_cast<Acc4D*>(acc), n_bins,
-                                static_cast<double*>(out), add, clear, replicas, stride);
-    return cudaLaunchKernelEx(&cfg, k_acc_scan_to_traces<float>, static_cast<float4*>(acc), n_bins,
-                              static_cast<float*>(out), add, clear, replicas, stride);
+      return cudaLaunchKernelEx(&cfg, k_acc_scan_to_traces<double>, static_cast<Acc4D*>(acc),
+                                static_cast<Acc4D*>(edges), row, n_bins, static_cast<double*>(out), add, clear,
+                                replicas, stride);
+    return cudaLaunchKernelEx(&cfg, k_acc_scan_to_traces<float>, static_cast<float4*>(acc),
+                              static_cast<float4*>(acc) + n_bins, row, n_bins, static_cast<float*>(out), add, clear,
+                              replicas, stride);
   }
   if (precision == C8R_FP64) {
     k_acc_to_traces_f64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(static_cast<Acc4D*>(acc), n, n_bins,

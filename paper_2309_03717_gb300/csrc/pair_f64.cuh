@@ -139,7 +139,7 @@ struct OpsF64 {
   static constexpr bool kFastBins = false;
   static constexpr int kBwdMinBlocks = 2;
   static constexpr int kBwdGridBlocks = 2;
-  static constexpr int kAccRows = FORM == C8R_ZHS ? 2 : 1;  // as the plain media's kernels (OpsF64Plain)
+  static constexpr int kAccRows = 1;      // no box deposits
 
   using Ant = AntRec;
   static __device__ __forceinline__ void stage_ant(AntRec* p, const AntRec& A, const MedParams&) { *p = A; }
@@ -745,7 +745,7 @@ struct OpsF64Plain {
   static constexpr int kFwdThreads = kTileT;
   static constexpr bool kDefers = FORM == C8R_ENDPOINT;  // near-Cherenkov pairs, as OpsF64
   static constexpr bool kFastBins = false;
-  static constexpr int kAccRows = FORM == C8R_ZHS ? 2 : 1;  // ZHS: box edges in the second row
+  static constexpr int kAccRows = 1;  // (ZHS: the box edges lie apart, FwdShape::edge_off)
 
   // an emission point of the track
   struct Point {
@@ -1013,8 +1013,9 @@ cudaError_t forward_f64(int formalism, const void* tiles, int64_t n_tiles, const
     using O = decltype(ops);
     a.replicas = shape.replicas > 1 ? shape.replicas : 1;
     a.replica_stride = (int64_t)n_ant * M.n_bins * O::kAccRows;
-    const int64_t ctas =
-        forward_grid(a, shape, sm_count * forward_blocks_per_sm<O>(shape.a_tile), sizeof(Acc4D) * O::kAccRows);
+    a.edge_off = shape.edge_off;
+    const int64_t ctas = forward_grid(a, shape, sm_count * forward_blocks_per_sm<O>(shape.a_tile),
+                                      sizeof(Acc4D) * (shape.edge_off ? 2 : 1));
     return launch_forward_ops<O>(a, ctas, st);
   };
   if constexpr (!LIN) {
