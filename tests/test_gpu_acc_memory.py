@@ -1,6 +1,8 @@
 """The accumulator's memory: what a layout takes of the device, and that the copies
 and the row of box edges are a help, not a need: without room for them the traces
 are the same."""
+import json
+
 import numpy as np
 import pytest
 
@@ -157,4 +159,26 @@ def test_captured_pushes_and_fetches(formalism, precision):
     push.replay()
     fetch.replay()
     assert rel_l2(out.double().cpu().numpy(), some) < tol
+    p.close()
+
+
+def test_moving_antennas_zeroes_the_copies_in_use(tmp_path):
+    """64 antennas x 2048 bins keep 16 copies of 2 MB, of which a push of 3000 tracks
+    uses two: moving the antennas afterwards zeroes those (and a few counters)."""
+    from torch.profiler import ProfilerActivity, profile
+    from paper_2309_03717_gb300.c8r import RadioProcess
+    ant = synth.antennas_star(8, n_radii=8)
+    p = RadioProcess(synth.AIR_EXPONENTIAL, ant, synth.trace_start_ns(ant), 2048, 0.2, "endpoint", "mixed")
+    tracks = to_device(synth.make_tracks(3000, 5, 0.0))
+    for _ in range(2):  # (the profiler's first session can come up empty)
+        p.push(tracks)
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            p.set_antenna_positions(p.ant_xyz + [0.5, 0.0, 0.0])
+            torch.cuda.synchronize()
+    path = str(tmp_path / "trace.json")
+    prof.export_chrome_trace(path)
+    sets = [e["args"]["bytes"] for e in json.load(open(path))["traceEvents"] if e.get("cat") == "gpu_memset"]
+    assert sets and max(sets) == 2 * 64 * 2048 * 16, sets
+    assert not p.traces().any()
     p.close()
