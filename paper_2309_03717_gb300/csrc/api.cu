@@ -266,14 +266,16 @@ struct c8r_ctx {
   size_t acc_bytes = 0;      // of all copies (shape.replicas of them)
   // copies that may hold deposits (the first copies_used; the others are zero),
   // which is what a fetch sums and a reset zeroes.  Work captured into a CUDA
-  // graph runs when the host does not see it: once anything was captured, every
-  // copy counts as used for good
-  int copies_used = 1;
-  bool copies_all = false;
+  // graph runs when the host does not see it: the copies of captured pushes
+  // (copies_replayed) count as used for good, and a captured fetch or reset takes
+  // every copy, whatever the pushes before its replays will have used
+  int copies_used = 1, copies_replayed = 1;
   // FP64 ZHS: box edges, [copies][n_ant][n_bins], from the first push with boxes on
   // where there is room, and whether they may hold any (as copies_used)
   void* d_edges = nullptr;
   bool edges_used = false, edges_refused = false;
+  bool edges_replayed = false;   // by captured pushes
+  bool fetch_captured = false;   // (or a reset) on the present accumulator
   int floor_copies = 1;  // that every push uses (floor_replicas)
   void* d_stage = nullptr;   // [n_ant][3][n_bins] staging for copies to host
   void* d_gbm = nullptr;     // backward: dL/dtraces, bin-major [n_ant][n_bins] accumulator elements
@@ -384,23 +386,35 @@ void form_fetch(c8r_ctx* c, cudaStream_t st) {
   c->form_pending = true;
 }
 
-// copies of the accumulator that work enqueued on st has to reckon with
-int copies_in_use(c8r_ctx* c, cudaStream_t st) {
-  if (capturing(st)) c->copies_all = true;
-  return c->copies_all ? c->shape.replicas : c->copies_used;
+// what a fetch or a reset enqueued on st has to reckon with: copies of the
+// accumulator, and its box edges if they may hold any
+struct InUse {
+  int copies;
+  void* edges;
+  bool replayed;  // the work runs from a graph
+};
+InUse acc_in_use(c8r_ctx* c, cudaStream_t st) {
+  if (capturing(st)) {
+    c->fetch_captured = true;
+    return {c->shape.replicas, c->d_edges, true};
+  }
+  return {c->copies_used > c->copies_replayed ? c->copies_used : c->copies_replayed,
+          c->edges_used || c->edges_replayed ? c->d_edges : nullptr, false};
 }
-// and its box edges, if they may hold any (after copies_in_use)
-void* edges_in_use(c8r_ctx* c) { return c->edges_used || c->copies_all ? c->d_edges : nullptr; }
+// the accumulator has been zeroed
+void acc_zeroed(c8r_ctx* c, const InUse& u) {
+  if (u.replayed) return;
+  c->copies_used = 1;
+  c->edges_used = false;
+}
 
 // zero the accumulator
 cudaError_t zero_acc(c8r_ctx* c, cudaStream_t st) {
-  const int n = copies_in_use(c, st);
-  const size_t bytes = c->acc_bytes / c->shape.replicas * n;
+  const InUse u = acc_in_use(c, st);
+  const size_t bytes = c->acc_bytes / c->shape.replicas * u.copies;
   cudaError_t e = cudaMemsetAsync(c->d_acc, 0, bytes, st);
-  if (e == cudaSuccess && edges_in_use(c)) e = cudaMemsetAsync(c->d_edges, 0, bytes, st);
-  if (e != cudaSuccess) return e;
-  c->copies_used = 1;
-  c->edges_used = false;
+  if (e == cudaSuccess && u.edges) e = cudaMemsetAsync(u.edges, 0, bytes, st);
+  if (e == cudaSuccess) acc_zeroed(c, u);
   return e;
 }
 
@@ -409,7 +423,7 @@ cudaError_t zero_acc(c8r_ctx* c, cudaStream_t st) {
 // as for its copies) the traces do not need.  Not from the middle of a capture, nor
 // once a captured fetch may be about that knows nothing of them
 bool ensure_edges(c8r_ctx* c, cudaStream_t st) {
-  if (c->d_edges || c->edges_refused || c->copies_all || capturing(st)) return c->d_edges != nullptr;
+  if (c->d_edges || c->edges_refused || c->fetch_captured || capturing(st)) return c->d_edges != nullptr;
   size_t mem_free = 0, mem_total = 0;
   cudaError_t e = cudaMemGetInfo(&mem_free, &mem_total);
   if (e == cudaSuccess && c->acc_bytes <= mem_free / 4) e = dev_malloc(&c->d_edges, c->acc_bytes);
@@ -463,7 +477,7 @@ void free_antenna_state(c8r_ctx* c) {
   if (c->d_acc) cudaFree(c->d_acc);
   if (c->d_edges) cudaFree(c->d_edges);
   c->d_edges = nullptr;
-  c->edges_used = c->edges_refused = false;
+  c->edges_used = c->edges_refused = c->edges_replayed = c->fetch_captured = false;
   if (c->d_stage) cudaFree(c->d_stage);
   if (c->d_gbm) cudaFree(c->d_gbm);
   c->d_gbm = nullptr;
@@ -710,8 +724,7 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   }
   while (c->shape.replicas > 1 && c->acc_bytes * c->shape.replicas > mem_free / 4) c->shape.replicas /= 2;
   c->acc_bytes *= c->shape.replicas;
-  c->copies_used = 1;
-  c->copies_all = false;
+  c->copies_used = c->copies_replayed = 1;
   cudaError_t e = dev_malloc(&c->d_ants, sizeof(AntRec) * n_ant);
   if (e == cudaSuccess) e = dev_malloc(&c->d_acc, c->acc_bytes);
   if (e == cudaSuccess) e = cudaMemset(c->d_acc, 0, c->acc_bytes);
@@ -778,12 +791,12 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
     rows = 2;
     shape.edge_off = (static_cast<char*>(c->d_edges) - static_cast<char*>(c->d_acc)) /
                      (int64_t)acc_elem_bytes(C8R_FP64);
-    c->edges_used = true;
+    (capturing(st) ? c->edges_replayed : c->edges_used) = true;
   }
   shape.replicas = push_replicas(c->precision, shape.replicas, n, c->n_bins, rows);
   if (shape.replicas < floor_copies) shape.replicas = floor_copies;
-  if (capturing(st)) c->copies_all = true;
-  if (shape.replicas > c->copies_used) c->copies_used = shape.replicas;
+  int& used = capturing(st) ? c->copies_replayed : c->copies_used;
+  if (shape.replicas > used) used = shape.replicas;
   for (int64_t off = 0; off < n; off += chunk) {
     const int64_t m = (n - off) < chunk ? (n - off) : chunk;
     TrackPtrs p = offset_tracks(t, off);
@@ -823,15 +836,12 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
 // reads and writes in turn
 constexpr size_t kFusedClear = (size_t)4 << 20;
 static cudaError_t fetch_acc(c8r_ctx* c, void* dst, bool clear, cudaStream_t st) {
-  const int n = copies_in_use(c, st);
-  void* edges = edges_in_use(c);
-  const bool fused = clear && c->acc_bytes / c->shape.replicas * n * (edges ? 2 : 1) <= kFusedClear;
+  const InUse u = acc_in_use(c, st);
+  const bool fused = clear && c->acc_bytes / c->shape.replicas * u.copies * (u.edges ? 2 : 1) <= kFusedClear;
   cudaError_t e = launch_acc_to_traces(c->precision, c->d_acc, c->n_ant, c->n_bins,
-                                       acc_rows(c->precision, c->formalism), dst, false, fused, st, n, edges);
-  if (e == cudaSuccess && fused) {
-    c->copies_used = 1;
-    c->edges_used = false;
-  }
+                                       acc_rows(c->precision, c->formalism), dst, false, fused, st, u.copies,
+                                       u.edges);
+  if (e == cudaSuccess && fused) acc_zeroed(c, u);
   if (e == cudaSuccess && clear && !fused) e = zero_acc(c, st);
   return e;
 }
