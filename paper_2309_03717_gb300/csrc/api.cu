@@ -347,14 +347,16 @@ void form_apply(c8r_ctx* c) {
                   ? 1
                   : 0;
 }
-void form_poll(c8r_ctx* c) {
+// `st`: the stream of the launch to come (an event may not be queried while it is
+// captured, which would end the capture: the counts then wait for a later push)
+void form_poll(c8r_ctx* c, cudaStream_t st) {
   if (c->form_mode != C8R_FORM_AUTO) {
     c->split = c->form_mode == C8R_FORM_SPLIT;
     form_apply(c);
     return;
   }
   form_apply(c);
-  if (!c->form_pending) return;
+  if (!c->form_pending || capturing(st)) return;
   const cudaError_t q = cudaEventQuery(c->ev_form);
   if (q == cudaErrorNotReady) {
     if (cudaPeekAtLastError() == cudaErrorNotReady) cudaGetLastError();
@@ -778,7 +780,7 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
   const int64_t chunk = n < c->chunk_tracks ? n : c->chunk_tracks;
   if ((r = ensure_tiles(c, chunk)) != C8R_OK) return r;
   const bool lin = c->deposit == C8R_DEPOSIT_LINEAR;
-  form_poll(c);
+  form_poll(c, st);
   FwdShape shape = c->shape;  // of this push: its antenna tile and the accumulator copies it uses
   if (c->user_a_tile == 0)
     shape.a_tile = push_a_tile(shape.a_tile, (chunk + kTileT - 1) / kTileT, c->n_ant, c->precision, c->formalism,
@@ -945,7 +947,7 @@ int c8r_stats(c8r_ctx* c, c8r_stats_t* out) {
   out->pairs = (int64_t)kept * c->n_ant;
   // the stream has drained: the votes' copy, if one was made, has landed
   if (c->form_pending) cudaEventSynchronize(c->ev_form);
-  form_poll(c);
+  form_poll(c, c->last_stream);
   out->arrival_form = c->split ? C8R_FORM_SPLIT : C8R_FORM_DIRECT;
   if (err != kErrNone) {
     cudaMemset(c->d_err, 0, sizeof(int));
@@ -1024,7 +1026,7 @@ int c8r_backward(c8r_ctx* c, const c8r_tracks* t, int64_t n, const void* grad_tr
     if (e == cudaSuccess && prefix) e = launch_bin_running_sums(c->d_gbm, c->n_ant, c->n_bins, c->d_gpre, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "gradient layout");
   }
-  form_poll(c);
+  form_poll(c, st);
   for (int64_t off = 0; off < n; off += chunk) {
     const int64_t m = (n - off) < chunk ? (n - off) : chunk;
     cudaError_t e = launch_ingest(c->precision, offset_tracks(t, off), m, c->d_tiles, c->M, nullptr, st);

@@ -120,7 +120,6 @@ def test_captured_pushes_and_fetches(formalism, precision):
     many = to_device(synth.make_tracks(60_000, 5, 0.0), dtype)
     few = {f: x[:500].contiguous() for f, x in many.items()}
     p = RadioProcess(synth.AIR_EXPONENTIAL, ant, synth.trace_start_ns(ant), 1000, 0.5, formalism, precision)
-    p.set_arrival_form("split")  # (the automatic form reads its counts back with an event query)
     out = torch.empty((2, 3, 1000), dtype=dtype, device="cuda")
     # a fetch captured before anything was pushed
     torch.cuda.synchronize()
