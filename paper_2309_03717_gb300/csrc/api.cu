@@ -114,7 +114,7 @@ void fill_antenna(AntRec& r, double x, double y, double z, double t_ref_ns, cons
   const double kff = M.kind == C8R_UNIFORM ? (double)M.s_h + (double)M.s_l : (double)M.kc_h + (double)M.kc_l;
   const double Ta = t_ref_ns / M.dt_ns + kff * z;
   split(Ta, r.Tah, r.Tal);
-  // error-bound constants of the FP32 arrival (arrival_bin_fast): twice the
+  // error-bound constants of the FP32 arrival (arrival_fast): twice the
   // bins per metre (n/(c dt), or (1 + N0)/(c dt) as an upper bound for the
   // exponential medium) times the neglected low part of the position, 16 u^2
   // |T_a| (u = 2^-24) for the float-float shifted times, and a floor of 1e-6

@@ -73,7 +73,7 @@ struct AntRec {
   float xh, yh, zh, xl, yl, zl;  // position as float-float
   float tauh, taul;              // t_ref / dt as float-float
   float Eah, Eal;                // Ea as float-float
-  // constants of the error bound of the FP32 arrival (arrival_bin_fast):
+  // constants of the error bound of the FP32 arrival (arrival_fast):
   // fb_abs = 2 x bins per metre x |low part of the position| + 16 u^2 |T_a| +
   // 1e-6 bin, and fb_rel_v = |z_l| / (1e-3 H), the relative error of the
   // refractivity term from the low part of the altitude (exponential medium;
@@ -135,7 +135,7 @@ struct MedParams {
 // approximate operations (2 ulp), with denormal arguments taken as zero.  The
 // plain rsqrtf, __fdividef and __expf cover denormals too and execute 4, 5 and
 // about 4 instructions for it, against 1, 2 and 2 here (counted on this part);
-// on normal arguments the values are the same, bit for bit (2^24 random pairs).
+// on normal arguments the values are the same, bit for bit (test_gpu_helpers).
 // No argument here is denormal: distances are above 1e-19 m, and what divides
 // is a distance, a product of distances or an altitude difference above
 // 1e-3 H.  A pair has two such roots and eight quotients (Endpoint), so the

@@ -15,8 +15,8 @@
 // L2-resident accumulator [antenna][bin][x, y, z, 0] with one native vector
 // reduction (atomicAdd on float4; three FP64 reductions in the FP64 path); a
 // constant run of bins (ZHS) is added as its two edges into a second row that
-// the fetch integrates.  The mixed accumulator has 1 to 16 copies (CTA range r
-// adds into copy r % copies, acc_replicas) that the fetch sums.  Shared-memory
+// the fetch integrates.  The accumulator has 1 to 16 copies (CTA range r adds into
+// copy r % copies, acc_replicas) that the fetch sums.  Shared-memory
 // float atomics are not used: they stall the issuing warp, while the global
 // reductions are fire-and-forget.
 #pragma once
@@ -78,7 +78,7 @@ struct AccOf<double> {
 };
 
 // CTA -> (antenna tile, track range).  Antenna tiles are grouped into blocks
-// whose accumulators fit comfortably in L2; inside a block the antenna tile
+// whose accumulator rows stay within kAccBudget; inside a block the antenna tile
 // varies fastest, so CTAs resident together read the same track range (L2
 // reuse of the track tiles) and add into a bounded set of accumulator rows.
 struct FwdGrid {

@@ -561,7 +561,7 @@ struct OpsMixed {
   static constexpr bool kDefers = FORM == C8R_ENDPOINT;
   // Endpoint with the one-bin deposit in the plain straight-line media: the
   // main pass takes each bin from the FP32 arrival with its error bound
-  // (arrival_bin_fast) and sets aside only the endpoints it cannot decide,
+  // (arrival_fast, decide_bins) and sets aside only the endpoints it cannot decide,
   // for the float-float arrival after the main pass
   static constexpr bool kFastBins =
       FORM == C8R_ENDPOINT && !LIN && (KIND == C8R_UNIFORM || KIND == C8R_EXPONENTIAL);
@@ -1100,7 +1100,7 @@ struct OpsMixed {
   // A near-Cherenkov pair (kFastBins) whose two linearised arrivals
   // u_m -/+ D_m (t1 - t0)/(2 dt) lie in one bin, or both before or both after
   // the window, contributes exactly 0 (reading C), and so does its adjoint.
-  // Decided here from FP32 midpoint geometry, as arrival_bin_fast decides a
+  // Decided here from FP32 midpoint geometry, as decide_bins decides a
   // bin: the midpoint d_m = (s0 + s1)/2 from the endpoints' FP32 d (the
   // float-float path's high part; its roundings move each component by at most
   // 2u |s_i| + u L_i / 2, which moves x = R - w by at most 6u x + u L1 / 2, so
