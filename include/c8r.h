@@ -184,9 +184,10 @@ int c8r_set_medium_spherical(c8r_ctx* ctx, double N0, double scale_height_m, dou
  * ZHS keeps a second row per antenna (box edges), and 1 to 16 copies of the whole
  * accumulator are kept, more for fewer antennas (up to 192 MB and a quarter of the
  * device's free memory in all), which the fetch sums; a push uses as many of them
- * as its tracks pay for.  FP64 ZHS allocates box edges of the accumulator's size at
- * the first push that has a use for them (one-bin deposit in the uniform or flat
- * exponential medium) where a quarter of the free memory holds them.  Replaces any previous antenna set and discards its
+ * as its tracks pay for.  FP64 ZHS with the one-bin deposit in the uniform or flat
+ * exponential medium allocates box edges of the accumulator's size where a quarter
+ * of the free memory holds them (here, or at the first push that has a use for
+ * them when the medium or the deposit is set later).  Replaces any previous antenna set and discards its
  * traces (a call with the same
  * n_ant, n_bins, dt_ns, formalism and precision keeps the device memory and
  * only replaces the table, so moving an array between steps is cheap).  EINVAL on n_ant < 1,

@@ -360,12 +360,12 @@ class RadioProcess:
         self.formalism = formalism
         self.medium = dict(medium)
         self._apply_medium()
+        c8r_set_deposit(self.ctx, _DEPOSIT[deposit])  # (the accumulator's memory depends on both)
+        self.deposit = deposit
         c8r_set_antennas(self.ctx, self.ant_xyz, self.t_start_ns, n_bins, dt_ns, _FORMALISM[formalism],
                          _PRECISION[precision])
         if eps_C is not None:
             c8r_set_cherenkov_threshold(self.ctx, eps_C)
-        c8r_set_deposit(self.ctx, _DEPOSIT[deposit])
-        self.deposit = deposit
 
     def _apply_medium(self):
         m = self.medium

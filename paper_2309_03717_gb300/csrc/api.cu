@@ -420,6 +420,12 @@ cudaError_t zero_acc(c8r_ctx* c, cudaStream_t st) {
   return e;
 }
 
+// whether a push adds boxes into an accumulator that keeps their edges apart
+bool has_boxes(const c8r_ctx* c) {
+  return c->precision == C8R_FP64 && c->formalism == C8R_ZHS && c->deposit == C8R_DEPOSIT_BIN &&
+         (c->med_kind == C8R_UNIFORM || c->med_kind == C8R_EXPONENTIAL);
+}
+
 // whether a push on st can add boxes by their edges: they take as much memory as
 // the accumulator, which on a device that is nearly full (a quarter of what is free,
 // as for its copies) the traces do not need.  Not from the middle of a capture, nor
@@ -739,6 +745,7 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   c->pushed = 0;
   cudaMemset(c->d_kept, 0, sizeof(unsigned long long));
   form_reset(c);
+  if (c->medium_set && has_boxes(c)) ensure_edges(c, nullptr);  // (or by the first push that wants them: 60 us there)
   return rebuild_tables(c);
 }
 
@@ -786,10 +793,8 @@ int c8r_push_tracks(c8r_ctx* c, const c8r_tracks* t, int64_t n, void* stream) {
     shape.a_tile = push_a_tile(shape.a_tile, (chunk + kTileT - 1) / kTileT, c->n_ant, c->precision, c->formalism,
                                c->sm_count);
   const int floor_copies = c->floor_copies < shape.replicas ? c->floor_copies : shape.replicas;
-  const bool boxes = c->precision == C8R_FP64 && c->formalism == C8R_ZHS && !lin &&
-                     (c->med_kind == C8R_UNIFORM || c->med_kind == C8R_EXPONENTIAL);
   int rows = acc_rows(c->precision, c->formalism);
-  if (boxes && ensure_edges(c, st)) {
+  if (has_boxes(c) && ensure_edges(c, st)) {
     rows = 2;
     shape.edge_off = (static_cast<char*>(c->d_edges) - static_cast<char*>(c->d_acc)) /
                      (int64_t)acc_elem_bytes(C8R_FP64);

@@ -1,7 +1,9 @@
 // pair_f64.cuh -- per (track, antenna) arithmetic of the FP64 path: the plain
 // formulas of the two formalisms (§1) and the straight-line propagator (§2) in
 // FP64, in the order of their definitions (one exception: the ZHS factor
-// K_A/(R |D_m| dt) is formed once per interval rather than once per bin).  This
+// K_A/(R |D_m| dt) is formed once per interval rather than once per bin), and for
+// the one-bin deposit in the plain media with fewer and fused operations
+// (OpsF64Plain, which the adjoint's geometry and bins are taken from).  This
 // translation unit is compiled without FMA contraction so that every operation
 // rounds as written.
 #pragma once

@@ -38,6 +38,8 @@ def launched(work, kernel):
         work()
         torch.cuda.synchronize()
     names = [e.name for e in prof.events()]
+    if not names:
+        pytest.skip("the profiler records no kernels here")
     forms = set()
     for n in names:
         m = re.search(kernel + r"<c8r::OpsMixed<[^>]*>", n)
