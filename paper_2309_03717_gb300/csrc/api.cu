@@ -973,6 +973,7 @@ int c8r_arrivals(c8r_ctx* c, const c8r_tracks* t, int64_t n, int32_t* branch, in
   c->last_stream = st;
   const int64_t chunk = n < c->chunk_tracks ? n : c->chunk_tracks;
   if ((r = ensure_tiles(c, chunk)) != C8R_OK) return r;
+  form_poll(c, st);
   for (int64_t off = 0; off < n; off += chunk) {
     const int64_t m = (n - off) < chunk ? (n - off) : chunk;
     const int64_t j0 = off * c->n_ant;

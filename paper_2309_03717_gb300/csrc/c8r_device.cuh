@@ -1033,7 +1033,9 @@ using FieldM = FieldT<float>;
 // Every step uses explicit-rounding intrinsics so the forward and the adjoint
 // kernels, which inline this in different contexts, take identical branch
 // decisions.
-template <typename T>
+// FUSED: D's last product and sum as one operation (pairs only), see mul_apart and
+// OpsMixed::kFusedD.
+template <typename T, bool FUSED = false>
 __device__ __forceinline__ void field_mixed(const GeoT<T>& g, T bx, T by, T bz, T bmag, T om_nb, T n, FieldT<T>& f) {
   const T sx = g.s[0], sy = g.s[1], sz = g.s[2];
   // w = d x beta from the FP32 part of d (the low parts, ~2^-24 |d|, change D by
@@ -1046,7 +1048,10 @@ __device__ __forceinline__ void field_mixed(const GeoT<T>& g, T bx, T by, T bz, 
   const T invR = g.y;
   const T w2 = fma_rn(wx, wx, fma_rn(wy, wy, mul_rn(wz, wz)));
   const T den = mul_rn(R, fma_rn(bmag, R, bd));
-  f.D = add_rn(om_nb, mul_apart(mul_rn(n, w2), rcp_ap(den)));
+  if constexpr (FUSED)
+    f.D = fma_rn(mul_rn(n, w2), rcp_ap(den), om_nb);
+  else
+    f.D = add_rn(om_nb, mul_apart(mul_rn(n, w2), rcp_ap(den)));
   if constexpr (!kUsualForm<T>)
     if (!(bd >= 0.0f)) f.D = __fsub_rn(1.0f, __fmul_rn(__fmul_rn(n, bd), invR));
   // d x w = d (d.beta) - beta R^2  ->  V R^2

@@ -441,13 +441,11 @@ cudaError_t launch_arrivals_mixed(int formalism, const void* tiles, int64_t n, c
     k_arrivals<decltype(ops)><<<blocks, 256, 0, st>>>(tiles, n, ants, n_ant, M, branch, bin, frac);
     return cudaGetLastError();
   };
-  // the kernels of forward_mixed (the arrival form and an Endpoint's flat array
-  // change nothing that is listed)
+  // the kernels of forward_mixed
   if (formalism == C8R_ENDPOINT) {
     if (M.kind == C8R_EXPONENTIAL_RAY) return go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_RAY>{});
     if (M.kind == C8R_EXPONENTIAL_SPHERICAL) return go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL_SPHERICAL>{});
-    return M.kind == C8R_EXPONENTIAL ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>{})
-                                     : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
+    return with_endpoint_ops(M, go);
   }
   if (M.flat) {
     if (M.kind == C8R_EXPONENTIAL_RAY)

@@ -585,6 +585,12 @@ struct OpsMixed {
   // showers in a batch 2.99 -> 2.96 ms.  ZHS, one track per thread, 2e7-track
   // vertical shower: 31.96 -> 29.56 ms, and 28.50 with the z part as well
   static constexpr bool kFlat = FLAT && KIND != C8R_UNIFORM && (kFastBins || FORM == C8R_ZHS);
+  // the main pass's Doppler factor with its last product and sum fused: in the
+  // direct and axis kernels without a per-pair quotient, where the assembler had made
+  // them one operation; apart in the others, as in the plain arithmetic.  Either is
+  // within a rounding, but the near-Cherenkov decision is taken from it, so each
+  // kernel states which it has: its forward pass, adjoint and listing agree
+  static constexpr bool kFusedD = kFastBins && AF != kFormSplit && (KIND == C8R_UNIFORM || FLAT);
   // adjoint CTAs (128 threads) per SM the registers are set for (the linear
   // Endpoint adjoint carries the slide of each deposit as well)
   static constexpr int kBwdMinBlocks = (LIN && FORM == C8R_ENDPOINT) ? 4 : (kFastBins ? 5 : 6);
@@ -1030,7 +1036,8 @@ struct OpsMixed {
     else if constexpr (KIND == C8R_EXPONENTIAL)
       q = fast_quotient(M, A.Eh, A.El, g.s[2], t.Eh, t.El);
     float2 eps = arrival_fast<KIND, kAF>(M, g, S, P, t.Th, t.Tl, A.Th, A.Tl, A.fb_abs, A.fb_rel_v, q, 0.0f, uf);
-    field_mixed(g, bc<float2>(t.bx), bc<float2>(t.by), bc<float2>(t.bz), bc<float2>(t.bmag), t.om, t.n, f);
+    field_mixed<float2, kFusedD>(g, bc<float2>(t.bx), bc<float2>(t.by), bc<float2>(t.bz), bc<float2>(t.bmag), t.om,
+                                 t.n, f);
     // the usual forms: bd >= 0 (the Doppler factor); an altitude difference
     // beyond 1e-3 H, tested at 1.001e-3 H so that no rounding lets one through
     // (the refractivity quotient); an emission point above the antenna (the
@@ -1903,6 +1910,24 @@ struct OpsMixed {
 
 #undef TF
 
+// The one-bin Endpoint kernels of the plain media come in the arrival forms (M.axis,
+// M.split) and, in the exponential medium, for a flat antenna array (M.flat,
+// OpsMixed::kFlat)
+template <class F>
+cudaError_t with_endpoint_ops(const MedParams& M, F go) {
+  if (M.kind != C8R_EXPONENTIAL)
+    return M.axis    ? go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>{})
+           : M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{})
+                     : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
+  if (M.flat)
+    return M.axis    ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis, true>{})
+           : M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit, true>{})
+                     : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{});
+  return M.axis    ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis>{})
+         : M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{})
+                   : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>{});
+}
+
 // forward and adjoint launches for one deposit shape (one-bin, or linear in a
 // translation unit of its own so that the two compile in parallel)
 template <bool LIN>
@@ -1928,24 +1953,7 @@ cudaError_t forward_mixed(int formalism, const void* tiles, int64_t n_tiles, con
            : M.flat                  ? go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, LIN, kFormDirect, true>{})
                                      : go(OpsMixed<C8R_ZHS, C8R_EXPONENTIAL_RAY, LIN>{});
   if constexpr (!LIN) {
-    // the one-bin Endpoint kernels come in the arrival forms (M.axis, M.split)
-    // and, in the exponential medium, for a flat antenna array (M.flat,
-    // OpsMixed::kFlat)
-    if (formalism == C8R_ENDPOINT) {
-      if (M.axis) {
-        if (!ex) return go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>{});
-        return M.flat ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis, true>{})
-                      : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis>{});
-      }
-      if (!ex)
-        return M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{})
-                       : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM>{});
-      if (M.split)
-        return M.flat ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit, true>{})
-                      : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{});
-      return M.flat ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{})
-                    : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL>{});
-    }
+    if (formalism == C8R_ENDPOINT) return with_endpoint_ops(M, go);
   }
   if (formalism == C8R_ENDPOINT)
     return ex ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, LIN>{}) : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, LIN>{});
@@ -1965,19 +1973,8 @@ cudaError_t backward_mixed(int formalism, BwdArgs& a, const FwdShape& shape, int
     return ex ? launch_backward_ops<OpsMixed<C8R_ZHS, C8R_EXPONENTIAL, LIN>>(a, shape, sm_count, st)
               : launch_backward_ops<OpsMixed<C8R_ZHS, C8R_UNIFORM, LIN>>(a, shape, sm_count, st);
   }
-  if constexpr (!LIN) {
-    auto go = [&](auto ops) { return launch_backward_ops<decltype(ops)>(a, shape, sm_count, st); };
-    if (ex && a.M.flat)
-      return a.M.axis    ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis, true>{})
-             : a.M.split ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit, true>{})
-                         : go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormDirect, true>{});
-    if (a.M.axis)
-      return ex ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormAxis>{})
-                : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormAxis>{});
-    if (a.M.split)
-      return ex ? go(OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, false, kFormSplit>{})
-                : go(OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, false, kFormSplit>{});
-  }
+  if constexpr (!LIN)
+    return with_endpoint_ops(a.M, [&](auto ops) { return launch_backward_ops<decltype(ops)>(a, shape, sm_count, st); });
   return ex ? launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_EXPONENTIAL, LIN>>(a, shape, sm_count, st)
             : launch_backward_ops<OpsMixed<C8R_ENDPOINT, C8R_UNIFORM, LIN>>(a, shape, sm_count, st);
 }
