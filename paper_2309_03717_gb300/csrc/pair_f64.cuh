@@ -390,6 +390,7 @@ struct OpsF64 {
       if (!Plain::eval(tr.t, tr.t.p[0], A, M, e)) return;
       typename Plain::Interval v;
       Plain::interval(tr.t, e, N, v);
+      if (v.one && v.lo.bin < 0) return;  // (also NaN: out of FP64's range)
       Plain::geometry(tr.t.p[0], A, e, gm);
       c = e.c;
       Dm = e.D;
@@ -668,7 +669,7 @@ struct OpsF64 {
       typename Plain::Eval em;
       typename Plain::Near v;
       if (!Plain::near_arrivals(tr.t, T, l, A, M, pm, em, v)) return;
-      if (v.a.k == v.b.k) return;
+      if (v.a.k == v.b.k || (v.a.bin < 0 && v.b.bin < 0)) return;  // (also NaN, as in adj_zhs)
       double gv[3];
       for (int cc = 0; cc < 3; ++cc)
         gv[cc] = (v.a.bin >= 0 ? (&G[v.a.bin].x)[cc] : 0.0) - (v.b.bin >= 0 ? (&G[v.b.bin].x)[cc] : 0.0);

@@ -26,7 +26,8 @@ def gradients(p, tracks, G):
     n = len(tracks["x0"])
     dev = to_device(tracks)
     p.push(dev)
-    tg = {f: torch.zeros(n, dtype=torch.float32, device="cuda") for f in c8r.GRAD_FIELDS}
+    gdt = torch.float64 if p.precision == "fp64" else torch.float32
+    tg = {f: torch.zeros(n, dtype=gdt, device="cuda") for f in c8r.GRAD_FIELDS}
     ag = torch.zeros((p.n_ant, 3), dtype=torch.float64, device="cuda")
     dn = torch.zeros(1, dtype=torch.float64, device="cuda")
     c8r.c8r_backward(p.ctx, dev, G, tg, ag, dn)
@@ -109,3 +110,31 @@ def test_fp64_emission_point_whose_distance_overflows(hills, formalism, medium):
         p.close()
     assert np.abs(out[0]).max() > 0 and np.isfinite(out[1]).all()
     assert np.abs(out[1] - out[0]).max() <= 1e-12 * np.abs(out[0]).max()
+
+
+@pytest.mark.parametrize("medium", [synth.AIR_EXPONENTIAL, UNIFORM])
+@pytest.mark.parametrize("formalism", ["endpoint", "zhs"])
+@pytest.mark.parametrize("precision,far", [("fp64", 1.0e200), ("mixed", 1.0e25)])
+def test_adjoint_of_emission_points_out_of_range(precision, far, formalism, medium):
+    """Tracks whose squared distance overflows pass the filter and have no part in
+    any gradient: as with those tracks dropped, to the order of the additions (FP32:
+    200 of them; FP64: 1e-12)."""
+    from paper_2309_03717_gb300 import c8r
+    dtype = np.float64 if precision == "fp64" else np.float32
+    tracks = {f: x.astype(dtype) for f, x in synth.make_tracks(200, 31, 0.0).items()}
+    ant = synth.antennas_star(8, n_radii=2)[:9].copy()
+    G = torch.from_numpy(np.random.default_rng(3).normal(size=(len(ant), 3, 1024)).astype(dtype)).cuda()
+    out = []
+    for dropped in (True, False):
+        t = {f: x.copy() for f, x in tracks.items()}
+        if dropped:
+            t["q"][::7] = 0.0
+        else:
+            t["x0"][::7] = far
+            t["x1"][::7] = 1.1 * far
+        p = c8r.RadioProcess(medium, ant, synth.trace_start_ns(ant, 0.0), 1024, 0.2, formalism, precision)
+        out.append(gradients(p, t, G))
+    for f in out[0]:
+        assert np.isfinite(out[1][f]).all(), f
+        tol = 1e-12 if precision == "fp64" else 200 * 2.0 ** -24
+        assert np.abs(out[1][f] - out[0][f]).max() <= tol * np.abs(out[0][f]).max(), f
