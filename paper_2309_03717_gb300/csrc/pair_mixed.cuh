@@ -1126,10 +1126,6 @@ struct OpsMixed {
       const float x1 = TF(fm::X1), y1 = TF(fm::Y1), z1 = TF(fm::Z1);
       const float a0x = __fadd_rn(A.xh, -x0), a0y = __fadd_rn(A.yh, -y0), a0z = __fadd_rn(A.zh, -z0);
       const float a1x = __fadd_rn(A.xh, -x1), a1y = __fadd_rn(A.yh, -y1), a1z = __fadd_rn(A.zh, -z1);
-      // (adjoint) an endpoint on the antenna: not this form
-      if constexpr (ADJ) {
-        if (on_antenna(a0x, a0y, a0z) || on_antenna(a1x, a1y, a1z)) return false;
-      }
       GeoM g;
       g.s[0] = 0.5f * __fadd_rn(a0x, a1x);
       g.s[1] = 0.5f * __fadd_rn(a0y, a1y);
@@ -1141,6 +1137,10 @@ struct OpsMixed {
       g.R1 = 0.0f;
       if (g.R0 == 0.0f) return true;  // the midpoint on the antenna: no deposit
       const float L1 = fabsf(__fsub_rn(a0x, a1x)) + fabsf(__fsub_rn(a0y, a1y)) + fabsf(__fsub_rn(a0z, a1z));
+      // (adjoint) an endpoint on the antenna, at half the track's length from the
+      // midpoint: not this form
+      if constexpr (ADJ)
+        if (g.R0 <= L1) return false;
       const float bx = TF(fm::BX), by = TF(fm::BY), bz = TF(fm::BZ), bmag = TF(fm::BMAG);
       float Eh = 1.0f, El = 0.0f, nm1 = M.nm1f;
       if (KIND != C8R_UNIFORM) {
@@ -1434,11 +1434,6 @@ struct OpsMixed {
     dn = __fmaf_rn(dns.y, t.Eh.y, __fmaf_rn(dns.x, t.Eh.x, dn));
   }
 
-  // a squared distance of zero, also from components whose squares are denormal
-  static __device__ __forceinline__ bool on_antenna(float x, float y, float z) {
-    constexpr float none = 1.1e-19f;
-    return fabsf(x) < none && fabsf(y) < none && fabsf(z) < none;
-  }
   // of a pair that the adjoint's main pass set aside whole: the one endpoint with a
   // geometry where the other has none and that one is not near the Cherenkov angle
   // (kDeferEnd0 or kDeferEnd1), or 0
