@@ -270,9 +270,11 @@ struct c8r_ctx {
   // (copies_replayed) count as used for good, and a captured fetch or reset takes
   // every copy, whatever the pushes before its replays will have used
   int copies_used = 1, copies_replayed = 1;
-  // FP64 ZHS: box edges, [copies][n_ant][n_bins], from the first push with boxes on
-  // where there is room, and whether they may hold any (as copies_used)
+  // FP64 ZHS: box edges, [copies][n_ant][n_bins], where there is room: behind the
+  // accumulator in its allocation (edges_behind), or in one of their own from the
+  // first push with boxes on; and whether they may hold any (as copies_used)
   void* d_edges = nullptr;
+  bool edges_behind = false;
   bool edges_used = false, edges_refused = false;
   bool edges_replayed = false;   // by captured pushes
   bool fetch_captured = false;   // (or a reset) on the present accumulator
@@ -414,8 +416,13 @@ void acc_zeroed(c8r_ctx* c, const InUse& u) {
 cudaError_t zero_acc(c8r_ctx* c, cudaStream_t st) {
   const InUse u = acc_in_use(c, st);
   const size_t bytes = c->acc_bytes / c->shape.replicas * u.copies;
-  cudaError_t e = cudaMemsetAsync(c->d_acc, 0, bytes, st);
-  if (e == cudaSuccess && u.edges) e = cudaMemsetAsync(u.edges, 0, bytes, st);
+  cudaError_t e;
+  if (u.edges && c->edges_behind) {
+    e = cudaMemset2DAsync(c->d_acc, c->acc_bytes, 0, bytes, 2, st);  // one launch for both
+  } else {
+    e = cudaMemsetAsync(c->d_acc, 0, bytes, st);
+    if (e == cudaSuccess && u.edges) e = cudaMemsetAsync(u.edges, 0, bytes, st);
+  }
   if (e == cudaSuccess) acc_zeroed(c, u);
   return e;
 }
@@ -426,15 +433,25 @@ bool has_boxes(const c8r_ctx* c) {
          (c->med_kind == C8R_UNIFORM || c->med_kind == C8R_EXPONENTIAL);
 }
 
-// whether a push on st can add boxes by their edges: they take as much memory as
-// the accumulator, which on a device that is nearly full (a quarter of what is free,
-// as for its copies) the traces do not need.  Not from the middle of a capture, nor
-// once a captured fetch may be about that knows nothing of them
+// room for box edges: they take as much memory as the accumulator, which on a device
+// that is nearly full (a quarter of what is free, as for its copies) the traces do
+// not need
+bool room_for_edges(size_t bytes) {
+  size_t mem_free = 0, mem_total = 0;
+  if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return bytes <= mem_free / 4;
+}
+
+// whether a push on st can add boxes by their edges.  They are not allocated from the
+// middle of a capture, nor once a captured fetch may be about that knows nothing of
+// them
 bool ensure_edges(c8r_ctx* c, cudaStream_t st) {
   if (c->d_edges || c->edges_refused || c->fetch_captured || capturing(st)) return c->d_edges != nullptr;
-  size_t mem_free = 0, mem_total = 0;
-  cudaError_t e = cudaMemGetInfo(&mem_free, &mem_total);
-  if (e == cudaSuccess && c->acc_bytes <= mem_free / 4) e = dev_malloc(&c->d_edges, c->acc_bytes);
+  cudaError_t e = cudaSuccess;
+  if (room_for_edges(c->acc_bytes)) e = dev_malloc(&c->d_edges, c->acc_bytes);
   if (e == cudaSuccess && c->d_edges) e = cudaMemsetAsync(c->d_edges, 0, c->acc_bytes, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -483,9 +500,9 @@ int rebuild_tables(c8r_ctx* c) {
 void free_antenna_state(c8r_ctx* c) {
   if (c->d_ants) cudaFree(c->d_ants);
   if (c->d_acc) cudaFree(c->d_acc);
-  if (c->d_edges) cudaFree(c->d_edges);
+  if (c->d_edges && !c->edges_behind) cudaFree(c->d_edges);
   c->d_edges = nullptr;
-  c->edges_used = c->edges_refused = c->edges_replayed = c->fetch_captured = false;
+  c->edges_behind = c->edges_used = c->edges_refused = c->edges_replayed = c->fetch_captured = false;
   if (c->d_stage) cudaFree(c->d_stage);
   if (c->d_gbm) cudaFree(c->d_gbm);
   c->d_gbm = nullptr;
@@ -734,8 +751,17 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   c->acc_bytes *= c->shape.replicas;
   c->copies_used = c->copies_replayed = 1;
   cudaError_t e = dev_malloc(&c->d_ants, sizeof(AntRec) * n_ant);
-  if (e == cudaSuccess) e = dev_malloc(&c->d_acc, c->acc_bytes);
-  if (e == cudaSuccess) e = cudaMemset(c->d_acc, 0, c->acc_bytes);
+  // with boxes to come, the edges behind the accumulator (one launch zeroes both);
+  // set to have them later, the first push that wants them allocates them
+  const bool boxes = c->medium_set && has_boxes(c);
+  if (e == cudaSuccess && boxes) {
+    c->edges_behind = room_for_edges(c->acc_bytes) && dev_malloc(&c->d_acc, 2 * c->acc_bytes) == cudaSuccess;
+    c->edges_refused = !c->edges_behind;
+    cudaGetLastError();
+    if (c->edges_behind) c->d_edges = static_cast<char*>(c->d_acc) + c->acc_bytes;
+  }
+  if (e == cudaSuccess && !c->edges_behind) e = dev_malloc(&c->d_acc, c->acc_bytes);
+  if (e == cudaSuccess) e = cudaMemset(c->d_acc, 0, c->acc_bytes * (c->edges_behind ? 2 : 1));
   if (e != cudaSuccess) {
     cudaGetLastError();
     free_antenna_state(c);
@@ -745,7 +771,6 @@ int c8r_set_antennas(c8r_ctx* c, int32_t n_ant, const double* pos, const double*
   c->pushed = 0;
   cudaMemset(c->d_kept, 0, sizeof(unsigned long long));
   form_reset(c);
-  if (c->medium_set && has_boxes(c)) ensure_edges(c, nullptr);  // (or by the first push that wants them: 60 us there)
   return rebuild_tables(c);
 }
 

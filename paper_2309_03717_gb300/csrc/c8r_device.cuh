@@ -234,6 +234,13 @@ __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
   const T bb = sub_rn(s, a);
   e = add_rn(sub_rn(a, sub_rn(s, bb)), sub_rn(b, bb));
 }
+// a - b exactly: the negated operand keeps a packed product b out of fused sums
+template <typename T>
+__device__ __forceinline__ void two_diff(T a, T b, T& s, T& e) {
+  s = sub_rn(a, b);
+  const T bb = sub_rn(s, a);
+  e = sub_rn(sub_rn(a, sub_rn(s, bb)), add_rn(b, bb));
+}
 template <typename T>
 __device__ __forceinline__ void two_prod(T a, T b, T& p, T& e) {
   p = mul_rn(a, b);
@@ -1121,7 +1128,7 @@ __device__ __forceinline__ ffT<T> doppler_ff(const GeoT<T>& g, T bx, T by, T p2,
   const T ql = mul_rn(r, g.y);
   // n q = q + (n - 1) q, then D = 1 - n q
   T nh, nl;
-  two_sum(qh, mul_apart(nm1, qh), nh, nl);
+  two_diff(qh, mul_rn(neg(nm1), qh), nh, nl);
   nl = add_rn(nl, ql);
   T dh, dl;
   two_sum(bc<T>(1.0f), neg(nh), dh, dl);

@@ -28,9 +28,10 @@ size_t tile_bytes(int precision);
 inline size_t acc_elem_bytes(int precision) { return precision == C8R_FP64 ? 32 : 16; }
 // accumulator rows per antenna, box edges included (ZHS)
 inline int acc_rows(int formalism) { return formalism == C8R_ZHS ? 2 : 1; }
-// and of the accumulator itself: the FP64 path keeps the edges apart, in memory
-// allocated for pushes with boxes where there is room (only the one-bin deposit of
-// the plain media has boxes; without the edges they go in bin by bin)
+// and of the accumulator itself: the FP64 path keeps the edges apart, behind the
+// accumulator or in memory of their own, where there is room for them (only the
+// one-bin deposit of the plain media has boxes; without the edges they go in bin by
+// bin)
 inline int acc_rows(int precision, int formalism) { return precision == C8R_MIXED ? acc_rows(formalism) : 1; }
 // copies of the accumulator the forward kernel spreads its reductions over (CTA
 // range r adds into copy r % replicas; the fetch sums them).  Most reductions go

@@ -68,16 +68,16 @@ def test_fp64_zhs_without_room_for_the_edges(n_ant, late):
     ref = reference(synth.AIR_EXPONENTIAL, ant, n_bins, tracks)
     dev = to_device(tracks)
     try:
-        # the context's counters and error word, the antenna table and the
-        # accumulator, then the edges; in another medium first, the edges after a
-        # push's scratch
+        # the context's counters and error word, the antenna table, then the
+        # accumulator with its edges (and, that failing, without); in another medium
+        # first, the edges after a push's scratch
         if late:
             p = process(SPHERE, ant, n_bins)
             p.medium = dict(synth.AIR_EXPONENTIAL)
             p._apply_medium()
             c8r.c8r_inject_alloc_failures(1, 1)
         else:
-            c8r.c8r_inject_alloc_failures(4, 1)
+            c8r.c8r_inject_alloc_failures(3, 1)
             p = process(synth.AIR_EXPONENTIAL, ant, n_bins)
         p.push(dev)
     finally:
