@@ -290,6 +290,13 @@ int c8r_reset(c8r_ctx* ctx, void* cuda_stream);
 int c8r_backward(c8r_ctx* ctx, const c8r_tracks* tracks, int64_t n, const void* grad_traces,
                  const c8r_track_grads* out_tracks, double* out_ant_grad, double* out_dN0, void* cuda_stream);
 
+/* Zero the outputs of c8r_backward (the same pointers, for n tracks and the
+ * context's antennas) in one launch, for a caller who wants the gradients alone and
+ * not their sum with what was there.  EINVAL on a NULL pointer, n < 0 or a dtype that
+ * does not match the context; n == 0 zeroes the antenna and N0 gradients only. */
+int c8r_zero_gradients(c8r_ctx* ctx, const c8r_track_grads* out_tracks, int64_t n, double* out_ant_grad,
+                       double* out_dN0, void* cuda_stream);
+
 /* Kernel timing.  While enabled, every ingest and pair-kernel launch of
  * c8r_push_tracks is bracketed by CUDA events recorded on the launching stream.
  * c8r_profile_read synchronises and returns the summed device time (ms) and the

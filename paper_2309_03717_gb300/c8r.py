@@ -93,6 +93,7 @@ _SIGNATURES = [
     ("c8r_reset", ctypes.c_int, [_P, _P]),
     ("c8r_backward", ctypes.c_int, [_P, ctypes.POINTER(c8r_tracks), ctypes.c_int64, _P,
                                     ctypes.POINTER(c8r_track_grads), _P, _P, _P]),
+    ("c8r_zero_gradients", ctypes.c_int, [_P, ctypes.POINTER(c8r_track_grads), ctypes.c_int64, _P, _P, _P]),
     ("c8r_stats", ctypes.c_int, [_P, ctypes.POINTER(c8r_stats_t)]),
     ("c8r_profile", ctypes.c_int, [_P, ctypes.c_int]),
     ("c8r_profile_read", ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int64),
@@ -271,20 +272,31 @@ def c8r_arrivals(ctx, tracks: dict, n_ant: int, stream=None):
     return br, b, fr
 
 
+def _grads_struct(track_grads, n, ant_grad, dN0):
+    ts = [track_grads[f] for f in GRAD_FIELDS]
+    dt = ts[0].dtype
+    for t in ts:
+        if t.dtype != dt or t.numel() != n or not t.is_cuda or not t.is_contiguous():
+            raise ValueError("gradient arrays must be contiguous CUDA tensors matching the tracks")
+    if ant_grad.dtype != torch.float64 or dN0.dtype != torch.float64:
+        raise ValueError("ant_grad and dN0 are float64")
+    return c8r_track_grads(C8R_F64 if dt == torch.float64 else C8R_F32, *[t.data_ptr() for t in ts])
+
+
+def c8r_zero_gradients(ctx, track_grads: dict, ant_grad: torch.Tensor, dN0: torch.Tensor, stream=None):
+    """Zero the outputs of c8r_backward in one launch (ant_grad for the context's antennas)."""
+    n = track_grads["x0"].numel()
+    if not ant_grad.is_contiguous():
+        raise ValueError("ant_grad must be contiguous")
+    g = _grads_struct(track_grads, n, ant_grad, dN0)
+    return _check(ctx, load().c8r_zero_gradients(ctx, ctypes.byref(g), n, _ptr(ant_grad), _ptr(dN0), _stream(stream)))
+
+
 def c8r_backward(ctx, tracks: dict, grad_traces: torch.Tensor, track_grads: dict, ant_grad: torch.Tensor,
                  dN0: torch.Tensor, stream=None):
     s = tracks_struct(tracks)
     n = tracks["x0"].numel()
-    g = c8r_track_grads()
-    dt = track_grads["x0"].dtype
-    g.dtype = C8R_F64 if dt == torch.float64 else C8R_F32
-    for f in GRAD_FIELDS:
-        t = track_grads[f]
-        if t.dtype != dt or t.numel() != n or not t.is_cuda or not t.is_contiguous():
-            raise ValueError("gradient arrays must be contiguous CUDA tensors matching the tracks")
-        setattr(g, f, t.data_ptr())
-    if ant_grad.dtype != torch.float64 or dN0.dtype != torch.float64:
-        raise ValueError("ant_grad and dN0 are float64")
+    g = _grads_struct(track_grads, n, ant_grad, dN0)
     return _check(ctx, load().c8r_backward(ctx, ctypes.byref(s), n, _ptr(grad_traces.contiguous()),
                                            ctypes.byref(g), _ptr(ant_grad), _ptr(dN0), _stream(stream)))
 
@@ -481,18 +493,13 @@ class RadioTraces(torch.autograd.Function):
         process = ctx.process
         gdt = torch.float64 if process.precision == "fp64" else torch.float32
         n = tracks["x0"].numel()
-        # every gradient a tensor of its own, zeroed by one launch per element type (a
-        # fill per gradient is what a small step would wait for: 5000 tracks x 13
-        # antennas 485 us per step, with a fill each 600)
+        # every gradient a tensor of its own, all zeroed by one launch (a fill per
+        # gradient is what a small step would wait for: 5000 tracks x 13 antennas 485 us
+        # per step, with a fill each 600)
         tg = {f: torch.empty(n, dtype=gdt, device=process.device) for f in GRAD_FIELDS}
         ag = torch.empty((process.n_ant, 3), dtype=torch.float64, device=process.device)
         dn = torch.empty((), dtype=torch.float64, device=process.device)
-        sums = [ag, dn]
-        if gdt == torch.float64:
-            sums += tg.values()
-        else:
-            torch._foreach_zero_(list(tg.values()))
-        torch._foreach_zero_(sums)
+        c8r_zero_gradients(process.ctx, tg, ag, dn)
         g = grad_out.to(process.trace_dtype).contiguous()
         c8r_backward(process.ctx, tracks, g, tg, ag, dn)
         grads = [tg[f].to(tracks[f].dtype) for f in GRAD_FIELDS] + [torch.zeros_like(tracks["q"])]
