@@ -175,9 +175,10 @@ __device__ __forceinline__ float exp_ap(float x) {
 // (counted on this part), while the FP32 pipe's rate per value stays the same.
 // One exception, whatever -fmad says: the assembler makes one fused operation of
 // a packed product that goes into packed sums only, which it never does with the
-// plain ones.  Where such a sum decides a bin or a branch that other kernels form from
-// plain values, mul_apart keeps the product rounded: two plain multiplications, an
-// issue slot more.
+// plain ones.  Where such a sum decides a bin or a branch that other kernels form
+// from plain values, the product is kept rounded: as two plain multiplications
+// (mul_apart, an issue slot more), or with its sign turned (two_diff, none);
+// test_gpu_bin_edges holds the outcome.
 // The pair kernels are bound by issue, so the per-pair arithmetic is written
 // once for T = float or float2 and the main passes run it on pairs: a pair's
 // two endpoints (Endpoint).  Comparisons and the approximate reciprocals take
